@@ -53,7 +53,11 @@ typedef enum {
   FRLAP_ETIMEOUT = 8     /* a bounded device-side wait expired */
 } frlap_status;
 
-/* Arithmetic of the FFT apply.  F64: IEEE double everywhere.  F32: single
+/* Arithmetic of the FFT apply.  F64: IEEE double vectors and symbol; the transforms
+ * run in 64-bit fixed point with one exponent per line (58 bits below a line's
+ * largest value, against a double's 53), which GB300's integer pipes do several
+ * times faster than its FP64 pipe.  Vectors of any finite scale; a non-finite
+ * entry makes the whole product NaN.  F32: single
  * precision FFT stages and symbol.  MIXED: a plan that holds both, so
  * that the iterative-refinement solver can run FP32 inner applies and FP64
  * outer residuals (coefficients and symbol are always generated in FP64).
@@ -241,12 +245,8 @@ frlap_status frlap_pcg_solve(const frlap_plan* plan, const double* d_f, double* 
                              void* stream);
 
 /* r = f - A x and ||r||_2 / ||f||_2 in FP64: the true relative residual that decides frlap_pcg_solve's
- * convergence (the paper solves its systems by CG, Sec. 5.3), with the same apply.  F64 and MIXED plans: the native FP64 apply.
- * Double-float plans: forward transforms and symbol product in FP64, inverse transforms in
- * double-float.  The forward transforms' rounding reaches A x multiplied by up to lambda_max, the
- * inverse ones' only relative to A x itself; so near a solution (||A x|| far below lambda_max ||x||)
- * this is as accurate as native FP64 and about 1.7x faster (2D plans with a 16384-point y embedding
- * use native FP64).  Far from a solution it is as accurate as the double-float apply.
+ * convergence (the paper solves its systems by CG, Sec. 5.3), with the same apply: the FP64 engine,
+ * on double-float plans too.
  * d_f, d_x: device FP64 vectors of the plan's unknowns (x-fastest); d_r: device, the residual, or NULL
  * for the norm only (must not overlap d_f or d_x); d_work: frlap_workspace_bytes(plan, FRLAP_OP_PCG).
  * Synchronises `stream` to return *relres.  FRLAP_EINVAL: NULL plan, d_f, d_x or relres, an F32 plan,
@@ -385,7 +385,7 @@ frlap_status frlap_allen_cahn_batch(int nbatch, const frlap_plan* const* plans, 
  * time-out path.  The paper has no counterpart. */
 frlap_status frlap_set_loop_pass_limit(unsigned max_passes);
 
-/* The first apply stage of the FP64 and double-float engines stages its input rows in shared
+/* The first apply stage of the double-float engine stages its input rows in shared
  * memory by bulk asynchronous copies and waits for each on an mbarrier.  Every such wait is
  * bounded (about a second); a wait that gives up is counted, and that kernel returns without
  * storing its remaining tiles (the call's result is then wrong).  frlap_async_wait_report returns

@@ -102,11 +102,9 @@ frlap_status frlap_async_wait_report(unsigned long long* timeouts) {
     FRLAP_CUDA_TRY(fn(&c));
     total += c;
   }
-  for (auto fn : {dft16_wait_collect, hyb_wait_collect}) {
-    unsigned long long c = 0ull;
-    FRLAP_CUDA_TRY(fn(&c));
-    total += c;
-  }
+  unsigned long long cd = 0ull;
+  FRLAP_CUDA_TRY(dft16_wait_collect(&cd));
+  total += cd;
   *timeouts = total;
   return FRLAP_OK;
 }
@@ -136,8 +134,8 @@ frlap_status frlap_bounds_check_report(int* enabled, unsigned long long* violati
                                        unsigned long long* first_address) {
   if (!violations) return fail(FRLAP_EINVAL, "violations is NULL");
   unsigned long long total = 0ull, first = ~0ull;
-  cudaError_t (*collect[4])(unsigned long long*, unsigned long long*) = {bc_collect<float>, bc_collect<double>,
-                                                                         bc_collect<dfl>, hyb_bc_collect};
+  cudaError_t (*collect[3])(unsigned long long*, unsigned long long*) = {bc_collect<float>, bc_collect<double>,
+                                                                         bc_collect<dfl>};
   for (auto fn : collect) {
     unsigned long long c = 0ull, f = ~0ull;
     FRLAP_CUDA_TRY(fn(&c, &f));
@@ -209,6 +207,7 @@ frlap_status frlap_plan_destroy(frlap_plan* plan) {
     cudaFree(plan->tw64[r]);
     cudaFree(plan->tw32[r]);
     cudaFree(plan->twdf[r]);
+    cudaFree(plan->twq[r]);
   }
   if (plan->side) cudaStreamDestroy(plan->side);
   delete plan;
@@ -285,6 +284,12 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
       return cleanup(FRLAP_ENOMEM, "plan allocation failed");
     cudaError_t e = twiddle_launch(p->P[r], p->tw64[r], p->tw32[r], s);
     if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
+    if (prec != FRLAP_F32) {
+      if (cudaMalloc(&p->twq[r], ntw * sizeof(int4)) != cudaSuccess)
+        return cleanup(FRLAP_ENOMEM, "plan allocation failed");
+      e = to_q_launch(p->tw64[r], p->twq[r], (size_t)ntw, s);
+      if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
+    }
     if (p->df64) {
       if (cudaMalloc(&p->twdf[r], ntw * sizeof(cdf)) != cudaSuccess)
         return cleanup(FRLAP_ENOMEM, "plan allocation failed");

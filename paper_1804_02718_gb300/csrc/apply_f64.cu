@@ -1,7 +1,6 @@
-// FP64 instances of the FFT apply and of the spectrum transforms used by the learned
-// preconditioner (kernels and launchers in apply_impl.cuh), plus the engine-independent
-// entry points.
-#include "apply_impl.cuh"
+// The FP64 engine's apply and the spectrum transforms of the learned preconditioner (kernels and launchers in
+// apply_q.cuh, dispatch in apply_impl.cuh), plus the engine-independent entry points.
+#include "apply_q.cuh"
 
 namespace frlap {
 
@@ -13,6 +12,7 @@ size_t apply_work_bytes(const Plan& p, int real_bytes) {
   const size_t cb = 2 * (size_t)real_bytes;
   size_t b = align256(p.s1_elems * cb);
   b += align256(p.s2_elems * cb);
+  if (real_bytes == 8) b += q_exp_layout(p).total * sizeof(int);  // the FP64 engine's exponents
   return b;
 }
 
@@ -31,10 +31,6 @@ size_t spectrum_elems(const Plan& p) {
   const size_t Hx1 = p.P[0] / 2 + 1;
   return (p.d == 2) ? Hx1 * p.P[1] : Hx1 * p.P[1] * p.P[2];
 }
-
-template cudaError_t spectrum_forward<double>(const Plan&, const double*, double2*, void*, cudaStream_t);
-template cudaError_t spectrum_inverse<double>(const Plan&, const double2*, const double*, double*, void*,
-                                              cudaStream_t);
 
 template cudaError_t autotune_engine<double>(Plan&, int, double*, double*, void*, cudaStream_t);
 

@@ -14,8 +14,8 @@
 // Every stage reads and writes whole contiguous lines or TL-wide contiguous
 // tiles; every global index below is bounded by the line/tile validity tests.
 //
-// This header holds the kernel and launcher templates; apply_f32.cu, apply_f64.cu and
-// apply_dfl.cu instantiate them per engine (three translation units, built in parallel).
+// This header holds the kernel and launcher templates; apply_f32.cu and apply_dfl.cu instantiate them, one
+// translation unit per engine.  The FP64 engine has kernels of its own (apply_q.cuh, apply_f64.cu).
 #pragma once
 
 #include <type_traits>
@@ -207,13 +207,13 @@ template <typename T>
 constexpr bool kFusedSplitC2R = std::is_same<T, float>::value;
 
 // The first stage runs as the persistent k_r2c_pf (its input rows' loads overlap the previous
-// tile's arithmetic) in the FP64 and double-float engines for transforms of up to 1024 points,
-// as measured: double-float 255^3 r2c 235 -> 221 us per 2-vector launch, while the 2048-point
+// tile's arithmetic) in the double-float engine for transforms of up to 1024 points,
+// as measured: 255^3 r2c 235 -> 221 us per 2-vector launch, while the 2048-point
 // rows of 2047^2 keep k_r2c_T (71 against 77 us per vector).  FP32 keeps k_r2c_T everywhere: its
 // first stage is bound by shared-memory and store throughput, not load latency (persistent form
 // at 255^3: 44.7 -> 51.0 us per launch; at 2047^2: 21.3 -> 21.0 us per vector).  -1: never.
 template <typename T>
-constexpr int kR2CPersistentMaxLogH = std::is_same<T, float>::value ? -1 : 10;
+constexpr int kR2CPersistentMaxLogH = std::is_same<T, dfl>::value ? 10 : -1;
 template <typename T>
 inline bool use_r2c_pf(int logH, const void* u) {
   return logH <= kR2CPersistentMaxLogH<T> && (reinterpret_cast<uintptr_t>(u) % sizeof(io_t<T>)) == 0;
@@ -766,55 +766,6 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_colmul(cplx<T>* __restrict__ 
   else store_line(v, data, ncols, n, ld, logP, TL);
 }
 
-// The middle stage of the residual apply of double-float plans (apply_launch_b<double, dfl>): the
-// forward transform and the symbol product in FP64, then each value split into a double-float pair
-// and the inverse transform in double-float.  The column is read as FP64 and written back in place
-// as double-float (16 bytes per complex value either way).  Rounding in the forward transform
-// reaches the product multiplied by up to lambda_max, so that transform keeps FP64; the inverse
-// transform's rounding is relative to the product itself, where double-float's 2^-48 suffices.
-template <int REM>
-__global__ void __launch_bounds__(kMaxCta<double>, 1)
-    k_colmul_hyb(double2* __restrict__ data, int ncols, int n, size_t ld, int logP, int TL,
-                 const double* __restrict__ lam, LamMap map, const double2* __restrict__ tw64,
-                 const cdf* __restrict__ twdf, const int* __restrict__ skip, Batch bt) {
-  {
-    const size_t bi = blockIdx.y;
-    data += bi * bt.in;
-    lam += bi * bt.lam;
-    if (skip) skip += bi * bt.skip;
-  }
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  double2* smem = reinterpret_cast<double2*>(smem_raw);
-  if (skip && FRLAP_GLD(skip)) return;
-  const int P = 1 << logP, G = P >> 4;
-  const int l = threadIdx.x / G, lane = threadIdx.x % G;
-  const int col = blockIdx.x * TL + l;
-  const bool valid = col < ncols;
-  double2* buf = smem + (size_t)l * sline(P);
-  const double2* line = data + (size_t)(valid ? col : 0) * ld;
-  double2 v[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int i = lane + m * G;
-    v[m] = (m < 8 && valid && i < n) ? ld_stream(&line[i]) : czero<double2>();
-  }
-  fft_regs<double, -1, true, REM>(v, buf, logP, lane, tw64, logP, false);
-  const int c = valid ? col : 0;
-  const double* __restrict__ lrow =
-      map.d == 2 ? lam + (size_t)c * map.Hy1
-                 : lam + ((size_t)(c >> map.logPy) * map.Hy1 + min(c & (map.Py - 1), map.Py - (c & (map.Py - 1)))) *
-                             map.Hz1;
-  cdf w[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int k = lane + m * G;
-    const double2 t = ld_stream(&lrow[min(k, P - k)]) * v[m];
-    w[m] = make_cdf(df_from(t.x), df_from(t.y));
-  }
-  fft_regs<dfl, 1, false, REM>(w, reinterpret_cast<cdf*>(buf), logP, lane, twdf, logP, true);
-  store_line(w, reinterpret_cast<cdf*>(data), ncols, n, ld, logP, TL);
-}
-
 // groups of contiguous lines of length n -> pad, FFT, transposed store out[g][k][line]
 template <typename T, int REM, int LOGL = 0, bool ODD = false>
 __global__ void __launch_bounds__(kMaxCta<T>, 1) k_c2cT_fwd(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, int nlines, int tiles, int n,
@@ -931,68 +882,6 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_c2cT_inv(const cplx<T>* __res
   }
 }
 
-
-// lines of length n (stride ld) -> zero-pad to P, forward FFT, write all P outputs (stride ldo)
-template <typename T>
-__global__ void __launch_bounds__(kMaxCta<T>, 1)
-    k_col_fwd(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, int ncols, int n, size_t ld, size_t ldo,
-              int logP, int TL, const cplx<T>* __restrict__ tw, int logPtab) {
-  using C = cplx<T>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* smem = reinterpret_cast<C*>(smem_raw);
-  const int P = 1 << logP, G = P >> 4;
-  const int l = threadIdx.x / G, lane = threadIdx.x % G;
-  const int col = blockIdx.x * TL + l;
-  const bool valid = col < ncols;
-  C* buf = smem + (size_t)l * sline(P);
-  const C* src = in + (size_t)(valid ? col : 0) * ld;
-  load_line<C>(buf, src, lane, G, n, valid);
-  __syncthreads();
-  fft_line<T, -1, true, false>(buf, logP, lane, tw, logPtab);
-  if (valid) {
-    C* dst = out + (size_t)col * ldo;
-    for (int i = lane; i < P; i += G) FRLAP_GST(dst + i, buf[spad(i)]);
-  }
-}
-
-// lines of P spectrum values (stride ld) -> * multiplier, inverse FFT, crop to n, write (stride ldo)
-template <typename T>
-__global__ void __launch_bounds__(kMaxCta<T>, 1)
-    k_col_mulinv(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, int ncols, int n, size_t ld, size_t ldo,
-                 int logP, int TL, const T* __restrict__ lam, LamMap map, const cplx<T>* __restrict__ tw,
-                 int logPtab) {
-  using C = cplx<T>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* smem = reinterpret_cast<C*>(smem_raw);
-  const int P = 1 << logP, G = P >> 4;
-  const int l = threadIdx.x / G, lane = threadIdx.x % G;
-  const int col = blockIdx.x * TL + l;
-  const bool valid = col < ncols;
-  C* buf = smem + (size_t)l * sline(P);
-  const C* src = in + (size_t)(valid ? col : 0) * ld;
-  // the multiplier is in natural octant order here (it comes from the learning kernels)
-  size_t lam_base;
-  int lam_stride;
-  if (map.d == 2) {
-    lam_base = valid ? col : 0;
-    lam_stride = map.Hx1;
-  } else {
-    const int c = valid ? col : 0;
-    const int kx = c >> map.logPy, ky = c & (map.Py - 1);
-    lam_base = (size_t)min(ky, map.Py - ky) * map.Hx1 + kx;
-    lam_stride = map.Hy1 * map.Hx1;
-  }
-  for (int k = lane; k < P; k += G) {
-    const int kf = min(k, P - k);
-    buf[spad(k)] = valid ? FRLAP_GLD(lam + lam_base + (size_t)kf * lam_stride) * FRLAP_GLD(src + k) : czero<C>();
-  }
-  __syncthreads();
-  fft_line<T, 1, false, true>(buf, logP, lane, tw, logPtab);
-  if (valid) {
-    C* dst = out + (size_t)col * ldo;
-    for (int i = lane; i < n; i += G) FRLAP_GST(dst + i, buf[spad(i)]);
-  }
-}
 
 // Lines per CTA for a line of `len` complex slots: as many as fit in
 // `budget` bytes of shared memory and 256 threads (at least one), rounded down to a
@@ -1128,36 +1017,22 @@ cudaError_t launch_r2c_pf(const io_t<T>* u, cplx<T>* S1, int nrows, int nx, size
   }
 }
 
-// The hybrid middle stage (k_colmul_hyb), one instance per REM; a template so that only the
-// translation unit that runs it compiles it.
-template <int UNUSED = 0>
-cudaError_t launch_colmul_hyb(double2* data, int ncols, int n, size_t ld, int logP, int tl, const double* lam,
-                              LamMap map, const double2* tw64, const cdf* twdf, const int* skip, Batch b, int grid,
-                              int B, size_t sm, cudaStream_t s) {
-  const int G = 1 << (logP - 4);
-  return with_rem(logP, [&](auto tag) {
-    constexpr int REM = decltype(tag)::value;
-    cudaError_t e = set_smem(k_colmul_hyb<REM>, sm);
-    if (e != cudaSuccess) return e;
-    k_colmul_hyb<REM><<<dim3(grid, B), tl * G, sm, s>>>(data, ncols, n, ld, logP, tl, lam, map, tw64, twdf, skip, b);
-    return cudaGetLastError();
-  });
-}
+// The same in the FP64 engine (apply_q.cuh), which only its own translation unit compiles.
+template <typename T>
+cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstride, void* work, cudaStream_t s,
+                             const int* skip, int skip_stride, cudaEvent_t const* ev, const T* lam_override,
+                             size_t lam_stride);
 
-// TI: the engine of the inverse transforms (the last stage, the 3D inverse y stage and the middle
-// stage's inverse half); TI = T but for the residual apply of double-float plans, <double, dfl>
-// (k_colmul_hyb), which plans with the split middle stage do not take.
-template <typename T, typename TI = T>
-static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<TI>* y, size_t vstride, void* work,
+template <typename T>
+static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T>* y, size_t vstride, void* work,
                                   cudaStream_t s, const int* skip, int skip_stride, cudaEvent_t const* ev,
                                   const T* lam_override, size_t lam_stride, bool odd = false) {
-  constexpr bool kHyb = !std::is_same<T, TI>::value;
-  static_assert(!kHyb || (std::is_same<T, double>::value && std::is_same<TI, dfl>::value),
-                "apply_launch_b: the only mixed form is FP64 forward, double-float inverse");
-  if (kHyb && (odd || (p.d == 2 && p.P[1] > kMaxLine))) return cudaErrorNotSupported;
   // odd: the pipeline on odd extensions (a multiplier in the sine basis, see k_r2c_T); the FP32
   // engine only, P_r = 2(n_r + 1) on every axis (the callers check)
   if (odd && (!std::is_same<T, float>::value || p.P[1] > kMaxLine)) return cudaErrorNotSupported;
+  if constexpr (std::is_same<T, double>::value) {
+    return q_apply_launch_b<T>(p, B, u, y, vstride, work, s, skip, skip_stride, ev, lam_override, lam_stride);
+  } else {
   int stage = 0;
   auto mark = [&]() -> cudaError_t {
     if (ev && ev[stage]) {
@@ -1173,11 +1048,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
   const int* tuned = p.tl_tuned[engine_index<T>()];
   const C* tw[3];
   for (int r = 0; r < 3; ++r) tw[r] = twiddle_table<T>(p, r);
-  using CI = cplx<TI>;
-  static_assert(sizeof(CI) == sizeof(C), "apply_launch_b: both engines keep the same bytes per value");
-  const int* tunedI = p.tl_tuned[engine_index<TI>()];
-  const CI* twI[3];
-  for (int r = 0; r < 3; ++r) twI[r] = twiddle_table<TI>(p, r);
   const T* lam = lam_override ? lam_override : symbol_table<T>(p);
   C* S1 = reinterpret_cast<C*>(work);
   C* S2 = reinterpret_cast<C*>(reinterpret_cast<unsigned char*>(work) + align256(p.s1_elems * eb));
@@ -1197,8 +1067,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
     r.add(work, (size_t)B * apply_work_bytes(p, sizeof(T)));
     r.add(lam, ((size_t)(B - 1) * lam_stride + p.lam_count) * sizeof(T));
     for (int a = 0; a < p.d; ++a) r.add(tw[a], (size_t)twiddle_entries(p.P[a]) * sizeof(C));
-    if (kHyb)
-      for (int a = 0; a < p.d; ++a) r.add(twI[a], (size_t)twiddle_entries(p.P[a]) * sizeof(CI));
     if (skip) r.add(skip, ((size_t)(B - 1) * skip_stride + 1) * sizeof(int));
     cudaError_t e = r.commit(s);
     if (e != cudaSuccess) return e;
@@ -1275,17 +1143,13 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
     Batch b_split = b_ws;  // columns in S1, the even half in S2 (same per-instance stride)
     cudaError_t e;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (kHyb) {
-      return cudaErrorNotSupported;  // refused above; no split instances in the hybrid's unit
-    } else {
-      if ((e = set_smem(k_colmul_split<T, false>, sm)) != cudaSuccess) return e;
-      if ((e = set_smem(k_colmul_split<T, true>, sm)) != cudaSuccess) return e;
-      k_colmul_split<T, false><<<dim3(grid, B), tl * G, sm, s>>>(S1, S2, ncols, ny, ld1, tl, lam, map.Hy1, tw[1],
-                                                                skip, b_split);
-      k_colmul_split<T, true><<<dim3(grid, B), tl * G, sm, s>>>(S1, S2, ncols, ny, ld1, tl, lam, map.Hy1, tw[1],
-                                                               skip, b_split);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    if ((e = set_smem(k_colmul_split<T, false>, sm)) != cudaSuccess) return e;
+    if ((e = set_smem(k_colmul_split<T, true>, sm)) != cudaSuccess) return e;
+    k_colmul_split<T, false><<<dim3(grid, B), tl * G, sm, s>>>(S1, S2, ncols, ny, ld1, tl, lam, map.Hy1, tw[1],
+                                                              skip, b_split);
+    k_colmul_split<T, true><<<dim3(grid, B), tl * G, sm, s>>>(S1, S2, ncols, ny, ld1, tl, lam, map.Hy1, tw[1],
+                                                             skip, b_split);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   } else if (p.d == 2) {
     const int G = p.P[1] >> 4;
     const int tl = pick_tl_tuned(tuned[1], sline(p.P[1]), eb, G, budget, (long long)(Hx + 1) * B);
@@ -1294,11 +1158,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
     const int ncols = Hx + 1;
     const int grid = (ncols + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (kHyb) {
-      e = launch_colmul_hyb(reinterpret_cast<double2*>(S1), ncols, ny, ld1, logPy, tl,
-                            reinterpret_cast<const double*>(lam), map, reinterpret_cast<const double2*>(tw[1]),
-                            reinterpret_cast<const cdf*>(twI[1]), skip, b_ws, grid, B, sm, s);
-    } else {
     if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPy, [&](auto tag) {
@@ -1318,7 +1177,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
         k_colmul<T, REM, LP><<<dim3(grid, B), tl * G, sm, s>>>(S1, ncols, ny, ld1, logPy, tl, lam, map, tw[1], logPy, skip, b_ws);
         return cudaGetLastError();
       });
-    }
     if (e != cudaSuccess) return e;
   } else {
     const int Py = p.P[1], Pz = p.P[2];
@@ -1362,11 +1220,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
       const int ncols = (Hx + 1) * Py;
       const int grid = (ncols + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (kHyb) {
-      e = launch_colmul_hyb(reinterpret_cast<double2*>(S2), ncols, nz, (size_t)nz, logPz, tl,
-                            reinterpret_cast<const double*>(lam), map, reinterpret_cast<const double2*>(tw[2]),
-                            reinterpret_cast<const cdf*>(twI[2]), skip, b_ws, grid, B, sm, s);
-    } else {
     if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPz, [&](auto tag) {
@@ -1386,74 +1239,71 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
       k_colmul<T, REM, LP><<<dim3(grid, B), tl * G, sm, s>>>(S2, ncols, nz, (size_t)nz, logPz, tl, lam, map, tw[2], logPz, skip, b_ws);
       return cudaGetLastError();
     });
-    }
     if (e != cudaSuccess) return e;
     }
-    // ---- stage 4: S2[kx][ky][z] -> IFFT_y -> S1[kx][z][y] (engine TI)
+    // ---- stage 4: S2[kx][ky][z] -> IFFT_y -> S1[kx][z][y]
     {
-      CI* S1i = reinterpret_cast<CI*>(S1);
-      CI* S2i = reinterpret_cast<CI*>(S2);
       const int G = Py >> 4;
-      const int tl = pick_tl_tuned(tunedI[3], sline(Py), eb, G, budget, (long long)nz * (Hx + 1) * B);
+      const int tl = pick_tl_tuned(tuned[3], sline(Py), eb, G, budget, (long long)nz * (Hx + 1) * B);
       const size_t sm = (size_t)tl * sline(Py) * eb;
       cudaError_t e;
       const int tiles = (nz + tl - 1) / tl;
       const int grid = (Hx + 1) * tiles;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<TI, float>::value) {
+    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPy, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
-          cudaError_t e2 = set_smem(k_c2cT_inv<TI, REM, 0, true>, sm);
+          cudaError_t e2 = set_smem(k_c2cT_inv<T, REM, 0, true>, sm);
           if (e2 != cudaSuccess) return e2;
-          k_c2cT_inv<TI, REM, 0, true><<<dim3(grid, B), tl * G, sm, s>>>(S2i, S1i, nz, tiles, ny, (size_t)Py * nz, nz,
-                                                                          (size_t)nz * ny, ny, logPy, tl, twI[1], logPy,
+          k_c2cT_inv<T, REM, 0, true><<<dim3(grid, B), tl * G, sm, s>>>(S2, S1, nz, tiles, ny, (size_t)Py * nz, nz,
+                                                                          (size_t)nz * ny, ny, logPy, tl, tw[1], logPy,
                                                                           skip, b_ws);
           return cudaGetLastError();
         });
     }
     if (!odd)
-    e = with_line_shape<TI, std::is_same<TI, float>::value>(logPy, [&](auto tag) {
+    e = with_line_shape<T, std::is_same<T, float>::value>(logPy, [&](auto tag) {
       constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
-      cudaError_t e2 = set_smem(k_c2cT_inv<TI, REM, LL>, sm);
+      cudaError_t e2 = set_smem(k_c2cT_inv<T, REM, LL>, sm);
       if (e2 != cudaSuccess) return e2;
-      k_c2cT_inv<TI, REM, LL><<<dim3(grid, B), tl * G, sm, s>>>(S2i, S1i, nz, tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, logPy, tl, twI[1], logPy, skip, b_ws);
+      k_c2cT_inv<T, REM, LL><<<dim3(grid, B), tl * G, sm, s>>>(S2, S1, nz, tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, logPy, tl, tw[1], logPy, skip, b_ws);
       return cudaGetLastError();
     });
     if (e != cudaSuccess) return e;
     }
   }
-  // ---- last stage: S1[kx][row] -> rows of y (engine TI)
+  // ---- last stage: S1[kx][row] -> rows of y 
   {
-    const CI* S1i = reinterpret_cast<const CI*>(S1);
     const int G = Hx >> 4;
-    const int tl = pick_tl_tuned(tunedI[p.d == 2 ? 2 : 4], sline(Hx), eb, G, budget, (long long)nrows * B);
+    const int tl = pick_tl_tuned(tuned[p.d == 2 ? 2 : 4], sline(Hx), eb, G, budget, (long long)nrows * B);
     const size_t sm = (size_t)tl * sline(Hx) * eb;
     cudaError_t e;
     const int grid = (nrows + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<TI, float>::value) {
+    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPx - 1, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
-          cudaError_t e2 = set_smem(k_c2r_T<TI, REM, 0, true>, sm);
+          cudaError_t e2 = set_smem(k_c2r_T<T, REM, 0, true>, sm);
           if (e2 != cudaSuccess) return e2;
-          k_c2r_T<TI, REM, 0, true><<<dim3(grid, B), tl * G, sm, s>>>(S1i, y, nrows, nx, ld1, nx, logPx - 1, tl, twI[0],
+          k_c2r_T<T, REM, 0, true><<<dim3(grid, B), tl * G, sm, s>>>(S1, y, nrows, nx, ld1, nx, logPx - 1, tl, tw[0],
                                                                        logPx, skip, b_out);
           return cudaGetLastError();
         });
     }
     if (!odd)
-      e = with_line_shape<TI, std::is_same<TI, float>::value>(logPx - 1, [&](auto tag) {
+      e = with_line_shape<T, std::is_same<T, float>::value>(logPx - 1, [&](auto tag) {
         constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
-        cudaError_t e2 = set_smem(k_c2r_T<TI, REM, LL>, sm);
+        cudaError_t e2 = set_smem(k_c2r_T<T, REM, LL>, sm);
         if (e2 != cudaSuccess) return e2;
-        k_c2r_T<TI, REM, LL><<<dim3(grid, B), tl * G, sm, s>>>(S1i, y, nrows, nx, ld1, nx, logPx - 1, tl, twI[0], logPx, skip, b_out);
+        k_c2r_T<T, REM, LL><<<dim3(grid, B), tl * G, sm, s>>>(S1, y, nrows, nx, ld1, nx, logPx - 1, tl, tw[0], logPx, skip, b_out);
         return cudaGetLastError();
       });
     if (e != cudaSuccess) return e;
   }
   return mark();
+  }
 }
 
 template <typename T>
@@ -1468,158 +1318,6 @@ cudaError_t apply_batch_launch(const Plan& p, int B, const io_t<T>* u, io_t<T>* 
                                cudaEvent_t const* ev) {
   return apply_launch_b<T>(p, B, u, y, vstride, work, s, skip, skip_stride, ev, lam, lam_stride);
 }
-
-// SP = F R^T u on the half spectrum: 2D [kx][ky], 3D [kx][ky][kz] (kx <= P_x/2, full ky, kz).
-template <typename T>
-cudaError_t spectrum_forward(const Plan& p, const T* u, cplx<T>* SP, void* work, cudaStream_t s) {
-  using C = cplx<T>;
-  const int eb = sizeof(C);
-  const int budget = 96 * 1024;
-  const C* tw[3];
-  for (int r = 0; r < 3; ++r) tw[r] = twiddle_table<T>(p, r);
-#ifdef FRLAP_BOUNDS_CHECK
-  {
-    BcRanges r;
-    r.add(u, p.M * sizeof(T));
-    r.add(SP, spectrum_elems(p) * sizeof(C));
-    r.add(work, apply_work_bytes(p, sizeof(T)));
-    for (int a = 0; a < p.d; ++a) r.add(tw[a], (size_t)twiddle_entries(p.P[a]) * sizeof(C));
-    cudaError_t e = r.commit(s);
-    if (e != cudaSuccess) return e;
-  }
-#endif
-  C* S1 = reinterpret_cast<C*>(work);
-  C* S2 = reinterpret_cast<C*>(reinterpret_cast<unsigned char*>(work) + align256(p.s1_elems * eb));
-  const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
-  const int Hx = p.P[0] / 2;
-  const int nrows = ny * (p.d == 3 ? nz : 1);
-  cudaError_t e;
-  {
-    const int G = Hx >> 4;
-    const int tl = pick_tl(sline(Hx), eb, G, budget, 64);
-    const size_t sm = (size_t)tl * r2c_line_stride<T>(Hx, tl) * eb;
-    e = with_rem(p.logP[0] - 1, [&](auto tag) {
-      constexpr int REM = decltype(tag)::value;
-      cudaError_t e2 = set_smem(k_r2c_T<T, REM>, sm);
-      if (e2 != cudaSuccess) return e2;
-      k_r2c_T<T, REM><<<(nrows + tl - 1) / tl, tl * G, sm, s>>>(u, S1, nrows, nx, nx, (size_t)nrows, p.logP[0] - 1, tl, tw[0], p.logP[0], nullptr, Batch{});
-      return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-  }
-  const C* lines = S1;
-  int ncols = Hx + 1, n = ny, logP = p.logP[1];
-  size_t ld = (size_t)nrows;
-  const C* twl = tw[1];
-  if (p.d == 3) {
-    const int Py = p.P[1];
-    const int G = Py >> 4;
-    const int tl = pick_tl(sline(Py), eb, G, budget, 64);
-    const size_t sm = (size_t)tl * sline(Py) * eb;
-    const int tiles = (nz + tl - 1) / tl;
-    e = with_rem(p.logP[1], [&](auto tag) {
-      constexpr int REM = decltype(tag)::value;
-      cudaError_t e2 = set_smem(k_c2cT_fwd<T, REM>, sm);
-      if (e2 != cudaSuccess) return e2;
-      k_c2cT_fwd<T, REM><<<(Hx + 1) * tiles, tl * G, sm, s>>>(S1, S2, nz, tiles, ny, (size_t)nz * ny, ny, (size_t)Py * nz, nz, p.logP[1], tl, tw[1], p.logP[1], nullptr, Batch{});
-      return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-    lines = S2;
-    ncols = (Hx + 1) * Py;
-    n = nz;
-    ld = (size_t)nz;
-    logP = p.logP[2];
-    twl = tw[2];
-  }
-  const int P = 1 << logP;
-  const int G = P >> 4;
-  const int tl = pick_tl(sline(P), eb, G, budget, 64);
-  const size_t sm = (size_t)tl * sline(P) * eb;
-  if ((e = set_smem(k_col_fwd<T>, sm)) != cudaSuccess) return e;
-  k_col_fwd<T><<<(ncols + tl - 1) / tl, tl * G, sm, s>>>(lines, SP, ncols, n, ld, (size_t)P, logP, tl, twl, logP);
-  return cudaGetLastError();
-}
-
-// y = R F^-1 (mult * SP), mult = a symbol octant with the 1/prod(P) factor folded in.
-template <typename T>
-cudaError_t spectrum_inverse(const Plan& p, const cplx<T>* SP, const T* mult, T* y, void* work, cudaStream_t s) {
-  using C = cplx<T>;
-  const int eb = sizeof(C);
-  const int budget = 96 * 1024;
-  const C* tw[3];
-  for (int r = 0; r < 3; ++r) tw[r] = twiddle_table<T>(p, r);
-#ifdef FRLAP_BOUNDS_CHECK
-  {
-    BcRanges r;
-    r.add(SP, spectrum_elems(p) * sizeof(C));
-    r.add(mult, p.lam_count * sizeof(T));
-    r.add(y, p.M * sizeof(T));
-    r.add(work, apply_work_bytes(p, sizeof(T)));
-    for (int a = 0; a < p.d; ++a) r.add(tw[a], (size_t)twiddle_entries(p.P[a]) * sizeof(C));
-    cudaError_t e = r.commit(s);
-    if (e != cudaSuccess) return e;
-  }
-#endif
-  C* S1 = reinterpret_cast<C*>(work);
-  C* S2 = reinterpret_cast<C*>(reinterpret_cast<unsigned char*>(work) + align256(p.s1_elems * eb));
-  const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
-  const int Hx = p.P[0] / 2;
-  const int nrows = ny * (p.d == 3 ? nz : 1);
-  LamMap map;
-  map.d = p.d;
-  map.Hx1 = Hx + 1;
-  map.logPy = p.logP[1];
-  map.Py = p.P[1];
-  map.Hy1 = p.P[1] / 2 + 1;
-  map.Hz1 = p.d == 3 ? p.P[2] / 2 + 1 : 1;
-  cudaError_t e;
-  {
-    const int logP = p.d == 2 ? p.logP[1] : p.logP[2];
-    const int P = 1 << logP;
-    const int G = P >> 4;
-    const int tl = pick_tl(sline(P), eb, G, budget, 64);
-    const size_t sm = (size_t)tl * sline(P) * eb;
-    if ((e = set_smem(k_col_mulinv<T>, sm)) != cudaSuccess) return e;
-    const int ncols = p.d == 2 ? Hx + 1 : (Hx + 1) * p.P[1];
-    const int n = p.d == 2 ? ny : nz;
-    C* dst = p.d == 2 ? S1 : S2;
-    const size_t ldo = p.d == 2 ? (size_t)nrows : (size_t)nz;
-    k_col_mulinv<T><<<(ncols + tl - 1) / tl, tl * G, sm, s>>>(SP, dst, ncols, n, (size_t)P, ldo, logP, tl, mult, map,
-                                                               p.d == 2 ? tw[1] : tw[2], logP);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (p.d == 3) {
-    const int Py = p.P[1];
-    const int G = Py >> 4;
-    const int tl = pick_tl(sline(Py), eb, G, budget, 64);
-    const size_t sm = (size_t)tl * sline(Py) * eb;
-    const int tiles = (nz + tl - 1) / tl;
-    e = with_rem(p.logP[1], [&](auto tag) {
-      constexpr int REM = decltype(tag)::value;
-      cudaError_t e2 = set_smem(k_c2cT_inv<T, REM>, sm);
-      if (e2 != cudaSuccess) return e2;
-      k_c2cT_inv<T, REM><<<(Hx + 1) * tiles, tl * G, sm, s>>>(S2, S1, nz, tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, p.logP[1], tl, tw[1], p.logP[1], nullptr, Batch{});
-      return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-  }
-  {
-    const int G = Hx >> 4;
-    const int tl = pick_tl(sline(Hx), eb, G, budget, 64);
-    const size_t sm = (size_t)tl * sline(Hx) * eb;
-    e = with_rem(p.logP[0] - 1, [&](auto tag) {
-      constexpr int REM = decltype(tag)::value;
-      cudaError_t e2 = set_smem(k_c2r_T<T, REM>, sm);
-      if (e2 != cudaSuccess) return e2;
-      k_c2r_T<T, REM><<<(nrows + tl - 1) / tl, tl * G, sm, s>>>(S1, y, nrows, nx, (size_t)nrows, nx, p.logP[0] - 1, tl, tw[0], p.logP[0], nullptr, Batch{});
-      return cudaGetLastError();
-    });
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 
 // Lines per CTA candidates of apply stage `st`: powers of two from whole warps up to the
 // compiled thread bound (kMaxCta), 64 lines, and 227 KB of shared memory.

@@ -1,0 +1,820 @@
+// The apply's stages in the FP64 engine: the pipeline of apply_impl.cuh on 64-bit block fixed point
+// (fft_q.cuh).  Vectors and symbol are FP64.  In the workspace a complex value is two 64-bit integers
+// below 2^58, in the same S1 / S2 layout and 16 bytes as an FP64 pair, and each line that a kernel wrote
+// has its exponent in an array behind S1 and S2:
+//   ex_row[row]           after the first stage, for S1[.][row]
+//   ex_line[kx n_z + z]   3D, for the y lines of both directions
+//   ex_col[kx] (2D), ex_col[kx P_y + ky] (3D) after the middle stage
+// A kernel whose lines run across those shifts its entries to the largest of their exponents as it loads
+// them: the bits it drops are below the rounding unit of the line that set that exponent.
+//
+// Native FP64 stages were bound by the FP64 pipe (84% busy) at a ninth of these stages' rate; conversions
+// from and to FP64 (64 cycles a warp) remain only at the vectors.
+#pragma once
+
+#include "apply_impl.cuh"
+#include "fft_q.cuh"
+
+namespace frlap {
+
+namespace {
+
+// Exponent arrays of one instance, in ints.
+struct QExpLayout {
+  size_t row, line, col, total;
+};
+inline QExpLayout q_exp_layout(const Plan& p) {
+  const size_t Hx1 = p.P[0] / 2 + 1;
+  QExpLayout l;
+  l.row = 0;
+  const size_t nrows = (size_t)p.n[1] * (p.d == 3 ? p.n[2] : 1);
+  l.line = align256(nrows * 4) / 4;
+  l.col = l.line + (p.d == 3 ? align256(Hx1 * p.n[2] * 4) / 4 : 0);
+  // 2D with the split middle stage: a second array for the even half
+  const size_t ncol = p.d == 3 ? Hx1 * p.P[1] : Hx1 * (p.P[1] > kMaxLine ? 2 : 1);
+  l.total = l.col + align256(ncol * 4) / 4;
+  return l;
+}
+
+__device__ __forceinline__ unsigned q_ord(int e) { return (unsigned)e ^ 0x80000000u; }
+__device__ __forceinline__ int q_unord(unsigned u) { return (int)(u ^ 0x80000000u); }
+// v 2^(e - top), e <= top
+__device__ __forceinline__ cq q_align(cq v, int e, int top) {
+  const int d = top - e > 63 ? 63 : top - e;
+  return {v.x >> d, v.y >> d};
+}
+
+#define FRLAP_Q_PROLOGUE(logLine)                                        \
+  extern __shared__ __align__(16) unsigned char smem_raw[];              \
+  __shared__ unsigned q_slot_words[kQSlots * kQLines];                   \
+  if (skip && FRLAP_GLD(skip)) return;                                   \
+  if ((logLine) > 9) {                                                   \
+    q_slots_clear(q_slot_words);                                         \
+    __syncthreads();                                                     \
+  }                                                                      \
+  cq* smem = reinterpret_cast<cq*>(smem_raw);
+
+template <int REM, int LOGL = 0>
+__global__ void __launch_bounds__(512, 1)
+    k_q_r2c(const double* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int nlines, int n, size_t ldo,
+            int logH, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  if constexpr (LOGL > 0) logH = LOGL;
+  {
+    const size_t bi = blockIdx.y;
+    in += bi * bt.in;
+    out += bi * bt.out;
+    ex += bi * ex_inst;
+    if (skip) skip += bi * bt.skip;
+  }
+  FRLAP_Q_PROLOGUE(logH)
+  const int H = 1 << logH, G = H >> 4, LS = sline(H);
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int line0 = blockIdx.x * TL, line = line0 + l;
+  const bool valid = line < nlines;
+  const double* src = in + (size_t)(valid ? line : 0) * n;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * LS;
+  // packed samples z[q] = x[2q] + i x[2q+1], as in k_r2c_T
+  double xr[8], xi[8];
+  const bool pair_aligned = (reinterpret_cast<uintptr_t>(src) % sizeof(double2)) == 0;
+  unsigned hm = 0u;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const int q = lane + m * G;
+    double a = 0.0, b = 0.0;
+    if (valid) {
+      if (pair_aligned && 2 * q + 1 < n) {
+        const double2 t = FRLAP_GLD(reinterpret_cast<const double2*>(src + 2 * q));
+        a = t.x;
+        b = t.y;
+      } else {
+        if (2 * q < n) a = FRLAP_GLD(src + 2 * q);
+        if (2 * q + 1 < n) b = FRLAP_GLD(src + 2 * q + 1);
+      }
+    }
+    xr[m] = a;
+    xi[m] = b;
+  }
+#pragma unroll
+  for (int m = 0; m < 8; ++m) hm = max(hm, max(q_mag(xr[m]), q_mag(xi[m])));
+  int si = 0;
+  const QIn qs = q_in_scale(q_reduce<true>(hm, logH, slots + si));
+  ++si;
+  cq v[16];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) v[m] = {q_in(xr[m], qs), q_in(xi[m], qs)};
+  int e = qs.e;
+  q_fft<-1, true, REM>(v, e, buf, logH, lane, tw, logH + 1, false, slots, si);
+  line_sync<double>(logH);
+#pragma unroll
+  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = {v[m].x >> 1, v[m].y >> 1};
+  line_sync<double>(logH);
+  // Real-data split in place, one product per pair (see r2c_tile): with a' = Z/2, X[k] = s + W^k d,
+  // X[H-k] = conj(s - W^k d), s = a' + b', d = -i (a' - b'); stored over 64, below 2^57.5.
+  for (int k = lane; k <= H / 2; k += G) {
+    const int km = H - k;
+    const cq a = buf[spad(k)];
+    const cq b = conjg(buf[spad(km & (H - 1))]);
+    const cq s = a + b, t = q_cmul<false>(mul_i<-1>(a - b), FRLAP_GLD(tw + k));
+    const cq s4 = {s.x >> 4, s.y >> 4};
+    buf[spad(k)] = q_shr_round<2>(s4 + t);
+    if (k != km) buf[spad(km)] = conjg(q_shr_round<2>(s4 - t));
+  }
+  if (valid && lane == 0) FRLAP_GST(ex + line, e + 6);
+  __syncthreads();
+  const int logTL = __ffs(TL) - 1;
+  const int lt = threadIdx.x & (TL - 1);
+  if (line0 + lt < nlines) {
+    const cq* trow = smem + (size_t)lt * LS;
+    int k = (int)threadIdx.x >> logTL;
+    cq* gp = out + (size_t)k * ldo + line0 + lt;
+    const size_t gstep = (size_t)G * ldo;
+#pragma unroll 4
+    for (; k <= H; k += G, gp += gstep) FRLAP_GST(gp, trow[spad(k)]);
+  }
+}
+
+// Entries v[m], m < M, of a line that runs across lines of other exponents: v = line[lane + m G] aligned to
+// the largest, which it returns.
+template <int M>
+__device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* ex, int lane, int G, int n, bool valid,
+                                              int logL, unsigned* slot) {
+  int e[M];
+  int top = kQZero;
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int i = lane + m * G;
+    const bool ok = valid && i < n;
+    v[m] = ok ? ld_stream(line + i) : cq{0, 0};
+    e[m] = ok ? FRLAP_GLD(ex + i) : kQZero;
+  }
+#pragma unroll
+  for (int m = 0; m < M; ++m) top = max(top, e[m]);
+  top = q_unord(q_reduce<true>(q_ord(top), logL, slot));
+#pragma unroll
+  for (int m = 0; m < M; ++m) v[m] = q_align(v[m], e[m], top);
+  return top;
+}
+
+// The symbol product in two steps.  v <- lambda v 2^(1020 - el), el = lambda's exponent field: the product
+// takes lambda's mantissa, so it has full precision whatever lambda's range along the line.  top collects the
+// largest leading bit of the line's lambda v.
+__device__ __forceinline__ void q_times(cq& v, int& el, double lam, int& top) {
+  const int h = __double2hiint(lam);
+  el = (h >> 20) & 0x7ff;
+  long long mant = (long long)(((unsigned long long)((unsigned)(h & 0xfffff) | 0x100000u) << 32) |
+                               (unsigned)__double2loint(lam))
+                   << 9;  // 2^61 <= mant < 2^62
+  if (el == 0) mant = 0;
+  if (h < 0) mant = -mant;
+  const QHalf w = q_half(mant);
+  v = {q_rmul(q_half(v.x), w), q_rmul(q_half(v.y), w)};
+  // leading bit of |v| above bit 31 (rounded up by at most one), plus 127
+  const int pos = __float_as_int(__uint2float_rn(q_bits(v))) >> 23;
+  top = max(top, el + max(pos, 126));
+}
+// All entries to the line's common exponent, components below 2^58.
+__device__ __forceinline__ void q_rescale(cq* v, const int* el, int& e, int top, int logL, unsigned* slot) {
+  top = (int)q_reduce<true>((unsigned)top, logL, slot);
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int s = el[m] + 152 - top;  // leading bits to bit 57 or below
+    const int sl = min(max(s, 0), 31), sr = min(max(-s, 0), 63);
+    v[m] = s >= 0 ? cq{q_shl(v[m].x, sl), q_shl(v[m].y, sl)} : cq{v[m].x >> sr, v[m].y >> sr};
+  }
+  e += top - 1172;
+}
+
+// A column's entries of one line: element i of instance-local column col at data[col ld + i].
+template <int REM, int LOGP = 0>
+__global__ void __launch_bounds__(512, 1)
+    k_q_colmul(cq* __restrict__ data, const int* __restrict__ ex_in, int* __restrict__ ex_out, int ncols, int n,
+               size_t ld, int logP, int TL, const double* __restrict__ lam, LamMap map, int nz,
+               const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  if constexpr (LOGP > 0) logP = LOGP;
+  {
+    const size_t bi = blockIdx.y;
+    data += bi * bt.in;
+    lam += bi * bt.lam;
+    ex_in += bi * ex_inst;
+    ex_out += bi * ex_inst;
+    if (skip) skip += bi * bt.skip;
+  }
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col = blockIdx.x * TL + l;
+  const bool valid = col < ncols;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * sline(P);
+  const int c = valid ? col : 0;
+  int si = 0;
+  cq v[16];
+  const int* exi = ex_in + (map.d == 2 ? 0 : (size_t)(c >> map.logPy) * nz);
+  int e = q_load_aligned<8>(v, data + (size_t)c * ld, exi, lane, G, n, valid, logP, slots + si);
+  ++si;
+  q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  const int ky = c & (map.Py - 1);
+  const double* lrow = map.d == 2 ? lam + (size_t)c * map.Hy1
+                                  : lam + ((size_t)(c >> map.logPy) * map.Hy1 + min(ky, map.Py - ky)) * map.Hz1;
+  {
+    int el[16];
+    int top = 0;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int k = lane + m * G;
+      q_times(v[m], el[m], ld_stream(&lrow[min(k, P - k)]), top);
+    }
+    q_rescale(v, el, e, top, logP, slots + si);
+    ++si;
+  }
+  q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  if (valid && lane == 0) FRLAP_GST(ex_out + col, e + 5);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) v[m] = q_shr_round<5>(v[m]);
+  store_line(v, data, ncols, n, ld, logP, TL);
+}
+
+// The middle stage of a 16384-point y embedding in two halves (see k_colmul_split).  ODD = false: the even
+// frequencies' half of the column into tmp; ODD = true: the odd half, added to it, in place.
+template <bool ODD>
+__global__ void __launch_bounds__(512, 1)
+    k_q_colmul_split(cq* __restrict__ data, cq* __restrict__ tmp, const int* __restrict__ ex_in,
+                     int* __restrict__ ex_out, int* __restrict__ ex_tmp, int ncols, int n, size_t ld, int TL,
+                     const double* __restrict__ lam, int Hy1, const int4* __restrict__ tw,
+                     const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  constexpr int logL = 13, L = 1 << logL, P = 2 * L, G = L >> 4, REM = logL & 3;
+  {
+    const size_t bi = blockIdx.y;
+    data += bi * bt.in;
+    tmp += bi * bt.out;
+    lam += bi * bt.lam;
+    ex_in += bi * ex_inst;
+    ex_out += bi * ex_inst;
+    ex_tmp += bi * ex_inst;
+    if (skip) skip += bi * bt.skip;
+  }
+  FRLAP_Q_PROLOGUE(logL)
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col = blockIdx.x * TL + l;
+  const bool valid = col < ncols;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * sline(L);
+  cq* line = data + (size_t)(valid ? col : 0) * ld;
+  cq* tline = tmp + (size_t)(valid ? col : 0) * ld;
+  int si = 0;
+  cq v[16];
+  int e = q_load_aligned<16>(v, line, ex_in, lane, G, n, valid, logL, slots + si);
+  ++si;
+  if constexpr (ODD) {  // times W_P^j: from below 2^62.5 (a shift by 4) back to below 2^58.5
+#pragma unroll
+    for (int m = 0; m < 16; ++m)
+      v[m] = q_cmul<false>(cq{q_shl(v[m].x, 4), q_shl(v[m].y, 4)}, FRLAP_GLD(tw + lane + m * G));
+  }
+  q_fft<-1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, false, slots, si);
+  // the half's symbol entries are every second one: gather through a strided row
+  const double* lrow = lam + (size_t)(valid ? col : 0) * Hy1;
+  {
+    int el[16];
+    int top = 0;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int k = 2 * (lane + m * G) + (ODD ? 1 : 0);
+      q_times(v[m], el[m], ld_stream(&lrow[min(k, P - k)]), top);
+    }
+    q_rescale(v, el, e, top, logL, slots + si);
+    ++si;
+  }
+  q_fft<1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, true, slots, si);
+  if (!valid) return;
+  if constexpr (!ODD) {
+    if (lane == 0) FRLAP_GST(ex_tmp + col, e + 5);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int j = lane + m * G;
+      if (j < n) FRLAP_GST(tline + j, q_shr_round<5>(v[m]));
+    }
+  } else {
+    // y_j = even_j + W_P^-j odd_j: magnitudes below 2^58 each at exponents et and e + 5
+    const int et = FRLAP_GLD(ex_tmp + col);
+    const int eo = e + 5;
+    const int top = max(et, eo);
+    if (lane == 0) FRLAP_GST(ex_out + col, top + 1);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int j = lane + m * G;
+      if (j < n) {
+        const cq o = q_shr_round<1>(q_cmul<true>(v[m], FRLAP_GLD(tw + j)));
+        FRLAP_GST(line + j, q_shr_round<1>(q_align(o, eo, top) + q_align(FRLAP_GLD(tline + j), et, top)));
+      }
+    }
+  }
+}
+
+// groups of contiguous lines of length n -> pad, FFT, transposed store out[g][k][line]
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_c2cT_fwd(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
+                 int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
+                 int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
+                 size_t ex_inst) {
+  {
+    const size_t bi = blockIdx.y;
+    in += bi * bt.in;
+    out += bi * bt.out;
+    ex_in += bi * ex_inst;
+    ex_out += bi * ex_inst;
+    if (skip) skip += bi * bt.skip;
+  }
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4, LS = sline(P);
+  const int g = blockIdx.x / tiles, tile = blockIdx.x % tiles;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int line0 = tile * TL, line = line0 + l;
+  const bool valid = line < nlines;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * LS;
+  const int c = valid ? line : 0;
+  int si = 0;
+  cq v[16];
+  // rows (z, y) of this line z: exponents ex_in[z n + y]
+  int e = q_load_aligned<8>(v, in + g * gin + (size_t)c * ldi, ex_in + (size_t)c * n, lane, G, n, valid, logP,
+                            slots + si);
+  ++si;
+  q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + 5);
+  line_sync<double>(logP);
+#pragma unroll
+  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = q_shr_round<5>(v[m]);
+  __syncthreads();
+  const int logTL = __ffs(TL) - 1;
+  const int lt = threadIdx.x & (TL - 1);
+  if (line0 + lt < nlines) {
+    const cq* trow = smem + (size_t)lt * LS;
+    int k = (int)threadIdx.x >> logTL;
+    cq* gp = out + g * gout + (size_t)k * ldo + line0 + lt;
+    const size_t gstep = (size_t)G * ldo;
+#pragma unroll 4
+    for (; k < P; k += G, gp += gstep) FRLAP_GST(gp, trow[spad(k)]);
+  }
+}
+
+// transposed in[g][k][line] (k < P) -> IFFT along k, crop to n, store out[g][line][i]
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_c2cT_inv(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
+                 int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
+                 int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
+                 size_t ex_inst) {
+  {
+    const size_t bi = blockIdx.y;
+    in += bi * bt.in;
+    out += bi * bt.out;
+    ex_in += bi * ex_inst;
+    ex_out += bi * ex_inst;
+    if (skip) skip += bi * bt.skip;
+  }
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4, LS = sline(P);
+  const int g = blockIdx.x / tiles, tile = blockIdx.x % tiles;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int line0 = tile * TL, line = line0 + l;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * LS;
+  int ek[16];
+  int e = kQZero;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    ek[m] = FRLAP_GLD(ex_in + (size_t)g * P + lane + m * G);
+    e = max(e, ek[m]);
+  }
+  load_transposed<cq>(smem, in + g * gin, TL * P, TL, LS, ldi, line0, nlines);
+  unsigned o = q_publish<true>(q_ord(e), logP, slots);
+  __syncthreads();
+  e = q_unord(q_fetch(o, logP, slots));
+  int si = 1;
+  cq v[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e);
+  q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  if (line < nlines) {
+    if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + 5);
+    cq* dst = out + g * gout + (size_t)line * ldo;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      const int i = lane + m * G;
+      if (i < n) FRLAP_GST(dst + i, q_shr_round<5>(v[m]));
+    }
+  }
+}
+
+// Last stage.  Bin k of row r has exponent ex[k ex_k + (r / rows_per) ].
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_c2r(const cq* __restrict__ in, double* __restrict__ out, const int* __restrict__ ex, int ex_k, int rows_per,
+            int nlines, int n, size_t ldi, int logH, int TL, const int4* __restrict__ tw,
+            const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  {
+    const size_t bi = blockIdx.y;
+    in += bi * bt.in;
+    out += bi * bt.out;
+    ex += bi * ex_inst;
+    if (skip) skip += bi * bt.skip;
+  }
+  FRLAP_Q_PROLOGUE(logH)
+  const int H = 1 << logH, G = H >> 4, LS = sline(H);
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int line0 = blockIdx.x * TL, line = line0 + l;
+  const bool valid = line < nlines;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * LS;
+  // this thread's pairs (k, H - k): k = lane + j G <= H/2 (j = 8: lane 0 alone)
+  int ea[9], eb[9];
+  int e = kQZero;
+  const int* exl = ex + (valid ? line / rows_per : 0);
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int k = lane + j * G;
+    if (k <= H / 2) {
+      ea[j] = FRLAP_GLD(exl + (size_t)k * ex_k);
+      eb[j] = FRLAP_GLD(exl + (size_t)(H - k) * ex_k);
+      e = max(e, max(ea[j], eb[j]));
+    }
+  }
+  load_transposed<cq>(smem, in, TL * (H + 1), TL, LS, ldi, line0, nlines);
+  unsigned o = q_publish<true>(q_ord(e), logH, slots);
+  __syncthreads();
+  e = q_unord(q_fetch(o, logH, slots));
+  int si = 1;
+  // repack in place (see k_c2r_T), over 4: Z[k] = A + i T, Z[H-k] = conj(A - i T), A = X[k] + conj X[H-k],
+  // T = W^-k (X[k] - conj X[H-k])
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int k = lane + j * G;
+    if (k <= H / 2) {
+      const int km = H - k;
+      const cq xk = q_align(buf[spad(k)], ea[j], e);
+      const cq b = conjg(q_align(buf[spad(km)], eb[j], e));
+      const cq A = q_shr_round<2>(xk + b), d = xk - b;
+      const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, FRLAP_GLD(tw + k)));
+      buf[spad(k)] = A + iT;
+      if (k != km && km != H) buf[spad(km)] = conjg(A - iT);
+    }
+  }
+  e += 2;
+  line_sync<double>(logH);
+  cq v[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) v[m] = buf[spad(lane + m * G)];
+  q_fft<1, false, REM>(v, e, buf, logH, lane, tw, logH + 1, true, slots, si);
+  if (!valid) return;
+  double* dst = out + (size_t)line * n;
+  const bool pair_aligned = (reinterpret_cast<uintptr_t>(dst) % sizeof(double2)) == 0;
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const int q = lane + m * G;
+    if (2 * q < n) {
+      const double a = q_out_any(v[m].x, e), b = q_out_any(v[m].y, e);
+      if (pair_aligned && 2 * q + 1 < n) {
+        FRLAP_GST(reinterpret_cast<double2*>(dst + 2 * q), make_double2(a, b));
+      } else {
+        FRLAP_GST(dst + 2 * q, a);
+        if (2 * q + 1 < n) FRLAP_GST(dst + 2 * q + 1, b);
+      }
+    }
+  }
+}
+
+// Spectrum columns of the learned preconditioner: columns of n entries -> zero-pad to P, forward FFT, all P
+// outputs in FP64 (stride ldo).
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_col_fwd(const cq* __restrict__ in, const int* __restrict__ ex, double2* __restrict__ out, int ncols, int n,
+                size_t ld, size_t ldo, int logP, int TL, int cols_per, const int4* __restrict__ tw,
+                const int* __restrict__ skip) {
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col = blockIdx.x * TL + l;
+  const bool valid = col < ncols;
+  const int c = valid ? col : 0;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * sline(P);
+  int si = 0;
+  cq v[16];
+  // exponents: 2D ex[i] for every column; 3D ex[(col / P_y) n + i]
+  int e = q_load_aligned<8>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)(c / cols_per) * n : 0), lane, G, n,
+                            valid, logP, slots + si);
+  ++si;
+  q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  if (!valid) return;
+  double2* dst = out + (size_t)col * ldo;
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    FRLAP_GST(dst + lane + m * G, make_double2(q_out_any(v[m].x, e), q_out_any(v[m].y, e)));
+}
+
+// Columns of P FP64 spectrum values times a multiplier (natural octant order) -> inverse FFT, crop to n.
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_col_mulinv(const double2* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int ncols, int n,
+                   size_t ld, size_t ldo, int logP, int TL, const double* __restrict__ lam, LamMap map,
+                   const int4* __restrict__ tw, const int* __restrict__ skip) {
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col = blockIdx.x * TL + l;
+  const bool valid = col < ncols;
+  const int c = valid ? col : 0;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * sline(P);
+  const double2* src = in + (size_t)c * ld;
+  size_t lam_base;
+  int lam_stride;
+  if (map.d == 2) {
+    lam_base = c;
+    lam_stride = map.Hx1;
+  } else {
+    const int kx = c >> map.logPy, ky = c & (map.Py - 1);
+    lam_base = (size_t)min(ky, map.Py - ky) * map.Hx1 + kx;
+    lam_stride = map.Hy1 * map.Hx1;
+  }
+  double2 x[16];
+  unsigned hm = 0u;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int k = lane + m * G;
+    x[m] = valid ? FRLAP_GLD(lam + lam_base + (size_t)min(k, P - k) * lam_stride) * FRLAP_GLD(src + k)
+                 : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int m = 0; m < 16; ++m) hm = max(hm, max(q_mag(x[m].x), q_mag(x[m].y)));
+  int si = 0;
+  const QIn qs = q_in_scale(q_reduce<true>(hm, logP, slots + si));
+  ++si;
+  cq v[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
+  int e = qs.e;
+  q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  if (valid && lane == 0) FRLAP_GST(ex + col, e + 5);
+#pragma unroll
+  for (int m = 0; m < 8; ++m) v[m] = q_shr_round<5>(v[m]);
+  store_line(v, out, ncols, n, ldo, logP, TL);
+}
+
+}  // namespace
+}  // namespace frlap
+
+namespace frlap {
+
+// Workspace arrays of one instance: S1, S2 (16-byte complex entries), then the exponents.
+struct QWork {
+  cq* S1;
+  cq* S2;
+  int *row, *line, *col;
+  size_t stride;     // to the next instance, in complex entries
+  size_t ex_stride;  // the same in ints
+};
+inline QWork q_work(const Plan& p, void* work) {
+  unsigned char* w = reinterpret_cast<unsigned char*>(work);
+  const QExpLayout l = q_exp_layout(p);
+  QWork q;
+  q.S1 = reinterpret_cast<cq*>(w);
+  q.S2 = reinterpret_cast<cq*>(w + align256(p.s1_elems * 16));
+  int* ex = reinterpret_cast<int*>(w + align256(p.s1_elems * 16) + align256(p.s2_elems * 16));
+  q.row = ex + l.row;
+  q.line = ex + l.line;
+  q.col = ex + l.col;
+  q.stride = apply_work_bytes(p, 8) / 16;
+  q.ex_stride = q.stride * 4;
+  return q;
+}
+
+// One launch: the kernel's shared memory limit, then the grid of (tiles, instances).
+template <typename K, typename... A>
+static cudaError_t q_launch(K kern, unsigned grid, int B, int threads, size_t sm, cudaStream_t s, A... args) {
+  cudaError_t e = set_smem(kern, sm);
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(grid, B), threads, sm, s>>>(args...);
+  return cudaGetLastError();
+}
+
+// Lines per CTA and the launch numbers that follow, for `lines` lines (per group: `tiles`) of length L.
+struct QShape {
+  int tl, threads, tiles;
+  size_t sm;
+};
+static QShape q_shape(int tuned, int L, long long lines_total, int lines_per_group) {
+  const int G = L >> 4;
+  QShape q;
+  q.tl = pick_tl_tuned(tuned, sline(L), 16, G, 96 * 1024, lines_total);
+  q.threads = q.tl * G;
+  q.tiles = (lines_per_group + q.tl - 1) / q.tl;
+  q.sm = (size_t)q.tl * sline(L) * 16;
+  return q;
+}
+
+static LamMap q_lam_map(const Plan& p) {
+  LamMap map;
+  map.d = p.d;
+  map.Hx1 = p.P[0] / 2 + 1;
+  map.logPy = p.logP[1];
+  map.Py = p.P[1];
+  map.Hy1 = p.P[1] / 2 + 1;
+  map.Hz1 = p.d == 3 ? p.P[2] / 2 + 1 : 1;
+  return map;
+}
+
+#ifdef FRLAP_BOUNDS_CHECK
+static cudaError_t q_register(const Plan& p, BcRanges r, void* work, int B, cudaStream_t s) {
+  r.add(work, (size_t)B * apply_work_bytes(p, 8));
+  for (int a = 0; a < p.d; ++a) r.add(p.twq[a], (size_t)twiddle_entries(p.P[a]) * sizeof(int4));
+  return r.commit(s);
+}
+#endif
+
+// The stages, one launch each over B instances (per-instance strides in elements).
+static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const double* u, size_t ustride, int tuned,
+                               const int* skip, int skip_stride, cudaStream_t s) {
+  const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
+  const QShape q = q_shape(tuned, H, (long long)nrows * B, nrows);
+  Batch b;
+  b.in = ustride;
+  b.out = w.stride;
+  b.skip = skip_stride;
+  return with_rem(p.logP[0] - 1, [&](auto tag) {
+    return q_launch(k_q_r2c<decltype(tag)::value>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row, nrows, p.n[0],
+                    (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
+  });
+}
+static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
+                                  cudaStream_t s) {
+  const int Py = p.P[1], ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1;
+  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1 * B, nz);
+  Batch b;
+  b.in = b.out = w.stride;
+  b.skip = skip_stride;
+  return with_rem(p.logP[1], [&](auto tag) {
+    return q_launch(k_q_c2cT_fwd<decltype(tag)::value>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, w.S2,
+                    (const int*)w.row, w.line, nz, q.tiles, ny, (size_t)nz * ny, ny, (size_t)Py * nz, nz, p.logP[1],
+                    q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
+  });
+}
+static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
+                                  cudaStream_t s) {
+  const int Py = p.P[1], ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1;
+  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1 * B, nz);
+  Batch b;
+  b.in = b.out = w.stride;
+  b.skip = skip_stride;
+  return with_rem(p.logP[1], [&](auto tag) {
+    return q_launch(k_q_c2cT_inv<decltype(tag)::value>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S2, w.S1,
+                    (const int*)w.col, w.line, nz, q.tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, p.logP[1],
+                    q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
+  });
+}
+static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, size_t ystride, int tuned,
+                               const int* skip, int skip_stride, cudaStream_t s) {
+  const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
+  const QShape q = q_shape(tuned, H, (long long)nrows * B, nrows);
+  Batch b;
+  b.in = w.stride;
+  b.out = ystride;
+  b.skip = skip_stride;
+  return with_rem(p.logP[0] - 1, [&](auto tag) {
+    return q_launch(k_q_c2r<decltype(tag)::value>, q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, y,
+                    (const int*)(p.d == 3 ? w.line : w.col), p.d == 3 ? p.n[2] : 1, p.d == 3 ? p.n[1] : nrows, nrows,
+                    p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
+  });
+}
+
+template <typename T>
+cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstride, void* work, cudaStream_t s,
+                             const int* skip, int skip_stride, cudaEvent_t const* ev, const T* lam_override,
+                             size_t lam_stride) {
+  static_assert(std::is_same<T, double>::value, "the FP64 engine");
+  int stage = 0;
+  auto mark = [&]() -> cudaError_t {
+    if (ev && ev[stage]) {
+      cudaError_t e = cudaEventRecord(ev[stage], s);
+      if (e != cudaSuccess) return e;
+    }
+    ++stage;
+    return cudaSuccess;
+  };
+  const int* tuned = p.tl_tuned[engine_index<T>()];
+  const double* lam = lam_override ? lam_override : p.lamL64;
+  const QWork w = q_work(p, work);
+  const int ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1, nrows = ny * nz;
+  const LamMap map = q_lam_map(p);
+  cudaError_t e;
+#ifdef FRLAP_BOUNDS_CHECK
+  {
+    BcRanges r;
+    const size_t vext = ((size_t)(B - 1) * vstride + p.M) * sizeof(double);
+    r.add(u, vext);
+    r.add(y, vext);
+    r.add(lam, ((size_t)(B - 1) * lam_stride + p.lam_count) * sizeof(double));
+    if (skip) r.add(skip, ((size_t)(B - 1) * skip_stride + 1) * sizeof(int));
+    if ((e = q_register(p, r, work, B, s)) != cudaSuccess) return e;
+  }
+#endif
+  Batch b;
+  b.in = b.out = w.stride;
+  b.lam = lam_stride;
+  b.skip = skip_stride;
+  if ((e = mark()) != cudaSuccess) return e;
+  if ((e = q_stage_r2c(p, w, B, u, vstride, tuned[0], skip, skip_stride, s)) != cudaSuccess) return e;
+  if ((e = mark()) != cudaSuccess) return e;
+  if (p.d == 2 && p.P[1] > kMaxLine) {
+    const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1 * B, Hx1);
+    int* ex_tmp = w.col + Hx1;
+    e = q_launch(k_q_colmul_split<false>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col, ex_tmp,
+                 Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);
+    if (e == cudaSuccess)
+      e = q_launch(k_q_colmul_split<true>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col,
+                   ex_tmp, Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);
+    if (e != cudaSuccess) return e;
+  } else {
+    if (p.d == 3) {
+      if ((e = q_stage_yz_fwd(p, w, B, tuned[1], skip, skip_stride, s)) != cudaSuccess) return e;
+      if ((e = mark()) != cudaSuccess) return e;
+    }
+    // the middle stage: columns over y in S1 (2D), over z in S2 (3D)
+    const int ax = p.d == 3 ? 2 : 1;
+    const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
+    const QShape q = q_shape(tuned[p.d == 3 ? 2 : 1], p.P[ax], (long long)ncols * B, ncols);
+    e = with_line_shape<T, true>(p.logP[ax], [&](auto tag) {
+      constexpr int REM = decltype(tag)::rem, LP = decltype(tag)::logp;
+      return q_launch(k_q_colmul<REM, LP>, q.tiles, B, q.threads, q.sm, s, p.d == 3 ? w.S2 : w.S1,
+                      (const int*)(p.d == 3 ? w.line : w.row), w.col, ncols, p.n[ax], (size_t)(p.d == 3 ? nz : nrows),
+                      p.logP[ax], q.tl, lam, map, nz, (const int4*)p.twq[ax], skip, b, w.ex_stride);
+    });
+    if (e != cudaSuccess) return e;
+    if (p.d == 3) {
+      if ((e = mark()) != cudaSuccess) return e;
+      if ((e = q_stage_yz_inv(p, w, B, tuned[3], skip, skip_stride, s)) != cudaSuccess) return e;
+    }
+  }
+  if ((e = mark()) != cudaSuccess) return e;
+  if ((e = q_stage_c2r(p, w, B, y, vstride, tuned[p.d == 2 ? 2 : 4], skip, skip_stride, s)) != cudaSuccess) return e;
+  return mark();
+}
+
+// SP = F R^T u on the half spectrum in FP64: 2D [kx][ky], 3D [kx][ky][kz] (kx <= P_x/2, full ky, kz).
+template <>
+cudaError_t spectrum_forward<double>(const Plan& p, const double* u, double2* SP, void* work, cudaStream_t s) {
+  cudaError_t e;
+#ifdef FRLAP_BOUNDS_CHECK
+  {
+    BcRanges r;
+    r.add(u, p.M * sizeof(double));
+    r.add(SP, spectrum_elems(p) * sizeof(double2));
+    if ((e = q_register(p, r, work, 1, s)) != cudaSuccess) return e;
+  }
+#endif
+  const QWork w = q_work(p, work);
+  if ((e = q_stage_r2c(p, w, 1, u, 0, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  if (p.d == 3 && (e = q_stage_yz_fwd(p, w, 1, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
+  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
+  const QShape q = q_shape(0, p.P[ax], ncols, ncols);
+  return with_rem(p.logP[ax], [&](auto tag) {
+    return q_launch(k_q_col_fwd<decltype(tag)::value>, q.tiles, 1, q.threads, q.sm, s,
+                    (const cq*)(p.d == 3 ? w.S2 : w.S1), (const int*)(p.d == 3 ? w.line : w.row), SP, ncols, p.n[ax],
+                    (size_t)(p.d == 3 ? p.n[2] : nrows), (size_t)p.P[ax], p.logP[ax], q.tl, p.d == 3 ? p.P[1] : 0,
+                    (const int4*)p.twq[ax], (const int*)nullptr);
+  });
+}
+
+// y = R F^-1 (mult * SP), mult = a symbol octant with the 1/prod(P) factor folded in.
+template <>
+cudaError_t spectrum_inverse<double>(const Plan& p, const double2* SP, const double* mult, double* y, void* work,
+                                     cudaStream_t s) {
+  cudaError_t e;
+#ifdef FRLAP_BOUNDS_CHECK
+  {
+    BcRanges r;
+    r.add(SP, spectrum_elems(p) * sizeof(double2));
+    r.add(mult, p.lam_count * sizeof(double));
+    r.add(y, p.M * sizeof(double));
+    if ((e = q_register(p, r, work, 1, s)) != cudaSuccess) return e;
+  }
+#endif
+  const QWork w = q_work(p, work);
+  const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
+  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
+  const QShape q = q_shape(0, p.P[ax], ncols, ncols);
+  const LamMap map = q_lam_map(p);
+  e = with_rem(p.logP[ax], [&](auto tag) {
+    return q_launch(k_q_col_mulinv<decltype(tag)::value>, q.tiles, 1, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
+                    w.col, ncols, p.n[ax], (size_t)p.P[ax], (size_t)(p.d == 3 ? p.n[2] : nrows), p.logP[ax], q.tl, mult,
+                    map, (const int4*)p.twq[ax], (const int*)nullptr);
+  });
+  if (e != cudaSuccess) return e;
+  if (p.d == 3 && (e = q_stage_yz_inv(p, w, 1, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  return q_stage_c2r(p, w, 1, y, 0, 0, nullptr, 0, s);
+}
+
+}  // namespace frlap

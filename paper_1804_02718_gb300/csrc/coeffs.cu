@@ -10,6 +10,7 @@
 // which integrates the radial variable in closed form and leaves a smooth
 // (d-1)-dimensional integral.  Gauss-Legendre nodes are computed on the device by
 // Newton's method on the three-term Legendre recurrence.
+#include <limits.h>
 #include <math.h>
 
 #include <type_traits>
@@ -506,6 +507,29 @@ __global__ void k_to_cdf(const double2* __restrict__ src, cdf* dst, size_t n) {
 // double-float copy of a complex table (twiddles), n values, in the paired layout of cdf
 cudaError_t to_cdf_launch(const double2* src, cdf* dst, size_t n, cudaStream_t st) {
   k_to_cdf<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, dst, n);
+  return cudaGetLastError();
+}
+
+namespace {
+// x in [-1, 1] with 60 fraction bits as h 2^32 + l, both signed; a low half of -2^31 takes one unit more,
+// so that a half can be negated
+__device__ __forceinline__ int2 q60(double x) {
+  long long v = __double2ll_rn(x * 0x1p60);
+  if ((int)v == INT_MIN) ++v;
+  const int l = (int)v;
+  return make_int2((int)((v - (long long)l) >> 32), l);
+}
+__global__ void k_to_q(const double2* __restrict__ src, int4* dst, size_t n) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int2 a = q60(src[i].x), b = q60(src[i].y);
+  dst[i] = make_int4(a.x, a.y, b.x, b.y);
+}
+}  // namespace
+
+// fixed-point copy of a complex table (twiddles), n values, in the layout of Plan::twq
+cudaError_t to_q_launch(const double2* src, int4* dst, size_t n, cudaStream_t st) {
+  k_to_q<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, dst, n);
   return cudaGetLastError();
 }
 

@@ -258,6 +258,9 @@ struct Plan {
   double2* tw64[3] = {nullptr, nullptr, nullptr};
   float2* tw32[3] = {nullptr, nullptr, nullptr};
   cdf* twdf[3] = {nullptr, nullptr, nullptr};      // the same twiddles as double-floats
+  // the same in fixed point (60 fraction bits, signed 32-bit halves: re high, re low, im high, im low), for
+  // the FP64 engine (all plans but F32)
+  int4* twq[3] = {nullptr, nullptr, nullptr};
   dfl* lamdf = nullptr;        // line-major, as double-floats (DF64 plans)
   bool df64 = false;           // FP64-precision vectors are applied with double-float FFTs
   // workspace layout of one apply, in complex elements of the apply precision
@@ -287,11 +290,6 @@ cudaError_t bc_collect(unsigned long long* count, unsigned long long* first);
 cudaError_t bc_selftest(unsigned long long* flagged);
 // Runs one bounded mbarrier wait that nothing completes; *timeouts = waits that gave up (1 expected).
 cudaError_t wait_selftest(unsigned long long* timeouts);
-// the residual apply of double-float plans (FP64 forward, double-float inverse transforms; see
-// apply_hyb.cu); cudaErrorNotSupported for other plans and for plans with a split middle stage
-cudaError_t apply_residual_hyb(const Plan& p, const double* u, double* y, void* work, cudaStream_t s);
-cudaError_t hyb_wait_collect(unsigned long long* count);
-cudaError_t hyb_bc_collect(unsigned long long* count, unsigned long long* first);
 // radix-16 stages on CUDA cores (engine 0) or tensor cores (engine 1); see dft16_tc.cu
 cudaError_t dft16_stages_launch(int engine, const float* in, float* out, int ntiles, int reps, cudaStream_t s);
 cudaError_t dft16_wait_collect(unsigned long long* count);
@@ -346,6 +344,7 @@ cudaError_t scale_symbol_launch(double* lam64, float* lam32, size_t n, double s,
 template <typename To>
 cudaError_t line_symbol_launch(const Plan& p, const double* oct, To* dst, double s, cudaStream_t st);
 cudaError_t to_df_launch(const double* src, dfl* dst, size_t n, cudaStream_t st);
+cudaError_t to_q_launch(const double2* src, int4* dst, size_t n, cudaStream_t st);
 cudaError_t to_cdf_launch(const double2* src, cdf* dst, size_t n, cudaStream_t st);
 // even DFT of the octant along every axis (used for both the operator and preconditioner symbols)
 cudaError_t symbol_axes_launch(const Plan& p, double* lam_oct, cudaStream_t s);

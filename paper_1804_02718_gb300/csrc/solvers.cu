@@ -460,24 +460,13 @@ static cudaError_t apply_T(const Plan& p, const T* u, T* y, void* work, cudaStre
 }
 
 // The residuals f - B x that restart a solve or decide its convergence.  The iterations may run
-// on double-float (48-bit products, 5.6x faster than native FP64), but a residual computed with it
-// carries the forward transforms' rounding times up to lambda_max (about 5e-15 lambda_max ||x||),
-// which at 2047^2 already sits near 1e-10 ||f||.  So the forward transforms of a residual run in
-// native FP64: on double-float plans the hybrid apply (FP64 forward, double-float inverse
-// transforms, apply_hyb.cu), as accurate as native FP64 near a solution and 1.7x faster; native FP64
-// throughout on F64 plans and on plans with a split middle stage.  A restart from such a residual
-// removes the recurrence's drift, as in iterative refinement.
+// on double-float (48-bit products), but a residual computed with it carries the transforms' rounding times
+// up to lambda_max (about 5e-15 lambda_max ||x||), which at 2047^2 already sits near 1e-10 ||f||.  So a
+// residual takes the FP64 engine on every plan.  A restart from such a residual removes the recurrence's
+// drift, as in iterative refinement.
 template <typename T>
 static cudaError_t apply_residual(const Plan& p, const T* u, T* y, void* work, cudaStream_t s) {
-  if constexpr (sizeof(T) == 8) {
-    if (p.df64) {
-      const cudaError_t e = apply_residual_hyb(p, u, y, work, s);
-      if (e != cudaErrorNotSupported) return e;
-    }
-    return apply_launch<double>(p, u, y, work, s, nullptr);
-  } else {
-    return apply_launch<float>(p, u, y, work, s, nullptr);
-  }
+  return apply_launch<T>(p, u, y, work, s, nullptr);
 }
 
 // workspace of one (P)CG solve in precision T:

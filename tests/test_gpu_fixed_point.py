@@ -1,0 +1,113 @@
+"""The FP64 engine's block fixed-point transforms: accuracy, exact scaling, zeros and non-finite values.
+
+The reference is the defining sum y_i = -c sum_j a_|i-j| u_j (eqs. A-2D / A-3D) in extended precision, at
+sampled rows, so it shares no transform with the library.  Tolerance, per entry, for i.i.d. N(0,1) input:
+2^-49 lambda_max.  An FP64 FFT product of such a vector (rms 1) has an entrywise error of about
+2^-53 sqrt(2 log2(prod P)) <= 2^-50.5 lambda_max in the mean square; the fixed-point unit is 2^-58 of a
+line's largest value, below that, and the factor 2^1.5 covers the largest of 40 samples.
+"""
+import numpy as np
+import pytest
+
+import frlap_inputs as inp
+
+pytestmark = pytest.mark.gpu
+
+# every transform length the plans admit, on rows and on columns, with ragged ends; 3D with its y and z lines
+SHAPES = [(32, 32), (17, 40), (40, 17), (100, 70), (130, 9), (9, 130), (300, 257), (256, 513), (600, 12), (12, 600),
+          (1025, 5), (5, 1025), (2049, 6), (6, 2049), (4097, 3), (3, 4097), (2, 2),
+          (12, 7, 9), (33, 9, 17), (5, 70, 6), (6, 5, 130), (40, 40, 40), (3, 300, 4)]
+
+
+def _operator(fl, Ns, alpha, prec):
+    from oracle import scheme
+
+    d, N = len(Ns), max(Ns)
+    h = 2.0 / N
+    coef = fl.frlap_coeffs(d, alpha, 2.0, h, Ns).cpu().numpy()
+    plan = fl.Plan(d, alpha, h, Ns, prec=prec)
+    lam_max = float(plan.symbol().abs().max()) * float(np.prod([float(p) for p in plan.P]))
+    return plan, coef, scheme.c_d_alpha(d, alpha), lam_max
+
+
+@pytest.mark.parametrize("Ns", SHAPES)
+def test_entries_against_the_defining_sum(frlap, Ns):
+    import torch
+
+    plan, coef, c, lam_max = _operator(frlap, Ns, 1.3, frlap.FRLAP_F64)
+    u = inp.normal_field(Ns, seed=11)
+    y = frlap.frlap_apply(plan, torch.from_numpy(u).cuda()).cpu().numpy()
+    rng = np.random.default_rng(3)
+    ul = u.astype(np.longdouble)
+    grids = [np.arange(n) for n in u.shape]
+    worst = 0.0
+    for _ in range(40):
+        i = [int(rng.integers(n)) for n in u.shape]
+        a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
+        ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
+        worst = max(worst, abs(float(y[tuple(i)] - ref)))
+    assert worst < 2.0 ** -49 * lam_max, (worst / lam_max)
+
+
+@pytest.mark.parametrize("Ns", [(100, 70), (600, 40), (12, 40, 9)])
+@pytest.mark.parametrize("e", [-960, -40, 900])
+def test_scaling_by_a_power_of_two_is_exact(frlap, Ns, e):
+    """Fixed point with an exponent per line: 2^e u gives the same integers, so 2^e y exactly."""
+    import torch
+
+    plan, _, _, _ = _operator(frlap, Ns, 1.3, frlap.FRLAP_F64)
+    u = torch.from_numpy(inp.normal_field(Ns, seed=5)).cuda()
+    y = frlap.frlap_apply(plan, u)
+    ys = frlap.frlap_apply(plan, u * 2.0 ** e)  # (torch.ldexp on the GPU takes an inexact power)
+    assert torch.equal(ys, y * 2.0 ** e)
+
+
+def test_rows_of_very_different_scales(frlap):
+    """Rows between 1e-120 and 1: every row's error stays relative to the whole vector, and the product is
+    that of the sum of the parts."""
+    import torch
+
+    Ns = (70, 100)
+    plan, coef, c, lam_max = _operator(frlap, Ns, 0.8, frlap.FRLAP_F64)
+    u = inp.normal_field(Ns, seed=7)
+    u *= 10.0 ** -np.linspace(0, 120, u.shape[0])[:, None]
+    u[10] = 0.0
+    y = frlap.frlap_apply(plan, torch.from_numpy(u).cuda()).cpu().numpy()
+    ul = u.astype(np.longdouble)
+    grids = [np.arange(n) for n in u.shape]
+    for i in [(0, 0), (1, 40), (10, 3), (50, 68), (98, 20)]:
+        a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
+        ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
+        assert abs(float(y[i] - ref)) < 2.0 ** -49 * lam_max
+
+
+@pytest.mark.parametrize("Ns", [(100, 70), (12, 40, 9)])
+def test_zero_and_non_finite_inputs(frlap, Ns):
+    import torch
+
+    plan, _, _, _ = _operator(frlap, Ns, 1.1, frlap.FRLAP_F64)
+    u = torch.zeros(plan.shape, dtype=torch.float64, device="cuda")
+    assert torch.equal(frlap.frlap_apply(plan, u), u)
+    for bad in (float("nan"), float("inf"), -float("inf")):
+        v = u.clone()
+        v.view(-1)[plan.M // 2] = bad
+        assert bool(torch.isnan(frlap.frlap_apply(plan, v)).all())
+    tiny = torch.full(plan.shape, 5e-324, dtype=torch.float64, device="cuda")
+    assert bool(torch.isfinite(frlap.frlap_apply(plan, tiny)).all())
+
+
+def test_split_middle_stage(frlap):
+    """A 16384-point y embedding (two half-length transforms), against the defining sum at sampled rows."""
+    import torch
+
+    Ns = (6, 4200)
+    plan, coef, c, lam_max = _operator(frlap, Ns, 1.3, frlap.FRLAP_F64)
+    assert plan.P[1] == 16384
+    u = inp.normal_field(Ns, seed=2)
+    y = frlap.frlap_apply(plan, torch.from_numpy(u).cuda()).cpu().numpy()
+    ul = u.astype(np.longdouble)
+    grids = [np.arange(n) for n in u.shape]
+    for i in [(0, 0), (17, 4), (2100, 2), (4095, 0), (4096, 1), (4198, 4)]:
+        a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
+        ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
+        assert abs(float(y[i] - ref)) < 2.0 ** -49 * lam_max
