@@ -8,8 +8,7 @@
 // the singular point xi = 0; the origin element and the far field are reduced
 // by splitting the cube into d pyramids (on each, one coordinate is the largest),
 // which integrates the radial variable in closed form and leaves a smooth
-// (d-1)-dimensional integral.  Gauss-Legendre nodes are computed on the device by
-// Newton's method on the three-term Legendre recurrence.
+// (d-1)-dimensional integral.
 #include <limits.h>
 #include <math.h>
 
@@ -22,50 +21,51 @@ namespace frlap {
 
 namespace {
 
-// orders used by the element rule and by the pyramid integrals
+// Gauss-Legendre rules of the orders below on [0, 1], weights summing to 1, one after another; a kernel
+// argument (read as constants).  Newton's method on the three-term recurrence, on the host once per process:
+// on the device, 83 threads of one warp group in serial FP64 took 1.7 ms of each plan's creation.
 constexpr int kNumQ = 6;
-__constant__ int c_q[kNumQ] = {4, 5, 8, 14, 20, 32};
-constexpr int kQTotal = 83;
-
-// nodes on [0,1] and weights summing to 1, one thread per node
-__global__ void k_gauss(double* nodes, double* weights) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= kQTotal) return;
-  int qi = 0;
-  int off[kNumQ + 1] = {0, 4, 9, 17, 31, 51, 83};
-  while (t >= off[qi + 1]) ++qi;
-  const int q = c_q[qi];
-  const int i = t - off[qi];
-  double x = cos(M_PI * (i + 0.75) / (q + 0.5));
-  double dP = 1.0;
-  for (int it = 0; it < 100; ++it) {
-    double p0 = 1.0, p1 = x;
-    for (int k = 2; k <= q; ++k) {
-      const double p2 = ((2.0 * k - 1.0) * x * p1 - (k - 1.0) * p0) / k;
-      p0 = p1;
-      p1 = p2;
+__host__ __device__ constexpr int rule_q(int r) {
+  return r == 0 ? 4 : r == 1 ? 5 : r == 2 ? 8 : r == 3 ? 14 : r == 4 ? 20 : 32;
+}
+__host__ __device__ constexpr int rule_off(int r) { return r == 0 ? 0 : rule_off(r - 1) + rule_q(r - 1); }
+constexpr int kQTotal = rule_off(kNumQ);
+struct GaussRules {
+  double x[kQTotal], w[kQTotal];
+};
+GaussRules make_gauss_rules() {
+  GaussRules g;
+  for (int r = 0; r < kNumQ; ++r) {
+    const int q = rule_q(r);
+    for (int i = 0; i < q; ++i) {
+      double x = cos(M_PI * (i + 0.75) / (q + 0.5)), dP = 1.0;
+      for (int it = 0; it < 20; ++it) {
+        double p0 = 1.0, p1 = x;
+        for (int k = 2; k <= q; ++k) {
+          const double p2 = ((2.0 * k - 1.0) * x * p1 - (k - 1.0) * p0) / k;
+          p0 = p1;
+          p1 = p2;
+        }
+        dP = q * (x * p1 - p0) / (x * x - 1.0);
+        const double dx = p1 / dP;
+        x -= dx;
+        if (fabs(dx) < 1e-15) break;  // quadratic: the step after a 1e-8 one is the last that changes x
+      }
+      g.x[rule_off(r) + i] = 0.5 * (1.0 - x);
+      g.w[rule_off(r) + i] = 1.0 / ((1.0 - x * x) * dP * dP);  // (2 / ((1 - x^2) P'^2)) / 2
     }
-    dP = q * (x * p1 - p0) / (x * x - 1.0);
-    const double dx = p1 / dP;
-    x -= dx;
-    if (fabs(dx) < 1e-17) break;
   }
-  {
-    double p0 = 1.0, p1 = x;
-    for (int k = 2; k <= q; ++k) {
-      const double p2 = ((2.0 * k - 1.0) * x * p1 - (k - 1.0) * p0) / k;
-      p0 = p1;
-      p1 = p2;
-    }
-    dP = q * (x * p1 - p0) / (x * x - 1.0);
-  }
-  nodes[t] = 0.5 * (1.0 - x);
-  weights[t] = 1.0 / ((1.0 - x * x) * dP * dP);  // (2/((1-x^2)P'^2)) / 2
+  return g;
+}
+const GaussRules& gauss_rules() {
+  static const GaussRules g = make_gauss_rules();
+  return g;
 }
 
-__device__ __forceinline__ int q_index(int dist) {
-  // Gauss-Legendre order for an element whose lower corner has max-norm dist >= 1;
-  // the error decays like (2 dist)^(-2q)
+// Elements of max-norm distance at most kNear (and at least 1) by k_elements_near, beyond by k_elements_far.
+// The order falls with the distance; the error decays like (2 dist)^(-2q).
+constexpr int kNear = 24, kMid = 96;
+__host__ __device__ __forceinline__ int q_index(int dist) {
   if (dist <= 2) return 4;   // 20 points
   if (dist <= 6) return 3;   // 14
   if (dist <= 24) return 2;  // 8
@@ -73,9 +73,114 @@ __device__ __forceinline__ int q_index(int dist) {
   return 0;                  // 4
 }
 
+// |xi|^-p and the tensor rule are symmetric under permutations of the coordinates, so w_k = w_{sorted k}:
+// only elements with k[0] <= k[1] (<= k[2]) are integrated, and k_fill_permuted copies them to the others
+// (2D: half, 3D: a sixth of the work).
+
+// Near elements, one per CTA, their 64 to 400 (3D: 512 to 8000) powers spread over its threads: with one
+// thread per element the nearest ones' serial powers set the kernel's time (512^2: 1.5 ms).
 template <int D>
-__global__ void k_element_weights(double* w, int N, double p, const double* __restrict__ gn,
-                                  const double* __restrict__ gw) {
+__global__ void __launch_bounds__(128) k_elements_near(double* w, int N, int side, double p, GaussRules g) {
+  int k[3] = {0, 0, 0};
+  int rest = blockIdx.x;
+  for (int r = 0; r < D; ++r) {
+    k[r] = rest % side;
+    rest /= side;
+  }
+  for (int r = 0; r + 1 < D; ++r)
+    if (k[r] > k[r + 1]) return;
+  const int dist = k[D - 1];
+  if (dist == 0) return;  // origin element: k_pyramid
+  const int qi = q_index(dist), q = rule_q(qi);
+  const double *xn = g.x + rule_off(qi), *xw = g.w + rule_off(qi);
+  const double mp = -0.5 * p;
+  const int cnt = D == 2 ? q * q : q * q * q;
+  double acc = 0.0;
+  for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+    const int i = t % q, j = (t / q) % q;
+    const double a = k[0] + xn[i], b = k[1] + xn[j];
+    double r2 = a * a + b * b, wt = xw[i] * xw[j];
+    if (D == 3) {
+      const int l = t / (q * q);
+      const double c = k[2] + xn[l];
+      r2 += c * c;
+      wt *= xw[l];
+    }
+    acc += wt * pow(r2, mp);
+  }
+  __shared__ double red[128];
+  red[threadIdx.x] = acc;
+  __syncthreads();
+  for (int st = 64; st > 0; st >>= 1) {
+    if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    size_t e = 0, stride = 1;
+    for (int r = 0; r < D; ++r) {
+      e += (size_t)k[r] * stride;
+      stride *= N;
+    }
+    w[e] = red[0];
+  }
+}
+
+// Binomial coefficients of (1 + delta)^(-p/2).
+constexpr int kFarTerms = 13;
+struct FarSeries {
+  double c[kFarTerms];
+};
+
+// Far elements, a thread each: one power at the element's centre c, and at the nodes c + t the series
+// |c + t|^-p = |c|^-p (1 + delta)^(-p/2), delta = (2 c.t + |t|^2) / |c|^2 in Horner form.  |delta| <= 1 / dist:
+// 10 terms beyond 96 and 13 beyond 24 leave less than 1e-17.  (16 powers a thread, of about 80 FP64
+// instructions each at 76 cycles, were the kernel's time: 512^2 1.48 ms.)
+template <int D, int Q, int NT>
+__device__ __forceinline__ double far_element(const int* k, double mp, const double* xn, const double* xw,
+                                              const FarSeries& s) {
+  double c[3], r2 = 0.0;
+#pragma unroll
+  for (int r = 0; r < D; ++r) {
+    c[r] = k[r] + 0.5;
+    r2 = fma(c[r], c[r], r2);
+  }
+  const double inv = 1.0 / r2;
+  double d[3][Q];  // (2 c_r t + t^2) / |c|^2
+#pragma unroll
+  for (int r = 0; r < D; ++r)
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const double t = xn[i] - 0.5;
+      d[r][i] = t * fma(2.0, c[r], t) * inv;
+    }
+  auto series = [&](double x) {
+    double v = s.c[NT - 1];
+#pragma unroll
+    for (int n = NT - 2; n >= 0; --n) v = fma(v, x, s.c[n]);
+    return v;
+  };
+  double acc = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < Q; ++i) {
+    double s1 = 0.0;
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+      const double dij = d[0][i] + d[1][j];
+      if (D == 2) {
+        s1 += xw[j] * series(dij);
+      } else {
+        double s2 = 0.0;
+#pragma unroll 1
+        for (int l = 0; l < Q; ++l) s2 += xw[l] * series(dij + d[2][l]);
+        s1 += xw[j] * s2;
+      }
+    }
+    acc += xw[i] * s1;
+  }
+  return acc * pow(r2, mp);
+}
+template <int D>
+__global__ void __launch_bounds__(128) k_elements_far(double* w, int N, double p, GaussRules g, FarSeries s) {
   const size_t total = (D == 2) ? (size_t)N * N : (size_t)N * N * N;
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
@@ -85,48 +190,13 @@ __global__ void k_element_weights(double* w, int N, double p, const double* __re
     k[r] = (int)(rest % N);
     rest /= N;
   }
-  // |xi|^-p and the tensor rule are symmetric under permutations of the coordinates, so
-  // w_k = w_{sorted k}: only elements with k[0] <= k[1] (<= k[2]) are integrated here, and
-  // k_fill_permuted copies them to the others (2D: half, 3D: a sixth of the work).
   for (int r = 0; r + 1 < D; ++r)
     if (k[r] > k[r + 1]) return;
-  int dist = k[D - 1];
-  if (dist == 0) return;  // origin element: k_pyramid
-  const int qi = q_index(dist);
-  int off[kNumQ + 1] = {0, 4, 9, 17, 31, 51, 83};
-  const int q = off[qi + 1] - off[qi];
-  const double* xn = gn + off[qi];
-  const double* xw = gw + off[qi];
+  const int dist = k[D - 1];
+  if (dist <= kNear) return;
   const double mp = -0.5 * p;
-  double acc = 0.0;
-  if (D == 2) {
-    for (int i = 0; i < q; ++i) {
-      const double a = k[0] + xn[i];
-      double s = 0.0;
-      for (int j = 0; j < q; ++j) {
-        const double b = k[1] + xn[j];
-        s += xw[j] * pow(a * a + b * b, mp);
-      }
-      acc += xw[i] * s;
-    }
-  } else {
-    for (int i = 0; i < q; ++i) {
-      const double a = k[0] + xn[i];
-      double s1 = 0.0;
-      for (int j = 0; j < q; ++j) {
-        const double b = k[1] + xn[j];
-        const double ab = a * a + b * b;
-        double s2 = 0.0;
-        for (int l = 0; l < q; ++l) {
-          const double c = k[2] + xn[l];
-          s2 += xw[l] * pow(ab + c * c, mp);
-        }
-        s1 += xw[j] * s2;
-      }
-      acc += xw[i] * s1;
-    }
-  }
-  w[e] = acc;
+  w[e] = dist <= kMid ? far_element<D, 5, 13>(k, mp, g.x + rule_off(1), g.w + rule_off(1), s)
+                      : far_element<D, 4, 10>(k, mp, g.x + rule_off(0), g.w + rule_off(0), s);
 }
 
 // w[e] = w[index of the sorted coordinates of element e], for every element whose coordinates are
@@ -163,10 +233,10 @@ __global__ void k_fill_permuted(double* w, int N) {
 
 // pyramid reductions: out[0] = w_0 = d/(d-p) int_{[0,1]^(d-1)} (1+|s|^2)^(-p/2),
 // out[1] = W_D2 = d N^-alpha / alpha int_{[0,1]^(d-1)} (1+|s|^2)^(-(d+alpha)/2)   (h = 1)
-__global__ void k_pyramid(int d, double p, double alpha, int N, const double* __restrict__ gn,
-                          const double* __restrict__ gw, double* out, double* w) {
-  const int off = 51;  // offset of the 32-point rule in the node table
+__global__ void k_pyramid(int d, double p, double alpha, int N, GaussRules g, double* out, double* w) {
+  const int off = rule_off(5);  // the 32-point rule
   const int q = 32;
+  const double *gn = g.x, *gw = g.w;
   const int cnt = (d == 2) ? q : q * q;
   double s0 = 0.0, s1 = 0.0;
   for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
@@ -243,7 +313,8 @@ __global__ void k_assemble(const double* __restrict__ w, int N, double gamma, do
         for (int r = 0; r < D; ++r) unit = unit && k[r] <= 1;
         if (unit) kappa = (ksum == 1) ? ((D == 2) ? 1.0 : 5.0 / 3.0) : -1.0;
       }
-      const double a = ldexp(1.0, sigma - D) / pow(k2, 0.5 * gamma) * (WT + kappa * pyr[0]);
+      const double kg = gamma == 2.0 ? k2 : pow(k2, 0.5 * gamma);
+      const double a = ldexp(1.0, sigma - D) / kg * (WT + kappa * pyr[0]);
       coef[e] = a * hscale;
       contrib = ldexp(a, D - sigma);
     }
@@ -388,7 +459,7 @@ size_t coeffs_scratch_bytes(int d, int Nmax) {
   const size_t N1 = (size_t)Nmax + 1;
   const size_t nco = (d == 2) ? N1 * N1 : N1 * N1 * N1;
   const size_t nparts = (nco + 255) / 256;
-  return align256(nel * 8) + align256(nparts * 8) + align256(2 * kQTotal * 8) + 256;
+  return align256(nel * 8) + align256(nparts * 8) + 256;
 }
 
 cudaError_t coeffs_launch(int d, double alpha, double gamma, double h, int N, double* coef, void* scratch,
@@ -402,23 +473,26 @@ cudaError_t coeffs_launch(int d, double alpha, double gamma, double h, int N, do
   sp += align256(nel * 8);
   double* partial = reinterpret_cast<double*>(sp);
   sp += align256((size_t)nparts * 8);
-  double* gn = reinterpret_cast<double*>(sp);
-  double* gw = gn + kQTotal;
-  sp += align256(2 * kQTotal * 8);
   double* pyr = reinterpret_cast<double*>(sp);
   const double p = d + alpha - gamma;
   const double hscale = pow(h, -alpha);
-  k_gauss<<<1, 128, 0, s>>>(gn, gw);
-  const int bs = 256;
-  const unsigned gridw = (unsigned)((nel + bs - 1) / bs);
+  const GaussRules& g = gauss_rules();
+  FarSeries far;
+  far.c[0] = 1.0;
+  for (int n = 1; n < kFarTerms; ++n) far.c[n] = far.c[n - 1] * (-0.5 * p - (n - 1)) / n;
+  const int side = N < kNear + 1 ? N : kNear + 1;
+  const unsigned near = (unsigned)(d == 2 ? side * side : side * side * side);
+  const unsigned gridf = (unsigned)((nel + 127) / 128), gridw = (unsigned)((nel + 255) / 256);
   if (d == 2) {
-    k_element_weights<2><<<gridw, bs, 0, s>>>(w, N, p, gn, gw);
-    k_fill_permuted<2><<<gridw, bs, 0, s>>>(w, N);
+    k_elements_near<2><<<near, 128, 0, s>>>(w, N, side, p, g);
+    if (N > kNear + 1) k_elements_far<2><<<gridf, 128, 0, s>>>(w, N, p, g, far);
+    k_fill_permuted<2><<<gridw, 256, 0, s>>>(w, N);
   } else {
-    k_element_weights<3><<<gridw, bs, 0, s>>>(w, N, p, gn, gw);
-    k_fill_permuted<3><<<gridw, bs, 0, s>>>(w, N);
+    k_elements_near<3><<<near, 128, 0, s>>>(w, N, side, p, g);
+    if (N > kNear + 1) k_elements_far<3><<<gridf, 128, 0, s>>>(w, N, p, g, far);
+    k_fill_permuted<3><<<gridw, 256, 0, s>>>(w, N);
   }
-  k_pyramid<<<1, 256, 0, s>>>(d, p, alpha, N, gn, gw, pyr, w);
+  k_pyramid<<<1, 256, 0, s>>>(d, p, alpha, N, g, pyr, w);
   if (d == 2) k_assemble<2><<<nparts, 256, 0, s>>>(w, N, gamma, hscale, pyr, coef, partial);
   else k_assemble<3><<<nparts, 256, 0, s>>>(w, N, gamma, hscale, pyr, coef, partial);
   k_diag<<<1, 256, 0, s>>>(partial, nparts, d, pyr, hscale, coef);
