@@ -36,12 +36,19 @@ inline QExpLayout q_exp_layout(const Plan& p) {
   return l;
 }
 
+// A transform's output is stored below 2^57.5.
+template <int REM>
+constexpr int kQStore = 5 - kQDrop<REM>;
+
 __device__ __forceinline__ unsigned q_ord(int e) { return (unsigned)e ^ 0x80000000u; }
 __device__ __forceinline__ int q_unord(unsigned u) { return (int)(u ^ 0x80000000u); }
-// v 2^(e - top), e <= top
-__device__ __forceinline__ cq q_align(cq v, int e, int top) {
-  const int d = top - e > 63 ? 63 : top - e;
-  return {v.x >> d, v.y >> d};
+// v 2^(e - top), e <= top, rounded down or, with up, up.  Callers alternate up with the parity of a frequency
+// index along which a line's exponent (and so the offset of a rounding) is the same: the offset then sits at
+// the middle of the axis' embedding, outside the box, instead of adding up at its first point.
+__device__ __forceinline__ cq q_align(cq v, int e, int top, bool up) {
+  const int d = min(top - e, 63);
+  const unsigned c = up ? (1u << min(d, 31)) - 1u : 0u;
+  return {(v.x + c) >> d, (v.y + c) >> d};
 }
 
 #define FRLAP_Q_PROLOGUE(logLine)                                        \
@@ -107,20 +114,31 @@ __global__ void __launch_bounds__(512, 1)
   q_fft<-1, true, REM>(v, e, buf, logH, lane, tw, logH + 1, false, slots, si);
   line_sync<double>(logH);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = {v[m].x >> 1, v[m].y >> 1};
+  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = v[m];
   line_sync<double>(logH);
-  // Real-data split in place, one product per pair (see r2c_tile): with a' = Z/2, X[k] = s + W^k d,
-  // X[H-k] = conj(s - W^k d), s = a' + b', d = -i (a' - b'); stored over 64, below 2^57.5.
+  // Real-data split in place, one product per pair (see r2c_tile): X[k] = s + W^k d,
+  // X[H-k] = conj(s - W^k d), s = (a + b) / 2, d = -i (a - b) / 2; stored below 2^57.5, that is over 2^(6 - D),
+  // D = kQDrop.  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of the downward
+  // shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in a + b.
+  constexpr int D = kQDrop<REM>;
   for (int k = lane; k <= H / 2; k += G) {
     const int km = H - k;
     const cq a = buf[spad(k)];
     const cq b = conjg(buf[spad(km & (H - 1))]);
-    const cq s = a + b, t = q_cmul<false>(mul_i<-1>(a - b), FRLAP_GLD(tw + k));
-    const cq s4 = {s.x >> 4, s.y >> 4};
-    buf[spad(k)] = q_shr_round<2>(s4 + t);
-    if (k != km) buf[spad(km)] = conjg(q_shr_round<2>(s4 - t));
+    cq d, s;
+    if constexpr (D == 0) {
+      d = {(a.x >> 1) - (b.x >> 1), (a.y >> 1) - (b.y >> 1)};
+      s = {((a.x >> 2) + (b.x >> 2) + 4) >> 3, ((a.y >> 2) + (b.y >> 2) + 4) >> 3};
+    } else {
+      d = a - b;
+      d = {d.x << (D - 1), d.y << (D - 1)};
+      s = q_shr_even<5 - D>(a + b);
+    }
+    const cq t = q_cmul<false>(mul_i<-1>(d), FRLAP_GLD(tw + k));
+    buf[spad(k)] = q_shr_even<2>(s + t);
+    if (k != km) buf[spad(km)] = conjg(q_shr_even<2>(s - t));
   }
-  if (valid && lane == 0) FRLAP_GST(ex + line, e + 6);
+  if (valid && lane == 0) FRLAP_GST(ex + line, e + 6 - D);
   __syncthreads();
   const int logTL = __ffs(TL) - 1;
   const int lt = threadIdx.x & (TL - 1);
@@ -135,10 +153,10 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // Entries v[m], m < M, of a line that runs across lines of other exponents: v = line[lane + m G] aligned to
-// the largest, which it returns.
+// the largest, which it returns (up: see q_align).
 template <int M>
-__device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* ex, int lane, int G, int n, bool valid,
-                                              int logL, unsigned* slot) {
+__device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* ex, bool up, int lane, int G, int n,
+                                              bool valid, int logL, unsigned* slot) {
   int e[M];
   int top = kQZero;
 #pragma unroll
@@ -152,35 +170,60 @@ __device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* 
   for (int m = 0; m < M; ++m) top = max(top, e[m]);
   top = q_unord(q_reduce<true>(q_ord(top), logL, slot));
 #pragma unroll
-  for (int m = 0; m < M; ++m) v[m] = q_align(v[m], e[m], top);
+  for (int m = 0; m < M; ++m) v[m] = q_align(v[m], e[m], top, up);
   return top;
 }
 
-// The symbol product in two steps.  v <- lambda v 2^(1020 - el), el = lambda's exponent field: the product
-// takes lambda's mantissa, so it has full precision whatever lambda's range along the line.  top collects the
-// largest leading bit of the line's lambda v.
-__device__ __forceinline__ void q_times(cq& v, int& el, double lam, int& top) {
-  const int h = __double2hiint(lam);
-  el = (h >> 20) & 0x7ff;
-  long long mant = (long long)(((unsigned long long)((unsigned)(h & 0xfffff) | 0x100000u) << 32) |
-                               (unsigned)__double2loint(lam))
-                   << 9;  // 2^61 <= mant < 2^62
-  if (el == 0) mant = 0;
-  if (h < 0) mant = -mant;
-  const QHalf w = q_half(mant);
-  v = {q_rmul(q_half(v.x), w), q_rmul(q_half(v.y), w)};
-  // leading bit of |v| above bit 31 (rounded up by at most one), plus 127
-  const int pos = __float_as_int(__uint2float_rn(q_bits(v))) >> 23;
-  top = max(top, el + max(pos, 126));
+// Loads that stay where they are written (not merged with an earlier one of the same address).
+__device__ __forceinline__ unsigned q_ld_hi(const double* p) {
+#ifdef FRLAP_BOUNDS_CHECK
+  if (!bc_ok(p, 8)) return 0u;
+#endif
+  unsigned h;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(h) : "l"(reinterpret_cast<const unsigned*>(p) + 1));
+  return h;
 }
-// All entries to the line's common exponent, components below 2^58.
-__device__ __forceinline__ void q_rescale(cq* v, const int* el, int& e, int top, int logL, unsigned* slot) {
+__device__ __forceinline__ double q_ld(const double* p) {
+#ifdef FRLAP_BOUNDS_CHECK
+  if (!bc_ok(p, 8)) return 0.0;
+#endif
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
+// The symbol product v <- lambda v at a common exponent for the line, components below 2^58.  lambda enters by
+// its mantissa, so every entry has full precision whatever lambda's range along the line; the line's
+// exponent is what its largest |lambda_k| |v_k| needs.  lambda is positive: A is strictly diagonally dominant
+// and so is its circulant embedding (a zero from underflow acts as 2^-1022).
+// lrow[idx(m)] is entry m's lambda; its words are read twice (the second time from L1), since held over the
+// reduction they spill.
+template <typename I>
+__device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict__ lrow, I idx, int logL,
+                                         unsigned* slot) {
+  int top = 0;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const unsigned h = q_ld_hi(lrow + idx(m));
+    // leading bit of |v| above bit 31 (the conversion rounds it up by at most one), plus 127
+    const int pos = __float_as_int(__uint2float_rn(q_bits(v[m]))) >> 23;
+    top = max(top, (int)(h >> 20) + max(pos, 126));
+  }
   top = (int)q_reduce<true>((unsigned)top, logL, slot);
 #pragma unroll
   for (int m = 0; m < 16; ++m) {
-    const int s = el[m] + 152 - top;  // leading bits to bit 57 or below
-    const int sl = min(max(s, 0), 31), sr = min(max(-s, 0), 63);
-    v[m] = s >= 0 ? cq{q_shl(v[m].x, sl), q_shl(v[m].y, sl)} : cq{v[m].x >> sr, v[m].y >> sr};
+    // lambda v = (mant v / 2^64) 2^(el - 1020), 2^61 <= mant < 2^62, and |v| 2^(el - top + 127) < 2^33: the
+    // shift s = el - top + 152 brings the product below 2^58.  A right shift is one of the mantissa (its
+    // dropped bits weigh less than a unit of the product), a left one is one of v.
+    const double lam = q_ld(lrow + idx(m));
+    const unsigned h = (unsigned)__double2hiint(lam), l = (unsigned)__double2loint(lam);
+    const int s = (int)(h >> 20) - top + 152;
+    unsigned long long mant =
+        ((unsigned long long)__funnelshift_l(l, (h & 0xfffffu) | 0x100000u, 9) << 32) | (l << 9);
+    mant >>= min(max(-s, 0), 63);
+    const int sl = min(max(s, 0), 31);
+    const QHalf w = q_half((long long)mant);
+    v[m] = {q_rmul(q_half(q_shl(v[m].x, sl)), w), q_rmul(q_half(q_shl(v[m].y, sl)), w)};
   }
   e += top - 1172;
 }
@@ -210,28 +253,20 @@ __global__ void __launch_bounds__(512, 1)
   const int c = valid ? col : 0;
   int si = 0;
   cq v[16];
-  const int* exi = ex_in + (map.d == 2 ? 0 : (size_t)(c >> map.logPy) * nz);
-  int e = q_load_aligned<8>(v, data + (size_t)c * ld, exi, lane, G, n, valid, logP, slots + si);
+  const int kx = map.d == 2 ? c : c >> map.logPy;
+  const int* exi = ex_in + (map.d == 2 ? 0 : (size_t)kx * nz);
+  int e = q_load_aligned<8>(v, data + (size_t)c * ld, exi, kx & 1, lane, G, n, valid, logP, slots + si);
   ++si;
   q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
   const int ky = c & (map.Py - 1);
   const double* lrow = map.d == 2 ? lam + (size_t)c * map.Hy1
-                                  : lam + ((size_t)(c >> map.logPy) * map.Hy1 + min(ky, map.Py - ky)) * map.Hz1;
-  {
-    int el[16];
-    int top = 0;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int k = lane + m * G;
-      q_times(v[m], el[m], ld_stream(&lrow[min(k, P - k)]), top);
-    }
-    q_rescale(v, el, e, top, logP, slots + si);
-    ++si;
-  }
+                                  : lam + ((size_t)kx * map.Hy1 + min(ky, map.Py - ky)) * map.Hz1;
+  q_symbol(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, logP, slots + si);
+  ++si;
   q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  if (valid && lane == 0) FRLAP_GST(ex_out + col, e + 5);
+  if (valid && lane == 0) FRLAP_GST(ex_out + col, e + kQStore<REM>);
 #pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = q_shr_round<5>(v[m]);
+  for (int m = 0; m < 8; ++m) v[m] = q_shr_even<kQStore<REM>>(v[m]);
   store_line(v, data, ncols, n, ld, logP, TL);
 }
 
@@ -264,7 +299,7 @@ __global__ void __launch_bounds__(512, 1)
   cq* tline = tmp + (size_t)(valid ? col : 0) * ld;
   int si = 0;
   cq v[16];
-  int e = q_load_aligned<16>(v, line, ex_in, lane, G, n, valid, logL, slots + si);
+  int e = q_load_aligned<16>(v, line, ex_in, col & 1, lane, G, n, valid, logL, slots + si);
   ++si;
   if constexpr (ODD) {  // times W_P^j: from below 2^62.5 (a shift by 4) back to below 2^58.5
 #pragma unroll
@@ -272,40 +307,38 @@ __global__ void __launch_bounds__(512, 1)
       v[m] = q_cmul<false>(cq{q_shl(v[m].x, 4), q_shl(v[m].y, 4)}, FRLAP_GLD(tw + lane + m * G));
   }
   q_fft<-1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, false, slots, si);
-  // the half's symbol entries are every second one: gather through a strided row
+  // the half's symbol entries are every second one
   const double* lrow = lam + (size_t)(valid ? col : 0) * Hy1;
-  {
-    int el[16];
-    int top = 0;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int k = 2 * (lane + m * G) + (ODD ? 1 : 0);
-      q_times(v[m], el[m], ld_stream(&lrow[min(k, P - k)]), top);
-    }
-    q_rescale(v, el, e, top, logL, slots + si);
-    ++si;
-  }
+  q_symbol(
+      v, e, lrow,
+      [&](int m) {
+        const int k = 2 * (lane + m * G) + (ODD ? 1 : 0);
+        return min(k, P - k);
+      },
+      logL, slots + si);
+  ++si;
   q_fft<1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, true, slots, si);
   if (!valid) return;
   if constexpr (!ODD) {
-    if (lane == 0) FRLAP_GST(ex_tmp + col, e + 5);
+    if (lane == 0) FRLAP_GST(ex_tmp + col, e + kQStore<REM>);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int j = lane + m * G;
-      if (j < n) FRLAP_GST(tline + j, q_shr_round<5>(v[m]));
+      if (j < n) FRLAP_GST(tline + j, q_shr_even<kQStore<REM>>(v[m]));
     }
   } else {
-    // y_j = even_j + W_P^-j odd_j: magnitudes below 2^58 each at exponents et and e + 5
+    // y_j = even_j + W_P^-j odd_j, magnitudes below 2^58 each at exponents et and eo: the odd half, below
+    // 2^59.5, up by 2 before its product (which divides by 16)
     const int et = FRLAP_GLD(ex_tmp + col);
-    const int eo = e + 5;
+    const int eo = e + 2;
     const int top = max(et, eo);
     if (lane == 0) FRLAP_GST(ex_out + col, top + 1);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int j = lane + m * G;
       if (j < n) {
-        const cq o = q_shr_round<1>(q_cmul<true>(v[m], FRLAP_GLD(tw + j)));
-        FRLAP_GST(line + j, q_shr_round<1>(q_align(o, eo, top) + q_align(FRLAP_GLD(tline + j), et, top)));
+        const cq o = q_cmul<true>(cq{v[m].x << 2, v[m].y << 2}, FRLAP_GLD(tw + j));
+        FRLAP_GST(line + j, q_shr_even<1>(q_align(o, eo, top, col & 1) + q_align(FRLAP_GLD(tline + j), et, top, col & 1)));
       }
     }
   }
@@ -338,14 +371,14 @@ __global__ void __launch_bounds__(512, 1)
   int si = 0;
   cq v[16];
   // rows (z, y) of this line z: exponents ex_in[z n + y]
-  int e = q_load_aligned<8>(v, in + g * gin + (size_t)c * ldi, ex_in + (size_t)c * n, lane, G, n, valid, logP,
-                            slots + si);
+  int e = q_load_aligned<8>(v, in + g * gin + (size_t)c * ldi, ex_in + (size_t)c * n, g & 1, lane, G, n, valid,
+                            logP, slots + si);
   ++si;
   q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + 5);
+  if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + kQStore<REM>);
   line_sync<double>(logP);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = q_shr_round<5>(v[m]);
+  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = q_shr_even<kQStore<REM>>(v[m]);
   __syncthreads();
   const int logTL = __ffs(TL) - 1;
   const int lt = threadIdx.x & (TL - 1);
@@ -395,15 +428,15 @@ __global__ void __launch_bounds__(512, 1)
   int si = 1;
   cq v[16];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e);
+  for (int m = 0; m < 16; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
   q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
   if (line < nlines) {
-    if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + 5);
+    if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + kQStore<REM>);
     cq* dst = out + g * gout + (size_t)line * ldo;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int i = lane + m * G;
-      if (i < n) FRLAP_GST(dst + i, q_shr_round<5>(v[m]));
+      if (i < n) FRLAP_GST(dst + i, q_shr_even<kQStore<REM>>(v[m]));
     }
   }
 }
@@ -453,9 +486,9 @@ __global__ void __launch_bounds__(512, 1)
     const int k = lane + j * G;
     if (k <= H / 2) {
       const int km = H - k;
-      const cq xk = q_align(buf[spad(k)], ea[j], e);
-      const cq b = conjg(q_align(buf[spad(km)], eb[j], e));
-      const cq A = q_shr_round<2>(xk + b), d = xk - b;
+      const cq xk = q_align(buf[spad(k)], ea[j], e, k & 1);
+      const cq b = conjg(q_align(buf[spad(km)], eb[j], e, k & 1));
+      const cq A = q_shr_even<2>(xk + b), d = xk - b;
       const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, FRLAP_GLD(tw + k)));
       buf[spad(k)] = A + iT;
       if (k != km && km != H) buf[spad(km)] = conjg(A - iT);
@@ -503,8 +536,9 @@ __global__ void __launch_bounds__(512, 1)
   int si = 0;
   cq v[16];
   // exponents: 2D ex[i] for every column; 3D ex[(col / P_y) n + i]
-  int e = q_load_aligned<8>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)(c / cols_per) * n : 0), lane, G, n,
-                            valid, logP, slots + si);
+  const int kx = cols_per ? c / cols_per : c;
+  int e = q_load_aligned<8>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)kx * n : 0), kx & 1, lane, G, n, valid,
+                            logP, slots + si);
   ++si;
   q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
   if (!valid) return;
@@ -557,9 +591,9 @@ __global__ void __launch_bounds__(512, 1)
   for (int m = 0; m < 16; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
   int e = qs.e;
   q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  if (valid && lane == 0) FRLAP_GST(ex + col, e + 5);
+  if (valid && lane == 0) FRLAP_GST(ex + col, e + kQStore<REM>);
 #pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = q_shr_round<5>(v[m]);
+  for (int m = 0; m < 8; ++m) v[m] = q_shr_even<kQStore<REM>>(v[m]);
   store_line(v, out, ncols, n, ldo, logP, TL);
 }
 

@@ -41,31 +41,33 @@ __host__ __device__ __forceinline__ QHalf q_half(long long a) {
 __device__ __forceinline__ long long q_wide(int a, int b) { return (long long)a * b; }
 
 // Products a w / 2^64 as a1 w1 + (a1 w0 + a0 w1) / 2^32 on the signed halves: one 64-bit and two high
-// 32-bit products (a0 w0 stays below the unit).  A high product rounds down, by 1/2 in the mean; a
-// component that adds k of them more than it subtracts gets + k / 2.  (Summing the cross products in 64
-// bits and rounding once is slightly more exact, 6.8e-17 against 7.3e-17, but takes multiply-adds with
-// 64-bit addends, 5.5 cycles each against 4: 3.04 against 2.58 ps.)
+// 32-bit products (a0 w0 stays below the unit).  A high product rounds down; a sum takes them in pairs, one
+// as p and one as -(-p), which rounds up, so that the offsets cancel and zero stays zero.  (Summing the cross
+// products in 64 bits and rounding once is no more exact and takes multiply-adds with 64-bit addends, 5.5
+// cycles each against 4: 3.04 against 2.72 ps per point and stage.)
 
 // a w (CONJ = false) or a conj(w), over 16 (w: 60 fraction bits)
 template <bool CONJ>
 __device__ __forceinline__ cq q_cmul(cq a, int4 w) {
   const QHalf x = q_half(a.x), y = q_half(a.y);
-  const int nih = -w.z;
-  const int xr = __mulhi(x.h, w.y) + __mulhi(x.l, w.x), yi = __mulhi(y.h, w.w) + __mulhi(y.l, w.z);
-  const int xi = __mulhi(x.h, w.w) + __mulhi(x.l, w.z), yr = __mulhi(y.h, w.y) + __mulhi(y.l, w.x);
+  const int nrh = -w.x, nih = -w.z;
   cq r;
   if constexpr (!CONJ) {
-    r.x = q_wide(x.h, w.x) + (q_wide(y.h, nih) + (long long)(xr - yi));
-    r.y = q_wide(x.h, w.z) + (q_wide(y.h, w.x) + (long long)(xi + yr + 2));
+    const int mx = __mulhi(x.h, w.y) - __mulhi(x.l, nrh) - __mulhi(y.h, w.w) + __mulhi(y.l, nih);
+    const int my = __mulhi(x.h, w.w) - __mulhi(x.l, nih) + __mulhi(y.h, w.y) - __mulhi(y.l, nrh);
+    r.x = q_wide(x.h, w.x) + (q_wide(y.h, nih) + (long long)mx);
+    r.y = q_wide(x.h, w.z) + (q_wide(y.h, w.x) + (long long)my);
   } else {
-    r.x = q_wide(x.h, w.x) + (q_wide(y.h, w.z) + (long long)(xr + yi + 2));
-    r.y = q_wide(y.h, w.x) + (q_wide(x.h, nih) + (long long)(yr - xi));
+    const int mx = __mulhi(x.h, w.y) - __mulhi(x.l, nrh) + __mulhi(y.h, w.w) - __mulhi(y.l, nih);
+    const int my = __mulhi(y.h, w.y) - __mulhi(y.l, nrh) - __mulhi(x.h, w.w) + __mulhi(x.l, nih);
+    r.x = q_wide(x.h, w.x) + (q_wide(y.h, w.z) + (long long)mx);
+    r.y = q_wide(x.h, nih) + (q_wide(y.h, w.x) + (long long)my);
   }
   return r;
 }
 // a w / 2^64 for a real w
 __device__ __forceinline__ long long q_rmul(QHalf a, QHalf w) {
-  return q_wide(a.h, w.h) + (long long)(__mulhi(a.h, w.l) + __mulhi(a.l, w.h) + 1);
+  return q_wide(a.h, w.h) + (long long)(__mulhi(a.h, w.l) - __mulhi(a.l, -w.h));
 }
 
 // Constants of the 8- and 16-point DFTs with 64 fraction bits: 1 - cos(pi/8), sin(pi/8), 1 - 1/sqrt 2
@@ -78,7 +80,7 @@ constexpr int qlo(long long w) { return (int)(w & 0xffffffffLL); }
 __device__ __forceinline__ long long q_r2(long long a) {
   const QHalf t = q_half(a);
   constexpr int h = qhi(kQ1mR2), l = qlo(kQ1mR2);
-  return a + (q_wide(t.h, -h) - (long long)(__mulhi(t.h, l) + __mulhi(t.l, h) + 1));
+  return a + (q_wide(t.h, -h) - (long long)(__mulhi(t.h, l) - __mulhi(t.l, -h)));
 }
 // a cos(pi/8) + b sin(pi/8) and a cos(pi/8) - b sin(pi/8)
 __device__ __forceinline__ long long q_cs_add(long long a, long long b) {
@@ -90,7 +92,7 @@ __device__ __forceinline__ long long q_cs_add(long long a, long long b) {
 __device__ __forceinline__ long long q_cs_sub(long long a, long long b) {
   const QHalf s = q_half(a), t = q_half(b);
   constexpr int ch = qhi(kQ1mC1), cl = qlo(kQ1mC1), sh = qhi(kQS1), sl = qlo(kQS1);
-  const int m = __mulhi(t.h, sl) + __mulhi(t.l, sh) + __mulhi(s.h, cl) + __mulhi(s.l, ch) + 2;
+  const int m = (__mulhi(t.h, sl) - __mulhi(t.l, -sh)) + (__mulhi(s.h, cl) - __mulhi(s.l, -ch));
   return a + (q_wide(s.h, -ch) + (q_wide(t.h, -sh) - (long long)m));
 }
 // v W_16^m, m = 1, 2, 3, 6, 9 (W = exp(SIGN 2 pi i / 16))
@@ -221,6 +223,17 @@ __device__ __forceinline__ cq q_shr_round(cq a) {
   return {q_shr_round<SH>(a.x), q_shr_round<SH>(a.y)};
 }
 
+// To nearest, ties to even where few bits go: ties are frequent there, and rounding them all one way puts
+// the same offset on every bin of a spectrum, an error concentrated at one grid point.
+template <int SH>
+__device__ __forceinline__ long long q_shr_even(long long a) {
+  return SH >= 4 ? q_shr_round<SH>(a) : (a + ((1LL << (SH - 1)) - 1 + ((a >> SH) & 1))) >> SH;
+}
+template <int SH>
+__device__ __forceinline__ cq q_shr_even(cq a) {
+  return {q_shr_even<SH>(a.x), q_shr_even<SH>(a.y)};
+}
+
 // ---- double <-> fixed point.  Scaling by a power of two is an addition to the exponent field.
 
 // Exponents that mark a line with a non-finite entry, and a line of zeros: further stages shift an
@@ -295,8 +308,13 @@ __device__ __forceinline__ void q_last_stage(cq* v, int lane, int G, const int4*
   }
 }
 
+// Bits that a line's transform of log2 length = REM mod 4 ends below 2^62.5: a last stage of radix 2 or 4
+// grows by that, but its products divide by 16.
+template <int REM>
+constexpr int kQDrop = REM == 1 ? 3 : REM == 2 ? 2 : 0;
+
 // As fft_regs: v[m] = x[lane + m G] on entry (components below 2^58), X[lane + m G] on exit (magnitudes
-// below 2^62.5); e, the line's exponent, follows.  ZIN: v[8..15] are zero.  slots: the line's reduction
+// below 2^(62.5 - kQDrop)); e, the line's exponent, follows.  ZIN: v[8..15] are zero.  slots: the line's reduction
 // words, used from index si on.
 template <int SIGN, bool ZIN, int REM>
 __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
