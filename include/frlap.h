@@ -377,7 +377,7 @@ frlap_status frlap_allen_cahn_batch(int nbatch, const frlap_plan* const* plans, 
                                     void* d_work, void* stream);
 
 /* Process-wide cap on the passes of the graph-launched loops: the conditional WHILE
- * node of frlap_pcg_solve's CG (after its first 8 iterations) and of
+ * node of frlap_pcg_solve's CG (after its first 8 iterations; 16 with a preconditioner and no limit) and of
  * frlap_allen_cahn_batch.  Each loop stops after min(its own bound, max_passes)
  * passes; a loop that stops there with work left returns FRLAP_ETIMEOUT, leaving
  * the context usable.  0 (the default) keeps the loops' own bounds.  For callers

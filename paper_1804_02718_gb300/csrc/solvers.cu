@@ -22,11 +22,14 @@ namespace frlap {
 
 namespace {
 
-constexpr int kBlocks = 2 * 152;  // grid of the vector kernels: two CTAs per SM (four measured slower)
+constexpr int kBlocks = 2 * 152;  // largest grid of the vector kernels: two CTAs per SM (four measured slower)
 constexpr int kThreads = 512;
-// grid for n elements: two CTAs per SM, fewer for short vectors (the reductions use gridDim.x)
+// CTA size and grid for n elements (the reductions use gridDim.x).  A CTA's FP64 tree costs each of its warps
+// five additions at 76 cycles, so a short vector takes CTAs of 128 threads, one warp per SM sub-partition,
+// with up to four elements a thread: 127^2 k_cg_update 9.2 -> 6.1 us, k_cg_pq 7.2 -> 4.8 us.
+inline unsigned vthreads(size_t n) { return n <= (size_t)kBlocks * 128 * 4 ? 128u : (unsigned)kThreads; }
 inline unsigned vgrid(size_t n) {
-  const size_t b = (n + kThreads - 1) / kThreads;
+  const size_t t = vthreads(n), b = (n + t - 1) / t;
   return (unsigned)(b < 1 ? 1 : (b > (size_t)kBlocks ? (size_t)kBlocks : b));
 }
 
@@ -58,18 +61,22 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return t;  // valid in thread 0
 }
 
-// Two block sums, then the last block to arrive reduces all partials in block order.
+// NS = 1 or 2 block sums, then the last block to arrive reduces all partials in block order.
 // Returns true in thread 0 of the last block, with the totals in *ta, *tb.
-__device__ __forceinline__ bool grid_sum2(double a, double b, double* partials, unsigned* counter, double* ta,
+template <int NS>
+__device__ __forceinline__ bool grid_sum(double a, double b, double* partials, unsigned* counter, double* ta,
                                           double* tb) {
   __shared__ double red[32];
   __shared__ bool is_last;
   const double sa = block_sum(a, red);
-  __syncthreads();
-  const double sb = block_sum(b, red);
+  double sb = 0.0;
+  if (NS == 2) {
+    __syncthreads();
+    sb = block_sum(b, red);
+  }
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = sa;
-    partials[gridDim.x + blockIdx.x] = sb;
+    if (NS == 2) partials[gridDim.x + blockIdx.x] = sb;
     __threadfence();
     is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
@@ -78,15 +85,18 @@ __device__ __forceinline__ bool grid_sum2(double a, double b, double* partials, 
   double va = 0.0, vb = 0.0;
   for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
     va += *((volatile double*)&partials[i]);
-    vb += *((volatile double*)&partials[gridDim.x + i]);
+    if (NS == 2) vb += *((volatile double*)&partials[gridDim.x + i]);
   }
   __syncthreads();
   const double xa = block_sum(va, red);
-  __syncthreads();
-  const double xb = block_sum(vb, red);
+  double xb = 0.0;
+  if (NS == 2) {
+    __syncthreads();
+    xb = block_sum(vb, red);
+  }
   if (threadIdx.x == 0) {
     *ta = xa;
-    *tb = xb;
+    if (NS == 2) *tb = xb;
     *counter = 0u;
   }
   return threadIdx.x == 0;
@@ -128,7 +138,7 @@ __global__ void k_cg_init(const T* __restrict__ f, const T* __restrict__ x, cons
     b += fi * fi;
   }
   double ta, tb;
-  if (grid_sum2(a, b, partials, &S->counter, &ta, &tb)) {
+  if (grid_sum<2>(a, b, partials, &S->counter, &ta, &tb)) {
     S->rr = ta;
     S->fnorm2 = tb;
     S->tol2 = rtol * rtol * tb;
@@ -170,7 +180,7 @@ __global__ void k_pcg_start(const T* __restrict__ r, const TP* __restrict__ zp, 
     }
   }
   double ta, tb;
-  if (grid_sum2((double)a, 0.0, partials, &S->counter, &ta, &tb)) {
+  if (grid_sum<1>((double)a, 0.0, partials, &S->counter, &ta, &tb)) {
     S->rz = ta;
     if (zp && !(ta > 0.0) && !S->done) {
       S->status = isfinite(ta) ? FRLAP_EBREAKDOWN : FRLAP_ENAN;
@@ -212,7 +222,7 @@ __global__ void k_cg_pq(const T* __restrict__ p, T* q, size_t n, double* partial
     }
   }
   double ta, tb;
-  if (grid_sum2((double)a, 0.0, partials, &S->counter, &ta, &tb)) {
+  if (grid_sum<1>((double)a, 0.0, partials, &S->counter, &ta, &tb)) {
     S->pq = ta;
     if (!(ta > 0.0) || !isfinite(ta)) {
       S->status = isfinite(ta) ? FRLAP_EBREAKDOWN : FRLAP_ENAN;
@@ -258,7 +268,7 @@ __global__ void k_cg_update(T* x, T* r, const T* __restrict__ p, const T* __rest
     }
   }
   double ta, tb;
-  if (grid_sum2((double)a, 0.0, partials, &S->counter, &ta, &tb)) {
+  if (grid_sum<1>((double)a, 0.0, partials, &S->counter, &ta, &tb)) {
     if (!precond) {
       S->beta = ta / S->rz;
       S->rz = ta;
@@ -306,7 +316,7 @@ __global__ void k_pcg_beta(const T* __restrict__ r, const TP* __restrict__ zp, c
     }
   }
   double ta, tb;
-  if (grid_sum2((double)a, (double)b, partials, &S->counter, &ta, &tb)) {
+  if (grid_sum<2>((double)a, (double)b, partials, &S->counter, &ta, &tb)) {
     if (!(ta > 0.0) || !isfinite(ta)) {
       S->status = isfinite(ta) ? FRLAP_EBREAKDOWN : FRLAP_ENAN;
       S->done = 1;
@@ -317,9 +327,23 @@ __global__ void k_pcg_beta(const T* __restrict__ r, const TP* __restrict__ zp, c
   }
 }
 
+// Loop control of the graph-launched iterations, in the last kernel of the body: another pass while the solve
+// runs, after at most max_passes passes (0: a plain launch, no loop).
+struct LoopControl {
+  unsigned max_passes;
+  cudaGraphConditionalHandle h;
+};
+__device__ __forceinline__ void loop_control(CgState* S, const LoopControl& lc) {
+  if (lc.max_passes == 0u || blockIdx.x != 0 || threadIdx.x != 0) return;
+  const unsigned c = S->passes + 1u;
+  S->passes = c;
+  cudaGraphSetConditional(lc.h, (!S->done && c < lc.max_passes) ? 1u : 0u);
+}
+
 // p = z + beta p (z: the preconditioner output, or r itself)
 template <typename T, typename TZ>
-__global__ void k_cg_dir(const TZ* __restrict__ z, T* p, size_t n, const CgState* S) {
+__global__ void k_cg_dir(const TZ* __restrict__ z, T* p, size_t n, CgState* S, LoopControl lc) {
+  loop_control(S, lc);
   if (S->done) return;
   using A = acc_t<T>;
   const A b = (A)S->beta;
@@ -353,13 +377,6 @@ __global__ void k_set_state(CgState* S, double sigma, double s) {
   S->passes = 0u;
 }
 
-// loop control of the graph-launched CG: another pass while the solve runs (bounded)
-__global__ void k_cg_control(CgState* S, unsigned max_passes, cudaGraphConditionalHandle h) {
-  const unsigned c = S->passes + 1u;
-  S->passes = c;
-  cudaGraphSetConditional(h, (!S->done && c < max_passes) ? 1u : 0u);
-}
-
 // true residual norms: out[0] = ||f - (sigma x + s q)||^2, out[1] = ||f||^2
 __global__ void k_resid(const double* __restrict__ f, const double* __restrict__ x, const double* __restrict__ q,
                         size_t n, double sigma, double s, double* partials, unsigned* counter, double* out,
@@ -372,7 +389,7 @@ __global__ void k_resid(const double* __restrict__ f, const double* __restrict__
     b += f[i] * f[i];
   }
   double ta, tb;
-  if (grid_sum2(a, b, partials, counter, &ta, &tb)) {
+  if (grid_sum<2>(a, b, partials, counter, &ta, &tb)) {
     out[0] = ta;
     out[1] = tb;
     if (rnorm_scale) *rnorm_scale = sqrt(ta);
@@ -548,29 +565,29 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
   k_set_state<<<1, 1, 0, st>>>(S, sigma, s);
   FRLAP_LAUNCH_CHECK("k_set_state");
   if (use_x0) {
-    // use_x0 = 1: the plan's engine; 2: native FP64 (a restart, which must see the true residual)
-    cudaError_t e = use_x0 == 2 ? apply_residual<T>(p, x, q, b.awork, st) : apply_T<T>(p, x, q, b.awork, st, nullptr);
+    // use_x0 = 1: A x by the plan's engine; 2: a restart, q already holds A x from true_residual (this workspace)
+    const cudaError_t e = use_x0 == 2 ? cudaSuccess : apply_T<T>(p, x, q, b.awork, st, nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "apply (initial residual)");
   }
   float* r32 = (mu && sizeof(T) == 8) ? b.r32 : nullptr;  // FP64 solves hand the preconditioner an FP32 r
-  k_cg_init<T><<<vgrid(n), kThreads, 0, st>>>(f, x, q, r, n, b.partials, S, rtol, use_x0, r32);
+  k_cg_init<T><<<vgrid(n), vthreads(n), 0, st>>>(f, x, q, r, n, b.partials, S, rtol, use_x0, r32);
   FRLAP_LAUNCH_CHECK("k_cg_init");
   if (mu) {
     cudaError_t e = precondition<T>(p, b, mu, odd, st);
     if (e != cudaSuccess) return cuda_fail(e, "preconditioner");
-    k_pcg_start<T, float><<<vgrid(n), kThreads, 0, st>>>(r, b.z32, pv, n, b.partials, S);
+    k_pcg_start<T, float><<<vgrid(n), vthreads(n), 0, st>>>(r, b.z32, pv, n, b.partials, S);
   } else {
-    k_pcg_start<T, T><<<vgrid(n), kThreads, 0, st>>>(r, nullptr, pv, n, b.partials, S);
+    k_pcg_start<T, T><<<vgrid(n), vthreads(n), 0, st>>>(r, nullptr, pv, n, b.partials, S);
   }
   FRLAP_LAUNCH_CHECK("k_pcg_start");
   if (snap && nsnap > 0) FRLAP_CUDA_TRY(cudaMemcpyAsync(snap, x, n * sizeof(T), cudaMemcpyDeviceToDevice, st));
   const int* done = &S->done;
   // one iteration on stream `ss`; the snapshot copy (training pairs) needs the host's count
-  auto iteration = [&](cudaStream_t ss, int it) -> cudaError_t {
+  auto iteration = [&](cudaStream_t ss, int it, LoopControl lc = LoopControl{}) -> cudaError_t {
     cudaError_t e = apply_T<T>(p, pv, q, b.awork, ss, done);
     if (e != cudaSuccess) return e;
-    k_cg_pq<T><<<vgrid(n), kThreads, 0, ss>>>(pv, q, n, b.partials, S);
-    k_cg_update<T><<<vgrid(n), kThreads, 0, ss>>>(x, r, pv, q, n, b.partials, S, maxit, mu != nullptr, r32);
+    k_cg_pq<T><<<vgrid(n), vthreads(n), 0, ss>>>(pv, q, n, b.partials, S);
+    k_cg_update<T><<<vgrid(n), vthreads(n), 0, ss>>>(x, r, pv, q, n, b.partials, S, maxit, mu != nullptr, r32);
     if (snap && it + 1 < nsnap) {
       e = cudaMemcpyAsync(snap + (size_t)(it + 1) * n, x, n * sizeof(T), cudaMemcpyDeviceToDevice, ss);
       if (e != cudaSuccess) return e;
@@ -578,16 +595,17 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
     if (mu) {
       e = precondition<T>(p, b, mu, odd, ss);
       if (e != cudaSuccess) return e;
-      k_pcg_beta<T, float><<<vgrid(n), kThreads, 0, ss>>>(r, b.z32, q, n, b.partials, S);
-      k_cg_dir<T, float><<<vgrid(n), kThreads, 0, ss>>>(b.z32, pv, n, S);
+      k_pcg_beta<T, float><<<vgrid(n), vthreads(n), 0, ss>>>(r, b.z32, q, n, b.partials, S);
+      k_cg_dir<T, float><<<vgrid(n), vthreads(n), 0, ss>>>(b.z32, pv, n, S, lc);
     } else {
-      k_cg_dir<T, T><<<vgrid(n), kThreads, 0, ss>>>(r, pv, n, S);
+      k_cg_dir<T, T><<<vgrid(n), vthreads(n), 0, ss>>>(r, pv, n, S, lc);
     }
     return cudaGetLastError();
   };
-  // The first iterations run as plain launches; when the solve goes on (and takes no
-  // snapshots), the rest runs as one CUDA-graph launch: a conditional WHILE node whose body
-  // is one iteration plus k_cg_control, which ends the loop once the update kernel has set
+  // The first iterations run as plain launches, eight at a time (a preconditioned solve, which takes 7 to 16
+  // as a rule, gets a second eight, cheaper than building the graph, unless a pass limit is set); when the solve goes on (and takes
+  // no snapshots), the rest runs as one CUDA-graph launch: a conditional WHILE node whose body
+  // is one iteration, whose last kernel (loop_control) ends the loop once the update kernel has set
   // `done` (converged, breakdown or maxit), and after at most maxit + 2 passes regardless.
   const int chunk = 8;
   int launched = 0;
@@ -601,7 +619,7 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
     FRLAP_CUDA_TRY(cudaStreamSynchronize(st));
     if (hS->done) return FRLAP_OK;
     if (launched > maxit + chunk) return FRLAP_OK;  // cannot happen: the update kernel stops at maxit
-    if (!snap) break;
+    if (!snap && launched >= (mu && loop_pass_limit() == 0u ? 2 * chunk : chunk)) break;
   }
   cudaStream_t cs = nullptr;
   cudaGraph_t graph = nullptr;
@@ -621,11 +639,7 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
     e = cudaStreamBeginCaptureToGraph(cs, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                       cudaStreamCaptureModeRelaxed);
   if (e == cudaSuccess) {
-    cudaError_t eb = iteration(cs, launched);
-    if (eb == cudaSuccess) {
-      k_cg_control<<<1, 1, 0, cs>>>(S, capped_passes((unsigned)maxit + 2u), h);
-      eb = cudaGetLastError();
-    }
+    const cudaError_t eb = iteration(cs, launched, LoopControl{capped_passes((unsigned)maxit + 2u), h});
     cudaGraph_t captured = nullptr;
     e = cudaStreamEndCapture(cs, &captured);
     if (eb != cudaSuccess) e = eb;
@@ -660,7 +674,7 @@ static frlap_status true_residual(const Plan& p, const double* f, const double* 
                            : apply64(p, x, q, b.awork, st, nullptr);
   if (e != cudaSuccess) return cuda_fail(e, "apply (true residual)");
   double* out = &S->alpha;  // reuse two scalar slots (alpha, beta) for the norms
-  k_resid<<<vgrid(p.M), kThreads, 0, st>>>(f, x, q, p.M, sigma, s, b.partials, &S->counter, out, rvec, rnorm_dev);
+  k_resid<<<vgrid(p.M), vthreads(p.M), 0, st>>>(f, x, q, p.M, sigma, s, b.partials, &S->counter, out, rvec, rnorm_dev);
   FRLAP_LAUNCH_CHECK("k_resid");
   double h[2];
   FRLAP_CUDA_TRY(cudaMemcpyAsync(h, out, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -693,7 +707,7 @@ frlap_status cg_pairs_impl(const Plan& p, const double* f, int K, double rtol, d
   const int np = hS.iters < K ? hS.iters : K;
   for (int j = 0; j < np; ++j) {
     double* Ej = E + (size_t)j * p.M;
-    k_err_from_snap<<<vgrid(p.M), kThreads, 0, st>>>(Ej, x, p.M);
+    k_err_from_snap<<<vgrid(p.M), vthreads(p.M), 0, st>>>(Ej, x, p.M);
     FRLAP_LAUNCH_CHECK("k_err_from_snap");
     cudaError_t e = apply64(p, Ej, R + (size_t)j * p.M, b.awork, st, nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "apply (training pairs)");
@@ -737,8 +751,8 @@ frlap_status pcg_solve_impl(const Plan& p, const double* f, double* x, double rt
   const CgBufs b = carve(p, work, 8);
   unsigned long long* slot = reinterpret_cast<unsigned long long*>(&b.S->alpha);  // alpha, beta: two slots
   FRLAP_CUDA_TRY(cudaMemsetAsync(slot, 0, 2 * sizeof(unsigned long long), st));
-  k_maxabs<<<vgrid(p.M), kThreads, 0, st>>>(f, p.M, slot);
-  k_maxabs<<<vgrid(p.M), kThreads, 0, st>>>(x, p.M, slot + 1);
+  k_maxabs<<<vgrid(p.M), vthreads(p.M), 0, st>>>(f, p.M, slot);
+  k_maxabs<<<vgrid(p.M), vthreads(p.M), 0, st>>>(x, p.M, slot + 1);
   FRLAP_LAUNCH_CHECK("k_maxabs");
   unsigned long long bits[2] = {0ull, 0ull};
   FRLAP_CUDA_TRY(cudaMemcpyAsync(bits, slot, sizeof(bits), cudaMemcpyDeviceToHost, st));
@@ -754,12 +768,12 @@ frlap_status pcg_solve_impl(const Plan& p, const double* f, double* x, double rt
   if (e == 0)
     return pcg_solve_core(p, f, x, rtol, maxit, solver, mu, inner_rtol, iters, relres, work, st, x0_zero);
   double* fs = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(work) + pcg_base_bytes(p));
-  k_scale_pow2<<<vgrid(p.M), kThreads, 0, st>>>(f, fs, p.M, -e);
-  if (!x0_zero) k_scale_pow2<<<vgrid(p.M), kThreads, 0, st>>>(x, x, p.M, -e);
+  k_scale_pow2<<<vgrid(p.M), vthreads(p.M), 0, st>>>(f, fs, p.M, -e);
+  if (!x0_zero) k_scale_pow2<<<vgrid(p.M), vthreads(p.M), 0, st>>>(x, x, p.M, -e);
   FRLAP_LAUNCH_CHECK("k_scale_pow2");
   const frlap_status rc = pcg_solve_core(p, fs, x, rtol, maxit, solver, mu, inner_rtol, iters, relres, work, st,
                                          x0_zero);
-  k_scale_pow2<<<vgrid(p.M), kThreads, 0, st>>>(x, x, p.M, e);
+  k_scale_pow2<<<vgrid(p.M), vthreads(p.M), 0, st>>>(x, x, p.M, e);
   cudaError_t ce = cudaGetLastError();
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess) return cuda_fail(ce, "k_scale_pow2 (solution)");
@@ -823,13 +837,13 @@ static frlap_status pcg_solve_core(const Plan& p, const double* f, double* x, do
     prev = rel;
     if (!isfinite(rel)) return fail(FRLAP_ENAN, "non-finite residual in iterative refinement");
     if (rel <= rtol || outer == max_outer || total >= maxit) break;
-    k_to_f32<<<vgrid(p.M), kThreads, 0, st>>>(r64, rnorm, r32, d32, p.M);
+    k_to_f32<<<vgrid(p.M), vthreads(p.M), 0, st>>>(r64, rnorm, r32, d32, p.M);
     FRLAP_LAUNCH_CHECK("k_to_f32");
     rc = run_cg<float>(p, r32, d32, 0.0, 1.0, inner_rtol, maxit - total, 0, mu, odd, work32, st, &hS);
     if (rc != FRLAP_OK) return rc;
     total += hS.iters;
     if (hS.status == FRLAP_ENAN) return fail(FRLAP_ENAN, "non-finite value in the FP32 inner solve");
-    k_correct<<<vgrid(p.M), kThreads, 0, st>>>(x, d32, rnorm, p.M);
+    k_correct<<<vgrid(p.M), vthreads(p.M), 0, st>>>(x, d32, rnorm, p.M);
     FRLAP_LAUNCH_CHECK("k_correct");
   }
   if (iters) *iters = total;
@@ -866,7 +880,7 @@ frlap_status allen_cahn_cn_impl(const Plan& p, double* ub, double tau, double de
   for (int step = 0; step < nsteps; ++step) {
     cudaError_t e = apply64(p, ub, aub, b.awork, st, nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "apply (Crank-Nicolson right-hand side)");
-    k_cn_rhs<<<vgrid(p.M), kThreads, 0, st>>>(ub, aub, rhs, p.M, tau, kdel);
+    k_cn_rhs<<<vgrid(p.M), vthreads(p.M), 0, st>>>(ub, aub, rhs, p.M, tau, kdel);
     FRLAP_LAUNCH_CHECK("k_cn_rhs");
     frlap_status rc = run_cg<double>(p, rhs, ub, 1.0, 0.5 * tau, rtol, 100000, 1, mu, mu != nullptr, cgw, st, &hS);
     if (rc != FRLAP_OK) return rc;
@@ -903,7 +917,7 @@ frlap_status allen_cahn_impl(const Plan& p, double* u, double tau, double eps, i
   int total = 0;
   CgState hS;
   for (int step = 0; step < nsteps; ++step) {
-    k_ac_rhs<<<vgrid(p.M), kThreads, 0, st>>>(u, rhs, p.M, tau);
+    k_ac_rhs<<<vgrid(p.M), vthreads(p.M), 0, st>>>(u, rhs, p.M, tau);
     FRLAP_LAUNCH_CHECK("k_ac_rhs");
     frlap_status rc = run_cg<double>(p, rhs, u, 1.0, tau * eps * eps, rtol, 100000, 1, mu, mu != nullptr, cgw, st,
                                      &hS);
