@@ -7,11 +7,11 @@
 // stacked, so each kernel below handles a whole group (blockIdx.y = instance).
 //
 // Control flow lives on the device.  The graph is one conditional WHILE node whose
-// body runs one CG iteration for every instance that is still solving, then an
-// `advance` kernel that, for each instance whose solve has just ended, copies the
-// solution into u and sets up the next step (or marks the instance finished),
-// then a kernel that keeps the loop going while any instance is unfinished.  The
-// loop count is bounded: each solve stops after maxit iterations, and the control
+// body runs one CG iteration for every instance that is still solving; its last
+// kernel, for each instance whose solve has just ended, copies the solution into u
+// and sets up the next step (or marks the instance finished).  The groups' kernels are
+// parallel branches of the body.  Then a kernel keeps the loop going while any instance is
+// unfinished.  The loop count is bounded: each solve stops after maxit iterations, and the control
 // kernel also stops the loop after nsteps * (maxit + 2) + 8 passes (or the lower limit set by
 // frlap_set_loop_pass_limit), reporting FRLAP_ETIMEOUT.
 #include <math.h>
@@ -24,8 +24,22 @@ namespace frlap {
 
 namespace {
 
-constexpr int kAcBlocks = 32;  // blocks per instance for the vector kernels
+constexpr int kAcMaxBlocks = 304;  // CTAs per instance of the vector kernels, at most
 constexpr int kAcThreads = 256;
+// CTAs per instance for a group of B instances of M unknowns: about four per SM over the group, each with at
+// least one pass of kU elements a thread (32 per instance whatever the group left four 1023^2 instances 8
+// warps per SM in flight).  With the groups as parallel branches and k_ac_next for two kernels, 12 instances
+// x 4 steps on 255^2, 511^2 and 1023^2: 20.0 -> 14.4 ms.
+inline int ac_blocks(size_t M, size_t B) {
+  const size_t want = (4 * 152 + B - 1) / B, most = (M + 4 * kAcThreads - 1) / (4 * kAcThreads);
+  const size_t b = want < most ? want : most;
+  return (int)(b < 1 ? 1 : b > (size_t)kAcMaxBlocks ? (size_t)kAcMaxBlocks : b);
+}
+#ifdef FRLAP_BOUNDS_CHECK
+constexpr int kAcStreams = 1;  // (the checked build registers one launching call's ranges at a time)
+#else
+constexpr int kAcStreams = 4;  // groups run side by side on up to this many streams
+#endif
 
 struct AcState {
   double rr, pq, alpha, beta, tol2;
@@ -77,7 +91,6 @@ __device__ __forceinline__ bool inst_sum(double v, double* partials, unsigned* c
   return threadIdx.x == 0;
 }
 
-#define INST_LOOP(i, n) for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (size_t)gridDim.x * blockDim.x)
 // The iteration kernels take kU elements per thread and pass, one grid apart, all loaded before any
 // arithmetic (several loads in flight per warp; see the CG kernels); the u-th is base + u * gstride.
 constexpr int kU = 4;
@@ -113,61 +126,6 @@ __device__ __forceinline__ bool inst_sum2(double a, double b, double* pa, double
     *counter = 0u;
   }
   return threadIdx.x == 0;
-}
-
-// Start of a solve.  The first step: rhs = u + tau (u - u^3), x = 0, r = p = rhs.  After a solve:
-// u <- x, and the next step starts from x = u^{n+1} itself (warm start).  Its initial residual
-// needs no apply: the finished solve's recursive residual is r = rhs_old - B x, so
-// rhs_new - B x = rhs_new - rhs_old + r, with rhs_old recomputed from the old u.
-__global__ void k_ac_advance(double* u, double* x, double* r, double* p, size_t M, size_t vs, AcState* S,
-                             double* partials, double* partials2, int nsteps, double tau, double rtol) {
-  const int b = blockIdx.y;
-  AcState* st = S + b;
-  if (!st->done || st->finished) return;
-  const bool fresh = st->fresh != 0;
-  const bool last_step = !fresh && st->step + 1 >= nsteps;
-  u += b * vs;
-  x += b * vs;
-  r += b * vs;
-  p += b * vs;
-  double acc_r = 0.0, acc_h = 0.0;
-  INST_LOOP(i, M) {
-    if (fresh) {
-      const double v = u[i];
-      const double rh = v + tau * (v - v * v * v);
-      x[i] = 0.0;
-      r[i] = rh;
-      p[i] = rh;
-      acc_r += rh * rh;
-      acc_h += rh * rh;
-    } else {
-      const double uo = u[i], v = x[i];
-      u[i] = v;
-      if (!last_step) {
-        const double rh_old = uo + tau * (uo - uo * uo * uo);
-        const double rh = v + tau * (v - v * v * v);
-        const double r0 = rh - rh_old + r[i];
-        r[i] = r0;
-        p[i] = r0;
-        acc_r += r0 * r0;
-        acc_h += rh * rh;
-      }
-    }
-  }
-  double tot_r, tot_h;
-  if (inst_sum2(acc_r, acc_h, partials + (size_t)b * gridDim.x, partials2 + (size_t)b * gridDim.x, &st->counter,
-                &tot_r, &tot_h)) {
-    if (!fresh) st->step += 1;
-    st->fresh = 0;
-    if (st->step >= nsteps) {
-      st->finished = 1;
-    } else {
-      st->rr = tot_r;
-      st->tol2 = rtol * rtol * tot_h;
-      st->iters = 0;
-      st->done = (tot_r <= st->tol2) ? 1 : 0;
-    }
-  }
 }
 
 // q <- p + s q ; pq ; alpha
@@ -264,26 +222,94 @@ __global__ void k_ac_update(double* x, double* r, const double* __restrict__ p, 
   }
 }
 
-__global__ void k_ac_dir(const double* __restrict__ r, double* p, size_t M, size_t vs, const AcState* S) {
+// End of a pass: an instance still solving takes its next direction, p = r + beta p.  One whose solve has ended
+// starts the next.  The first step: rhs = u + tau (u - u^3), x = 0, r = p = rhs.  After a solve: u <- x, and
+// the next step starts from x = u^{n+1} itself (warm start).  Its initial residual needs no apply: the
+// finished solve's recursive residual is r = rhs_old - B x, so rhs_new - B x = rhs_new - rhs_old + r, with
+// rhs_old recomputed from the old u.
+__global__ void k_ac_next(double* u, double* x, double* r, double* p, size_t M,
+                          size_t vs, AcState* S, double* partials, double* partials2, int nsteps, double tau,
+                          double rtol) {
   const int b = blockIdx.y;
-  if (S[b].done) return;
+  AcState* st = S + b;
+  if (st->finished) return;
+  u += b * vs;
+  x += b * vs;
   r += b * vs;
   p += b * vs;
-  const double be = S[b].beta;
-  INST_LOOP_U(b0, M) {
-    double rv[kU], pv[kU];
+  if (!st->done) {
+    const double be = st->beta;
+    INST_LOOP_U(b0, M) {
+      double rv[kU], pv[kU];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const size_t i = b0 + u * gstride;
+      for (int k = 0; k < kU; ++k) {
+        const size_t i = b0 + k * gstride;
+        if (i < M) {
+          rv[k] = r[i];
+          pv[k] = p[i];
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kU; ++k) {
+        const size_t i = b0 + k * gstride;
+        if (i < M) p[i] = rv[k] + be * pv[k];
+      }
+    }
+    return;
+  }
+  const bool fresh = st->fresh != 0;
+  const bool last_step = !fresh && st->step + 1 >= nsteps;
+  double acc_r = 0.0, acc_h = 0.0;
+  INST_LOOP_U(b0, M) {
+    double uv[kU], xv[kU], rv[kU];
+#pragma unroll
+    for (int k = 0; k < kU; ++k) {
+      const size_t i = b0 + k * gstride;
       if (i < M) {
-        rv[u] = r[i];
-        pv[u] = p[i];
+        uv[k] = u[i];
+        if (!fresh) {
+          xv[k] = x[i];
+          rv[k] = r[i];
+        }
       }
     }
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const size_t i = b0 + u * gstride;
-      if (i < M) p[i] = rv[u] + be * pv[u];
+    for (int k = 0; k < kU; ++k) {
+      const size_t i = b0 + k * gstride;
+      if (i >= M) continue;
+      if (fresh) {
+        const double rh = uv[k] + tau * (uv[k] - uv[k] * uv[k] * uv[k]);
+        x[i] = 0.0;
+        r[i] = rh;
+        p[i] = rh;
+        acc_r += rh * rh;
+        acc_h += rh * rh;
+      } else {
+        u[i] = xv[k];
+        if (!last_step) {
+          const double rh_old = uv[k] + tau * (uv[k] - uv[k] * uv[k] * uv[k]);
+          const double rh = xv[k] + tau * (xv[k] - xv[k] * xv[k] * xv[k]);
+          const double r0 = rh - rh_old + rv[k];
+          r[i] = r0;
+          p[i] = r0;
+          acc_r += r0 * r0;
+          acc_h += rh * rh;
+        }
+      }
+    }
+  }
+  double tot_r, tot_h;
+  if (inst_sum2(acc_r, acc_h, partials + (size_t)b * gridDim.x, partials2 + (size_t)b * gridDim.x, &st->counter,
+                &tot_r, &tot_h)) {
+    if (!fresh) st->step += 1;
+    st->fresh = 0;
+    if (st->step >= nsteps) {
+      st->finished = 1;
+    } else {
+      st->rr = tot_r;
+      st->tol2 = rtol * rtol * tot_h;
+      st->iters = 0;
+      st->done = (tot_r <= st->tol2) ? 1 : 0;
     }
   }
 }
@@ -333,8 +359,8 @@ struct Group {
   double* p;
   double* q;
   void* awork;          // [B][apply work]
-  double* partials;     // [B][kAcBlocks]
-  double* partials2;    // [B][kAcBlocks] (the second sum of k_ac_advance)
+  double* partials;     // [B][kAcMaxBlocks]
+  double* partials2;    // [B][kAcMaxBlocks] (the second sum of k_ac_next)
   AcState* S;           // points into the global state array
 };
 
@@ -378,7 +404,7 @@ size_t group_bytes(const Group& g) {
   const Plan& p = *g.plan;
   const size_t B = g.idx.size();
   return B * (align256(p.lam_count * 8) + 5 * align256(p.M * 8) + apply_work_bytes(p, 8) +
-              2 * align256(kAcBlocks * sizeof(double)));
+              2 * align256(kAcMaxBlocks * sizeof(double)));
 }
 
 }  // namespace
@@ -419,9 +445,9 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
     g.awork = w;
     w += B * g.work_stride;
     g.partials = reinterpret_cast<double*>(w);
-    w += B * align256(kAcBlocks * sizeof(double));
+    w += B * align256(kAcMaxBlocks * sizeof(double));
     g.partials2 = reinterpret_cast<double*>(w);
-    w += B * align256(kAcBlocks * sizeof(double));
+    w += B * align256(kAcMaxBlocks * sizeof(double));
     g.S = S_all + soff;
     soff += (int)B;
   }
@@ -431,6 +457,13 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
   cudaEvent_t ev0, ev1;
   cudaEventCreateWithFlags(&ev0, cudaEventDisableTiming);
   cudaEventCreateWithFlags(&ev1, cudaEventDisableTiming);
+  const int ns = (int)(groups.size() < (size_t)kAcStreams ? groups.size() : (size_t)kAcStreams) - 1;  // side streams
+  cudaStream_t side[kAcStreams] = {};
+  cudaEvent_t ev_side[kAcStreams] = {};
+  for (int k = 0; k < ns; ++k) {
+    cudaStreamCreateWithFlags(&side[k], cudaStreamNonBlocking);
+    cudaEventCreateWithFlags(&ev_side[k], cudaEventDisableTiming);
+  }
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   frlap_status rc = FRLAP_OK;
@@ -439,6 +472,10 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
     if (graph) cudaGraphDestroy(graph);
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
+    for (int k = 0; k < ns; ++k) {
+      cudaEventDestroy(ev_side[k]);
+      cudaStreamDestroy(side[k]);
+    }
     cudaStreamDestroy(s);
   };
   do {
@@ -504,21 +541,31 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
     }
     const double sc = tau * eps * eps;
     const int sstride = (int)(sizeof(AcState) / sizeof(int));
-    for (auto& g : groups) {
+    // The groups share nothing but the control kernel: they are captured on streams of their own, parallel
+    // branches of the body, so the kernels of the small ones fill the tails of the large ones.
+    cudaError_t eb = cudaEventRecord(ev0, s);
+    for (int k = 0; k < ns && eb == cudaSuccess; ++k) eb = cudaStreamWaitEvent(side[k], ev0, 0);
+    for (size_t gi = 0; gi < groups.size() && eb == cudaSuccess; ++gi) {
+      Group& g = groups[gi];
       const Plan& p = *g.plan;
       const int B = (int)g.idx.size();
-      batch_apply(p, B, g.p, g.q, g.vs, g.awork, s, &g.S[0].done, sstride, g.lam, align256(p.lam_count * 8) / 8);
-      const dim3 grid(kAcBlocks, B);
-      k_ac_pq<<<grid, kAcThreads, 0, s>>>(g.p, g.q, g.M, g.vs, g.S, g.partials, sc);
-      k_ac_update<<<grid, kAcThreads, 0, s>>>(g.x, g.r, g.p, g.q, g.M, g.vs, g.S, g.partials, maxit);
-      k_ac_dir<<<grid, kAcThreads, 0, s>>>(g.r, g.p, g.M, g.vs, g.S);
-      k_ac_advance<<<grid, kAcThreads, 0, s>>>(g.u, g.x, g.r, g.p, g.M, g.vs, g.S, g.partials, g.partials2, nsteps,
-                                                tau, rtol);
+      const cudaStream_t gs = gi % (ns + 1) == 0 ? s : side[gi % (ns + 1) - 1];
+      eb = batch_apply(p, B, g.p, g.q, g.vs, g.awork, gs, &g.S[0].done, sstride, g.lam, align256(p.lam_count * 8) / 8);
+      const dim3 grid(ac_blocks(g.M, B), B);
+      k_ac_pq<<<grid, kAcThreads, 0, gs>>>(g.p, g.q, g.M, g.vs, g.S, g.partials, sc);
+      k_ac_update<<<grid, kAcThreads, 0, gs>>>(g.x, g.r, g.p, g.q, g.M, g.vs, g.S, g.partials, maxit);
+      k_ac_next<<<grid, kAcThreads, 0, gs>>>(g.u, g.x, g.r, g.p, g.M, g.vs, g.S, g.partials, g.partials2, nsteps, tau,
+                                             rtol);
+    }
+    for (int k = 0; k < ns && eb == cudaSuccess; ++k) {
+      eb = cudaEventRecord(ev_side[k], side[k]);
+      if (eb == cudaSuccess) eb = cudaStreamWaitEvent(s, ev_side[k], 0);
     }
     const unsigned max_passes = capped_passes((unsigned)nsteps * (unsigned)(maxit + 2) + 8u);
     k_ac_control<<<1, 256, 0, s>>>(S_all, nb, passes, max_passes, timeout, h);
     cudaGraph_t captured = nullptr;
     cudaError_t ecap = cudaGetLastError();
+    if (ecap == cudaSuccess) ecap = eb;
     e = cudaStreamEndCapture(s, &captured);
     if (ecap != cudaSuccess || e != cudaSuccess) {
       rc = cuda_fail(ecap != cudaSuccess ? ecap : e, "capture of the loop body");
