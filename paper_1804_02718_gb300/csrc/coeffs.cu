@@ -38,21 +38,20 @@ GaussRules make_gauss_rules() {
   for (int r = 0; r < kNumQ; ++r) {
     const int q = rule_q(r);
     for (int i = 0; i < q; ++i) {
-      double x = cos(M_PI * (i + 0.75) / (q + 0.5)), dP = 1.0;
-      for (int it = 0; it < 20; ++it) {
-        double p0 = 1.0, p1 = x;
+      // in extended precision: an error of a rule is one of every element's integral alike
+      long double x = cosl(3.14159265358979323846L * (i + 0.75L) / (q + 0.5L)), dP = 1.0L;
+      for (int it = 0; it < 12; ++it) {  // quadratic: five steps reach the rounding level
+        long double p0 = 1.0L, p1 = x;
         for (int k = 2; k <= q; ++k) {
-          const double p2 = ((2.0 * k - 1.0) * x * p1 - (k - 1.0) * p0) / k;
+          const long double p2 = ((2.0L * k - 1.0L) * x * p1 - (k - 1.0L) * p0) / k;
           p0 = p1;
           p1 = p2;
         }
-        dP = q * (x * p1 - p0) / (x * x - 1.0);
-        const double dx = p1 / dP;
-        x -= dx;
-        if (fabs(dx) < 1e-15) break;  // quadratic: the step after a 1e-8 one is the last that changes x
+        dP = q * (x * p1 - p0) / (x * x - 1.0L);
+        x -= p1 / dP;
       }
-      g.x[rule_off(r) + i] = 0.5 * (1.0 - x);
-      g.w[rule_off(r) + i] = 1.0 / ((1.0 - x * x) * dP * dP);  // (2 / ((1 - x^2) P'^2)) / 2
+      g.x[rule_off(r) + i] = (double)(0.5L * (1.0L - x));
+      g.w[rule_off(r) + i] = (double)(1.0L / ((1.0L - x * x) * dP * dP));  // (2 / ((1 - x^2) P'^2)) / 2
     }
   }
   return g;
