@@ -524,7 +524,10 @@ template <int REM>
 __global__ void __launch_bounds__(512, 1)
     k_q_col_fwd(const cq* __restrict__ in, const int* __restrict__ ex, double2* __restrict__ out, int ncols, int n,
                 size_t ld, size_t ldo, int logP, int TL, int cols_per, const int4* __restrict__ tw,
-                const int* __restrict__ skip) {
+                const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  in += blockIdx.y * bt.in;
+  out += blockIdx.y * bt.out;
+  ex += blockIdx.y * ex_inst;
   FRLAP_Q_PROLOGUE(logP)
   const int P = 1 << logP, G = P >> 4;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
@@ -553,7 +556,10 @@ template <int REM>
 __global__ void __launch_bounds__(512, 1)
     k_q_col_mulinv(const double2* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int ncols, int n,
                    size_t ld, size_t ldo, int logP, int TL, const double* __restrict__ lam, LamMap map,
-                   const int4* __restrict__ tw, const int* __restrict__ skip) {
+                   const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  in += blockIdx.y * bt.in;
+  out += blockIdx.y * bt.out;
+  ex += blockIdx.y * ex_inst;
   FRLAP_Q_PROLOGUE(logP)
   const int P = 1 << logP, G = P >> 4;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
@@ -797,58 +803,63 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstr
 }
 
 // SP = F R^T u on the half spectrum in FP64: 2D [kx][ky], 3D [kx][ky][kz] (kx <= P_x/2, full ky, kz).
-template <>
-cudaError_t spectrum_forward<double>(const Plan& p, const double* u, double2* SP, void* work, cudaStream_t s) {
+cudaError_t spectrum_forward(const Plan& p, int nb, const double* u, double2* SP, size_t sstride, void* work,
+                             cudaStream_t s) {
   cudaError_t e;
 #ifdef FRLAP_BOUNDS_CHECK
   {
     BcRanges r;
-    r.add(u, p.M * sizeof(double));
-    r.add(SP, spectrum_elems(p) * sizeof(double2));
-    if ((e = q_register(p, r, work, 1, s)) != cudaSuccess) return e;
+    r.add(u, nb * p.M * sizeof(double));
+    r.add(SP, nb * sstride * sizeof(double2));
+    if ((e = q_register(p, r, work, nb, s)) != cudaSuccess) return e;
   }
 #endif
   const QWork w = q_work(p, work);
-  if ((e = q_stage_r2c(p, w, 1, u, 0, 0, nullptr, 0, s)) != cudaSuccess) return e;
-  if (p.d == 3 && (e = q_stage_yz_fwd(p, w, 1, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  if ((e = q_stage_r2c(p, w, nb, u, p.M, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  if (p.d == 3 && (e = q_stage_yz_fwd(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
   const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
   const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-  const QShape q = q_shape(0, p.P[ax], ncols, ncols);
+  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
+  Batch b;
+  b.in = w.stride;
+  b.out = sstride;
   return with_rem(p.logP[ax], [&](auto tag) {
-    return q_launch(k_q_col_fwd<decltype(tag)::value>, q.tiles, 1, q.threads, q.sm, s,
+    return q_launch(k_q_col_fwd<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s,
                     (const cq*)(p.d == 3 ? w.S2 : w.S1), (const int*)(p.d == 3 ? w.line : w.row), SP, ncols, p.n[ax],
                     (size_t)(p.d == 3 ? p.n[2] : nrows), (size_t)p.P[ax], p.logP[ax], q.tl, p.d == 3 ? p.P[1] : 0,
-                    (const int4*)p.twq[ax], (const int*)nullptr);
+                    (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
   });
 }
 
 // y = R F^-1 (mult * SP), mult = a symbol octant with the 1/prod(P) factor folded in.
-template <>
-cudaError_t spectrum_inverse<double>(const Plan& p, const double2* SP, const double* mult, double* y, void* work,
-                                     cudaStream_t s) {
+cudaError_t spectrum_inverse(const Plan& p, int nb, const double2* SP, size_t sstride, const double* mult, double* y,
+                             void* work, cudaStream_t s) {
   cudaError_t e;
 #ifdef FRLAP_BOUNDS_CHECK
   {
     BcRanges r;
-    r.add(SP, spectrum_elems(p) * sizeof(double2));
+    r.add(SP, nb * sstride * sizeof(double2));
     r.add(mult, p.lam_count * sizeof(double));
-    r.add(y, p.M * sizeof(double));
-    if ((e = q_register(p, r, work, 1, s)) != cudaSuccess) return e;
+    r.add(y, nb * p.M * sizeof(double));
+    if ((e = q_register(p, r, work, nb, s)) != cudaSuccess) return e;
   }
 #endif
   const QWork w = q_work(p, work);
   const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
   const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-  const QShape q = q_shape(0, p.P[ax], ncols, ncols);
+  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
   const LamMap map = q_lam_map(p);
+  Batch b;
+  b.in = sstride;
+  b.out = w.stride;
   e = with_rem(p.logP[ax], [&](auto tag) {
-    return q_launch(k_q_col_mulinv<decltype(tag)::value>, q.tiles, 1, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
+    return q_launch(k_q_col_mulinv<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
                     w.col, ncols, p.n[ax], (size_t)p.P[ax], (size_t)(p.d == 3 ? p.n[2] : nrows), p.logP[ax], q.tl, mult,
-                    map, (const int4*)p.twq[ax], (const int*)nullptr);
+                    map, (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
   });
   if (e != cudaSuccess) return e;
-  if (p.d == 3 && (e = q_stage_yz_inv(p, w, 1, 0, nullptr, 0, s)) != cudaSuccess) return e;
-  return q_stage_c2r(p, w, 1, y, 0, 0, nullptr, 0, s);
+  if (p.d == 3 && (e = q_stage_yz_inv(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  return q_stage_c2r(p, w, nb, y, p.M, 0, nullptr, 0, s);
 }
 
 }  // namespace frlap

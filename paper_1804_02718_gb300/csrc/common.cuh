@@ -313,12 +313,13 @@ template <typename T>
 cudaError_t apply_batch_launch(const Plan& p, int B, const io_t<T>* u, io_t<T>* y, size_t vstride, void* work,
                                cudaStream_t s, const int* skip, int skip_stride, const T* lam, size_t lam_stride,
                                cudaEvent_t const* ev = nullptr);
-// forward half spectrum F R^T u (2D [kx][ky], 3D [kx][ky][kz]) and its multiplied inverse; same workspace as apply
+// Forward half spectra F R^T u (2D [kx][ky], 3D [kx][ky][kz]) of nb vectors back to back, sstride complex entries
+// apart, and their inverse after a multiplier, in the FP64 engine; work: nb apply workspaces.
 size_t spectrum_elems(const Plan& p);
-template <typename T>
-cudaError_t spectrum_forward(const Plan& p, const T* u, cplx<T>* SP, void* work, cudaStream_t s);
-template <typename T>
-cudaError_t spectrum_inverse(const Plan& p, const cplx<T>* SP, const T* mult, T* y, void* work, cudaStream_t s);
+cudaError_t spectrum_forward(const Plan& p, int nb, const double* u, double2* SP, size_t sstride, void* work,
+                             cudaStream_t s);
+cudaError_t spectrum_inverse(const Plan& p, int nb, const double2* SP, size_t sstride, const double* mult, double* y,
+                             void* work, cudaStream_t s);
 
 // coefficient / symbol generation (coeffs.cu)
 cudaError_t coeffs_launch(int d, double alpha, double gamma, double h, int Nmax, double* coef, void* scratch,

@@ -50,11 +50,13 @@ __device__ __forceinline__ void features(const Oct& o, size_t f, float* phi) {
   phi[3] = (o.d == 3) ? kz * o.iz : 0.0f;
 }
 
-// m(f) = exp(s(f)) / lambda(f); optional caches of the two hidden layers for backprop
+// m(f) = exp(s(f)) / lambda(f); optional caches of the two hidden layers for backprop, [HID][F] so that a
+// warp's stores of one unit are contiguous.  The weights are read four per shared-memory load (one per load
+// took 98 us at 257 x 257 entries).
 __global__ void __launch_bounds__(128) k_mlp_fwd(const float* __restrict__ params, Oct o, const double* __restrict__ lam,
                                                  double lamscale, size_t F, double* m, double* m_scaled,
                                                  double mscale, float* h1c, float* h2c) {
-  __shared__ float W[NPAR];
+  __shared__ __align__(16) float W[NPAR + 3];
   for (int i = threadIdx.x; i < NPAR; i += blockDim.x) W[i] = params[i];
   __syncthreads();
   const size_t f = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -62,21 +64,32 @@ __global__ void __launch_bounds__(128) k_mlp_fwd(const float* __restrict__ param
   float phi[NF];
   features(o, f, phi);
   float h1[HID];
+  static_assert(NF == 4 && OW1 % 4 == 0 && OW2 % 4 == 0 && HID % 4 == 0, "float4 rows");
 #pragma unroll
   for (int h = 0; h < HID; ++h) {
+    const float4 w = *reinterpret_cast<const float4*>(&W[OW1 + h * NF]);
     float a = W[OB1 + h];
-#pragma unroll
-    for (int j = 0; j < NF; ++j) a = fmaf(W[OW1 + h * NF + j], phi[j], a);
+    a = fmaf(w.x, phi[0], a);
+    a = fmaf(w.y, phi[1], a);
+    a = fmaf(w.z, phi[2], a);
+    a = fmaf(w.w, phi[3], a);
     h1[h] = tanhf(a);
-    if (h1c) h1c[f * HID + h] = h1[h];
+    if (h1c) h1c[h * F + f] = h1[h];
   }
   float s = W[OB3];
+#pragma unroll 2
   for (int q = 0; q < HID; ++q) {
     float a = W[OB2 + q];
 #pragma unroll
-    for (int i = 0; i < HID; ++i) a = fmaf(W[OW2 + q * HID + i], h1[i], a);
+    for (int i = 0; i < HID; i += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(&W[OW2 + q * HID + i]);
+      a = fmaf(w.x, h1[i], a);
+      a = fmaf(w.y, h1[i + 1], a);
+      a = fmaf(w.z, h1[i + 2], a);
+      a = fmaf(w.w, h1[i + 3], a);
+    }
     const float h2 = tanhf(a);
-    if (h2c) h2c[f * HID + q] = h2;
+    if (h2c) h2c[q * F + f] = h2;
     s = fmaf(W[OW3 + q], h2, s);
   }
   const double l = lam[f] * lamscale;
@@ -85,86 +98,149 @@ __global__ void __launch_bounds__(128) k_mlp_fwd(const float* __restrict__ param
   if (m_scaled) m_scaled[f] = mv * mscale;
 }
 
-// per-block partial gradients of sum_f g_s(f) s(f), g_s = g_m * m; 64 entries per block, 256 threads
-constexpr int BENT = 64;
-__global__ void __launch_bounds__(256) k_mlp_bwd(const float* __restrict__ params, Oct o,
-                                                 const double* __restrict__ g_m, const double* __restrict__ m,
-                                                 const float* __restrict__ h1c, const float* __restrict__ h2c,
-                                                 size_t F, float* partial) {
+// Gradient of sum_f g_s(f) s(f), g_s = g_m * m.  A CTA walks tiles of BENT = 64 entries; per tile the two
+// 64 x 64 x 64 products run as register tiles (4 x 4 outputs a thread, operands four per load; one operand
+// per load was 115 us at 257 x 257 entries), their FP32 sums over the tile's entries added to FP64
+// accumulators in registers.  partial[CTA][NPAR].
+constexpr int BENT = 64, BST = BENT + 4;  // row stride of a tile in shared memory: 16-byte rows, spread banks
+constexpr int kBwdCtas = 304;
+constexpr size_t kBwdSmem = (size_t)(HID * BST + 4 * BENT * BST + BENT * NF + BENT) * sizeof(float);
+__global__ void __launch_bounds__(256, 2) k_mlp_bwd(const float* __restrict__ params, Oct o,
+                                                    const double* __restrict__ g_m, const double* __restrict__ m,
+                                                    const float* __restrict__ h1c, const float* __restrict__ h2c,
+                                                    size_t F, double* partial) {
+  static_assert(HID == 64 && BENT == 64, "16 x 16 threads of 4 x 4 outputs");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* W2 = reinterpret_cast<float*>(smem_raw);  // [HID][HID]
-  float* sh1 = W2 + HID * HID;                      // [BENT][HID]
-  float* sh2 = sh1 + BENT * HID;
-  float* sga2 = sh2 + BENT * HID;
-  float* sga1 = sga2 + BENT * HID;
-  float* sphi = sga1 + BENT * HID;                  // [BENT][NF]
-  float* sgs = sphi + BENT * NF;                    // [BENT]
-  for (int i = threadIdx.x; i < HID * HID; i += blockDim.x) W2[i] = params[OW2 + i];
-  const size_t f0 = (size_t)blockIdx.x * BENT;
-  // load caches and per-entry output gradient
-  for (int i = threadIdx.x; i < BENT * HID; i += blockDim.x) {
-    const int e = i / HID, h = i % HID;
-    const size_t f = f0 + e;
-    const bool v = f < F;
-    sh1[i] = v ? h1c[f * HID + h] : 0.0f;
-    sh2[i] = v ? h2c[f * HID + h] : 0.0f;
-  }
-  for (int e = threadIdx.x; e < BENT; e += blockDim.x) {
-    const size_t f = f0 + e;
-    float phi[NF];
-    features(o, f < F ? f : 0, phi);
-    for (int j = 0; j < NF; ++j) sphi[e * NF + j] = phi[j];
-    sgs[e] = (f < F) ? (float)(g_m[f] * m[f]) : 0.0f;
-  }
-  __syncthreads();
-  // g_a2[e][q] = g_s[e] w3[q] (1 - h2^2)
-  for (int i = threadIdx.x; i < BENT * HID; i += blockDim.x) {
-    const int e = i / HID, q = i % HID;
-    const float h2 = sh2[i];
-    sga2[i] = sgs[e] * params[OW3 + q] * (1.0f - h2 * h2);
-  }
-  __syncthreads();
-  // g_a1[e][h] = (sum_q W2[q][h] g_a2[e][q]) (1 - h1^2)
-  for (int i = threadIdx.x; i < BENT * HID; i += blockDim.x) {
-    const int e = i / HID, h = i % HID;
-    float a = 0.0f;
-    for (int q = 0; q < HID; ++q) a = fmaf(W2[q * HID + h], sga2[e * HID + q], a);
-    const float h1 = sh1[i];
-    sga1[i] = a * (1.0f - h1 * h1);
-  }
-  __syncthreads();
-  float* out = partial + (size_t)blockIdx.x * NPAR;
-  for (int p = threadIdx.x; p < NPAR; p += blockDim.x) {
-    float acc = 0.0f;
-    if (p < OB1) {  // W1[h][j]
-      const int h = p / NF, j = p % NF;
-      for (int e = 0; e < BENT; ++e) acc = fmaf(sga1[e * HID + h], sphi[e * NF + j], acc);
-    } else if (p < OW2) {  // b1
-      const int h = p - OB1;
-      for (int e = 0; e < BENT; ++e) acc += sga1[e * HID + h];
-    } else if (p < OB2) {  // W2[q][i]
-      const int q = (p - OW2) / HID, i = (p - OW2) % HID;
-      for (int e = 0; e < BENT; ++e) acc = fmaf(sga2[e * HID + q], sh1[e * HID + i], acc);
-    } else if (p < OW3) {  // b2
-      const int q = p - OB2;
-      for (int e = 0; e < BENT; ++e) acc += sga2[e * HID + q];
-    } else if (p < OB3) {  // w3
-      const int q = p - OW3;
-      for (int e = 0; e < BENT; ++e) acc = fmaf(sgs[e], sh2[e * HID + q], acc);
-    } else {  // b3
-      for (int e = 0; e < BENT; ++e) acc += sgs[e];
+  float* W2 = reinterpret_cast<float*>(smem_raw);  // [q][h]
+  float* sh1 = W2 + HID * BST;                     // [e][h] (and the next three)
+  float* sh2 = sh1 + BENT * BST;
+  float* sga2 = sh2 + BENT * BST;
+  float* sga1 = sga2 + BENT * BST;
+  float* sphi = sga1 + BENT * BST;                 // [e][NF]
+  float* sgs = sphi + BENT * NF;                   // [e]
+  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+  for (int i = t; i < HID * HID; i += 256) W2[(i >> 6) * BST + (i & 63)] = params[OW2 + i];
+  double acc2[4][4] = {};  // W2[4 ty + i][4 tx + j]
+  double acc1 = 0.0;       // W1[t / NF][t % NF]
+  double accb = 0.0;       // t < 64: b1, < 128: b2, < 192: w3, 192: b3
+  const size_t ntiles = (F + BENT - 1) / BENT;
+  for (size_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const size_t f0 = tile * BENT;
+    __syncthreads();  // the previous tile's readers are done
+    for (int i = t; i < BENT * HID; i += 256) {
+      const int e = i & 63, h = i >> 6;
+      const size_t f = f0 + e;
+      sh1[e * BST + h] = f < F ? h1c[(size_t)h * F + f] : 0.0f;
+      sh2[e * BST + h] = f < F ? h2c[(size_t)h * F + f] : 0.0f;
     }
-    out[p] = acc;
+    if (t < BENT) {
+      const size_t f = f0 + t;
+      float phi[NF];
+      features(o, f < F ? f : 0, phi);
+      for (int j = 0; j < NF; ++j) sphi[t * NF + j] = phi[j];
+      sgs[t] = (f < F) ? (float)(g_m[f] * m[f]) : 0.0f;
+    }
+    __syncthreads();
+    // g_a2[e][q] = g_s[e] w3[q] (1 - h2^2)
+    for (int i = t; i < BENT * HID; i += 256) {
+      const int e = i >> 6, q = i & 63;
+      const float h2 = sh2[e * BST + q];
+      sga2[e * BST + q] = sgs[e] * params[OW3 + q] * (1.0f - h2 * h2);
+    }
+    __syncthreads();
+    // g_a1[e][h] = (sum_q W2[q][h] g_a2[e][q]) (1 - h1^2): rows e = 4 ty + i, columns h = 4 tx + j
+    {
+      float a[4][4] = {};
+#pragma unroll 4
+      for (int q = 0; q < HID; q += 4) {
+        float4 g[4], w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) g[i] = *reinterpret_cast<const float4*>(&sga2[(4 * ty + i) * BST + q]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = *reinterpret_cast<const float4*>(&W2[(q + k) * BST + 4 * tx]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float gq[4] = {g[i].x, g[i].y, g[i].z, g[i].w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            a[i][0] = fmaf(w[k].x, gq[k], a[i][0]);
+            a[i][1] = fmaf(w[k].y, gq[k], a[i][1]);
+            a[i][2] = fmaf(w[k].z, gq[k], a[i][2]);
+            a[i][3] = fmaf(w[k].w, gq[k], a[i][3]);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 h1 = *reinterpret_cast<const float4*>(&sh1[(4 * ty + i) * BST + 4 * tx]);
+        *reinterpret_cast<float4*>(&sga1[(4 * ty + i) * BST + 4 * tx]) =
+            make_float4(a[i][0] * (1.0f - h1.x * h1.x), a[i][1] * (1.0f - h1.y * h1.y),
+                        a[i][2] * (1.0f - h1.z * h1.z), a[i][3] * (1.0f - h1.w * h1.w));
+      }
+    }
+    // W2[q][i]: sum_e g_a2[e][q] h1[e][i], q = 4 ty + i, columns 4 tx + j
+    {
+      float a[4][4] = {};
+#pragma unroll 8
+      for (int e = 0; e < BENT; ++e) {
+        const float4 g = *reinterpret_cast<const float4*>(&sga2[e * BST + 4 * ty]);
+        const float4 h = *reinterpret_cast<const float4*>(&sh1[e * BST + 4 * tx]);
+        const float gq[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          a[i][0] = fmaf(gq[i], h.x, a[i][0]);
+          a[i][1] = fmaf(gq[i], h.y, a[i][1]);
+          a[i][2] = fmaf(gq[i], h.z, a[i][2]);
+          a[i][3] = fmaf(gq[i], h.w, a[i][3]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc2[i][j] += (double)a[i][j];
+    }
+    __syncthreads();  // g_a1 is complete
+    float a1 = 0.0f, ab = 0.0f;
+    for (int e = 0; e < BENT; ++e) a1 = fmaf(sga1[e * BST + t / NF], sphi[e * NF + t % NF], a1);
+    if (t < 64) {
+      for (int e = 0; e < BENT; ++e) ab += sga1[e * BST + t];
+    } else if (t < 128) {
+      for (int e = 0; e < BENT; ++e) ab += sga2[e * BST + t - 64];
+    } else if (t < 192) {
+      for (int e = 0; e < BENT; ++e) ab = fmaf(sgs[e], sh2[e * BST + t - 128], ab);
+    } else if (t == 192) {
+      for (int e = 0; e < BENT; ++e) ab += sgs[e];
+    }
+    acc1 += (double)a1;
+    accb += (double)ab;
   }
+  double* out = partial + (size_t)blockIdx.x * NPAR;
+  out[OW1 + t] = acc1;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[OW2 + (4 * ty + i) * HID + 4 * tx + j] = acc2[i][j];
+  if (t < 64) out[OB1 + t] = accb;
+  else if (t < 128) out[OB2 + t - 64] = accb;
+  else if (t < 192) out[OW3 + t - 128] = accb;
+  else if (t == 192) out[OB3] = accb;
 }
+static_assert(HID * NF == 256, "one W1 entry per thread of k_mlp_bwd");
 
-// grad[p] = sum over blocks of the partials (FP64 accumulation, fixed order)
-__global__ void k_param_reduce(const float* __restrict__ partial, int nblocks, float* grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= NPAR) return;
+// grad[p] = sum over the CTAs of the partials, in a fixed order: 32 parameters per CTA, 8 threads each
+__global__ void __launch_bounds__(256) k_param_reduce(const double* __restrict__ partial, int nblocks, float* grad) {
+  __shared__ double red[8][33];
+  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
   double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) acc += (double)partial[(size_t)b * NPAR + p];
-  grad[p] = (float)acc;
+  if (p < NPAR)
+    for (int b = seg; b < nblocks; b += 8) acc += partial[(size_t)b * NPAR + p];
+  red[seg][lane] = acc;
+  __syncthreads();
+  if (seg == 0 && p < NPAR) {
+    for (int k = 1; k < 8; ++k) acc += red[k][lane];
+    grad[p] = (float)acc;
+  }
 }
 
 __device__ __forceinline__ double bsum(double v, double* red) {
@@ -181,31 +257,44 @@ __device__ __forceinline__ double bsum(double v, double* red) {
   return t;
 }
 
-// one block: out[0] = r.z, out[1] = z.w, out[2] = r.e
-__global__ void k_dots3(const double* __restrict__ r, const double* __restrict__ z, const double* __restrict__ w,
-                        const double* __restrict__ e, size_t n, double* out) {
+// part[pair][k][block]: the blocks' sums of r.z, z.w and r.e of each pair (blockIdx.y)
+constexpr int kDotBlocks = 64;
+__global__ void __launch_bounds__(256) k_dots3(const double* __restrict__ r, const double* __restrict__ z,
+                                               const double* __restrict__ w, const double* __restrict__ e, size_t n,
+                                               double* part) {
   __shared__ double red[32];
+  const size_t off = blockIdx.y * n;
   double a = 0.0, b = 0.0, c = 0.0;
-  for (size_t i = threadIdx.x; i < n; i += blockDim.x) {
-    const double ri = r[i], zi = z[i];
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const double ri = r[off + i], zi = z[off + i];
     a += ri * zi;
-    b += zi * w[i];
-    c += ri * e[i];
+    b += zi * w[off + i];
+    c += ri * e[off + i];
   }
   const double ta = bsum(a, red);
   const double tb = bsum(b, red);
   const double tc = bsum(c, red);
   if (threadIdx.x == 0) {
+    double* out = part + (size_t)blockIdx.y * 3 * kDotBlocks + blockIdx.x;
     out[0] = ta;
-    out[1] = tb;
-    out[2] = tc;
+    out[kDotBlocks] = tb;
+    out[2 * kDotBlocks] = tc;
   }
 }
+// dots[3 pair + k]: the blocks' sums added in a fixed order (one warp per dot product)
+__global__ void k_dots3_sum(const double* __restrict__ part, double* dots) {
+  const double* p = part + (size_t)blockIdx.x * kDotBlocks;
+  double v = p[threadIdx.x] + p[threadIdx.x + 32];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (threadIdx.x == 0) dots[blockIdx.x] = v;
+}
+static_assert(kDotBlocks == 64, "k_dots3_sum");
 
-// g_m[f] += (x weight) * sum over the y (z) mirror images of
+// g_m[f] += (x weight) * sum over nb pairs and the y (z) mirror images of
 //           [ -(2/c) |R|^2 + (1/c) 2 Re(conj(W) R) ] / (B prod(P))
-__global__ void k_grad_accum(const double2* __restrict__ SR, const double2* __restrict__ SW, Oct o, int Py, int Pz,
-                             const double* __restrict__ dots, int B, double invP, double* g_m) {
+__global__ void k_grad_accum(const double2* __restrict__ SR, const double2* __restrict__ SW, size_t sstride, Oct o,
+                             int Py, int Pz, const double* __restrict__ dots, int nb, int B, double invP,
+                             double* g_m) {
   const size_t F = (size_t)o.Hx1 * o.Hy1 * o.Hz1;
   const size_t f = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= F) return;
@@ -214,30 +303,36 @@ __global__ void k_grad_accum(const double2* __restrict__ SR, const double2* __re
   const int kz = (int)(f / ((size_t)o.Hx1 * o.Hy1));
   const int ny_img = (ky == 0 || 2 * ky == Py) ? 1 : 2;
   const int nz_img = (o.d == 2) ? 1 : ((kz == 0 || 2 * kz == Pz) ? 1 : 2);
-  const double c = dots[2];
-  if (!(c > 0.0)) return;  // degenerate pair (zero error): no contribution
-  const double ca = -2.0 / c, cb = 2.0 / c;
-  double acc = 0.0;
-  for (int i = 0; i < ny_img; ++i) {
-    const int yy = i == 0 ? ky : Py - ky;
-    for (int j = 0; j < nz_img; ++j) {
-      const int zz = j == 0 ? kz : Pz - kz;
-      const size_t idx = (o.d == 2) ? (size_t)kx * Py + yy : ((size_t)kx * Py + yy) * Pz + zz;
-      const double2 rv = SR[idx], wv = SW[idx];
-      acc += ca * (rv.x * rv.x + rv.y * rv.y) + cb * (wv.x * rv.x + wv.y * rv.y);
-    }
-  }
   const double wx = (kx == 0 || kx == o.Hx1 - 1) ? 1.0 : 2.0;
-  g_m[f] += wx * acc * invP / B;
+  double g = g_m[f];
+  for (int pair = 0; pair < nb; ++pair) {
+    const double c = dots[3 * pair + 2];
+    if (!(c > 0.0)) continue;  // degenerate pair (zero error): no contribution
+    const double ca = -2.0 / c, cb = 2.0 / c;
+    double acc = 0.0;
+    for (int i = 0; i < ny_img; ++i) {
+      const int yy = i == 0 ? ky : Py - ky;
+      for (int j = 0; j < nz_img; ++j) {
+        const int zz = j == 0 ? kz : Pz - kz;
+        const size_t idx =
+            pair * sstride + ((o.d == 2) ? (size_t)kx * Py + yy : ((size_t)kx * Py + yy) * Pz + zz);
+        const double2 rv = SR[idx], wv = SW[idx];
+        acc += ca * (rv.x * rv.x + rv.y * rv.y) + cb * (wv.x * rv.x + wv.y * rv.y);
+      }
+    }
+    g += wx * acc * invP / B;
+  }
+  g_m[f] = g;
 }
 
 __global__ void k_loss(const double* __restrict__ dots, int B, double* loss) {
-  double L = 0.0;
-  for (int i = 0; i < B; ++i) {
+  double L = 0.0;  // one warp; lane i takes pairs i, i + 32, ...
+  for (int i = threadIdx.x; i < B; i += 32) {
     const double a = dots[3 * i], b = dots[3 * i + 1], c = dots[3 * i + 2];
     if (c > 0.0) L += (1.0 - 2.0 * a / c + b / c) / B;
   }
-  *loss = L;
+  for (int o = 16; o > 0; o >>= 1) L += __shfl_down_sync(0xffffffffu, L, o);
+  if (threadIdx.x == 0) *loss = L;
 }
 
 __global__ void k_adam(float* p, const float* __restrict__ g, float* m1, float* m2, int n, float lr, float b1, float b2,
@@ -271,62 +366,58 @@ double prodP(const Plan& p) {
   return s;
 }
 
+// Pairs whose transforms share a launch: their spectra and workspaces are held at once.
+constexpr int kLearnChunk = 8;
+
 struct LearnBufs {
-  void* awork;
-  double2* SR;
+  void* awork;    // [chunk] apply workspaces
+  double2* SR;    // [chunk] spectra, sstride entries apart
   double2* SD;
-  double* z;
+  size_t sstride;
+  double* z;      // [chunk][M]
   double* w;
   double* m;
   double* ms;
   double* gm;
   float* h1;
   float* h2;
-  float* partial;
+  double* partial;
+  double* dpart;
   double* norms;
+  size_t bytes;
 };
 
 LearnBufs carve_learn(const Plan& p, void* work, int B) {
   LearnBufs b;
-  const size_t F = p.lam_count;
-  const size_t nblk = (F + BENT - 1) / BENT;
-  unsigned char* w = reinterpret_cast<unsigned char*>(work);
-  b.awork = w;
-  w += apply_work_bytes(p, 8);
-  b.SR = reinterpret_cast<double2*>(w);
-  w += align256(spectrum_elems(p) * 16);
-  b.SD = reinterpret_cast<double2*>(w);
-  w += align256(spectrum_elems(p) * 16);
-  b.z = reinterpret_cast<double*>(w);
-  w += align256(p.M * 8);
-  b.w = reinterpret_cast<double*>(w);
-  w += align256(p.M * 8);
-  b.m = reinterpret_cast<double*>(w);
-  w += align256(F * 8);
-  b.ms = reinterpret_cast<double*>(w);
-  w += align256(F * 8);
-  b.gm = reinterpret_cast<double*>(w);
-  w += align256(F * 8);
-  b.h1 = reinterpret_cast<float*>(w);
-  w += align256(F * HID * 4);
-  b.h2 = reinterpret_cast<float*>(w);
-  w += align256(F * HID * 4);
-  b.partial = reinterpret_cast<float*>(w);
-  w += align256(nblk * NPAR * 4);
-  b.norms = reinterpret_cast<double*>(w);
-  (void)B;
+  const size_t F = p.lam_count, C = B < kLearnChunk ? B : kLearnChunk;
+  unsigned char* const w0 = reinterpret_cast<unsigned char*>(work);
+  unsigned char* w = w0;
+  auto take = [&](size_t bytes) {
+    unsigned char* q = w;
+    w += align256(bytes);
+    return q;
+  };
+  b.sstride = align256(spectrum_elems(p) * 16) / 16;
+  b.awork = take(C * apply_work_bytes(p, 8));
+  b.SR = reinterpret_cast<double2*>(take(C * b.sstride * 16));
+  b.SD = reinterpret_cast<double2*>(take(C * b.sstride * 16));
+  b.z = reinterpret_cast<double*>(take(C * p.M * 8));
+  b.w = reinterpret_cast<double*>(take(C * p.M * 8));
+  b.m = reinterpret_cast<double*>(take(F * 8));
+  b.ms = reinterpret_cast<double*>(take(F * 8));
+  b.gm = reinterpret_cast<double*>(take(F * 8));
+  b.h1 = reinterpret_cast<float*>(take(F * HID * 4));
+  b.h2 = reinterpret_cast<float*>(take(F * HID * 4));
+  b.partial = reinterpret_cast<double*>(take((size_t)kBwdCtas * NPAR * 8));
+  b.dpart = reinterpret_cast<double*>(take(C * 3 * kDotBlocks * 8));
+  b.norms = reinterpret_cast<double*>(take((size_t)3 * B * 8));
+  b.bytes = (size_t)(w - w0);
   return b;
 }
 
 }  // namespace
 
-size_t learn_work_bytes(const Plan& p, int B) {
-  const size_t F = p.lam_count;
-  const size_t nblk = (F + BENT - 1) / BENT;
-  return apply_work_bytes(p, 8) + 2 * align256(spectrum_elems(p) * 16) + 2 * align256(p.M * 8) +
-         3 * align256(F * 8) + 2 * align256(F * HID * 4) + align256(nblk * NPAR * 4) + align256((size_t)3 * B * 8) +
-         256;
-}
+size_t learn_work_bytes(const Plan& p, int B) { return carve_learn(p, nullptr, B).bytes + 256; }
 
 cudaError_t mlp_multiplier_launch(const Plan& p, const float* params, double* m, cudaStream_t s) {
   const Oct o = make_oct(p);
@@ -347,27 +438,31 @@ cudaError_t learn_grad_launch(const Plan& p, const float* params, const double* 
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   if ((err = cudaMemsetAsync(b.gm, 0, F * sizeof(double), s)) != cudaSuccess) return err;
   const int Py = p.P[1], Pz = (p.d == 3) ? p.P[2] : 1;
-  for (int i = 0; i < B; ++i) {
+  for (int i = 0; i < B; i += kLearnChunk) {
+    const int nb = B - i < kLearnChunk ? B - i : kLearnChunk;
     const double* ri = r + (size_t)i * p.M;
     const double* ei = e + (size_t)i * p.M;
-    if ((err = spectrum_forward<double>(p, ri, b.SR, b.awork, s)) != cudaSuccess) return err;
-    if ((err = spectrum_inverse<double>(p, b.SR, b.ms, b.z, b.awork, s)) != cudaSuccess) return err;
-    if ((err = apply_launch<double>(p, b.z, b.w, b.awork, s, nullptr)) != cudaSuccess) return err;
-    if ((err = spectrum_forward<double>(p, b.w, b.SD, b.awork, s)) != cudaSuccess) return err;
-    k_dots3<<<1, 1024, 0, s>>>(ri, b.z, b.w, ei, p.M, b.norms + 3 * i);
+    if ((err = spectrum_forward(p, nb, ri, b.SR, b.sstride, b.awork, s)) != cudaSuccess) return err;
+    if ((err = spectrum_inverse(p, nb, b.SR, b.sstride, b.ms, b.z, b.awork, s)) != cudaSuccess) return err;
+    if ((err = apply_batch_launch<double>(p, nb, b.z, b.w, p.M, b.awork, s, nullptr, 0, nullptr, 0)) != cudaSuccess)
+      return err;
+    if ((err = spectrum_forward(p, nb, b.w, b.SD, b.sstride, b.awork, s)) != cudaSuccess) return err;
+    k_dots3<<<dim3(kDotBlocks, nb), 256, 0, s>>>(ri, b.z, b.w, ei, p.M, b.dpart);
+    k_dots3_sum<<<3 * nb, 32, 0, s>>>(b.dpart, b.norms + 3 * i);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    k_grad_accum<<<(unsigned)((F + 255) / 256), 256, 0, s>>>(b.SR, b.SD, o, Py, Pz, b.norms + 3 * i, B, 1.0 / PP,
-                                                            b.gm);
+    k_grad_accum<<<(unsigned)((F + 255) / 256), 256, 0, s>>>(b.SR, b.SD, b.sstride, o, Py, Pz, b.norms + 3 * i, nb, B,
+                                                            1.0 / PP, b.gm);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
-  k_loss<<<1, 1, 0, s>>>(b.norms, B, loss);
-  const int nblk = (int)((F + BENT - 1) / BENT);
-  const size_t sm = (size_t)(HID * HID + 4 * BENT * HID + BENT * NF + BENT) * sizeof(float);
-  if ((err = cudaFuncSetAttribute(k_mlp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+  k_loss<<<1, 32, 0, s>>>(b.norms, B, loss);
+  const size_t ntiles = (F + BENT - 1) / BENT;
+  const int ctas = ntiles < (size_t)kBwdCtas ? (int)ntiles : kBwdCtas;
+  if ((err = cudaFuncSetAttribute(k_mlp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem)) !=
+      cudaSuccess)
     return err;
-  k_mlp_bwd<<<nblk, 256, sm, s>>>(params, o, b.gm, b.m, b.h1, b.h2, F, b.partial);
+  k_mlp_bwd<<<ctas, 256, kBwdSmem, s>>>(params, o, b.gm, b.m, b.h1, b.h2, F, b.partial);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  k_param_reduce<<<(NPAR + 255) / 256, 256, 0, s>>>(b.partial, nblk, grad);
+  k_param_reduce<<<(NPAR + 31) / 32, 256, 0, s>>>(b.partial, ctas, grad);
   return cudaGetLastError();
 }
 
