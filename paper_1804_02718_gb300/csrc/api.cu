@@ -196,19 +196,10 @@ frlap_status frlap_coeffs(int d, double alpha, double gamma, double h, const int
 
 frlap_status frlap_plan_destroy(frlap_plan* plan) {
   if (!plan) return FRLAP_OK;
-  cudaFree(plan->lam64);
-  cudaFree(plan->lamL64);
-  cudaFree(plan->lam32);
+  cudaFree(plan->tables);
   cudaFree(plan->mu_strang);
   cudaFree(plan->mu_learned);
   cudaFree(plan->mu_tau);
-  cudaFree(plan->lamdf);
-  for (int r = 0; r < 3; ++r) {
-    cudaFree(plan->tw64[r]);
-    cudaFree(plan->tw32[r]);
-    cudaFree(plan->twdf[r]);
-    cudaFree(plan->twq[r]);
-  }
   if (plan->side) cudaStreamDestroy(plan->side);
   delete plan;
   return FRLAP_OK;
@@ -259,45 +250,60 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   p->s2_elems = (d == 3) ? (size_t)Hx1 * p->P[1] * p->n[2] : (p->P[1] > kMaxLine ? p->s1_elems : 0);
 
   cudaStream_t s = (cudaStream_t)stream;
-  double* coef = nullptr;
-  void* scratch = nullptr;
   const size_t N1 = (size_t)p->Nmax + 1;
   const size_t ncoef = (d == 2) ? N1 * N1 : N1 * N1 * N1;
+  // One allocation for all of the plan's tables and one for the scratch: each cudaMalloc and cudaFree costs
+  // some 20 to 50 us of host time and a free synchronises (512^2 plan: 14 and 16 of them).
+  size_t bytes = 0;
+  auto reserve = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += align256(n);
+    return at;
+  };
+  const size_t o_lam64 = reserve(p->lam_count * sizeof(double)), o_lamL64 = reserve(p->lam_count * sizeof(double));
+  const size_t o_lam32 = prec != FRLAP_F64 ? reserve(p->lam_count * sizeof(float)) : 0;
+  const size_t o_lamdf = p->df64 ? reserve(p->lam_count * sizeof(dfl)) : 0;
+  size_t o_tw64[3], o_tw32[3], o_twq[3], o_twdf[3];
+  for (int r = 0; r < d; ++r) {
+    const size_t ntw = (size_t)twiddle_entries(p->P[r]);
+    o_tw64[r] = reserve(ntw * sizeof(double2));
+    o_tw32[r] = reserve(ntw * sizeof(float2));
+    o_twq[r] = prec != FRLAP_F32 ? reserve(ntw * sizeof(int4)) : 0;
+    o_twdf[r] = p->df64 ? reserve(ntw * sizeof(cdf)) : 0;
+  }
+  unsigned char* scratch = nullptr;
   auto cleanup = [&](frlap_status code, const std::string& msg) {
     cudaStreamSynchronize(s);
-    if (coef) cudaFree(coef);
-    if (scratch) cudaFree(scratch);
+    cudaFree(scratch);
     frlap_plan_destroy(p);
     return fail(code, msg);
   };
-  if (cudaMalloc(&coef, ncoef * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&scratch, coeffs_scratch_bytes(d, p->Nmax)) != cudaSuccess ||
-      cudaMalloc(&p->lam64, p->lam_count * sizeof(double)) != cudaSuccess ||
-      cudaMalloc(&p->lamL64, p->lam_count * sizeof(double)) != cudaSuccess)
+  if (cudaMalloc(&p->tables, bytes) != cudaSuccess ||
+      cudaMalloc(&scratch, align256(ncoef * sizeof(double)) + coeffs_scratch_bytes(d, p->Nmax)) != cudaSuccess)
     return cleanup(FRLAP_ENOMEM, "plan allocation failed");
-  if (prec != FRLAP_F64 && cudaMalloc(&p->lam32, p->lam_count * sizeof(float)) != cudaSuccess)
-    return cleanup(FRLAP_ENOMEM, "plan allocation failed");
+  double* coef = reinterpret_cast<double*>(scratch);
+  void* coef_scratch = scratch + align256(ncoef * sizeof(double));
+  unsigned char* const t = static_cast<unsigned char*>(p->tables);
+  p->lam64 = reinterpret_cast<double*>(t + o_lam64);
+  p->lamL64 = reinterpret_cast<double*>(t + o_lamL64);
+  if (prec != FRLAP_F64) p->lam32 = reinterpret_cast<float*>(t + o_lam32);
+  if (p->df64) p->lamdf = reinterpret_cast<dfl*>(t + o_lamdf);
   for (int r = 0; r < d; ++r) {
-    const int ntw = twiddle_entries(p->P[r]);
-    if (cudaMalloc(&p->tw64[r], ntw * sizeof(double2)) != cudaSuccess ||
-        cudaMalloc(&p->tw32[r], ntw * sizeof(float2)) != cudaSuccess)
-      return cleanup(FRLAP_ENOMEM, "plan allocation failed");
+    const size_t ntw = (size_t)twiddle_entries(p->P[r]);
+    p->tw64[r] = reinterpret_cast<double2*>(t + o_tw64[r]);
+    p->tw32[r] = reinterpret_cast<float2*>(t + o_tw32[r]);
     cudaError_t e = twiddle_launch(p->P[r], p->tw64[r], p->tw32[r], s);
+    if (e == cudaSuccess && prec != FRLAP_F32) {
+      p->twq[r] = reinterpret_cast<int4*>(t + o_twq[r]);
+      e = to_q_launch(p->tw64[r], p->twq[r], ntw, s);
+    }
+    if (e == cudaSuccess && p->df64) {
+      p->twdf[r] = reinterpret_cast<cdf*>(t + o_twdf[r]);
+      e = to_cdf_launch(p->tw64[r], p->twdf[r], ntw, s);
+    }
     if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
-    if (prec != FRLAP_F32) {
-      if (cudaMalloc(&p->twq[r], ntw * sizeof(int4)) != cudaSuccess)
-        return cleanup(FRLAP_ENOMEM, "plan allocation failed");
-      e = to_q_launch(p->tw64[r], p->twq[r], (size_t)ntw, s);
-      if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
-    }
-    if (p->df64) {
-      if (cudaMalloc(&p->twdf[r], ntw * sizeof(cdf)) != cudaSuccess)
-        return cleanup(FRLAP_ENOMEM, "plan allocation failed");
-      e = to_cdf_launch(p->tw64[r], p->twdf[r], (size_t)ntw, s);
-      if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
-    }
   }
-  cudaError_t e = coeffs_launch(d, alpha, gamma, h, p->Nmax, coef, scratch, s);
+  cudaError_t e = coeffs_launch(d, alpha, gamma, h, p->Nmax, coef, coef_scratch, s);
   if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("coefficients: ") + cudaGetErrorString(e));
   e = symbol_launch(*p, coef, p->lam64, s);
   if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("symbol: ") + cudaGetErrorString(e));
@@ -309,16 +315,11 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   if (e == cudaSuccess && p->lam32) e = line_symbol_launch<float>(*p, p->lam64, p->lam32, 1.0, s);
   if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("symbol copy: ") + cudaGetErrorString(e));
   if (p->df64) {
-    if (cudaMalloc(&p->lamdf, p->lam_count * sizeof(dfl)) != cudaSuccess)
-      return cleanup(FRLAP_ENOMEM, "plan allocation failed");
     e = line_symbol_launch<dfl>(*p, p->lam64, p->lamdf, 1.0, s);
     if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("symbol copy: ") + cudaGetErrorString(e));
   }
   e = cudaStreamSynchronize(s);
-  cudaFree(coef);
   cudaFree(scratch);
-  coef = nullptr;
-  scratch = nullptr;
   if (e != cudaSuccess) {
     frlap_plan_destroy(p);
     return cuda_fail(e, "plan creation");

@@ -245,6 +245,7 @@ struct Plan {
   int prec;        // frlap_prec
   size_t M;        // number of unknowns
   size_t lam_count;            // prod (P_r/2 + 1) over the used axes
+  void* tables = nullptr;      // one allocation: the symbols and twiddles below
   // The symbol octant lambda(kx, ky[, kz]), k_r = 0..P_r/2, with 1/prod(P) folded in.
   // lam64 is in natural order ([ky][kx] / [kz][ky][kx], kx fastest).  The tables the
   // apply's middle stage reads (lamL64, lam32, lamdf and the preconditioner multipliers)
