@@ -115,13 +115,16 @@ __global__ void __launch_bounds__(512, 1)
   line_sync<double>(logH);
 #pragma unroll
   for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = v[m];
+  int4 wk[8];  // W^k of this thread's pairs, in flight over the barrier
+#pragma unroll
+  for (int j = 0; j < 8; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
   line_sync<double>(logH);
   // Real-data split in place, one product per pair (see r2c_tile): X[k] = s + W^k d,
   // X[H-k] = conj(s - W^k d), s = (a + b) / 2, d = -i (a - b) / 2; stored below 2^57.5, that is over 2^(6 - D),
   // D = kQDrop.  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of the downward
   // shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in a + b.
   constexpr int D = kQDrop<REM>;
-  for (int k = lane; k <= H / 2; k += G) {
+  auto split = [&](int k, const int4 wk) {
     const int km = H - k;
     const cq a = buf[spad(k)];
     const cq b = conjg(buf[spad(km & (H - 1))]);
@@ -134,10 +137,13 @@ __global__ void __launch_bounds__(512, 1)
       d = {d.x << (D - 1), d.y << (D - 1)};
       s = q_shr_even<5 - D>(a + b);
     }
-    const cq t = q_cmul<false>(mul_i<-1>(d), FRLAP_GLD(tw + k));
+    const cq t = q_cmul<false>(mul_i<-1>(d), wk);
     buf[spad(k)] = q_shr_even<2>(s + t);
     if (k != km) buf[spad(km)] = conjg(q_shr_even<2>(s - t));
-  }
+  };
+#pragma unroll
+  for (int j = 0; j < 8; ++j) split(lane + j * G, wk[j]);
+  if (lane == 0) split(H / 2, FRLAP_GLD(tw + H / 2));
   if (valid && lane == 0) FRLAP_GST(ex + line, e + 6 - D);
   __syncthreads();
   const int logTL = __ffs(TL) - 1;
@@ -476,6 +482,9 @@ __global__ void __launch_bounds__(512, 1)
   }
   load_transposed<cq>(smem, in, TL * (H + 1), TL, LS, ldi, line0, nlines);
   unsigned o = q_publish<true>(q_ord(e), logH, slots);
+  int4 wk[8];  // W^k of this thread's pairs, in flight over the barrier
+#pragma unroll
+  for (int j = 0; j < 8; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
   __syncthreads();
   e = q_unord(q_fetch(o, logH, slots));
   int si = 1;
@@ -489,7 +498,7 @@ __global__ void __launch_bounds__(512, 1)
       const cq xk = q_align(buf[spad(k)], ea[j], e, k & 1);
       const cq b = conjg(q_align(buf[spad(km)], eb[j], e, k & 1));
       const cq A = q_shr_even<2>(xk + b), d = xk - b;
-      const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, FRLAP_GLD(tw + k)));
+      const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, j < 8 ? wk[j & 7] : FRLAP_GLD(tw + k)));
       buf[spad(k)] = A + iT;
       if (k != km && km != H) buf[spad(km)] = conjg(A - iT);
     }

@@ -366,8 +366,14 @@ double prodP(const Plan& p) {
   return s;
 }
 
-// Pairs whose transforms share a launch: their spectra and workspaces are held at once.
-constexpr int kLearnChunk = 8;
+// Pairs whose transforms share a launch: their spectra and workspaces are held at once, so at most eight, and
+// on large grids no more than 2 GB of them (one pair at least).
+int learn_chunk(const Plan& p, int B) {
+  const size_t pair = apply_work_bytes(p, 8) + 2 * align256(spectrum_elems(p) * 16) + 2 * p.M * 8;
+  const size_t fit = ((size_t)2 << 30) / pair;
+  const int c = fit < 1 ? 1 : fit > 8 ? 8 : (int)fit;
+  return B < c ? B : c;
+}
 
 struct LearnBufs {
   void* awork;    // [chunk] apply workspaces
@@ -389,7 +395,7 @@ struct LearnBufs {
 
 LearnBufs carve_learn(const Plan& p, void* work, int B) {
   LearnBufs b;
-  const size_t F = p.lam_count, C = B < kLearnChunk ? B : kLearnChunk;
+  const size_t F = p.lam_count, C = learn_chunk(p, B);
   unsigned char* const w0 = reinterpret_cast<unsigned char*>(work);
   unsigned char* w = w0;
   auto take = [&](size_t bytes) {
@@ -438,8 +444,9 @@ cudaError_t learn_grad_launch(const Plan& p, const float* params, const double* 
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   if ((err = cudaMemsetAsync(b.gm, 0, F * sizeof(double), s)) != cudaSuccess) return err;
   const int Py = p.P[1], Pz = (p.d == 3) ? p.P[2] : 1;
-  for (int i = 0; i < B; i += kLearnChunk) {
-    const int nb = B - i < kLearnChunk ? B - i : kLearnChunk;
+  const int C = learn_chunk(p, B);
+  for (int i = 0; i < B; i += C) {
+    const int nb = B - i < C ? B - i : C;
     const double* ri = r + (size_t)i * p.M;
     const double* ei = e + (size_t)i * p.M;
     if ((err = spectrum_forward(p, nb, ri, b.SR, b.sstride, b.awork, s)) != cudaSuccess) return err;
