@@ -351,12 +351,13 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // groups of contiguous lines of length n -> pad, FFT, transposed store out[g][k][line]
-template <int REM>
+template <int REM, int LOGL = 0>
 __global__ void __launch_bounds__(512, 1)
     k_q_c2cT_fwd(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
                  int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
                  int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
                  size_t ex_inst) {
+  if constexpr (LOGL > 0) logP = LOGL;
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -399,12 +400,13 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // transposed in[g][k][line] (k < P) -> IFFT along k, crop to n, store out[g][line][i]
-template <int REM>
+template <int REM, int LOGL = 0>
 __global__ void __launch_bounds__(512, 1)
     k_q_c2cT_inv(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
                  int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
                  int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
                  size_t ex_inst) {
+  if constexpr (LOGL > 0) logP = LOGL;
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -448,11 +450,12 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // Last stage.  Bin k of row r has exponent ex[k ex_k + (r / rows_per) ].
-template <int REM>
+template <int REM, int LOGL = 0>
 __global__ void __launch_bounds__(512, 1)
     k_q_c2r(const cq* __restrict__ in, double* __restrict__ out, const int* __restrict__ ex, int ex_k, int rows_per,
             int nlines, int n, size_t ldi, int logH, int TL, const int4* __restrict__ tw,
             const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  if constexpr (LOGL > 0) logH = LOGL;
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -692,8 +695,8 @@ static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const doubl
   b.in = ustride;
   b.out = w.stride;
   b.skip = skip_stride;
-  return with_rem(p.logP[0] - 1, [&](auto tag) {
-    return q_launch(k_q_r2c<decltype(tag)::value>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row, nrows, p.n[0],
+  return with_line_shape<double, true>(p.logP[0] - 1, [&](auto tag) {
+    return q_launch(k_q_r2c<decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row, nrows, p.n[0],
                     (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
   });
 }
@@ -704,8 +707,8 @@ static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tune
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
-  return with_rem(p.logP[1], [&](auto tag) {
-    return q_launch(k_q_c2cT_fwd<decltype(tag)::value>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, w.S2,
+  return with_line_shape<double, true>(p.logP[1], [&](auto tag) {
+    return q_launch(k_q_c2cT_fwd<decltype(tag)::rem, decltype(tag)::logp>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, w.S2,
                     (const int*)w.row, w.line, nz, q.tiles, ny, (size_t)nz * ny, ny, (size_t)Py * nz, nz, p.logP[1],
                     q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
   });
@@ -717,8 +720,8 @@ static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tune
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
-  return with_rem(p.logP[1], [&](auto tag) {
-    return q_launch(k_q_c2cT_inv<decltype(tag)::value>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S2, w.S1,
+  return with_line_shape<double, true>(p.logP[1], [&](auto tag) {
+    return q_launch(k_q_c2cT_inv<decltype(tag)::rem, decltype(tag)::logp>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S2, w.S1,
                     (const int*)w.col, w.line, nz, q.tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, p.logP[1],
                     q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
   });
@@ -731,8 +734,8 @@ static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, 
   b.in = w.stride;
   b.out = ystride;
   b.skip = skip_stride;
-  return with_rem(p.logP[0] - 1, [&](auto tag) {
-    return q_launch(k_q_c2r<decltype(tag)::value>, q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, y,
+  return with_line_shape<double, true>(p.logP[0] - 1, [&](auto tag) {
+    return q_launch(k_q_c2r<decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, y,
                     (const int*)(p.d == 3 ? w.line : w.col), p.d == 3 ? p.n[2] : 1, p.d == 3 ? p.n[1] : nrows, nrows,
                     p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
   });
