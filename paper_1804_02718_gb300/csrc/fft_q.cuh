@@ -283,13 +283,23 @@ __device__ __forceinline__ double q_out_any(long long v, int e) {
 
 // ---- the transform
 
+// A twiddle, loaded where it stands in the code: hoisted over a stage, a stage's fifteen spill.
+__device__ __forceinline__ int4 q_ld_tw(const int4* p) {
+#ifdef FRLAP_BOUNDS_CHECK
+  if (!bc_ok(p, sizeof(int4))) return make_int4(0, 0, 0, 0);
+#endif
+  int4 v;
+  asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 template <int SIGN>
 __device__ __forceinline__ void q_stage16(cq* v, int lane, int logNs, const int4* __restrict__ tw, int logPtab) {
   const int Ns = 1 << logNs, k = lane & (Ns - 1);
   const int4* st = tw + (1 << logPtab) + 15 * (Ns - 1) - Ns + k;  // layout: twiddle_entries
   v[0] = q_shr_round<4>(v[0]);
 #pragma unroll
-  for (int r = 1; r < 16; ++r) v[r] = q_cmul<(SIGN > 0)>(v[r], FRLAP_GLD(st + r * Ns));
+  for (int r = 1; r < 16; ++r) v[r] = q_cmul<(SIGN > 0)>(v[r], q_ld_tw(st + r * Ns));
   q_dft16<SIGN>(v);
 }
 template <int R, int SIGN>
@@ -301,7 +311,7 @@ __device__ __forceinline__ void q_last_stage(cq* v, int lane, int G, const int4*
     cq t[R];
     t[0] = q_shr_round<4>(v[b]);
 #pragma unroll
-    for (int r = 1; r < R; ++r) t[r] = q_cmul<(SIGN > 0)>(v[b + r * B], FRLAP_GLD(tw + ((r * j) << shift)));
+    for (int r = 1; r < R; ++r) t[r] = q_cmul<(SIGN > 0)>(v[b + r * B], q_ld_tw(tw + ((r * j) << shift)));
     q_dftR<R, SIGN>(t);
 #pragma unroll
     for (int r = 0; r < R; ++r) v[b + r * B] = t[r];
