@@ -61,24 +61,16 @@ typedef enum {
  * precision FFT stages and symbol.  MIXED: a plan that holds both, so
  * that the iterative-refinement solver can run FP32 inner applies and FP64
  * outer residuals (coefficients and symbol are always generated in FP64).
- * DF64: FP64 vectors in memory, FFT stages in double-float arithmetic (pairs
- * of FP32 numbers, about 48 significant bits), which GB300 runs several times
- * faster than FP64 at an accuracy within the FP64 tolerance of the apply.
- * Double-float keeps FP32's exponent range: the FFT stages hold values up to
- * about 3.4e38 (larger ones become infinite) and lose low-order bits below
- * about 1e-31 (FP32's smallest normal number is 1.2e-38 and the low word sits
- * 2^-24 below the high one).  A DF64 apply is therefore accurate to the FP64
- * tolerance for inputs with 1e-25 <~ max|u_i| and lambda_max max|u_i| <~ 1e35;
- * outside that range use an F64 plan.  frlap_pcg_solve scales the system by the
- * power of two at or below 1/max|f_i| before its double-float iterations (an
- * exact scaling, undone on the solution), so its solves have no such limit; it
- * returns FRLAP_ENAN if the right-hand side itself is not finite.
+ * DF64: FP64 vectors and symbol as F64; the first stage sets a row's scale once
+ * instead of following its values: slightly faster, normwise within 2.1e-15 of F64
+ * (rows of one spike above noise; N(0,1) and smooth vectors 2.3e-16).  A non-finite
+ * right-hand side of frlap_pcg_solve returns FRLAP_ENAN; the system is solved
+ * scaled by the power of two at or below 1/max|f_i| (exactly, undone on the
+ * solution), so that FP32 preconditioners see values they can hold.
  * MIXED_DF64: MIXED with the FP64 side computed as in DF64.
- * In frlap_pcg_solve the iterations use the plan's engine, but the residuals
- * f - A x that restart a CG solve or decide convergence (the final check, and
- * the refinement residuals from 1e-6 relative on) are computed with the native
- * FP64 engine: double-float rounding, about 5e-15 lambda_max ||x||, would
- * otherwise set a residual floor near 1e-10 ||f|| at 2047^2. */
+ * In frlap_pcg_solve the iterations use the plan's engine; the residuals f - A x
+ * that restart a CG solve or decide convergence (the final check, and the
+ * refinement residuals from 1e-6 relative on) use the F64 one. */
 typedef enum { FRLAP_F64 = 0, FRLAP_F32 = 1, FRLAP_MIXED = 2, FRLAP_DF64 = 3, FRLAP_MIXED_DF64 = 4 } frlap_prec;
 
 /* Which scratch size frlap_workspace_bytes reports. */
@@ -179,7 +171,7 @@ frlap_status frlap_apply_batch(const frlap_plan* plan, int nbatch, const void* d
  * Synchronises `stream`: h_y is complete on return.  1 <= chunk <= 65535,
  * nbatch >= 1, else FRLAP_EINVAL. */
 /* Autotuner of the apply's launch shapes.  For each stage of the apply, and for each
- * engine the plan uses (FP32, and FP64 or double-float), times every admissible
+ * engine the plan uses (FP32, and F64 or DF64), times every admissible
  * number of FFT lines per CTA (powers of two up to 512 threads and 227 KB of shared
  * memory) on a batch of nbatch zero vectors, and keeps the fastest in the plan;
  * later applies, batched applies, solves and Allen-Cahn runs on the plan use it.
@@ -246,7 +238,7 @@ frlap_status frlap_pcg_solve(const frlap_plan* plan, const double* d_f, double* 
 
 /* r = f - A x and ||r||_2 / ||f||_2 in FP64: the true relative residual that decides frlap_pcg_solve's
  * convergence (the paper solves its systems by CG, Sec. 5.3), with the same apply: the FP64 engine,
- * on double-float plans too.
+ * on DF64 plans too.
  * d_f, d_x: device FP64 vectors of the plan's unknowns (x-fastest); d_r: device, the residual, or NULL
  * for the norm only (must not overlap d_f or d_x); d_work: frlap_workspace_bytes(plan, FRLAP_OP_PCG).
  * Synchronises `stream` to return *relres.  FRLAP_EINVAL: NULL plan, d_f, d_x or relres, an F32 plan,
@@ -385,12 +377,9 @@ frlap_status frlap_allen_cahn_batch(int nbatch, const frlap_plan* const* plans, 
  * time-out path.  The paper has no counterpart. */
 frlap_status frlap_set_loop_pass_limit(unsigned max_passes);
 
-/* The first apply stage of the double-float engine stages its input rows in shared
- * memory by bulk asynchronous copies and waits for each on an mbarrier.  Every such wait is
- * bounded (about a second); a wait that gives up is counted, and that kernel returns without
- * storing its remaining tiles (the call's result is then wrong).  frlap_async_wait_report returns
- * in *timeouts the count since the previous report (summed over the engines and the tensor-core
- * waits of frlap_dft16_stages, then reset).
+/* The tensor-core stage of frlap_dft16_stages waits for its products on an mbarrier, boundedly (about a
+ * second); a wait that gives up is counted, and that kernel leaves its tile unwritten.
+ * frlap_async_wait_report returns in *timeouts the count since the previous report (then reset).
  * Synchronises the device.  A tool for tests and health checks; the paper has no counterpart. */
 frlap_status frlap_async_wait_report(unsigned long long* timeouts);
 /* The give-up path of that wait: one warp waits on an mbarrier phase that nothing completes (no
@@ -424,7 +413,7 @@ frlap_status frlap_dft16_stages(int engine, const float* d_in, float* d_out, int
  * against the buffers its call registered (the call's vectors, workspace, symbol, twiddle tables and
  * skip flags); an access outside all of them is not performed (a load gives zero) but counted.
  * frlap_bounds_check_report returns in *violations the count since the previous report (summed
- * over the FP32, FP64 and double-float kernels, then reset) and in *first_address (may be NULL) the
+ * over the FP32 and FP64 kernels, then reset) and in *first_address (may be NULL) the
  * lowest such address; *enabled (may be NULL) is 1 in a checked build, 0 otherwise (where
  * *violations is always 0).  Synchronises the device.  A tool for tests, standing in for a memory
  * checker; the paper has no counterpart. */

@@ -391,12 +391,11 @@ std::vector<Group> make_groups(int nb, const frlap_plan* const* plans) {
   return g;
 }
 
-// the group's batched apply through its FP64 engine; lam holds the stacked symbols in that engine's type
+// the group's batched apply through its plans' engine; lam holds the stacked symbols
 cudaError_t batch_apply(const Plan& p, int B, const double* u, double* y, size_t vs, void* work, cudaStream_t s,
                         const int* skip, int skip_stride, const double* lam, size_t lam_stride) {
   if (p.df64)
-    return apply_batch_launch<dfl>(p, B, u, y, vs, work, s, skip, skip_stride, reinterpret_cast<const dfl*>(lam),
-                                   lam_stride);
+    return apply_batch_launch<df64>(p, B, u, y, vs, work, s, skip, skip_stride, lam, lam_stride);
   return apply_batch_launch<double>(p, B, u, y, vs, work, s, skip, skip_stride, lam, lam_stride);
 }
 
@@ -492,8 +491,7 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
         e = cudaMemcpyAsync(g.u + k * g.vs, u[g.idx[k]], p.M * 8, cudaMemcpyDeviceToDevice, s);
         if (e == cudaSuccess)
           e = cudaMemcpyAsync(g.lam + k * (align256(p.lam_count * 8) / 8),
-                              p.df64 ? static_cast<const void*>(pi->lamdf) : static_cast<const void*>(pi->lamL64),
-                              p.lam_count * 8, cudaMemcpyDeviceToDevice, s);
+                              pi->lamL64, p.lam_count * 8, cudaMemcpyDeviceToDevice, s);
       }
     }
     if (e != cudaSuccess) {

@@ -95,17 +95,10 @@ const char* frlap_last_error(void) { return g_last_error.c_str(); }
 
 frlap_status frlap_async_wait_report(unsigned long long* timeouts) {
   if (!timeouts) return fail(FRLAP_EINVAL, "timeouts is NULL");
-  unsigned long long total = 0ull;
-  cudaError_t (*collect[3])(unsigned long long*) = {wait_collect<float>, wait_collect<double>, wait_collect<dfl>};
-  for (auto fn : collect) {
-    unsigned long long c = 0ull;
-    FRLAP_CUDA_TRY(fn(&c));
-    total += c;
-  }
-  unsigned long long cd = 0ull;
+  unsigned long long c = 0ull, cd = 0ull;
+  FRLAP_CUDA_TRY(wait_collect(&c));
   FRLAP_CUDA_TRY(dft16_wait_collect(&cd));
-  total += cd;
-  *timeouts = total;
+  *timeouts = c + cd;
   return FRLAP_OK;
 }
 
@@ -134,8 +127,7 @@ frlap_status frlap_bounds_check_report(int* enabled, unsigned long long* violati
                                        unsigned long long* first_address) {
   if (!violations) return fail(FRLAP_EINVAL, "violations is NULL");
   unsigned long long total = 0ull, first = ~0ull;
-  cudaError_t (*collect[3])(unsigned long long*, unsigned long long*) = {bc_collect<float>, bc_collect<double>,
-                                                                         bc_collect<dfl>};
+  cudaError_t (*collect[2])(unsigned long long*, unsigned long long*) = {bc_collect<float>, bc_collect<double>};
   for (auto fn : collect) {
     unsigned long long c = 0ull, f = ~0ull;
     FRLAP_CUDA_TRY(fn(&c, &f));
@@ -262,14 +254,12 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   };
   const size_t o_lam64 = reserve(p->lam_count * sizeof(double)), o_lamL64 = reserve(p->lam_count * sizeof(double));
   const size_t o_lam32 = prec != FRLAP_F64 ? reserve(p->lam_count * sizeof(float)) : 0;
-  const size_t o_lamdf = p->df64 ? reserve(p->lam_count * sizeof(dfl)) : 0;
-  size_t o_tw64[3], o_tw32[3], o_twq[3], o_twdf[3];
+  size_t o_tw64[3], o_tw32[3], o_twq[3];
   for (int r = 0; r < d; ++r) {
     const size_t ntw = (size_t)twiddle_entries(p->P[r]);
     o_tw64[r] = reserve(ntw * sizeof(double2));
     o_tw32[r] = reserve(ntw * sizeof(float2));
     o_twq[r] = prec != FRLAP_F32 ? reserve(ntw * sizeof(int4)) : 0;
-    o_twdf[r] = p->df64 ? reserve(ntw * sizeof(cdf)) : 0;
   }
   unsigned char* scratch = nullptr;
   auto cleanup = [&](frlap_status code, const std::string& msg) {
@@ -287,7 +277,6 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   p->lam64 = reinterpret_cast<double*>(t + o_lam64);
   p->lamL64 = reinterpret_cast<double*>(t + o_lamL64);
   if (prec != FRLAP_F64) p->lam32 = reinterpret_cast<float*>(t + o_lam32);
-  if (p->df64) p->lamdf = reinterpret_cast<dfl*>(t + o_lamdf);
   for (int r = 0; r < d; ++r) {
     const size_t ntw = (size_t)twiddle_entries(p->P[r]);
     p->tw64[r] = reinterpret_cast<double2*>(t + o_tw64[r]);
@@ -296,10 +285,6 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
     if (e == cudaSuccess && prec != FRLAP_F32) {
       p->twq[r] = reinterpret_cast<int4*>(t + o_twq[r]);
       e = to_q_launch(p->tw64[r], p->twq[r], ntw, s);
-    }
-    if (e == cudaSuccess && p->df64) {
-      p->twdf[r] = reinterpret_cast<cdf*>(t + o_twdf[r]);
-      e = to_cdf_launch(p->tw64[r], p->twdf[r], ntw, s);
     }
     if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
   }
@@ -314,10 +299,6 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   e = line_symbol_launch<double>(*p, p->lam64, p->lamL64, 1.0, s);
   if (e == cudaSuccess && p->lam32) e = line_symbol_launch<float>(*p, p->lam64, p->lam32, 1.0, s);
   if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("symbol copy: ") + cudaGetErrorString(e));
-  if (p->df64) {
-    e = line_symbol_launch<dfl>(*p, p->lam64, p->lamdf, 1.0, s);
-    if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("symbol copy: ") + cudaGetErrorString(e));
-  }
   e = cudaStreamSynchronize(s);
   cudaFree(scratch);
   if (e != cudaSuccess) {
@@ -406,7 +387,7 @@ frlap_status frlap_apply_batch(const frlap_plan* plan, int nbatch, const void* d
     e = apply_batch_launch<float>(*plan, nbatch, (const float*)d_u, (float*)d_y, plan->M, d_work, s, nullptr, 0,
                                   nullptr, 0, ev);
   else if (plan->df64)
-    e = apply_batch_launch<dfl>(*plan, nbatch, (const double*)d_u, (double*)d_y, plan->M, d_work, s, nullptr, 0,
+    e = apply_batch_launch<df64>(*plan, nbatch, (const double*)d_u, (double*)d_y, plan->M, d_work, s, nullptr, 0,
                                 nullptr, 0, ev);
   else
     e = apply_batch_launch<double>(*plan, nbatch, (const double*)d_u, (double*)d_y, plan->M, d_work, s, nullptr, 0,
@@ -435,7 +416,7 @@ frlap_status frlap_plan_autotune(frlap_plan* plan, int nbatch, void* d_work, voi
   if (p == FRLAP_F64 || p == FRLAP_MIXED)
     e = autotune_engine<double>(*plan, nbatch, (double*)u, (double*)y, work, s);
   else if (p == FRLAP_DF64 || p == FRLAP_MIXED_DF64)
-    e = autotune_engine<dfl>(*plan, nbatch, (double*)u, (double*)y, work, s);
+    e = autotune_engine<df64>(*plan, nbatch, (double*)u, (double*)y, work, s);
   if (e == cudaSuccess && p != FRLAP_F64 && p != FRLAP_DF64)
     e = autotune_engine<float>(*plan, nbatch, (float*)u, (float*)y, work, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -548,7 +529,7 @@ frlap_status frlap_apply_host(const frlap_plan* plan, int nbatch, int chunk, con
         e = apply_batch_launch<float>(*plan, nb, (const float*)du[k], (float*)dy[k], plan->M, awork[k], ks, nullptr,
                                       0, nullptr, 0);
       else if (plan->df64)
-        e = apply_batch_launch<dfl>(*plan, nb, (const double*)du[k], (double*)dy[k], plan->M, awork[k], ks, nullptr,
+        e = apply_batch_launch<df64>(*plan, nb, (const double*)du[k], (double*)dy[k], plan->M, awork[k], ks, nullptr,
                                     0, nullptr, 0);
       else
         e = apply_batch_launch<double>(*plan, nb, (const double*)du[k], (double*)dy[k], plan->M, awork[k], ks,
@@ -642,7 +623,7 @@ frlap_status frlap_pcg_solve(const frlap_plan* plan, const double* d_f, double* 
 frlap_status frlap_residual(const frlap_plan* plan, const double* d_f, const double* d_x, double* d_r,
                             double* relres, void* d_work, void* stream) {
   if (!plan || !d_f || !d_x || !relres) return fail(FRLAP_EINVAL, "plan, d_f, d_x or relres is NULL");
-  if (plan->prec == FRLAP_F32) return fail(FRLAP_EINVAL, "the residual needs an F64, MIXED or double-float plan");
+  if (plan->prec == FRLAP_F32) return fail(FRLAP_EINVAL, "the residual needs an F64, MIXED or DF64 plan");
   const size_t vb = vector_bytes(*plan, false);
   if (d_r && (ranges_overlap(d_r, d_f, vb) || ranges_overlap(d_r, d_x, vb)))
     return fail(FRLAP_EINVAL, "d_r must not overlap d_f or d_x");

@@ -1,24 +1,20 @@
-// The FP64 engine's apply and the spectrum transforms of the learned preconditioner (kernels and launchers in
+// The FP64 and DF64 engines' apply and the spectrum transforms of the learned preconditioner (kernels and launchers in
 // apply_q.cuh, dispatch in apply_impl.cuh), plus the engine-independent entry points.
 #include "apply_q.cuh"
 
 namespace frlap {
 
-// instantiated in apply_dfl.cu
-extern template cudaError_t apply_launch<dfl>(const Plan&, const double*, double*, void*, cudaStream_t, const int*,
-                                              cudaEvent_t const*, const dfl*, bool);
-
 size_t apply_work_bytes(const Plan& p, int real_bytes) {
   const size_t cb = 2 * (size_t)real_bytes;
   size_t b = align256(p.s1_elems * cb);
   b += align256(p.s2_elems * cb);
-  if (real_bytes == 8) b += q_exp_layout(p).total * sizeof(int);  // the FP64 engine's exponents
+  if (real_bytes == 8) b += q_exp_layout(p).total * sizeof(int);  // the fixed-point engines' exponents
   return b;
 }
 
 cudaError_t apply64(const Plan& p, const double* u, double* y, void* work, cudaStream_t s, const int* skip,
                     cudaEvent_t const* ev) {
-  if (p.df64) return apply_launch<dfl>(p, u, y, work, s, skip, ev, nullptr);
+  if (p.df64) return apply_launch<df64>(p, u, y, work, s, skip, ev, nullptr);
   return apply_launch<double>(p, u, y, work, s, skip, ev, nullptr);
 }
 
@@ -26,16 +22,168 @@ template cudaError_t apply_batch_launch<double>(const Plan&, int, const double*,
                                                 const int*, int, const double*, size_t, cudaEvent_t const*);
 template cudaError_t apply_launch<double>(const Plan&, const double*, double*, void*, cudaStream_t, const int*,
                                           cudaEvent_t const*, const double*, bool);
+template cudaError_t apply_batch_launch<df64>(const Plan&, int, const double*, double*, size_t, void*, cudaStream_t,
+                                              const int*, int, const double*, size_t, cudaEvent_t const*);
+template cudaError_t apply_launch<df64>(const Plan&, const double*, double*, void*, cudaStream_t, const int*,
+                                        cudaEvent_t const*, const double*, bool);
 
 size_t spectrum_elems(const Plan& p) {
   const size_t Hx1 = p.P[0] / 2 + 1;
   return (p.d == 2) ? Hx1 * p.P[1] : Hx1 * p.P[1] * p.P[2];
 }
 
+namespace {
+
+// Spectrum columns of the learned preconditioner: columns of n entries -> zero-pad to P, forward FFT, all P
+// outputs in FP64 (stride ldo).
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_col_fwd(const cq* __restrict__ in, const int* __restrict__ ex, double2* __restrict__ out, int ncols, int n,
+                size_t ld, size_t ldo, int logP, int TL, int cols_per, const int4* __restrict__ tw,
+                const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  in += blockIdx.y * bt.in;
+  out += blockIdx.y * bt.out;
+  ex += blockIdx.y * ex_inst;
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col = blockIdx.x * TL + l;
+  const bool valid = col < ncols;
+  const int c = valid ? col : 0;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * sline(P);
+  int si = 0;
+  cq v[16];
+  // exponents: 2D ex[i] for every column; 3D ex[(col / P_y) n + i]
+  const int kx = cols_per ? c / cols_per : c;
+  int e = q_load_aligned<8>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)kx * n : 0), kx & 1, lane, G, n, valid,
+                            logP, slots + si);
+  ++si;
+  q_fft<true, -1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  if (!valid) return;
+  double2* dst = out + (size_t)col * ldo;
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    FRLAP_GST(dst + lane + m * G, make_double2(q_out_any(v[m].x, e), q_out_any(v[m].y, e)));
+}
+
+// Columns of P FP64 spectrum values times a multiplier (natural octant order) -> inverse FFT, crop to n.
+template <int REM>
+__global__ void __launch_bounds__(512, 1)
+    k_q_col_mulinv(const double2* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int ncols, int n,
+                   size_t ld, size_t ldo, int logP, int TL, const double* __restrict__ lam, LamMap map,
+                   const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
+  in += blockIdx.y * bt.in;
+  out += blockIdx.y * bt.out;
+  ex += blockIdx.y * ex_inst;
+  FRLAP_Q_PROLOGUE(logP)
+  const int P = 1 << logP, G = P >> 4;
+  const int l = threadIdx.x / G, lane = threadIdx.x % G;
+  const int col = blockIdx.x * TL + l;
+  const bool valid = col < ncols;
+  const int c = valid ? col : 0;
+  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
+  cq* buf = smem + (size_t)l * sline(P);
+  const double2* src = in + (size_t)c * ld;
+  size_t lam_base;
+  int lam_stride;
+  if (map.d == 2) {
+    lam_base = c;
+    lam_stride = map.Hx1;
+  } else {
+    const int kx = c >> map.logPy, ky = c & (map.Py - 1);
+    lam_base = (size_t)min(ky, map.Py - ky) * map.Hx1 + kx;
+    lam_stride = map.Hy1 * map.Hx1;
+  }
+  double2 x[16];
+  unsigned hm = 0u;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int k = lane + m * G;
+    x[m] = valid ? FRLAP_GLD(lam + lam_base + (size_t)min(k, P - k) * lam_stride) * FRLAP_GLD(src + k)
+                 : make_double2(0.0, 0.0);
+  }
+#pragma unroll
+  for (int m = 0; m < 16; ++m) hm = max(hm, max(q_mag(x[m].x), q_mag(x[m].y)));
+  int si = 0;
+  const QIn qs = q_in_scale(q_reduce<true>(hm, logP, slots + si));
+  ++si;
+  cq v[16];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
+  int e = qs.e;
+  q_fft<true, 1, false, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_store_scale<REM, 8>(v, e);
+  if (valid && lane == 0) FRLAP_GST(ex + col, e);
+  store_line(v, out, ncols, n, ldo, logP, TL);
+}
+
+}  // namespace
+
+// SP = F R^T u on the half spectrum in FP64: 2D [kx][ky], 3D [kx][ky][kz] (kx <= P_x/2, full ky, kz).
+cudaError_t spectrum_forward(const Plan& p, int nb, const double* u, double2* SP, size_t sstride, void* work,
+                             cudaStream_t s) {
+  cudaError_t e;
+#ifdef FRLAP_BOUNDS_CHECK
+  {
+    BcRanges r;
+    r.add(u, nb * p.M * sizeof(double));
+    r.add(SP, nb * sstride * sizeof(double2));
+    if ((e = q_register(p, r, work, nb, s)) != cudaSuccess) return e;
+  }
+#endif
+  const QWork w = q_work(p, work);
+  if ((e = q_stage_r2c<true>(p, w, nb, u, p.M, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  if (p.d == 3 && (e = q_stage_yz_fwd(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
+  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
+  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
+  Batch b;
+  b.in = w.stride;
+  b.out = sstride;
+  return with_rem(p.logP[ax], [&](auto tag) {
+    return q_launch(k_q_col_fwd<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s,
+                    (const cq*)(p.d == 3 ? w.S2 : w.S1), (const int*)(p.d == 3 ? w.line : w.row), SP, ncols, p.n[ax],
+                    (size_t)(p.d == 3 ? p.n[2] : nrows), (size_t)p.P[ax], p.logP[ax], q.tl, p.d == 3 ? p.P[1] : 0,
+                    (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
+  });
+}
+
+// y = R F^-1 (mult * SP), mult = a symbol octant with the 1/prod(P) factor folded in.
+cudaError_t spectrum_inverse(const Plan& p, int nb, const double2* SP, size_t sstride, const double* mult, double* y,
+                             void* work, cudaStream_t s) {
+  cudaError_t e;
+#ifdef FRLAP_BOUNDS_CHECK
+  {
+    BcRanges r;
+    r.add(SP, nb * sstride * sizeof(double2));
+    r.add(mult, p.lam_count * sizeof(double));
+    r.add(y, nb * p.M * sizeof(double));
+    if ((e = q_register(p, r, work, nb, s)) != cudaSuccess) return e;
+  }
+#endif
+  const QWork w = q_work(p, work);
+  const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
+  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
+  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
+  const LamMap map = q_lam_map(p);
+  Batch b;
+  b.in = sstride;
+  b.out = w.stride;
+  e = with_rem(p.logP[ax], [&](auto tag) {
+    return q_launch(k_q_col_mulinv<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
+                    w.col, ncols, p.n[ax], (size_t)p.P[ax], (size_t)(p.d == 3 ? p.n[2] : nrows), p.logP[ax], q.tl, mult,
+                    map, (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
+  });
+  if (e != cudaSuccess) return e;
+  if (p.d == 3 && (e = q_stage_yz_inv(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
+  return q_stage_c2r(p, w, nb, y, p.M, 0, nullptr, 0, s);
+}
+
 template cudaError_t autotune_engine<double>(Plan&, int, double*, double*, void*, cudaStream_t);
+template cudaError_t autotune_engine<df64>(Plan&, int, double*, double*, void*, cudaStream_t);
 
 template cudaError_t bc_collect<double>(unsigned long long*, unsigned long long*);
-template cudaError_t wait_collect<double>(unsigned long long*);
 
 #ifdef FRLAP_BOUNDS_CHECK
 static __device__ double g_bc_probe[16];
@@ -74,6 +222,49 @@ cudaError_t bc_selftest(unsigned long long* flagged) {
 #endif
 }
 
+namespace {
+
+// ---- the bounded mbarrier wait
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned arrivals) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(arrivals) : "memory");
+  // the initialised barrier is visible to the asynchronous proxy that completes its transactions
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+}
+
+// Waits until the phase of `bar` with the given parity has completed.  Each try suspends the
+// thread for at most about kWaitHintNs; after kWaitTries tries (about a second) it gives up and
+// returns false.
+constexpr unsigned kWaitHintNs = 1000;
+constexpr int kWaitTries = 1 << 20;
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
+  const unsigned a = smem_addr(bar);
+  for (int i = 0; i < kWaitTries; ++i) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(a), "r"(parity), "r"(kWaitHintNs)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+// Waits that gave up (wait_collect reads and resets it).
+__device__ unsigned long long g_wait_timeouts = 0ull;
+
+}  // namespace
+
+cudaError_t wait_collect(unsigned long long* count) {
+  cudaError_t e = cudaMemcpyFromSymbol(count, g_wait_timeouts, sizeof(*count));
+  if (e != cudaSuccess) return e;
+  const unsigned long long z = 0ull;
+  return cudaMemcpyToSymbol(g_wait_timeouts, &z, sizeof(z));
+}
+
 // The give-up path of the bounded mbarrier wait: one warp waits on a phase that nothing
 // completes (no arrival, no copy in flight), gives up after the wait's bound, and records it.
 __global__ void k_wait_selftest() {
@@ -86,12 +277,12 @@ __global__ void k_wait_selftest() {
 
 cudaError_t wait_selftest(unsigned long long* timeouts) {
   unsigned long long c = 0;
-  cudaError_t e = wait_collect<double>(&c);  // reset
+  cudaError_t e = wait_collect(&c);  // reset
   if (e != cudaSuccess) return e;
   k_wait_selftest<<<1, 32>>>();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
-  return wait_collect<double>(timeouts);
+  return wait_collect(timeouts);
 }
 
 }  // namespace frlap

@@ -14,8 +14,8 @@
 // Every stage reads and writes whole contiguous lines or TL-wide contiguous
 // tiles; every global index below is bounded by the line/tile validity tests.
 //
-// This header holds the kernel and launcher templates; apply_f32.cu and apply_dfl.cu instantiate them, one
-// translation unit per engine.  The FP64 engine has kernels of its own (apply_q.cuh, apply_f64.cu).
+// This header holds the FP32 engine's kernels and what the engines share.  The FP64-class engines have kernels of
+// their own (apply_q.cuh).  Two translation units: apply_f32.cu and apply_f64.cu.
 #pragma once
 
 #include <type_traits>
@@ -101,52 +101,6 @@ __device__ __forceinline__ void cp_async_elem(void* dst, const void* src, bool p
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// ---- bulk asynchronous copies completing on an mbarrier (the TMA unit's untiled copy)
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned arrivals) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(arrivals) : "memory");
-  // the initialised barrier is visible to the asynchronous proxy that completes its transactions
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-
-// One arrival that also raises the phase's expected transaction count by `bytes`.
-__device__ __forceinline__ void mbar_arrive_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-
-// dst (shared, 16-byte aligned) <- src (global, 16-byte aligned), `bytes` a multiple of 16; the
-// bytes count against bar's expected transactions.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                   smem_addr(dst)),
-               "l"(src), "r"(bytes), "r"(smem_addr(bar))
-               : "memory");
-}
-
-// Waits until the phase of `bar` with the given parity has completed.  Each try suspends the
-// thread for at most about kWaitHintNs; after kWaitTries tries (about a second) it gives up and
-// returns false.
-constexpr unsigned kWaitHintNs = 1000;
-constexpr int kWaitTries = 1 << 20;
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
-  const unsigned a = smem_addr(bar);
-  for (int i = 0; i < kWaitTries; ++i) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(a), "r"(parity), "r"(kWaitHintNs)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-// Waits that gave up (one copy per translation unit; wait_collect reads and resets it).
-static __device__ unsigned long long g_wait_timeouts = 0ull;
-
 // smem[l][spad(k)] = src[k * ld + line0 + l] for l < TL, k < total / TL (zero past nlines);
 // TL is a power of two dividing blockDim.x.  Thread t serves line t mod TL and rows
 // k = t / TL + j (blockDim.x / TL), walking its source column with a pointer increment.  Every
@@ -174,7 +128,7 @@ __device__ __forceinline__ void load_transposed(C* smem, const C* __restrict__ s
 
 // Threads per CTA the apply kernels are compiled for.  FP32 kernels fit 64 registers a thread,
 // so 1024-thread CTAs cost them no registers and let the transposed stages hold twice as many
-// lines per CTA; the FP64 and double-float kernels need 128 registers (512 threads).
+// lines per CTA; the fixed-point kernels need 128 registers (512 threads).
 template <typename T>
 constexpr int kMaxCta = std::is_same<T, float>::value ? 1024 : 512;
 
@@ -194,44 +148,10 @@ __host__ __device__ __forceinline__ int r2c_line_stride(int L, int TL) {
   return s;
 }
 
-// The real-data split of the first and last stages: computed per output element inside the
-// transposed store / the transform's register load (one complex product per element, no
-// shared-memory write-back), or in place per pair of bins (one product per pair, one more pass
-// over shared memory).  Per stage and engine, the faster measured form: the per-element form in
-// the forward stage of FP32 and double-float and in the inverse stage of FP32 (2047^2:
-// double-float r2c 99 -> 95 us, FP32 c2r 24 -> 22 us); the per-pair form where the extra
-// products cost more than the pass (native FP64; the double-float inverse, 75 against 86 us).
-template <typename T>
-constexpr bool kFusedSplitR2C = !std::is_same<T, double>::value;
-template <typename T>
-constexpr bool kFusedSplitC2R = std::is_same<T, float>::value;
-
-// The first stage runs as the persistent k_r2c_pf (its input rows' loads overlap the previous
-// tile's arithmetic) in the double-float engine for transforms of up to 1024 points,
-// as measured: 255^3 r2c 235 -> 221 us per 2-vector launch, while the 2048-point
-// rows of 2047^2 keep k_r2c_T (71 against 77 us per vector).  FP32 keeps k_r2c_T everywhere: its
-// first stage is bound by shared-memory and store throughput, not load latency (persistent form
-// at 255^3: 44.7 -> 51.0 us per launch; at 2047^2: 21.3 -> 21.0 us per vector).  -1: never.
-template <typename T>
-constexpr int kR2CPersistentMaxLogH = std::is_same<T, dfl>::value ? 10 : -1;
-template <typename T>
-inline bool use_r2c_pf(int logH, const void* u) {
-  return logH <= kR2CPersistentMaxLogH<T> && (reinterpret_cast<uintptr_t>(u) % sizeof(io_t<T>)) == 0;
-}
+// The real-data split of the first and last stages is computed per output element inside the transposed store /
+// the transform's register load (one complex product per element, no shared-memory write-back; 2047^2 last
+// stage 24 -> 22 us against one product per pair and a pass more over shared memory).
 constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory per CTA
-
-// Multiprocessors of the current device (cached per device).
-inline int device_sm_count() {
-  static int cached[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (cached[dev] == 0) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-    cached[dev] = n;
-  }
-  return cached[dev];
-}
 
 // The rest of the first stage for one tile of TL rows, once each thread holds its row's packed
 // samples in v (lane's q = lane + m G, see k_r2c_T): the half-length transform, the real-data
@@ -258,53 +178,22 @@ __device__ __forceinline__ void r2c_tile(cplx<T>* v, cplx<T>* smem, cplx<T>* __r
   const bool lt_ok = line0 + lt < nlines;
   const C* trow = smem + (size_t)lt * LS;
   const size_t gstep = (size_t)G * ldo;
-  if constexpr (kFusedSplitR2C<T>) {
-    // each output of the transposed store computes its own X[k] from the two bins it needs
-    // (one product per output, no write-back pass over shared memory)
-    __syncthreads();
-    if (lt_ok) {
-      int k = (int)threadIdx.x >> logTL;
-      C* gp = out + (size_t)k * ldo + line0 + lt;
-      if constexpr (std::is_same<T, float>::value) {
-        // FP32: the thread's bins are k0 + j G, and W^{k0 + j G} = W^{k0} W_32^j (one table load)
-        const C w0 = FRLAP_GLD(tw + k);
+  // each output of the transposed store computes its own X[k] from the two bins it needs
+  __syncthreads();
+  if (lt_ok) {
+    int k = (int)threadIdx.x >> logTL;
+    C* gp = out + (size_t)k * ldo + line0 + lt;
+    // the thread's bins are k0 + j G, and W^{k0 + j G} = W^{k0} W_32^j (one table load)
+    const C w0 = FRLAP_GLD(tw + k);
 #pragma unroll
-        for (int j = 0; j <= 16; ++j) {
-          const int kj = k + j * G;
-          if (kj <= H) {
-            const C a = trow[spad(kj & (H - 1))];
-            const C b = conjg(trow[spad((H - kj) & (H - 1))]);
-            const C wk = j == 0 ? w0 : cmul(w0, make_float2(c_w32.re[j], c_w32.im[j]));
-            FRLAP_GST(gp + (size_t)j * gstep, halve(a + b) + cmul(wk, halve(mul_i<-1>(a - b))));
-          }
-        }
-      } else {
-#pragma unroll 4
-        for (; k <= H; k += G, gp += gstep) {
-          const C a = trow[spad(k & (H - 1))];
-          const C b = conjg(trow[spad((H - k) & (H - 1))]);
-          FRLAP_GST(gp, halve(a + b) + cmul(FRLAP_GLD(tw + k), halve(mul_i<-1>(a - b))));
-        }
+    for (int j = 0; j <= 16; ++j) {
+      const int kj = k + j * G;
+      if (kj <= H) {
+        const C a = trow[spad(kj & (H - 1))];
+        const C b = conjg(trow[spad((H - kj) & (H - 1))]);
+        const C wk = j == 0 ? w0 : cmul(w0, make_float2(c_w32.re[j], c_w32.im[j]));
+        FRLAP_GST(gp + (size_t)j * gstep, halve(a + b) + cmul(wk, halve(mul_i<-1>(a - b))));
       }
-    }
-  } else {
-    line_sync<T>(logH);
-    // in place, one product per pair: X[k] = E + W^k O and X[H-k] = conj(E - W^k O)
-    for (int k = lane; k <= H / 2; k += G) {
-      const int km = H - k;
-      const C a = buf[spad(k)];
-      const C b = conjg(buf[spad(km & (H - 1))]);
-      const C e = halve(a + b);
-      const C t = cmul(FRLAP_GLD(tw + k), halve(mul_i<-1>(a - b)));
-      buf[spad(k)] = e + t;
-      if (k != km) buf[spad(km)] = conjg(e - t);
-    }
-    __syncthreads();
-    if (lt_ok) {
-      int k = (int)threadIdx.x >> logTL;
-      C* gp = out + (size_t)k * ldo + line0 + lt;
-#pragma unroll 4
-      for (; k <= H; k += G, gp += gstep) FRLAP_GST(gp, trow[spad(k)]);
     }
   }
 }
@@ -352,7 +241,7 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_r2c_T(const io_t<T>* __restri
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int q = lane + m * G;
-      v[m] = mk<C>(from_io<T>(odd_ext(src, 2 * q, n, H, valid)), from_io<T>(odd_ext(src, 2 * q + 1, n, H, valid)));
+      v[m] = mk<C>((odd_ext(src, 2 * q, n, H, valid)), (odd_ext(src, 2 * q + 1, n, H, valid)));
     }
     r2c_tile<T, REM, false>(v, smem, out, nlines, ldo, logH, TL, tw, logP, line0, l, lane);
     return;
@@ -374,132 +263,9 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_r2c_T(const io_t<T>* __restri
           if (2 * q + 1 < n) im = FRLAP_GLD(src + 2 * q + 1);
         }
       }
-      v[m] = mk<C>(from_io<T>(re), from_io<T>(im));
+      v[m] = mk<C>((re), (im));
     }
     r2c_tile<T, REM>(v, smem, out, nlines, ldo, logH, TL, tw, logP, line0, l, lane);
-  }
-}
-
-// Staging area of k_r2c_pf: the TL n elements of a tile's rows (E bytes each), shifted by the
-// tile start's offset from a 16-byte boundary (0..16/E - 1 elements), rounded up to 16 bytes;
-// then the mbarrier.
-template <int E>
-__host__ __device__ __forceinline__ int r2c_stage_elems(int TL, int n) {
-  constexpr int A = 16 / E;
-  return (TL * n + 2 * A - 2) / A * A;
-}
-// Byte offset of the staging area: after the TL transform lines, rounded up to 16 bytes (an
-// FP32 line of sline(H) complex elements is 8 bytes past a 16-byte boundary when TL is odd).
-template <typename T>
-__host__ __device__ __forceinline__ size_t r2c_stage_offset(int TL, int H) {
-  return ((size_t)TL * sline(H) * sizeof(cplx<T>) + 15) & ~(size_t)15;
-}
-template <typename T>
-size_t r2c_pf_smem_bytes(int TL, int H, int n) {
-  constexpr int E = (int)sizeof(io_t<T>);
-  return r2c_stage_offset<T>(TL, H) + (size_t)r2c_stage_elems<E>(TL, n) * E + 16;
-}
-
-// Persistent form of k_r2c_T for rows whose TL rows per tile are contiguous (row stride n).
-// CTA c takes the tiles t = c, c + gridDim.x, ... of all instances (t = instance * tiles +
-// tile).  A tile's rows reach a shared-memory staging area by one bulk asynchronous copy,
-// completing on an mbarrier, that thread 0 issues as soon as every thread holds the previous
-// tile's samples in registers: the copy runs during that tile's transform and transposed
-// store, so the loads' latency leaves the critical path.  The bulk copy moves the
-// 16-byte-aligned interior of the tile's span; the elements before and after it (a span that
-// does not start or end on a 16-byte boundary) are element-sized cp.async copies.
-template <typename T, int REM, int LOGL = 0>
-__global__ void __launch_bounds__(kMaxCta<T>, 1) k_r2c_pf(const io_t<T>* __restrict__ in, cplx<T>* __restrict__ out, int nlines, int n,
-                         size_t ldo, int logH, int TL, const cplx<T>* __restrict__ tw, int logP,
-                         const int* __restrict__ skip, Batch bt, int ninst) {
-  static_assert(LOGL == 0 || (LOGL & 3) == REM, "REM = LOGL mod 4");
-  if constexpr (LOGL > 0) {  // transform length fixed at compile time
-    logH = LOGL;
-    logP = LOGL + 1;
-  }
-  using C = cplx<T>;
-  using IO = io_t<T>;
-  constexpr int E = (int)sizeof(IO);
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* smem = reinterpret_cast<C*>(smem_raw);
-  const int H = 1 << logH, G = H >> 4;
-  const int l = threadIdx.x / G, lane = threadIdx.x % G;
-  IO* stage = reinterpret_cast<IO*>(smem_raw + r2c_stage_offset<T>(TL, H));  // 16-byte aligned
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(stage + r2c_stage_elems<E>(TL, n));
-  const int ntiles = (nlines + TL - 1) / TL;
-  const long long total = (long long)ntiles * ninst;
-  // tile t: its instance, first row, and the address of its first element
-  auto tile_src = [&](long long t, int& b, int& line0) {
-    b = (int)(t / ntiles);
-    line0 = (int)(t - (long long)b * ntiles) * TL;
-    return in + (size_t)b * bt.in + (size_t)line0 * n;
-  };
-  // thread 0: start the copies of tile t into the staging area (element j at stage[j + off])
-  auto issue = [&](long long t) {
-    int b, line0;
-    const IO* src = tile_src(t, b, line0);
-    if (skip && FRLAP_GLD(skip + (size_t)b * bt.skip)) {  // a skipped instance: nothing to copy
-      mbar_arrive_tx(bar, 0u);
-      return;
-    }
-    const int cnt = min(TL, nlines - line0) * n;
-    const uintptr_t a = reinterpret_cast<uintptr_t>(src);
-    const int off = (int)((a & 15) / E);
-    const uintptr_t a1 = (a + 15) & ~(uintptr_t)15, e0 = (a + (uintptr_t)cnt * E) & ~(uintptr_t)15;
-    unsigned bytes = e0 > a1 ? (unsigned)(e0 - a1) : 0u;
-    const int h = min((int)((a1 - a) / E), cnt);                         // elements before the bulk part
-    const int tl0 = bytes ? (int)((e0 - a) / E) : h;                     // first element after it
-#ifdef FRLAP_BOUNDS_CHECK
-    if (bytes && !bc_ok(reinterpret_cast<const void*>(a1), bytes)) bytes = 0u;
-#endif
-    for (int j = 0; j < h; ++j) cp_async_elem<E>(stage + j + off, src + j, FRLAP_GOK(src + j));
-    for (int j = tl0; j < cnt; ++j) cp_async_elem<E>(stage + j + off, src + j, FRLAP_GOK(src + j));
-    mbar_arrive_tx(bar, bytes);
-    if (bytes) bulk_g2s(stage + h + off, reinterpret_cast<const void*>(a1), bytes, bar);
-  };
-  if (threadIdx.x == 0) mbar_init(bar, 1);
-  __syncthreads();
-  long long t = blockIdx.x;
-  if (threadIdx.x == 0 && t < total) issue(t);
-  unsigned parity = 0;
-  for (; t < total; t += gridDim.x) {
-    cp_async_wait_all();  // thread 0's element copies of this tile
-    const bool ok = mbar_wait(bar, parity);
-    parity ^= 1;
-    if (!__syncthreads_and(ok)) {  // the staging copy did not complete in time: record and stop
-      if (threadIdx.x == 0) atomicAdd(&g_wait_timeouts, 1ull);
-      return;
-    }
-    int b, line0;
-    const IO* src = tile_src(t, b, line0);
-    const bool skipped = skip && FRLAP_GLD(skip + (size_t)b * bt.skip);
-    const int off = (int)((reinterpret_cast<uintptr_t>(src) & 15) / E);
-    const bool valid = line0 + l < nlines;
-    // packed samples z[q] = x[2q] + i x[2q+1] of row line0 + l, as in k_r2c_T
-    const IO* row = stage + (size_t)l * n + off;
-    const bool pair_aligned = ((l * n + off) & 1) == 0;
-    using IO2 = io_pair<T>;
-    C v[16];
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int q = lane + m * G;
-      IO re = IO(0), im = IO(0);
-      if (m < 8 && valid) {
-        if (pair_aligned && 2 * q + 1 < n) {
-          const IO2 p2 = *reinterpret_cast<const IO2*>(row + 2 * q);
-          re = p2.x;
-          im = p2.y;
-        } else {
-          if (2 * q < n) re = row[2 * q];
-          if (2 * q + 1 < n) im = row[2 * q + 1];
-        }
-      }
-      v[m] = mk<C>(from_io<T>(re), from_io<T>(im));
-    }
-    __syncthreads();  // the staging area is free: start the next tile's copy
-    if (threadIdx.x == 0 && t + gridDim.x < total) issue(t + gridDim.x);
-    if (!skipped)
-      r2c_tile<T, REM>(v, smem, out + (size_t)b * bt.out, nlines, ldo, logH, TL, tw, logP, line0, l, lane);
   }
 }
 
@@ -534,32 +300,16 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_c2r_T(const cplx<T>* __restri
   // repack: Z[k] = A + i T with A = X[k] + conj X[H-k], T = W^{-k} (X[k] - conj X[H-k]), so that
   // the unnormalised inverse half-length transform gives P (y[2j] + i y[2j+1])
   C v[16];
-  if constexpr (kFusedSplitC2R<T>) {
-    // straight into the registers the transform starts from (one product per element); the
-    // twiddle of bin lane + m G is W^{lane} W_32^m (one table load per thread)
-    const C w0 = FRLAP_GLD(tw + lane);
+  // straight into the registers the transform starts from (one product per element); the
+  // twiddle of bin lane + m G is W^{lane} W_32^m (one table load per thread)
+  const C w0 = FRLAP_GLD(tw + lane);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int k = lane + m * G;
-      const C xk = buf[spad(k)];
-      const C b = conjg(buf[spad(H - k)]);
-      const C wk = m == 0 ? w0 : cmul(w0, mk<C>(c_w32.re[m], c_w32.im[m]));
-      v[m] = (xk + b) + mul_i<1>(cmulc(xk - b, wk));
-    }
-  } else {
-    // in place, one product per pair; the partner is Z[H-k] = conj(A - i T)
-    for (int k = lane; k <= H / 2; k += G) {
-      const int km = H - k;
-      const C xk = buf[spad(k)];
-      const C b = conjg(buf[spad(km)]);
-      const C A = xk + b;
-      const C iT = mul_i<1>(cmulc(xk - b, FRLAP_GLD(tw + k)));
-      buf[spad(k)] = A + iT;
-      if (k != km && km != H) buf[spad(km)] = conjg(A - iT);
-    }
-    line_sync<T>(logH);
-#pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = buf[spad(lane + m * G)];
+  for (int m = 0; m < 16; ++m) {
+    const int k = lane + m * G;
+    const C xk = buf[spad(k)];
+    const C b = conjg(buf[spad(H - k)]);
+    const C wk = m == 0 ? w0 : cmul(w0, mk<C>(c_w32.re[m], c_w32.im[m]));
+    v[m] = (xk + b) + mul_i<1>(cmulc(xk - b, wk));
   }
   fft_regs<T, 1, false, REM>(v, buf, logH, lane, tw, logP, true);
   // v[m] = y[2q] + i y[2q+1] (times P), q = lane + m G; n <= H keeps only m < 8
@@ -569,8 +319,8 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_c2r_T(const cplx<T>* __restri
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
         const int q = lane + m * G;
-        if (q >= 1 && 2 * q <= n) FRLAP_GST(dst + (2 * q - 1), to_io<T>(re(v[m])));
-        if (2 * q + 1 <= n) FRLAP_GST(dst + 2 * q, to_io<T>(im(v[m])));
+        if (q >= 1 && 2 * q <= n) FRLAP_GST(dst + (2 * q - 1), (re(v[m])));
+        if (2 * q + 1 <= n) FRLAP_GST(dst + 2 * q, (im(v[m])));
       }
     }
   } else if (line < nlines) {
@@ -582,12 +332,12 @@ __global__ void __launch_bounds__(kMaxCta<T>, 1) k_c2r_T(const cplx<T>* __restri
       const int q = lane + m * G;
       if (pair_aligned && 2 * q + 1 < n) {
         IO2 t;
-        t.x = to_io<T>(re(v[m]));
-        t.y = to_io<T>(im(v[m]));
+        t.x = (re(v[m]));
+        t.y = (im(v[m]));
         FRLAP_GST(reinterpret_cast<IO2*>(dst + 2 * q), t);
       } else {
-        if (2 * q < n) FRLAP_GST(dst + 2 * q, to_io<T>(re(v[m])));
-        if (2 * q + 1 < n) FRLAP_GST(dst + 2 * q + 1, to_io<T>(im(v[m])));
+        if (2 * q < n) FRLAP_GST(dst + 2 * q, (re(v[m])));
+        if (2 * q + 1 < n) FRLAP_GST(dst + 2 * q + 1, (im(v[m])));
       }
     }
   }
@@ -916,6 +666,7 @@ int pick_tl_tuned(int tuned, int len, int elem_bytes, int G, int budget, long lo
   return tl;
 }
 
+// the engine's row of Plan::tl_tuned
 template <typename T>
 constexpr int engine_index() {
   return std::is_same<T, float>::value ? 0 : (std::is_same<T, double>::value ? 1 : 2);
@@ -947,90 +698,44 @@ struct ShapeTag {
   static constexpr int rem = R;
   static constexpr int logp = L;
 };
-// Transform shapes of the apply stages: with SPEC, every line length the plans allow (2^4 .. 2^13
-// points) runs a kernel with the length fixed at compile time; without, the run-time-length
-// kernel.  k_colmul is specialised for FP32 and double-float, the other stages for FP32 only
-// (the double-float ones are dominated by their arithmetic; their instances would double the
-// compile time).
-template <typename T, bool SPEC = !std::is_same<T, double>::value, typename F>
+// Transform shapes of the apply stages: every line length the plans allow (2^4 .. 2^13 points) runs a kernel
+// with the length fixed at compile time.
+template <typename F>
 cudaError_t with_line_shape(int logP, F&& f) {
-  if constexpr (SPEC) {
-    switch (logP) {
-      case 4: return f(ShapeTag<0, 4>{});
-      case 5: return f(ShapeTag<1, 5>{});
-      case 6: return f(ShapeTag<2, 6>{});
-      case 7: return f(ShapeTag<3, 7>{});
-      case 8: return f(ShapeTag<0, 8>{});
-      case 9: return f(ShapeTag<1, 9>{});
-      case 10: return f(ShapeTag<2, 10>{});
-      case 11: return f(ShapeTag<3, 11>{});
-      case 12: return f(ShapeTag<0, 12>{});
-      case 13: return f(ShapeTag<1, 13>{});
-      default: return cudaErrorInvalidValue;  // plan creation admits no longer line
-    }
-  } else {
-    return with_rem(logP, [&](auto t) { return f(ShapeTag<decltype(t)::value, 0>{}); });
+  switch (logP) {
+    case 4: return f(ShapeTag<0, 4>{});
+    case 5: return f(ShapeTag<1, 5>{});
+    case 6: return f(ShapeTag<2, 6>{});
+    case 7: return f(ShapeTag<3, 7>{});
+    case 8: return f(ShapeTag<0, 8>{});
+    case 9: return f(ShapeTag<1, 9>{});
+    case 10: return f(ShapeTag<2, 10>{});
+    case 11: return f(ShapeTag<3, 11>{});
+    case 12: return f(ShapeTag<0, 12>{});
+    case 13: return f(ShapeTag<1, 13>{});
+    default: return cudaErrorInvalidValue;  // plan creation admits no longer line
   }
 }
 
 }  // namespace
 
+// The FP64-class engines' stages (apply_q.cuh), which only their own translation unit compiles.
+template <typename T>
+cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, size_t vstride, void* work,
+                             cudaStream_t s, const int* skip, int skip_stride, cudaEvent_t const* ev,
+                             const double* lam_override, size_t lam_stride);
+
 // B instances of the same shape: u, y at stride `vstride` elements, workspace at stride
 // apply_work_bytes(p), symbols at stride lam_stride (0: all share one), skip flags at
 // stride skip_stride ints.
 template <typename T>
-static const cplx<T>* twiddle_table(const Plan& p, int r) {
-  if constexpr (std::is_same<T, double>::value) return p.tw64[r];
-  else if constexpr (std::is_same<T, float>::value) return p.tw32[r];
-  else return p.twdf[r];
-}
-
-template <typename T>
-static const T* symbol_table(const Plan& p) {
-  if constexpr (std::is_same<T, double>::value) return p.lamL64;
-  else if constexpr (std::is_same<T, float>::value) return p.lam32;
-  else return p.lamdf;
-}
-
-// The first stage as the persistent k_r2c_pf: as many CTAs as fit on the device at once, or one
-// per tile if there are fewer tiles.
-template <typename T>
-cudaError_t launch_r2c_pf(const io_t<T>* u, cplx<T>* S1, int nrows, int nx, size_t ld1, int logH, int tl, size_t sm,
-                          const cplx<T>* tw, const int* skip, Batch b_in, int B, cudaStream_t s) {
-  if constexpr (kR2CPersistentMaxLogH<T> < 0) {
-    return cudaErrorNotSupported;
-  } else {
-    const int G = 1 << (logH - 4);
-    return with_line_shape<T, std::is_same<T, float>::value>(logH, [&](auto tag) {
-      constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
-      cudaError_t e = set_smem(k_r2c_pf<T, REM, LL>, sm);
-      if (e != cudaSuccess) return e;
-      int occ = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_r2c_pf<T, REM, LL>, tl * G, sm);
-      if (e != cudaSuccess) return e;
-      const long long tiles = (long long)((nrows + tl - 1) / tl) * B;
-      const long long slots = (long long)(occ > 0 ? occ : 1) * device_sm_count();
-      const int grid = (int)(tiles < slots ? tiles : slots);
-      k_r2c_pf<T, REM, LL><<<grid, tl * G, sm, s>>>(u, S1, nrows, nx, ld1, logH, tl, tw, logH + 1, skip, b_in, B);
-      return cudaGetLastError();
-    });
-  }
-}
-
-// The same in the FP64 engine (apply_q.cuh), which only its own translation unit compiles.
-template <typename T>
-cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstride, void* work, cudaStream_t s,
-                             const int* skip, int skip_stride, cudaEvent_t const* ev, const T* lam_override,
-                             size_t lam_stride);
-
-template <typename T>
 static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T>* y, size_t vstride, void* work,
                                   cudaStream_t s, const int* skip, int skip_stride, cudaEvent_t const* ev,
-                                  const T* lam_override, size_t lam_stride, bool odd = false) {
+                                  const io_t<T>* lam_override, size_t lam_stride, bool odd = false) {
   // odd: the pipeline on odd extensions (a multiplier in the sine basis, see k_r2c_T); the FP32
   // engine only, P_r = 2(n_r + 1) on every axis (the callers check)
   if (odd && (!std::is_same<T, float>::value || p.P[1] > kMaxLine)) return cudaErrorNotSupported;
-  if constexpr (std::is_same<T, double>::value) {
+  if constexpr (!std::is_same<T, float>::value) {
     return q_apply_launch_b<T>(p, B, u, y, vstride, work, s, skip, skip_stride, ev, lam_override, lam_stride);
   } else {
   int stage = 0;
@@ -1046,9 +751,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
   const int eb = sizeof(C);
   const int budget = 96 * 1024;
   const int* tuned = p.tl_tuned[engine_index<T>()];
-  const C* tw[3];
-  for (int r = 0; r < 3; ++r) tw[r] = twiddle_table<T>(p, r);
-  const T* lam = lam_override ? lam_override : symbol_table<T>(p);
+  const C* const* tw = p.tw32;
+  const T* lam = lam_override ? lam_override : p.lam32;
   C* S1 = reinterpret_cast<C*>(work);
   C* S2 = reinterpret_cast<C*>(reinterpret_cast<unsigned char*>(work) + align256(p.s1_elems * eb));
   const int nx = p.n[0], ny = p.n[1], nz = p.n[2];
@@ -1088,24 +792,13 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
   b_out.skip = skip_stride;
 
   // ---- stage 1: rows of u -> S1[kx][row]
-  if (!odd && use_r2c_pf<T>(logPx - 1, u)) {
-    const int G = Hx >> 4;
-    const int q = G < 32 ? 32 / G : 1;
-    int tl = pick_tl_tuned(tuned[0], sline(Hx), eb, G, budget, (long long)nrows * B);
-    while (tl > q && r2c_pf_smem_bytes<T>(tl, Hx, nx) > kMaxSmem) tl /= 2;
-    const size_t sm = r2c_pf_smem_bytes<T>(tl, Hx, nx);
-    cudaError_t e;
-    if ((e = mark()) != cudaSuccess) return e;
-    e = launch_r2c_pf<T>(u, S1, nrows, nx, ld1, logPx - 1, tl, sm, tw[0], skip, b_in, B, s);
-    if (e != cudaSuccess) return e;
-  } else {
+  {
     const int G = Hx >> 4;
     const int tl = pick_tl_tuned(tuned[0], sline(Hx), eb, G, budget, (long long)nrows * B);
     const size_t sm = (size_t)tl * r2c_line_stride<T>(Hx, tl) * eb;
     cudaError_t e;
     const int grid = (nrows + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPx - 1, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
@@ -1115,9 +808,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
                                                                       logPx, skip, b_in);
           return cudaGetLastError();
         });
-    }
     if (!odd)
-      e = with_line_shape<T, std::is_same<T, float>::value>(logPx - 1, [&](auto tag) {
+      e = with_line_shape(logPx - 1, [&](auto tag) {
         constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
         cudaError_t e2 = set_smem(k_r2c_T<T, REM, LL>, sm);
         if (e2 != cudaSuccess) return e2;
@@ -1158,7 +850,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
     const int ncols = Hx + 1;
     const int grid = (ncols + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPy, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
@@ -1168,9 +859,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
                                                                        logPy, skip, b_ws);
           return cudaGetLastError();
         });
-    }
     if (!odd)
-      e = with_line_shape<T>(logPy, [&](auto tag) {
+      e = with_line_shape(logPy, [&](auto tag) {
         constexpr int REM = decltype(tag)::rem, LP = decltype(tag)::logp;
         cudaError_t e2 = set_smem(k_colmul<T, REM, LP>, sm);
         if (e2 != cudaSuccess) return e2;
@@ -1189,7 +879,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
       const int tiles = (nz + tl - 1) / tl;
       const int grid = (Hx + 1) * tiles;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPy, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
@@ -1200,9 +889,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
                                                                          skip, b_ws);
           return cudaGetLastError();
         });
-    }
     if (!odd)
-    e = with_line_shape<T, std::is_same<T, float>::value>(logPy, [&](auto tag) {
+    e = with_line_shape(logPy, [&](auto tag) {
       constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
       cudaError_t e2 = set_smem(k_c2cT_fwd<T, REM, LL>, sm);
       if (e2 != cudaSuccess) return e2;
@@ -1220,7 +908,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
       const int ncols = (Hx + 1) * Py;
       const int grid = (ncols + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPz, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
@@ -1230,9 +917,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
                                                                        tw[2], logPz, skip, b_ws);
           return cudaGetLastError();
         });
-    }
     if (!odd)
-    e = with_line_shape<T>(logPz, [&](auto tag) {
+    e = with_line_shape(logPz, [&](auto tag) {
       constexpr int REM = decltype(tag)::rem, LP = decltype(tag)::logp;
       cudaError_t e2 = set_smem(k_colmul<T, REM, LP>, sm);
       if (e2 != cudaSuccess) return e2;
@@ -1250,7 +936,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
       const int tiles = (nz + tl - 1) / tl;
       const int grid = (Hx + 1) * tiles;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPy, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
@@ -1261,9 +946,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
                                                                           skip, b_ws);
           return cudaGetLastError();
         });
-    }
     if (!odd)
-    e = with_line_shape<T, std::is_same<T, float>::value>(logPy, [&](auto tag) {
+    e = with_line_shape(logPy, [&](auto tag) {
       constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
       cudaError_t e2 = set_smem(k_c2cT_inv<T, REM, LL>, sm);
       if (e2 != cudaSuccess) return e2;
@@ -1281,7 +965,6 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
     cudaError_t e;
     const int grid = (nrows + tl - 1) / tl;
     if ((e = mark()) != cudaSuccess) return e;
-    if constexpr (std::is_same<T, float>::value) {
       if (odd)
         e = with_rem(logPx - 1, [&](auto tag) {
           constexpr int REM = decltype(tag)::value;
@@ -1291,9 +974,8 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
                                                                        logPx, skip, b_out);
           return cudaGetLastError();
         });
-    }
     if (!odd)
-      e = with_line_shape<T, std::is_same<T, float>::value>(logPx - 1, [&](auto tag) {
+      e = with_line_shape(logPx - 1, [&](auto tag) {
         constexpr int REM = decltype(tag)::rem, LL = decltype(tag)::logp;
         cudaError_t e2 = set_smem(k_c2r_T<T, REM, LL>, sm);
         if (e2 != cudaSuccess) return e2;
@@ -1308,20 +990,19 @@ static cudaError_t apply_launch_b(const Plan& p, int B, const io_t<T>* u, io_t<T
 
 template <typename T>
 cudaError_t apply_launch(const Plan& p, const io_t<T>* u, io_t<T>* y, void* work, cudaStream_t s, const int* skip,
-                         cudaEvent_t const* ev, const T* lam_override, bool odd) {
+                         cudaEvent_t const* ev, const io_t<T>* lam_override, bool odd) {
   return apply_launch_b<T>(p, 1, u, y, 0, work, s, skip, 0, ev, lam_override, 0, odd);
 }
 
 template <typename T>
 cudaError_t apply_batch_launch(const Plan& p, int B, const io_t<T>* u, io_t<T>* y, size_t vstride, void* work,
-                               cudaStream_t s, const int* skip, int skip_stride, const T* lam, size_t lam_stride,
+                               cudaStream_t s, const int* skip, int skip_stride, const io_t<T>* lam, size_t lam_stride,
                                cudaEvent_t const* ev) {
   return apply_launch_b<T>(p, B, u, y, vstride, work, s, skip, skip_stride, ev, lam, lam_stride);
 }
 
 // Lines per CTA candidates of apply stage `st`: powers of two from whole warps up to the
 // compiled thread bound (kMaxCta), 64 lines, and 227 KB of shared memory.
-template <typename T>
 static int stage_line_length(const Plan& p, int st) {
   const int Hx = p.P[0] / 2;
   if (p.d == 2) return st == 1 ? (p.P[1] > kMaxLine ? kMaxLine : p.P[1]) : Hx;
@@ -1333,7 +1014,7 @@ template <typename T>
 cudaError_t autotune_engine(Plan& p, int B, io_t<T>* u, io_t<T>* y, void* work, cudaStream_t s) {
   const int ns = p.d == 2 ? 3 : 5;
   const int eng = engine_index<T>();
-  const int eb = (int)sizeof(cplx<T>);
+  const int eb = 2 * (int)sizeof(io_t<T>);
   cudaEvent_t ev[6];
   for (int i = 0; i <= ns; ++i) {
     cudaError_t e = cudaEventCreate(&ev[i]);
@@ -1344,14 +1025,12 @@ cudaError_t autotune_engine(Plan& p, int B, io_t<T>* u, io_t<T>* y, void* work, 
   }
   cudaError_t e = cudaMemsetAsync(u, 0, (size_t)B * p.M * sizeof(io_t<T>), s);
   for (int st = 0; st < ns && e == cudaSuccess; ++st) {
-    const int L = stage_line_length<T>(p, st);
+    const int L = stage_line_length(p, st);
     const int G = L >> 4;
     int best = 0;
     float best_ms = 0.f;
     for (int t = 1; t <= 64 && e == cudaSuccess; t *= 2) {
-      const size_t smem = (st == 0 && use_r2c_pf<T>(p.logP[0] - 1, u)) ? r2c_pf_smem_bytes<T>(t, L, p.n[0])
-                          : st == 0                                     ? (size_t)t * r2c_line_stride<T>(L, t) * eb
-                                                                         : (size_t)t * sline(L) * eb;
+      const size_t smem = (size_t)t * (st == 0 ? r2c_line_stride<T>(L, t) : sline(L)) * eb;
       if (t * G > kMaxCta<T> || smem > kMaxSmem) break;
       if (G < 32 && t < 32 / G) continue;
       p.tl_tuned[eng][st] = t;
@@ -1374,18 +1053,8 @@ cudaError_t autotune_engine(Plan& p, int B, io_t<T>* u, io_t<T>* y, void* work, 
   return e;
 }
 
-// The give-up count and the bounds-check state of the including translation unit (every unit that
-// includes this header has its own), read and reset.
-[[maybe_unused]] static cudaError_t unit_wait_collect(unsigned long long* count) {
-  unsigned long long c = 0ull;
-  cudaError_t e = cudaMemcpyFromSymbol(&c, g_wait_timeouts, sizeof(c));
-  if (e != cudaSuccess) return e;
-  const unsigned long long z = 0ull;
-  e = cudaMemcpyToSymbol(g_wait_timeouts, &z, sizeof(z));
-  *count = c;
-  return e;
-}
-
+// The bounds-check state of the including translation unit (every unit that includes this header has its own),
+// read and reset.
 [[maybe_unused]] static cudaError_t unit_bc_collect(unsigned long long* count, unsigned long long* first) {
 #ifdef FRLAP_BOUNDS_CHECK
   BcState st;
@@ -1403,10 +1072,6 @@ cudaError_t autotune_engine(Plan& p, int B, io_t<T>* u, io_t<T>* y, void* work, 
 #endif
 }
 
-template <typename T>
-cudaError_t wait_collect(unsigned long long* count) {
-  return unit_wait_collect(count);
-}
 template <typename T>
 cudaError_t bc_collect(unsigned long long* count, unsigned long long* first) {
   return unit_bc_collect(count, first);

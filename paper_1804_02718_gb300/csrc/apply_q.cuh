@@ -1,5 +1,6 @@
-// The apply's stages in the FP64 engine: the pipeline of apply_impl.cuh on 64-bit block fixed point
-// (fft_q.cuh).  Vectors and symbol are FP64.  In the workspace a complex value is two 64-bit integers
+// The apply's stages in the FP64 and the DF64 engine: the pipeline of apply_impl.cuh on 64-bit block fixed point
+// (fft_q.cuh).  Vectors and symbol are FP64.  The DF64 engine's first stage sets a row's scale once (DYN =
+// false); the other stages are common.  In the workspace a complex value is two 64-bit integers
 // below 2^58, in the same S1 / S2 layout and 16 bytes as an FP64 pair, and each line that a kernel wrote
 // has its exponent in an array behind S1 and S2:
 //   ex_row[row]           after the first stage, for S1[.][row]
@@ -36,9 +37,14 @@ inline QExpLayout q_exp_layout(const Plan& p) {
   return l;
 }
 
-// A transform's output is stored below 2^57.5.
-template <int REM>
-constexpr int kQStore = 5 - kQDrop<REM>;
+// A transform's output v[0..N) to what is stored, components below 2^58, and its exponent.
+template <int REM, int N>
+__device__ __forceinline__ void q_store_scale(cq* v, int& e) {
+  constexpr int SH = 5 - kQDrop<REM>;
+#pragma unroll
+  for (int m = 0; m < N; ++m) v[m] = q_shr_even<SH>(v[m]);
+  e += SH;
+}
 
 __device__ __forceinline__ unsigned q_ord(int e) { return (unsigned)e ^ 0x80000000u; }
 __device__ __forceinline__ int q_unord(unsigned u) { return (int)(u ^ 0x80000000u); }
@@ -61,7 +67,7 @@ __device__ __forceinline__ cq q_align(cq v, int e, int top, bool up) {
   }                                                                      \
   cq* smem = reinterpret_cast<cq*>(smem_raw);
 
-template <int REM, int LOGL = 0>
+template <bool DYN, int REM, int LOGL = 0>
 __global__ void __launch_bounds__(512, 1)
     k_q_r2c(const double* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int nlines, int n, size_t ldo,
             int logH, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
@@ -111,7 +117,8 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
   for (int m = 0; m < 8; ++m) v[m] = {q_in(xr[m], qs), q_in(xi[m], qs)};
   int e = qs.e;
-  q_fft<-1, true, REM>(v, e, buf, logH, lane, tw, logH + 1, false, slots, si);
+  q_fft<DYN, -1, true, REM>(v, e, buf, logH, lane, tw, logH + 1, false, slots, si);
+  if constexpr (!DYN) q_fill<16>(v, e, logH, slots + si);
   line_sync<double>(logH);
 #pragma unroll
   for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = v[m];
@@ -121,9 +128,10 @@ __global__ void __launch_bounds__(512, 1)
   line_sync<double>(logH);
   // Real-data split in place, one product per pair (see r2c_tile): X[k] = s + W^k d,
   // X[H-k] = conj(s - W^k d), s = (a + b) / 2, d = -i (a - b) / 2; stored below 2^57.5, that is over 2^(6 - D),
-  // D = kQDrop.  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of the downward
-  // shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in a + b.
-  constexpr int D = kQDrop<REM>;
+  // D = kQDrop (0 after q_fill).  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of
+  // the downward shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in
+  // a + b.
+  constexpr int D = DYN ? kQDrop<REM> : 0;
   auto split = [&](int k, const int4 wk) {
     const int km = H - k;
     const cq a = buf[spad(k)];
@@ -263,16 +271,15 @@ __global__ void __launch_bounds__(512, 1)
   const int* exi = ex_in + (map.d == 2 ? 0 : (size_t)kx * nz);
   int e = q_load_aligned<8>(v, data + (size_t)c * ld, exi, kx & 1, lane, G, n, valid, logP, slots + si);
   ++si;
-  q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_fft<true, -1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
   const int ky = c & (map.Py - 1);
   const double* lrow = map.d == 2 ? lam + (size_t)c * map.Hy1
                                   : lam + ((size_t)kx * map.Hy1 + min(ky, map.Py - ky)) * map.Hz1;
   q_symbol(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, logP, slots + si);
   ++si;
-  q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  if (valid && lane == 0) FRLAP_GST(ex_out + col, e + kQStore<REM>);
-#pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = q_shr_even<kQStore<REM>>(v[m]);
+  q_fft<true, 1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  q_store_scale<REM, 8>(v, e);
+  if (valid && lane == 0) FRLAP_GST(ex_out + col, e);
   store_line(v, data, ncols, n, ld, logP, TL);
 }
 
@@ -312,7 +319,7 @@ __global__ void __launch_bounds__(512, 1)
     for (int m = 0; m < 16; ++m)
       v[m] = q_cmul<false>(cq{q_shl(v[m].x, 4), q_shl(v[m].y, 4)}, FRLAP_GLD(tw + lane + m * G));
   }
-  q_fft<-1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, false, slots, si);
+  q_fft<true, -1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, false, slots, si);
   // the half's symbol entries are every second one
   const double* lrow = lam + (size_t)(valid ? col : 0) * Hy1;
   q_symbol(
@@ -323,14 +330,15 @@ __global__ void __launch_bounds__(512, 1)
       },
       logL, slots + si);
   ++si;
-  q_fft<1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, true, slots, si);
+  q_fft<true, 1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, true, slots, si);
   if (!valid) return;
   if constexpr (!ODD) {
-    if (lane == 0) FRLAP_GST(ex_tmp + col, e + kQStore<REM>);
+    constexpr int SH = 5 - kQDrop<REM>;
+    if (lane == 0) FRLAP_GST(ex_tmp + col, e + SH);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int j = lane + m * G;
-      if (j < n) FRLAP_GST(tline + j, q_shr_even<kQStore<REM>>(v[m]));
+      if (j < n) FRLAP_GST(tline + j, q_shr_even<SH>(v[m]));
     }
   } else {
     // y_j = even_j + W_P^-j odd_j, magnitudes below 2^58 each at exponents et and eo: the odd half, below
@@ -381,11 +389,12 @@ __global__ void __launch_bounds__(512, 1)
   int e = q_load_aligned<8>(v, in + g * gin + (size_t)c * ldi, ex_in + (size_t)c * n, g & 1, lane, G, n, valid,
                             logP, slots + si);
   ++si;
-  q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + kQStore<REM>);
+  q_fft<true, -1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_store_scale<REM, 16>(v, e);
+  if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
   line_sync<double>(logP);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = q_shr_even<kQStore<REM>>(v[m]);
+  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = v[m];
   __syncthreads();
   const int logTL = __ffs(TL) - 1;
   const int lt = threadIdx.x & (TL - 1);
@@ -437,14 +446,15 @@ __global__ void __launch_bounds__(512, 1)
   cq v[16];
 #pragma unroll
   for (int m = 0; m < 16; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
-  q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  q_fft<true, 1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  q_store_scale<REM, 8>(v, e);
   if (line < nlines) {
-    if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e + kQStore<REM>);
+    if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
     cq* dst = out + g * gout + (size_t)line * ldo;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int i = lane + m * G;
-      if (i < n) FRLAP_GST(dst + i, q_shr_even<kQStore<REM>>(v[m]));
+      if (i < n) FRLAP_GST(dst + i, v[m]);
     }
   }
 }
@@ -511,7 +521,7 @@ __global__ void __launch_bounds__(512, 1)
   cq v[16];
 #pragma unroll
   for (int m = 0; m < 16; ++m) v[m] = buf[spad(lane + m * G)];
-  q_fft<1, false, REM>(v, e, buf, logH, lane, tw, logH + 1, true, slots, si);
+  q_fft<true, 1, false, REM>(v, e, buf, logH, lane, tw, logH + 1, true, slots, si);
   if (!valid) return;
   double* dst = out + (size_t)line * n;
   const bool pair_aligned = (reinterpret_cast<uintptr_t>(dst) % sizeof(double2)) == 0;
@@ -528,91 +538,6 @@ __global__ void __launch_bounds__(512, 1)
       }
     }
   }
-}
-
-// Spectrum columns of the learned preconditioner: columns of n entries -> zero-pad to P, forward FFT, all P
-// outputs in FP64 (stride ldo).
-template <int REM>
-__global__ void __launch_bounds__(512, 1)
-    k_q_col_fwd(const cq* __restrict__ in, const int* __restrict__ ex, double2* __restrict__ out, int ncols, int n,
-                size_t ld, size_t ldo, int logP, int TL, int cols_per, const int4* __restrict__ tw,
-                const int* __restrict__ skip, Batch bt, size_t ex_inst) {
-  in += blockIdx.y * bt.in;
-  out += blockIdx.y * bt.out;
-  ex += blockIdx.y * ex_inst;
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4;
-  const int l = threadIdx.x / G, lane = threadIdx.x % G;
-  const int col = blockIdx.x * TL + l;
-  const bool valid = col < ncols;
-  const int c = valid ? col : 0;
-  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
-  cq* buf = smem + (size_t)l * sline(P);
-  int si = 0;
-  cq v[16];
-  // exponents: 2D ex[i] for every column; 3D ex[(col / P_y) n + i]
-  const int kx = cols_per ? c / cols_per : c;
-  int e = q_load_aligned<8>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)kx * n : 0), kx & 1, lane, G, n, valid,
-                            logP, slots + si);
-  ++si;
-  q_fft<-1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  if (!valid) return;
-  double2* dst = out + (size_t)col * ldo;
-#pragma unroll
-  for (int m = 0; m < 16; ++m)
-    FRLAP_GST(dst + lane + m * G, make_double2(q_out_any(v[m].x, e), q_out_any(v[m].y, e)));
-}
-
-// Columns of P FP64 spectrum values times a multiplier (natural octant order) -> inverse FFT, crop to n.
-template <int REM>
-__global__ void __launch_bounds__(512, 1)
-    k_q_col_mulinv(const double2* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int ncols, int n,
-                   size_t ld, size_t ldo, int logP, int TL, const double* __restrict__ lam, LamMap map,
-                   const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
-  in += blockIdx.y * bt.in;
-  out += blockIdx.y * bt.out;
-  ex += blockIdx.y * ex_inst;
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4;
-  const int l = threadIdx.x / G, lane = threadIdx.x % G;
-  const int col = blockIdx.x * TL + l;
-  const bool valid = col < ncols;
-  const int c = valid ? col : 0;
-  unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
-  cq* buf = smem + (size_t)l * sline(P);
-  const double2* src = in + (size_t)c * ld;
-  size_t lam_base;
-  int lam_stride;
-  if (map.d == 2) {
-    lam_base = c;
-    lam_stride = map.Hx1;
-  } else {
-    const int kx = c >> map.logPy, ky = c & (map.Py - 1);
-    lam_base = (size_t)min(ky, map.Py - ky) * map.Hx1 + kx;
-    lam_stride = map.Hy1 * map.Hx1;
-  }
-  double2 x[16];
-  unsigned hm = 0u;
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int k = lane + m * G;
-    x[m] = valid ? FRLAP_GLD(lam + lam_base + (size_t)min(k, P - k) * lam_stride) * FRLAP_GLD(src + k)
-                 : make_double2(0.0, 0.0);
-  }
-#pragma unroll
-  for (int m = 0; m < 16; ++m) hm = max(hm, max(q_mag(x[m].x), q_mag(x[m].y)));
-  int si = 0;
-  const QIn qs = q_in_scale(q_reduce<true>(hm, logP, slots + si));
-  ++si;
-  cq v[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
-  int e = qs.e;
-  q_fft<1, false, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  if (valid && lane == 0) FRLAP_GST(ex + col, e + kQStore<REM>);
-#pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = q_shr_even<kQStore<REM>>(v[m]);
-  store_line(v, out, ncols, n, ldo, logP, TL);
 }
 
 }  // namespace
@@ -687,6 +612,7 @@ static cudaError_t q_register(const Plan& p, BcRanges r, void* work, int B, cuda
 #endif
 
 // The stages, one launch each over B instances (per-instance strides in elements).
+template <bool DYN>
 static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const double* u, size_t ustride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
   const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
@@ -695,9 +621,10 @@ static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const doubl
   b.in = ustride;
   b.out = w.stride;
   b.skip = skip_stride;
-  return with_line_shape<double, true>(p.logP[0] - 1, [&](auto tag) {
-    return q_launch(k_q_r2c<decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row, nrows, p.n[0],
-                    (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
+  return with_line_shape(p.logP[0] - 1, [&](auto tag) {
+    return q_launch(k_q_r2c<DYN, decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, u, w.S1,
+                    w.row, nrows, p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b,
+                    w.ex_stride);
   });
 }
 static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
@@ -707,7 +634,7 @@ static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tune
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
-  return with_line_shape<double, true>(p.logP[1], [&](auto tag) {
+  return with_line_shape(p.logP[1], [&](auto tag) {
     return q_launch(k_q_c2cT_fwd<decltype(tag)::rem, decltype(tag)::logp>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, w.S2,
                     (const int*)w.row, w.line, nz, q.tiles, ny, (size_t)nz * ny, ny, (size_t)Py * nz, nz, p.logP[1],
                     q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
@@ -720,7 +647,7 @@ static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tune
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
-  return with_line_shape<double, true>(p.logP[1], [&](auto tag) {
+  return with_line_shape(p.logP[1], [&](auto tag) {
     return q_launch(k_q_c2cT_inv<decltype(tag)::rem, decltype(tag)::logp>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S2, w.S1,
                     (const int*)w.col, w.line, nz, q.tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, p.logP[1],
                     q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
@@ -734,7 +661,7 @@ static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, 
   b.in = w.stride;
   b.out = ystride;
   b.skip = skip_stride;
-  return with_line_shape<double, true>(p.logP[0] - 1, [&](auto tag) {
+  return with_line_shape(p.logP[0] - 1, [&](auto tag) {
     return q_launch(k_q_c2r<decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, y,
                     (const int*)(p.d == 3 ? w.line : w.col), p.d == 3 ? p.n[2] : 1, p.d == 3 ? p.n[1] : nrows, nrows,
                     p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
@@ -742,10 +669,10 @@ static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, 
 }
 
 template <typename T>
-cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstride, void* work, cudaStream_t s,
-                             const int* skip, int skip_stride, cudaEvent_t const* ev, const T* lam_override,
-                             size_t lam_stride) {
-  static_assert(std::is_same<T, double>::value, "the FP64 engine");
+cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, size_t vstride, void* work,
+                             cudaStream_t s, const int* skip, int skip_stride, cudaEvent_t const* ev,
+                             const double* lam_override, size_t lam_stride) {
+  constexpr bool DYN = std::is_same<T, double>::value;
   int stage = 0;
   auto mark = [&]() -> cudaError_t {
     if (ev && ev[stage]) {
@@ -777,7 +704,7 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstr
   b.lam = lam_stride;
   b.skip = skip_stride;
   if ((e = mark()) != cudaSuccess) return e;
-  if ((e = q_stage_r2c(p, w, B, u, vstride, tuned[0], skip, skip_stride, s)) != cudaSuccess) return e;
+  if ((e = q_stage_r2c<DYN>(p, w, B, u, vstride, tuned[0], skip, skip_stride, s)) != cudaSuccess) return e;
   if ((e = mark()) != cudaSuccess) return e;
   if (p.d == 2 && p.P[1] > kMaxLine) {
     const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1 * B, Hx1);
@@ -797,7 +724,7 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstr
     const int ax = p.d == 3 ? 2 : 1;
     const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
     const QShape q = q_shape(tuned[p.d == 3 ? 2 : 1], p.P[ax], (long long)ncols * B, ncols);
-    e = with_line_shape<T, true>(p.logP[ax], [&](auto tag) {
+    e = with_line_shape(p.logP[ax], [&](auto tag) {
       constexpr int REM = decltype(tag)::rem, LP = decltype(tag)::logp;
       return q_launch(k_q_colmul<REM, LP>, q.tiles, B, q.threads, q.sm, s, p.d == 3 ? w.S2 : w.S1,
                       (const int*)(p.d == 3 ? w.line : w.row), w.col, ncols, p.n[ax], (size_t)(p.d == 3 ? nz : nrows),
@@ -812,66 +739,6 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const T* u, T* y, size_t vstr
   if ((e = mark()) != cudaSuccess) return e;
   if ((e = q_stage_c2r(p, w, B, y, vstride, tuned[p.d == 2 ? 2 : 4], skip, skip_stride, s)) != cudaSuccess) return e;
   return mark();
-}
-
-// SP = F R^T u on the half spectrum in FP64: 2D [kx][ky], 3D [kx][ky][kz] (kx <= P_x/2, full ky, kz).
-cudaError_t spectrum_forward(const Plan& p, int nb, const double* u, double2* SP, size_t sstride, void* work,
-                             cudaStream_t s) {
-  cudaError_t e;
-#ifdef FRLAP_BOUNDS_CHECK
-  {
-    BcRanges r;
-    r.add(u, nb * p.M * sizeof(double));
-    r.add(SP, nb * sstride * sizeof(double2));
-    if ((e = q_register(p, r, work, nb, s)) != cudaSuccess) return e;
-  }
-#endif
-  const QWork w = q_work(p, work);
-  if ((e = q_stage_r2c(p, w, nb, u, p.M, 0, nullptr, 0, s)) != cudaSuccess) return e;
-  if (p.d == 3 && (e = q_stage_yz_fwd(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
-  const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
-  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
-  Batch b;
-  b.in = w.stride;
-  b.out = sstride;
-  return with_rem(p.logP[ax], [&](auto tag) {
-    return q_launch(k_q_col_fwd<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s,
-                    (const cq*)(p.d == 3 ? w.S2 : w.S1), (const int*)(p.d == 3 ? w.line : w.row), SP, ncols, p.n[ax],
-                    (size_t)(p.d == 3 ? p.n[2] : nrows), (size_t)p.P[ax], p.logP[ax], q.tl, p.d == 3 ? p.P[1] : 0,
-                    (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
-  });
-}
-
-// y = R F^-1 (mult * SP), mult = a symbol octant with the 1/prod(P) factor folded in.
-cudaError_t spectrum_inverse(const Plan& p, int nb, const double2* SP, size_t sstride, const double* mult, double* y,
-                             void* work, cudaStream_t s) {
-  cudaError_t e;
-#ifdef FRLAP_BOUNDS_CHECK
-  {
-    BcRanges r;
-    r.add(SP, nb * sstride * sizeof(double2));
-    r.add(mult, p.lam_count * sizeof(double));
-    r.add(y, nb * p.M * sizeof(double));
-    if ((e = q_register(p, r, work, nb, s)) != cudaSuccess) return e;
-  }
-#endif
-  const QWork w = q_work(p, work);
-  const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
-  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
-  const LamMap map = q_lam_map(p);
-  Batch b;
-  b.in = sstride;
-  b.out = w.stride;
-  e = with_rem(p.logP[ax], [&](auto tag) {
-    return q_launch(k_q_col_mulinv<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
-                    w.col, ncols, p.n[ax], (size_t)p.P[ax], (size_t)(p.d == 3 ? p.n[2] : nrows), p.logP[ax], q.tl, mult,
-                    map, (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
-  });
-  if (e != cudaSuccess) return e;
-  if (p.d == 3 && (e = q_stage_yz_inv(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
-  return q_stage_c2r(p, w, nb, y, p.M, 0, nullptr, 0, s);
 }
 
 }  // namespace frlap

@@ -564,26 +564,6 @@ cudaError_t symbol_axes_launch(const Plan& p, double* lam, cudaStream_t s) {
 
 namespace frlap {
 namespace {
-__global__ void k_to_df(const double* __restrict__ src, dfl* dst, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = df_from(src[i]);
-}
-}  // namespace
-
-namespace {
-__global__ void k_to_cdf(const double2* __restrict__ src, cdf* dst, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = make_cdf(df_from(src[i].x), df_from(src[i].y));
-}
-}  // namespace
-
-// double-float copy of a complex table (twiddles), n values, in the paired layout of cdf
-cudaError_t to_cdf_launch(const double2* src, cdf* dst, size_t n, cudaStream_t st) {
-  k_to_cdf<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, dst, n);
-  return cudaGetLastError();
-}
-
-namespace {
 // x in [-1, 1] with 60 fraction bits as h 2^32 + l, both signed; a low half of -2^31 takes one unit more,
 // so that a half can be negated
 __device__ __forceinline__ int2 q60(double x) {
@@ -606,12 +586,6 @@ cudaError_t to_q_launch(const double2* src, int4* dst, size_t n, cudaStream_t st
   return cudaGetLastError();
 }
 
-// double-float copies of a symbol (n values)
-cudaError_t to_df_launch(const double* src, dfl* dst, size_t n, cudaStream_t st) {
-  k_to_df<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, dst, n);
-  return cudaGetLastError();
-}
-
 cudaError_t scale_symbol_launch(double* lam64, float* lam32, size_t n, double s, cudaStream_t st) {
   k_scale_copy<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(lam64, lam32, n, s);
   return cudaGetLastError();
@@ -620,8 +594,7 @@ cudaError_t scale_symbol_launch(double* lam64, float* lam32, size_t n, double s,
 namespace {
 template <typename To>
 __device__ __forceinline__ To from_double(double v) {
-  if constexpr (std::is_same<To, dfl>::value) return df_from(v);
-  else return (To)v;
+  return (To)v;
 }
 
 // natural octant [A][Bm][Cx] (Cx fastest) -> line-major [Cx][Bm][A] (A fastest), times s
@@ -647,5 +620,4 @@ cudaError_t line_symbol_launch(const Plan& p, const double* oct, To* dst, double
 }
 template cudaError_t line_symbol_launch<double>(const Plan&, const double*, double*, double, cudaStream_t);
 template cudaError_t line_symbol_launch<float>(const Plan&, const double*, float*, double, cudaStream_t);
-template cudaError_t line_symbol_launch<dfl>(const Plan&, const double*, dfl*, double, cudaStream_t);
 }  // namespace frlap

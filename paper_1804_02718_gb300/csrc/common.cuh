@@ -9,7 +9,6 @@
 #include <string>
 
 #include "../../include/frlap.h"
-#include "dfloat.cuh"
 
 namespace frlap {
 
@@ -42,7 +41,6 @@ inline unsigned capped_passes(unsigned derived) {
 template <typename T> struct cplx_t;
 template <> struct cplx_t<float> { using type = float2; };
 template <> struct cplx_t<double> { using type = double2; };
-template <> struct cplx_t<dfl> { using type = cdf; };
 template <typename T> using cplx = typename cplx_t<T>::type;
 
 #ifdef FRLAP_BOUNDS_CHECK
@@ -84,7 +82,7 @@ __device__ __forceinline__ void bc_st(V* p, const V& v) {
 #endif
 
 // Load of data a kernel reads once (cache-streaming: evict-first in L1 and L2), so that the
-// twiddle tables keep the L1.  8- and 16-byte values: float2 / float4 / double2 / cdf; 4 and 8
+// twiddle tables keep the L1.  8- and 16-byte values: float2 / float4 / double2 / a pair of 64-bit integers; 4 and 8
 // byte scalars.
 template <typename V>
 __device__ __forceinline__ V ld_stream(const V* p) {
@@ -127,31 +125,25 @@ __device__ __forceinline__ V ld_stream(const V* p) {
 #endif
 
 
-// storage type of the real grid vectors and of the symbol for each compute type:
-// FP32 and FP64 compute and store in their own type; double-float computes in
-// dfl, reads and writes FP64 vectors, and keeps its symbol/twiddles as dfl.
+// Engines of the apply: float (FP32), double (FP64 vectors and symbol, transforms in 64-bit fixed point whose
+// scale follows the data between stages) and this tag for the DF64 plans' one (the same with the scale set
+// once per transform).  io_t: the type of the engine's grid vectors and symbol.
+struct df64 {};
 template <typename T> struct io_t_ { using type = T; };
-template <> struct io_t_<dfl> { using type = double; };
+template <> struct io_t_<df64> { using type = double; };
 template <typename T> using io_t = typename io_t_<T>::type;
 
 // two consecutive grid values as one aligned vector (float2 / double2)
 template <typename T> using io_pair = typename std::conditional<sizeof(io_t<T>) == 4, float2, double2>::type;
 
-template <typename T> __device__ __forceinline__ T from_io(io_t<T> v) { return v; }
-template <> __device__ __forceinline__ dfl from_io<dfl>(double v) { return df_from(v); }
-template <typename T> __device__ __forceinline__ io_t<T> to_io(T v) { return v; }
-template <> __device__ __forceinline__ double to_io<dfl>(dfl v) { return df_to(v); }
-
 // the real type of a complex type
 template <typename C> struct real_of;
 template <> struct real_of<float2> { using type = float; };
 template <> struct real_of<double2> { using type = double; };
-template <> struct real_of<cdf> { using type = dfl; };
 template <typename C> using real_t = typename real_of<C>::type;
 
 __host__ __device__ __forceinline__ float2 make_cplx(float a, float b) { return make_float2(a, b); }
 __host__ __device__ __forceinline__ double2 make_cplx(double a, double b) { return make_double2(a, b); }
-__host__ __device__ __forceinline__ cdf make_cplx(dfl a, dfl b) { return make_cdf(a, b); }
 template <typename C> __host__ __device__ __forceinline__ C mk(real_t<C> a, real_t<C> b) { return make_cplx(a, b); }
 template <typename C> __host__ __device__ __forceinline__ C czero() {
   using T = real_t<C>;
@@ -162,8 +154,6 @@ __device__ __forceinline__ float re(float2 a) { return a.x; }
 __device__ __forceinline__ float im(float2 a) { return a.y; }
 __device__ __forceinline__ double re(double2 a) { return a.x; }
 __device__ __forceinline__ double im(double2 a) { return a.y; }
-__device__ __forceinline__ dfl re(cdf a) { return cdf_re(a); }
-__device__ __forceinline__ dfl im(cdf a) { return cdf_im(a); }
 // FP32 complex sums as single paired instructions (each component rounded as the scalar add;
 // a - b as b * (-1) + a, whose product is exact)
 __device__ __forceinline__ float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -171,21 +161,9 @@ __device__ __forceinline__ float2 operator-(float2 a, float2 b) { return __ffma2
 __device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 operator-(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 operator*(float s, float2 a) { return __fmul2_rn(make_float2(s, s), a); }
-// Sums that only feed another sum: plain for FP32 / FP64; without the closing renormalisation
-// for double-float (dfloat.cuh).
-__device__ __forceinline__ float2 add_lazy(float2 a, float2 b) { return a + b; }
-__device__ __forceinline__ float2 sub_lazy(float2 a, float2 b) { return a - b; }
-__device__ __forceinline__ double2 add_lazy(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 sub_lazy(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 // a / 2, exactly (a power-of-two scaling of each component)
 __device__ __forceinline__ float2 halve(float2 a) { return __fmul2_rn(a, make_float2(0.5f, 0.5f)); }
 __device__ __forceinline__ double2 halve(double2 a) { return make_double2(0.5 * a.x, 0.5 * a.y); }
-__device__ __forceinline__ cdf halve(cdf a) {
-  cdf r;
-  r.hi = p_mul(a.hi, p_bcast(0.5f));
-  r.lo = p_mul(a.lo, p_bcast(0.5f));
-  return r;
-}
 __device__ __forceinline__ double2 operator*(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
 
 // complex product a*b
@@ -202,33 +180,13 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -a.x * b.y));
 }
-// products that only feed a sum: as cmul / cmulc here, unrenormalised for double-float
-__device__ __forceinline__ float2 cmul_lazy(float2 a, float2 b) { return cmul(a, b); }
-__device__ __forceinline__ double2 cmul_lazy(double2 a, double2 b) { return cmul(a, b); }
-__device__ __forceinline__ float2 cmulc_lazy(float2 a, float2 b) { return cmulc(a, b); }
-__device__ __forceinline__ double2 cmulc_lazy(double2 a, double2 b) { return cmulc(a, b); }
 template <typename C> __device__ __forceinline__ C conjg(C a) { a.y = -a.y; return a; }
-template <> __device__ __forceinline__ cdf conjg<cdf>(cdf a) { return cdf_conj(a); }
 // multiply by -i (forward) or +i (inverse): sign = -1 gives -i*a
 template <int SIGN, typename C> __device__ __forceinline__ C mul_i(C a) {
   C r;
   if (SIGN < 0) { r.x = a.y; r.y = -a.x; } else { r.x = -a.y; r.y = a.x; }
   return r;
 }
-template <int SIGN> __device__ __forceinline__ cdf mul_i_cdf(cdf a) {
-  cdf r;
-  if (SIGN < 0) {
-    r.hi = make_float2(a.hi.y, -a.hi.x);
-    r.lo = make_float2(a.lo.y, -a.lo.x);
-  } else {
-    r.hi = make_float2(-a.hi.y, a.hi.x);
-    r.lo = make_float2(-a.lo.y, a.lo.x);
-  }
-  return r;
-}
-template <> __device__ __forceinline__ cdf mul_i<-1, cdf>(cdf a) { return mul_i_cdf<-1>(a); }
-template <> __device__ __forceinline__ cdf mul_i<1, cdf>(cdf a) { return mul_i_cdf<1>(a); }
-
 // ---------------------------------------------------------------- plan
 // Longest FFT line the transform kernels hold (one line of 2^13 points per 2^9 threads); longer
 // 2D embeddings (16384 points) split their middle stage into two halves of this length.
@@ -248,7 +206,7 @@ struct Plan {
   void* tables = nullptr;      // one allocation: the symbols and twiddles below
   // The symbol octant lambda(kx, ky[, kz]), k_r = 0..P_r/2, with 1/prod(P) folded in.
   // lam64 is in natural order ([ky][kx] / [kz][ky][kx], kx fastest).  The tables the
-  // apply's middle stage reads (lamL64, lam32, lamdf and the preconditioner multipliers)
+  // apply's middle stage reads (lamL64, lam32 and the preconditioner multipliers)
   // are line-major: axes reversed ([kx][ky] / [kx][ky][kz]), so that the folded line of
   // one column is contiguous.
   double* lam64 = nullptr;     // natural order, FP64 (always built)
@@ -258,12 +216,10 @@ struct Plan {
   // twiddle_entries(P_r): see there
   double2* tw64[3] = {nullptr, nullptr, nullptr};
   float2* tw32[3] = {nullptr, nullptr, nullptr};
-  cdf* twdf[3] = {nullptr, nullptr, nullptr};      // the same twiddles as double-floats
   // the same in fixed point (60 fraction bits, signed 32-bit halves: re high, re low, im high, im low), for
-  // the FP64 engine (all plans but F32)
+  // the fixed-point engines (all plans but F32)
   int4* twq[3] = {nullptr, nullptr, nullptr};
-  dfl* lamdf = nullptr;        // line-major, as double-floats (DF64 plans)
-  bool df64 = false;           // FP64-precision vectors are applied with double-float FFTs
+  bool df64 = false;           // DF64 / MIXED_DF64: FP64 vectors are applied by the df64 engine
   // workspace layout of one apply, in complex elements of the apply precision
   size_t s1_elems = 0, s2_elems = 0;
   cudaStream_t side = nullptr;  // internal stream for captured solver graphs
@@ -271,15 +227,12 @@ struct Plan {
   float* mu_strang = nullptr;   // inverse of the multilevel Strang circulant, embedded like A
   float* mu_learned = nullptr;  // learned Fourier multiplier
   float* mu_tau = nullptr;      // inverse of diag(S A S) in the sine basis S (applied on odd extensions)
-  // lines per CTA of each apply stage, per engine (0 FP32, 1 FP64, 2 double-float), set by
+  // lines per CTA of each apply stage, per engine (0 FP32, 1 F64, 2 DF64), set by
   // frlap_plan_autotune; 0 = the built-in choice
   int tl_tuned[3][5] = {};
 };
 
-// Bounded waits of the apply kernels on their asynchronous copies (mbarrier phases) that gave up
-// since the last call, per engine's translation unit (the counter is reset).  A kernel whose wait
-// gives up records it and returns without storing that tile's results.
-template <typename T>
+// The bounded mbarrier waits of wait_selftest's kernel that gave up since the last call (the counter is reset).
 cudaError_t wait_collect(unsigned long long* count);
 
 // Bounds-checked builds: accesses outside the registered ranges since the last call, summed per
@@ -295,13 +248,13 @@ cudaError_t wait_selftest(unsigned long long* timeouts);
 cudaError_t dft16_stages_launch(int engine, const float* in, float* out, int ntiles, int reps, cudaStream_t s);
 cudaError_t dft16_wait_collect(unsigned long long* count);
 
-// apply pipeline (apply.cu); work must hold apply_work_bytes(plan, sizeof(T)) bytes
-// T = compute type (float, double or dfl); vectors are io_t<T>, symbol overrides are T
+// apply pipeline (apply_impl.cuh, apply_q.cuh); work must hold apply_work_bytes(plan, sizeof(io_t<T>)) bytes
+// T = engine; vectors and symbol overrides are io_t<T>
 template <typename T>
 // odd: a multiplier lam_override in the sine basis (FP32, P_r = 2(n_r + 1); see k_r2c_T)
 cudaError_t apply_launch(const Plan& p, const io_t<T>* u, io_t<T>* y, void* work, cudaStream_t s, const int* skip,
-                         cudaEvent_t const* ev = nullptr, const T* lam_override = nullptr, bool odd = false);
-// FP64 vectors through the plan's FP64 engine (native double or double-float)
+                         cudaEvent_t const* ev = nullptr, const io_t<T>* lam_override = nullptr, bool odd = false);
+// FP64 vectors through the plan's own engine (double or df64)
 cudaError_t apply64(const Plan& p, const double* u, double* y, void* work, cudaStream_t s, const int* skip,
                     cudaEvent_t const* ev = nullptr);
 size_t apply_work_bytes(const Plan& p, int real_bytes);
@@ -312,7 +265,7 @@ cudaError_t autotune_engine(Plan& p, int B, io_t<T>* u, io_t<T>* y, void* work, 
 // B same-shape instances in one launch per stage (see apply.cu)
 template <typename T>
 cudaError_t apply_batch_launch(const Plan& p, int B, const io_t<T>* u, io_t<T>* y, size_t vstride, void* work,
-                               cudaStream_t s, const int* skip, int skip_stride, const T* lam, size_t lam_stride,
+                               cudaStream_t s, const int* skip, int skip_stride, const io_t<T>* lam, size_t lam_stride,
                                cudaEvent_t const* ev = nullptr);
 // Forward half spectra F R^T u (2D [kx][ky], 3D [kx][ky][kz]) of nb vectors back to back, sstride complex entries
 // apart, and their inverse after a multiplier, in the FP64 engine; work: nb apply workspaces.
@@ -332,7 +285,7 @@ cudaError_t symbol_launch(const Plan& p, const double* coef, double* lam_oct, cu
 cudaError_t shifted_tau_launch(const Plan& p, double sigma, double s, float* mu_b, cudaStream_t st);
 // the generator t_k = -c a_k (k_r <= n_r - 1, zero elsewhere) on the octant, natural order
 cudaError_t generator_octant_launch(const Plan& p, const double* coef, double* lam_oct, cudaStream_t s);
-// Entries of an FP64 / double-float twiddle table for embedding size P (a power of two >= 32).
+// Entries of a twiddle table for embedding size P (a power of two >= 32).
 // [0, P): W_P^m = exp(-2 pi i m / P).  Then, for Ns = 1, 2, 4, ..., P/16, the twiddles of a
 // radix-16 Stockham stage with Ns: W_{16 Ns}^{r k} (r = 1..15, k < Ns) at
 // P + 15 (Ns - 1) + (r - 1) Ns + k, so a warp's 32 consecutive k of one r are 32 consecutive
@@ -342,12 +295,10 @@ inline int twiddle_entries(int P) { return P + 15 * (P / 8 - 1); }
 // fills tw64 and tw32 (twiddle_entries(P) entries each; tw32 may be null)
 cudaError_t twiddle_launch(int P, double2* tw64, float2* tw32, cudaStream_t s);
 cudaError_t scale_symbol_launch(double* lam64, float* lam32, size_t n, double s, cudaStream_t st);
-// dst (line-major, converted to To) = s * oct (natural order); To = double, float or dfl
+// dst (line-major, converted to To) = s * oct (natural order); To = double or float
 template <typename To>
 cudaError_t line_symbol_launch(const Plan& p, const double* oct, To* dst, double s, cudaStream_t st);
-cudaError_t to_df_launch(const double* src, dfl* dst, size_t n, cudaStream_t st);
 cudaError_t to_q_launch(const double2* src, int4* dst, size_t n, cudaStream_t st);
-cudaError_t to_cdf_launch(const double2* src, cdf* dst, size_t n, cudaStream_t st);
 // even DFT of the octant along every axis (used for both the operator and preconditioner symbols)
 cudaError_t symbol_axes_launch(const Plan& p, double* lam_oct, cudaStream_t s);
 

@@ -66,11 +66,9 @@ __device__ __forceinline__ void dft2(C& a, C& b) {
   b = t;
 }
 
-// The first-level sums feed only the second level, so they skip the double-float
-// renormalisation (add_lazy); the outputs are normalised.
 template <int SIGN, typename C>
 __device__ __forceinline__ void dft4(C& a, C& b, C& c, C& d) {
-  C s0 = add_lazy(a, c), d0 = sub_lazy(a, c), s1 = add_lazy(b, d), d1 = mul_i<SIGN>(sub_lazy(b, d));
+  C s0 = a + c, d0 = a - c, s1 = b + d, d1 = mul_i<SIGN>(b - d);
   a = s0 + s1;
   c = s0 - s1;
   b = d0 + d1;
@@ -133,7 +131,7 @@ __device__ __forceinline__ void dft16_tail(C* v) {
     for (int j2 = 1; j2 < 4; ++j2) {
       const int m = j2 * k1;
       if (m == 4) v[4 * k1 + j2] = mul_i<SIGN>(v[4 * k1 + j2]);  // W16^4 = SIGN i
-      else v[4 * k1 + j2] = cmul_lazy(v[4 * k1 + j2], w16<SIGN, T>(m));  // feeds the second-level sums
+      else v[4 * k1 + j2] = cmul(v[4 * k1 + j2], w16<SIGN, T>(m));
     }
   // length-4 DFTs over j2 for each k1: X[k1 + 4 k2]
   C out[16];
@@ -225,11 +223,11 @@ __device__ __forceinline__ void twiddles16(cplx<T>* w, const cplx<T>* __restrict
 // (G <= 32) lies inside one warp, and a warp barrier suffices: the other warps of the CTA
 // proceed independently.  CTAs are whole warps (the launchers round their size to a
 // multiple of 32 threads) and every thread calls the transform, so the full-warp barrier
-// is well defined.  A longer line spans G/32 whole warps.  In the FP64 and double-float
-// engines such a line synchronises on its own named barrier (1 + its index in the CTA)
+// is well defined.  A longer line spans G/32 whole warps.  With 16-byte
+// elements such a line synchronises on its own named barrier (1 + its index in the CTA)
 // over its G threads when the CTA holds several lines (CTAs hold at most 512 threads, so
-// at most 8 such lines and barriers 1..8); this measured 4% faster for the 2048-point
-// double-float rows.  FP32 keeps the CTA barrier, which measured faster there.
+// at most 8 such lines and barriers 1..8), so that lines don't wait for each other
+// (a few percent on 2048-point rows).  FP32 keeps the CTA barrier, which measured faster there.
 template <typename T>
 __device__ __forceinline__ void line_sync(int logL) {
   if (logL <= 9) {
@@ -314,8 +312,8 @@ template <typename T, int SIGN, bool ZIN_ = false, bool HOUT_ = false>
 __device__ __forceinline__ void fft_line(cplx<T>* buf, int logL, int lane, const cplx<T>* __restrict__ tw,
                                          int logPtab) {
   // The pruned first/last stages pay off where arithmetic is the bottleneck (FP64); for
-  // FP32 and double-float they only add code (three copies of the radix-16 stage instead
-  // of one loop body), which measured slower, so they are used for FP64 only.
+  // FP32 they only add code (three copies of the radix-16 stage instead of one loop body),
+  // which measured slower, so they are used for FP64 only.
   constexpr bool ZIN = ZIN_ && std::is_same<T, double>::value;
   constexpr bool HOUT = HOUT_ && std::is_same<T, double>::value;
   const int rem = logL & 3;
@@ -411,7 +409,7 @@ __device__ __forceinline__ void regs_last_stage(cplx<T>* v, int lane, int G, con
       t[r] = v[b + r * B];
       if (r > 0) {
         const C wr = FRLAP_GLD(tw + ((r * j) << shift));
-        t[r] = (SIGN < 0) ? cmul_lazy(t[r], wr) : cmulc_lazy(t[r], wr);
+        t[r] = (SIGN < 0) ? cmul(t[r], wr) : cmulc(t[r], wr);
       }
     }
     dftR<R, SIGN, false>(t);
@@ -438,7 +436,7 @@ __device__ __forceinline__ void regs_stage16(cplx<T>* v, int lane, int logNs, co
     cplx<T> w[16];
     twiddles16<T>(w, tw, k, logNs, logPtab);
 #pragma unroll
-    for (int r = 1; r < 16; ++r) v[r] = (SIGN < 0) ? cmul_lazy(v[r], w[r]) : cmulc_lazy(v[r], w[r]);
+    for (int r = 1; r < 16; ++r) v[r] = (SIGN < 0) ? cmul(v[r], w[r]) : cmulc(v[r], w[r]);
   }
   dft16<SIGN>(v);
 }

@@ -14,6 +14,13 @@
 // FP64's 2^-53.  The scale follows the data and not a growth bound, so lines whose spectra are concentrated
 // (smooth fields) lose nothing.
 //
+// The DF64 engine sets the scale of the first stage's rows once, on entry, which saves the reductions and shifts
+// between its stages (a sixth of their integer operations): 1.6e-16 for N(0,1) data.  A smooth row loses
+// nothing, since its largest value grows by the bound; rows of one spike lose most (4096-point
+// axis, normwise against the FP64 engine: 5.8e-16, over noise at 1e-3 2.0e-15; the double-float arithmetic that
+// this replaced 5e-15 throughout).  (Columns and inverse transforms need the data's scale: the
+// columns of a smooth field at high frequencies, and spectra, lost up to 28 bits without it.)
+//
 // Between kernels a line's values are stored as integers below 2^58 with the line's exponent beside them
 // (apply_q.cuh); a kernel whose lines run across those aligns their exponents as it loads.
 #pragma once
@@ -214,6 +221,22 @@ __device__ __forceinline__ long long q_shl(long long a, int s) {  // 0 <= s <= 3
   const unsigned h = __funnelshift_l(l, (unsigned)(a >> 32), s);
   return (long long)(((unsigned long long)h << 32) | (l << s));
 }
+// Shift of a line with magnitude bits o to bits 0..61: components below 2^62, or magnitudes still below 2^62.5.
+__device__ __forceinline__ int q_fill_shift(unsigned o) {
+  const int sh = __clz((int)o) - 2;
+  return sh < 0 ? 0 : (sh > 30 ? 30 : sh);
+}
+// The line's entries v[0..N) (all threads') shifted so.
+template <int N>
+__device__ __forceinline__ void q_fill(cq* v, int& e, int logL, unsigned* slot) {
+  unsigned o = 0u;
+#pragma unroll
+  for (int m = 0; m < N; ++m) o |= q_bits(v[m]);
+  const int sh = q_fill_shift(q_reduce<false>(o, logL, slot));
+#pragma unroll
+  for (int m = 0; m < N; ++m) v[m] = {q_shl(v[m].x, sh), q_shl(v[m].y, sh)};
+  e -= sh;
+}
 template <int SH>
 __device__ __forceinline__ long long q_shr_round(long long a) {
   return (a + (1LL << (SH - 1))) >> SH;
@@ -324,12 +347,14 @@ template <int REM>
 constexpr int kQDrop = REM == 1 ? 3 : REM == 2 ? 2 : 0;
 
 // As fft_regs: v[m] = x[lane + m G] on entry (components below 2^58), X[lane + m G] on exit (magnitudes
-// below 2^(62.5 - kQDrop)); e, the line's exponent, follows.  ZIN: v[8..15] are zero.  slots: the line's reduction
+// below 2^(62.5 - kQDrop)); e, the line's exponent, follows.  DYN: the scale follows the data between stages;
+// else it stays as set on entry (lines with three twiddled stages excepted).  ZIN: v[8..15] are zero.  slots: the line's reduction
 // words, used from index si on.
-template <int SIGN, bool ZIN, int REM>
+template <bool DYN, int SIGN, bool ZIN, int REM>
 __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
                                       int logPtab, bool sync_first, unsigned* slots, int& si) {
   const int G = 1 << (logL - 4);
+  const bool dyn = DYN || (REM == 1 && logL > 12);
   if constexpr (ZIN) {
 #pragma unroll
     for (int m = 8; m < 16; ++m) v[m] = {0, 0};
@@ -337,9 +362,11 @@ __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane
   // between stages: write, agree on the scale, read, shift
   auto exchange = [&](int logNs, bool first8, bool pre_sync) {
     unsigned o = 0u;
+    if (dyn) {
 #pragma unroll
-    for (int m = 0; m < 16; ++m) o |= q_bits(v[m]);
-    o = q_publish<false>(o, logL, slots + si);
+      for (int m = 0; m < 16; ++m) o |= q_bits(v[m]);
+      o = q_publish<false>(o, logL, slots + si);
+    }
     if (pre_sync) line_sync<double>(logL);
     if (first8) {
 #pragma unroll
@@ -361,13 +388,14 @@ __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane
     const int rbase = spad(lane), rstep = G + (G >> 4);
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = buf[g16 ? rbase + m * rstep : spad(lane + m * G)];
-    // to bits 0..61: components below 2^62, or magnitudes still below 2^62.5
-    int sh = __clz((int)q_fetch(o, logL, slots + si)) - 2;
-    sh = sh < 0 ? 0 : (sh > 30 ? 30 : sh);
-    ++si;
+    e += 4;
+    if (dyn) {
+      const int sh = q_fill_shift(q_fetch(o, logL, slots + si));
+      ++si;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = {q_shl(v[m].x, sh), q_shl(v[m].y, sh)};
-    e += 4 - sh;
+      for (int m = 0; m < 16; ++m) v[m] = {q_shl(v[m].x, sh), q_shl(v[m].y, sh)};
+      e -= sh;
+    }
   };
   int logNs;
   if constexpr (REM == 3) {

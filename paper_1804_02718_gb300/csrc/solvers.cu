@@ -469,18 +469,16 @@ size_t vec_bytes(const Plan& p, int eb) { return align256(p.M * (size_t)eb); }
 }  // namespace
 
 // the apply of a CG in precision T: FP32 vectors through the FP32 engine, FP64
-// vectors through the plan's FP64 engine (native or double-float)
+// vectors through the plan's F64 or DF64 engine
 template <typename T>
 static cudaError_t apply_T(const Plan& p, const T* u, T* y, void* work, cudaStream_t s, const int* skip) {
   if constexpr (sizeof(T) == 8) return apply64(p, u, y, work, s, skip);
   else return apply_launch<float>(p, u, y, work, s, skip);
 }
 
-// The residuals f - B x that restart a solve or decide its convergence.  The iterations may run
-// on double-float (48-bit products), but a residual computed with it carries the transforms' rounding times
-// up to lambda_max (about 5e-15 lambda_max ||x||), which at 2047^2 already sits near 1e-10 ||f||.  So a
-// residual takes the FP64 engine on every plan.  A restart from such a residual removes the recurrence's
-// drift, as in iterative refinement.
+// The residuals f - B x that restart a solve or decide its convergence take the F64 engine on every plan: near a
+// solution an apply's rounding reaches the residual times up to lambda_max.  A restart from such a residual
+// removes the recurrence's drift, as in iterative refinement.
 template <typename T>
 static cudaError_t apply_residual(const Plan& p, const T* u, T* y, void* work, cudaStream_t s) {
   return apply_launch<T>(p, u, y, work, s, nullptr);
@@ -728,7 +726,7 @@ size_t ac_work_bytes(const Plan& p) {
   return cg_work_bytes(p, 8) + 2 * vec_bytes(p, 8) + align256(p.lam_count * sizeof(float)) + 256;
 }
 
-// Workspace of frlap_pcg_solve: the CG or refinement workspace, and on double-float plans the
+// Workspace of frlap_pcg_solve: the CG or refinement workspace, and on DF64 plans the
 // scaled right-hand side (one FP64 vector) behind it.
 static size_t pcg_base_bytes(const Plan& p) {
   if (p.prec == FRLAP_MIXED || p.prec == FRLAP_MIXED_DF64) return ir_work_bytes(p);
@@ -741,10 +739,9 @@ static frlap_status pcg_solve_core(const Plan& p, const double* f, double* x, do
                                    cudaStream_t st, bool x0_zero);
 
 // max |f_i| and max |x0_i| first (one synchronisation): a zero x0 needs no apply for the initial
-// residual (r = f), and on double-float plans, which keep FP32's exponent range, the system is
-// solved for 2^-e f with 2^e the power of two at or below max |f_i| (and x0 scaled alike), and x
-// is scaled back: every scaling is by a power of two, exact in FP64, so the solve is the same up
-// to the double-float range it now stays inside.
+// residual (r = f), and on DF64 plans, whose FP32 preconditioners and inner solves keep FP32's exponent
+// range, the system is solved for 2^-e f with 2^e the power of two at or below max |f_i| (and x0 scaled
+// alike), and x is scaled back: every scaling is by a power of two, exact in FP64.
 frlap_status pcg_solve_impl(const Plan& p, const double* f, double* x, double rtol, int maxit, int solver,
                             const float* mu, double inner_rtol, int* iters, double* relres, void* work,
                             cudaStream_t st) {
@@ -788,7 +785,7 @@ static frlap_status pcg_solve_core(const Plan& p, const double* f, double* x, do
   if (solver == FRLAP_SOLVE_CG) {
     // CG, then the true residual; if rounding left the true residual above rtol while the
     // recursive one met it, restart from the current x (at most 4 restarts, within maxit).
-    // A restart aims at rtol / 10: it starts from the native FP64 residual, so its own
+    // A restart aims at rtol / 10: it starts from the F64 engine's residual, so its own
     // recursive residual going well below rtol carries the true one below rtol too.
     int total = 0;
     double rel = 0.0;
@@ -826,7 +823,7 @@ static frlap_status pcg_solve_core(const Plan& p, const double* f, double* x, do
   double rel = 0.0;
   const int max_outer = 60;
   // Outer residuals use the plan's FP64-side engine while far from rtol; from 1e-6 on (and to
-  // decide convergence) the native FP64 engine computes them.
+  // decide convergence) the F64 engine computes them.
   double prev = 1.0;
   for (int outer = 0; outer <= max_outer; ++outer) {
     const bool native = prev <= 1e-6;

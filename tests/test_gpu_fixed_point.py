@@ -111,3 +111,28 @@ def test_split_middle_stage(frlap):
         a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
         ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
         assert abs(float(y[i] - ref)) < 2.0 ** -49 * lam_max
+
+
+@pytest.mark.parametrize("Ns", SHAPES)
+def test_df64_first_stage_entries(frlap, Ns):
+    """The DF64 engine's first stage, whose scale is set once per row.  With L points in a row (P <= 8192) its
+    unit after the last butterfly is 2^-60 L max|u|, and back on the grid that is sqrt(L) 2^-60 max|u| lambda_max
+    in the mean square: 2^-51.2 lambda_max at L = 8192 and max|u| = 5, three times that for the largest of 40
+    samples.  Beside the other stages' 2^-49 the bound is 2^-48 lambda_max."""
+    import torch
+
+    plan, coef, c, lam_max = _operator(frlap, Ns, 1.3, frlap.FRLAP_DF64)
+    u = inp.normal_field(Ns, seed=13)
+    B = 3  # a batch: its last CTA's rows are ragged
+    us = torch.stack([torch.from_numpy(u).cuda() * s for s in (1.0, 0.0, 2.0 ** -70)])
+    ys = frlap.frlap_apply_batch(plan, us).cpu().numpy()
+    assert ys.shape[0] == B and not ys[1].any()
+    assert np.array_equal(ys[2], ys[0] * 2.0 ** -70)
+    rng = np.random.default_rng(4)
+    ul = u.astype(np.longdouble)
+    grids = [np.arange(n) for n in u.shape]
+    for _ in range(40):
+        i = [int(rng.integers(n)) for n in u.shape]
+        a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
+        ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
+        assert abs(float(ys[0][tuple(i)] - ref)) < 2.0 ** -48 * lam_max
