@@ -36,7 +36,7 @@ namespace {
 
 // Spectrum columns of the learned preconditioner: columns of n entries -> zero-pad to P, forward FFT, all P
 // outputs in FP64 (stride ldo).
-template <int REM>
+template <int REM, int LOGP, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_col_fwd(const cq* __restrict__ in, const int* __restrict__ ex, double2* __restrict__ out, int ncols, int n,
                 size_t ld, size_t ldo, int logP, int TL, int cols_per, const int4* __restrict__ tw,
@@ -44,8 +44,10 @@ __global__ void __launch_bounds__(512, 1)
   in += blockIdx.y * bt.in;
   out += blockIdx.y * bt.out;
   ex += blockIdx.y * ex_inst;
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4;
+  logP = LOGP;
+  constexpr int lg = q_lg<E>(LOGP);
+  FRLAP_Q_PROLOGUE(lg)
+  const int P = 1 << logP, G = P / E;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int col = blockIdx.x * TL + l;
   const bool valid = col < ncols;
@@ -53,22 +55,22 @@ __global__ void __launch_bounds__(512, 1)
   unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
   cq* buf = smem + (size_t)l * sline(P);
   int si = 0;
-  cq v[16];
+  cq v[E];
   // exponents: 2D ex[i] for every column; 3D ex[(col / P_y) n + i]
   const int kx = cols_per ? c / cols_per : c;
-  int e = q_load_aligned<8>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)kx * n : 0), kx & 1, lane, G, n, valid,
-                            logP, slots + si);
+  int e = q_load_aligned<E / 2>(v, in + (size_t)c * ld, ex + (cols_per ? (size_t)kx * n : 0), kx & 1, lane, G, n, valid,
+                            lg, slots + si);
   ++si;
-  q_fft<true, -1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_fft<true, -1, true, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
   if (!valid) return;
   double2* dst = out + (size_t)col * ldo;
 #pragma unroll
-  for (int m = 0; m < 16; ++m)
+  for (int m = 0; m < E; ++m)
     FRLAP_GST(dst + lane + m * G, make_double2(q_out_any(v[m].x, e), q_out_any(v[m].y, e)));
 }
 
 // Columns of P FP64 spectrum values times a multiplier (natural octant order) -> inverse FFT, crop to n.
-template <int REM>
+template <int REM, int LOGP, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_col_mulinv(const double2* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int ncols, int n,
                    size_t ld, size_t ldo, int logP, int TL, const double* __restrict__ lam, LamMap map,
@@ -76,8 +78,10 @@ __global__ void __launch_bounds__(512, 1)
   in += blockIdx.y * bt.in;
   out += blockIdx.y * bt.out;
   ex += blockIdx.y * ex_inst;
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4;
+  logP = LOGP;
+  constexpr int lg = q_lg<E>(LOGP);
+  FRLAP_Q_PROLOGUE(lg)
+  const int P = 1 << logP, G = P / E;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int col = blockIdx.x * TL + l;
   const bool valid = col < ncols;
@@ -95,27 +99,27 @@ __global__ void __launch_bounds__(512, 1)
     lam_base = (size_t)min(ky, map.Py - ky) * map.Hx1 + kx;
     lam_stride = map.Hy1 * map.Hx1;
   }
-  double2 x[16];
+  double2 x[E];
   unsigned hm = 0u;
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const int k = lane + m * G;
     x[m] = valid ? FRLAP_GLD(lam + lam_base + (size_t)min(k, P - k) * lam_stride) * FRLAP_GLD(src + k)
                  : make_double2(0.0, 0.0);
   }
 #pragma unroll
-  for (int m = 0; m < 16; ++m) hm = max(hm, max(q_mag(x[m].x), q_mag(x[m].y)));
+  for (int m = 0; m < E; ++m) hm = max(hm, max(q_mag(x[m].x), q_mag(x[m].y)));
   int si = 0;
-  const QIn qs = q_in_scale(q_reduce<true>(hm, logP, slots + si));
+  const QIn qs = q_in_scale(q_reduce<true>(hm, lg, slots + si));
   ++si;
-  cq v[16];
+  cq v[E];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
+  for (int m = 0; m < E; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
   int e = qs.e;
-  q_fft<true, 1, false, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  q_store_scale<REM, 8>(v, e);
+  q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_store_scale<REM, E, E / 2>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex + col, e);
-  store_line(v, out, ncols, n, ldo, logP, TL);
+  store_line<E>(v, out, ncols, n, ldo, logP, TL);
 }
 
 }  // namespace
@@ -137,12 +141,13 @@ cudaError_t spectrum_forward(const Plan& p, int nb, const double* u, double2* SP
   if (p.d == 3 && (e = q_stage_yz_fwd(p, w, nb, 0, nullptr, 0, s)) != cudaSuccess) return e;
   const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
   const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
+  const QShape q = q_shape(0, p.P[ax], (long long)ncols, nb, ncols);
   Batch b;
   b.in = w.stride;
   b.out = sstride;
-  return with_rem(p.logP[ax], [&](auto tag) {
-    return q_launch(k_q_col_fwd<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s,
+  return q_with_shape(q, p.logP[ax], [&](auto tag) {
+    using K = decltype(tag);
+    return q_launch(k_q_col_fwd<K::rem, K::logp, K::e>, q.tiles, nb, q.threads, q.sm, s,
                     (const cq*)(p.d == 3 ? w.S2 : w.S1), (const int*)(p.d == 3 ? w.line : w.row), SP, ncols, p.n[ax],
                     (size_t)(p.d == 3 ? p.n[2] : nrows), (size_t)p.P[ax], p.logP[ax], q.tl, p.d == 3 ? p.P[1] : 0,
                     (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
@@ -165,13 +170,14 @@ cudaError_t spectrum_inverse(const Plan& p, int nb, const double2* SP, size_t ss
   const QWork w = q_work(p, work);
   const int ax = p.d == 3 ? 2 : 1, Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
   const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-  const QShape q = q_shape(0, p.P[ax], (long long)ncols * nb, ncols);
+  const QShape q = q_shape(0, p.P[ax], (long long)ncols, nb, ncols);
   const LamMap map = q_lam_map(p);
   Batch b;
   b.in = sstride;
   b.out = w.stride;
-  e = with_rem(p.logP[ax], [&](auto tag) {
-    return q_launch(k_q_col_mulinv<decltype(tag)::value>, q.tiles, nb, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
+  e = q_with_shape(q, p.logP[ax], [&](auto tag) {
+    using K = decltype(tag);
+    return q_launch(k_q_col_mulinv<K::rem, K::logp, K::e>, q.tiles, nb, q.threads, q.sm, s, SP, p.d == 3 ? w.S2 : w.S1,
                     w.col, ncols, p.n[ax], (size_t)p.P[ax], (size_t)(p.d == 3 ? p.n[2] : nrows), p.logP[ax], q.tl, mult,
                     map, (const int4*)p.twq[ax], (const int*)nullptr, b, w.ex_stride);
   });

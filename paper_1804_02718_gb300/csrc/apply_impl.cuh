@@ -426,18 +426,19 @@ __device__ __forceinline__ void store_line_odd(const C* v, C* __restrict__ data,
 // The cropped output of k_colmul: column blockIdx.x * TL + tid / G, elements lane + m G < n
 // (m < 8; n <= P/2).  The thread's column and lane are re-derived from
 // the special registers here, not kept live across both transforms (that spilled).
-template <typename C>
+template <int E = 16, typename C>
 __device__ __forceinline__ void store_line(const C* v, C* __restrict__ data, int ncols, int n, size_t ld, int logP,
                                            int TL) {
   unsigned tid;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
-  const int G = 1 << (logP - 4);
+  constexpr int LE = E == 4 ? 2 : 4;
+  const int G = 1 << (logP - LE);
   const int lane = (int)tid & (G - 1);
-  const int col = (int)blockIdx.x * TL + ((int)tid >> (logP - 4));
+  const int col = (int)blockIdx.x * TL + ((int)tid >> (logP - LE));
   if (col >= ncols) return;
   C* out = data + (size_t)col * ld;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+  for (int m = 0; m < E / 2; ++m) {
     const int i = lane + m * G;
     if (i < n) FRLAP_GST(out + i, v[m]);
   }

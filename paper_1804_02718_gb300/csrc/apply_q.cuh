@@ -38,9 +38,9 @@ inline QExpLayout q_exp_layout(const Plan& p) {
 }
 
 // A transform's output v[0..N) to what is stored, components below 2^58, and its exponent.
-template <int REM, int N>
+template <int REM, int E, int N>
 __device__ __forceinline__ void q_store_scale(cq* v, int& e) {
-  constexpr int SH = 5 - kQDrop<REM>;
+  constexpr int SH = 5 - kQDrop<REM, E>;
 #pragma unroll
   for (int m = 0; m < N; ++m) v[m] = q_shr_even<SH>(v[m]);
   e += SH;
@@ -67,11 +67,12 @@ __device__ __forceinline__ cq q_align(cq v, int e, int top, bool up) {
   }                                                                      \
   cq* smem = reinterpret_cast<cq*>(smem_raw);
 
-template <bool DYN, int REM, int LOGL = 0>
+template <bool DYN, int REM, int LOGL, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_r2c(const double* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int nlines, int n, size_t ldo,
             int logH, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
-  if constexpr (LOGL > 0) logH = LOGL;
+  logH = LOGL;
+  constexpr int lg = q_lg<E>(LOGL);
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -79,8 +80,8 @@ __global__ void __launch_bounds__(512, 1)
     ex += bi * ex_inst;
     if (skip) skip += bi * bt.skip;
   }
-  FRLAP_Q_PROLOGUE(logH)
-  const int H = 1 << logH, G = H >> 4, LS = sline(H);
+  FRLAP_Q_PROLOGUE(lg)
+  const int H = 1 << logH, G = H / E, LS = sline(H);
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int line0 = blockIdx.x * TL, line = line0 + l;
   const bool valid = line < nlines;
@@ -88,11 +89,11 @@ __global__ void __launch_bounds__(512, 1)
   unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
   cq* buf = smem + (size_t)l * LS;
   // packed samples z[q] = x[2q] + i x[2q+1], as in k_r2c_T
-  double xr[8], xi[8];
+  double xr[E / 2], xi[E / 2];
   const bool pair_aligned = (reinterpret_cast<uintptr_t>(src) % sizeof(double2)) == 0;
   unsigned hm = 0u;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+  for (int m = 0; m < E / 2; ++m) {
     const int q = lane + m * G;
     double a = 0.0, b = 0.0;
     if (valid) {
@@ -109,29 +110,29 @@ __global__ void __launch_bounds__(512, 1)
     xi[m] = b;
   }
 #pragma unroll
-  for (int m = 0; m < 8; ++m) hm = max(hm, max(q_mag(xr[m]), q_mag(xi[m])));
+  for (int m = 0; m < E / 2; ++m) hm = max(hm, max(q_mag(xr[m]), q_mag(xi[m])));
   int si = 0;
-  const QIn qs = q_in_scale(q_reduce<true>(hm, logH, slots + si));
+  const QIn qs = q_in_scale(q_reduce<true>(hm, lg, slots + si));
   ++si;
-  cq v[16];
+  cq v[E];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = {q_in(xr[m], qs), q_in(xi[m], qs)};
+  for (int m = 0; m < E / 2; ++m) v[m] = {q_in(xr[m], qs), q_in(xi[m], qs)};
   int e = qs.e;
-  q_fft<DYN, -1, true, REM>(v, e, buf, logH, lane, tw, logH + 1, false, slots, si);
-  if constexpr (!DYN) q_fill<16>(v, e, logH, slots + si);
-  line_sync<double>(logH);
+  q_fft<DYN, -1, true, REM, E>(v, e, buf, logH, lane, tw, logH + 1, false, slots, si);
+  if constexpr (!DYN) q_fill<E>(v, e, lg, slots + si);
+  line_sync<double>(lg);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = v[m];
-  int4 wk[8];  // W^k of this thread's pairs, in flight over the barrier
+  for (int m = 0; m < E; ++m) buf[spad(lane + m * G)] = v[m];
+  int4 wk[E / 2];  // W^k of this thread's pairs, in flight over the barrier
 #pragma unroll
-  for (int j = 0; j < 8; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
-  line_sync<double>(logH);
+  for (int j = 0; j < E / 2; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
+  line_sync<double>(lg);
   // Real-data split in place, one product per pair (see r2c_tile): X[k] = s + W^k d,
   // X[H-k] = conj(s - W^k d), s = (a + b) / 2, d = -i (a - b) / 2; stored below 2^57.5, that is over 2^(6 - D),
   // D = kQDrop (0 after q_fill).  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of
   // the downward shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in
   // a + b.
-  constexpr int D = DYN ? kQDrop<REM> : 0;
+  constexpr int D = DYN ? kQDrop<REM, E> : 0;
   auto split = [&](int k, const int4 wk) {
     const int km = H - k;
     const cq a = buf[spad(k)];
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(512, 1)
     if (k != km) buf[spad(km)] = conjg(q_shr_even<2>(s - t));
   };
 #pragma unroll
-  for (int j = 0; j < 8; ++j) split(lane + j * G, wk[j]);
+  for (int j = 0; j < E / 2; ++j) split(lane + j * G, wk[j]);
   if (lane == 0) split(H / 2, FRLAP_GLD(tw + H / 2));
   if (valid && lane == 0) FRLAP_GST(ex + line, e + 6 - D);
   __syncthreads();
@@ -212,12 +213,12 @@ __device__ __forceinline__ double q_ld(const double* p) {
 // and so is its circulant embedding (a zero from underflow acts as 2^-1022).
 // lrow[idx(m)] is entry m's lambda; its words are read twice (the second time from L1), since held over the
 // reduction they spill.
-template <typename I>
+template <int E, typename I>
 __device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict__ lrow, I idx, int logL,
                                          unsigned* slot) {
   int top = 0;
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const unsigned h = q_ld_hi(lrow + idx(m));
     // leading bit of |v| above bit 31 (the conversion rounds it up by at most one), plus 127
     const int pos = __float_as_int(__uint2float_rn(q_bits(v[m]))) >> 23;
@@ -225,7 +226,7 @@ __device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict
   }
   top = (int)q_reduce<true>((unsigned)top, logL, slot);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     // lambda v = (mant v / 2^64) 2^(el - 1020), 2^61 <= mant < 2^62, and |v| 2^(el - top + 127) < 2^33: the
     // shift s = el - top + 152 brings the product below 2^58.  A right shift is one of the mantissa (its
     // dropped bits weigh less than a unit of the product), a left one is one of v.
@@ -243,12 +244,13 @@ __device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict
 }
 
 // A column's entries of one line: element i of instance-local column col at data[col ld + i].
-template <int REM, int LOGP = 0>
+template <int REM, int LOGP, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_colmul(cq* __restrict__ data, const int* __restrict__ ex_in, int* __restrict__ ex_out, int ncols, int n,
                size_t ld, int logP, int TL, const double* __restrict__ lam, LamMap map, int nz,
                const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
-  if constexpr (LOGP > 0) logP = LOGP;
+  logP = LOGP;
+  constexpr int lg = q_lg<E>(LOGP);
   {
     const size_t bi = blockIdx.y;
     data += bi * bt.in;
@@ -257,8 +259,8 @@ __global__ void __launch_bounds__(512, 1)
     ex_out += bi * ex_inst;
     if (skip) skip += bi * bt.skip;
   }
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4;
+  FRLAP_Q_PROLOGUE(lg)
+  const int P = 1 << logP, G = P / E;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int col = blockIdx.x * TL + l;
   const bool valid = col < ncols;
@@ -266,21 +268,21 @@ __global__ void __launch_bounds__(512, 1)
   cq* buf = smem + (size_t)l * sline(P);
   const int c = valid ? col : 0;
   int si = 0;
-  cq v[16];
+  cq v[E];
   const int kx = map.d == 2 ? c : c >> map.logPy;
   const int* exi = ex_in + (map.d == 2 ? 0 : (size_t)kx * nz);
-  int e = q_load_aligned<8>(v, data + (size_t)c * ld, exi, kx & 1, lane, G, n, valid, logP, slots + si);
+  int e = q_load_aligned<E / 2>(v, data + (size_t)c * ld, exi, kx & 1, lane, G, n, valid, lg, slots + si);
   ++si;
-  q_fft<true, -1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_fft<true, -1, true, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
   const int ky = c & (map.Py - 1);
   const double* lrow = map.d == 2 ? lam + (size_t)c * map.Hy1
                                   : lam + ((size_t)kx * map.Hy1 + min(ky, map.Py - ky)) * map.Hz1;
-  q_symbol(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, logP, slots + si);
+  q_symbol<E>(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, lg, slots + si);
   ++si;
-  q_fft<true, 1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  q_store_scale<REM, 8>(v, e);
+  q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  q_store_scale<REM, E, E / 2>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex_out + col, e);
-  store_line(v, data, ncols, n, ld, logP, TL);
+  store_line<E>(v, data, ncols, n, ld, logP, TL);
 }
 
 // The middle stage of a 16384-point y embedding in two halves (see k_colmul_split).  ODD = false: the even
@@ -322,7 +324,7 @@ __global__ void __launch_bounds__(512, 1)
   q_fft<true, -1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, false, slots, si);
   // the half's symbol entries are every second one
   const double* lrow = lam + (size_t)(valid ? col : 0) * Hy1;
-  q_symbol(
+  q_symbol<16>(
       v, e, lrow,
       [&](int m) {
         const int k = 2 * (lane + m * G) + (ODD ? 1 : 0);
@@ -359,13 +361,14 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // groups of contiguous lines of length n -> pad, FFT, transposed store out[g][k][line]
-template <int REM, int LOGL = 0>
+template <int REM, int LOGL, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_c2cT_fwd(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
                  int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
                  int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
                  size_t ex_inst) {
-  if constexpr (LOGL > 0) logP = LOGL;
+  logP = LOGL;
+  constexpr int lg = q_lg<E>(LOGL);
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -374,8 +377,8 @@ __global__ void __launch_bounds__(512, 1)
     ex_out += bi * ex_inst;
     if (skip) skip += bi * bt.skip;
   }
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4, LS = sline(P);
+  FRLAP_Q_PROLOGUE(lg)
+  const int P = 1 << logP, G = P / E, LS = sline(P);
   const int g = blockIdx.x / tiles, tile = blockIdx.x % tiles;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int line0 = tile * TL, line = line0 + l;
@@ -384,17 +387,17 @@ __global__ void __launch_bounds__(512, 1)
   cq* buf = smem + (size_t)l * LS;
   const int c = valid ? line : 0;
   int si = 0;
-  cq v[16];
+  cq v[E];
   // rows (z, y) of this line z: exponents ex_in[z n + y]
-  int e = q_load_aligned<8>(v, in + g * gin + (size_t)c * ldi, ex_in + (size_t)c * n, g & 1, lane, G, n, valid,
-                            logP, slots + si);
+  int e = q_load_aligned<E / 2>(v, in + g * gin + (size_t)c * ldi, ex_in + (size_t)c * n, g & 1, lane, G, n, valid,
+                            lg, slots + si);
   ++si;
-  q_fft<true, -1, true, REM>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  q_store_scale<REM, 16>(v, e);
+  q_fft<true, -1, true, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
+  q_store_scale<REM, E, E>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
-  line_sync<double>(logP);
+  line_sync<double>(lg);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) buf[spad(lane + m * G)] = v[m];
+  for (int m = 0; m < E; ++m) buf[spad(lane + m * G)] = v[m];
   __syncthreads();
   const int logTL = __ffs(TL) - 1;
   const int lt = threadIdx.x & (TL - 1);
@@ -409,13 +412,14 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // transposed in[g][k][line] (k < P) -> IFFT along k, crop to n, store out[g][line][i]
-template <int REM, int LOGL = 0>
+template <int REM, int LOGL, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_c2cT_inv(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
                  int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
                  int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
                  size_t ex_inst) {
-  if constexpr (LOGL > 0) logP = LOGL;
+  logP = LOGL;
+  constexpr int lg = q_lg<E>(LOGL);
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -424,35 +428,35 @@ __global__ void __launch_bounds__(512, 1)
     ex_out += bi * ex_inst;
     if (skip) skip += bi * bt.skip;
   }
-  FRLAP_Q_PROLOGUE(logP)
-  const int P = 1 << logP, G = P >> 4, LS = sline(P);
+  FRLAP_Q_PROLOGUE(lg)
+  const int P = 1 << logP, G = P / E, LS = sline(P);
   const int g = blockIdx.x / tiles, tile = blockIdx.x % tiles;
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int line0 = tile * TL, line = line0 + l;
   unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
   cq* buf = smem + (size_t)l * LS;
-  int ek[16];
+  int ek[E];
   int e = kQZero;
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     ek[m] = FRLAP_GLD(ex_in + (size_t)g * P + lane + m * G);
     e = max(e, ek[m]);
   }
   load_transposed<cq>(smem, in + g * gin, TL * P, TL, LS, ldi, line0, nlines);
-  unsigned o = q_publish<true>(q_ord(e), logP, slots);
+  unsigned o = q_publish<true>(q_ord(e), lg, slots);
   __syncthreads();
-  e = q_unord(q_fetch(o, logP, slots));
+  e = q_unord(q_fetch(o, lg, slots));
   int si = 1;
-  cq v[16];
+  cq v[E];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
-  q_fft<true, 1, false, REM>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  q_store_scale<REM, 8>(v, e);
+  for (int m = 0; m < E; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
+  q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
+  q_store_scale<REM, E, E / 2>(v, e);
   if (line < nlines) {
     if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
     cq* dst = out + g * gout + (size_t)line * ldo;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
+    for (int m = 0; m < E / 2; ++m) {
       const int i = lane + m * G;
       if (i < n) FRLAP_GST(dst + i, v[m]);
     }
@@ -460,12 +464,13 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // Last stage.  Bin k of row r has exponent ex[k ex_k + (r / rows_per) ].
-template <int REM, int LOGL = 0>
+template <int REM, int LOGL, int E>
 __global__ void __launch_bounds__(512, 1)
     k_q_c2r(const cq* __restrict__ in, double* __restrict__ out, const int* __restrict__ ex, int ex_k, int rows_per,
             int nlines, int n, size_t ldi, int logH, int TL, const int4* __restrict__ tw,
             const int* __restrict__ skip, Batch bt, size_t ex_inst) {
-  if constexpr (LOGL > 0) logH = LOGL;
+  logH = LOGL;
+  constexpr int lg = q_lg<E>(LOGL);
   {
     const size_t bi = blockIdx.y;
     in += bi * bt.in;
@@ -473,19 +478,19 @@ __global__ void __launch_bounds__(512, 1)
     ex += bi * ex_inst;
     if (skip) skip += bi * bt.skip;
   }
-  FRLAP_Q_PROLOGUE(logH)
-  const int H = 1 << logH, G = H >> 4, LS = sline(H);
+  FRLAP_Q_PROLOGUE(lg)
+  const int H = 1 << logH, G = H / E, LS = sline(H);
   const int l = threadIdx.x / G, lane = threadIdx.x % G;
   const int line0 = blockIdx.x * TL, line = line0 + l;
   const bool valid = line < nlines;
   unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
   cq* buf = smem + (size_t)l * LS;
-  // this thread's pairs (k, H - k): k = lane + j G <= H/2 (j = 8: lane 0 alone)
-  int ea[9], eb[9];
+  // this thread's pairs (k, H - k): k = lane + j G <= H/2 (j = E/2: lane 0 alone)
+  int ea[E / 2 + 1], eb[E / 2 + 1];
   int e = kQZero;
   const int* exl = ex + (valid ? line / rows_per : 0);
 #pragma unroll
-  for (int j = 0; j < 9; ++j) {
+  for (int j = 0; j < E / 2 + 1; ++j) {
     const int k = lane + j * G;
     if (k <= H / 2) {
       ea[j] = FRLAP_GLD(exl + (size_t)k * ex_k);
@@ -494,39 +499,40 @@ __global__ void __launch_bounds__(512, 1)
     }
   }
   load_transposed<cq>(smem, in, TL * (H + 1), TL, LS, ldi, line0, nlines);
-  unsigned o = q_publish<true>(q_ord(e), logH, slots);
-  int4 wk[8];  // W^k of this thread's pairs, in flight over the barrier
+  unsigned o = q_publish<true>(q_ord(e), lg, slots);
+  int4 wk[E / 2];  // W^k of this thread's pairs, in flight over the barrier
 #pragma unroll
-  for (int j = 0; j < 8; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
+  for (int j = 0; j < E / 2; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
   __syncthreads();
-  e = q_unord(q_fetch(o, logH, slots));
+  e = q_unord(q_fetch(o, lg, slots));
   int si = 1;
   // repack in place (see k_c2r_T), over 4: Z[k] = A + i T, Z[H-k] = conj(A - i T), A = X[k] + conj X[H-k],
   // T = W^-k (X[k] - conj X[H-k])
 #pragma unroll
-  for (int j = 0; j < 9; ++j) {
+  for (int j = 0; j < E / 2 + 1; ++j) {
     const int k = lane + j * G;
     if (k <= H / 2) {
       const int km = H - k;
       const cq xk = q_align(buf[spad(k)], ea[j], e, k & 1);
       const cq b = conjg(q_align(buf[spad(km)], eb[j], e, k & 1));
       const cq A = q_shr_even<2>(xk + b), d = xk - b;
-      const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, j < 8 ? wk[j & 7] : FRLAP_GLD(tw + k)));
+      const int4 w = j < E / 2 ? wk[j & (E / 2 - 1)] : FRLAP_GLD(tw + k);
+      const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, w));
       buf[spad(k)] = A + iT;
       if (k != km && km != H) buf[spad(km)] = conjg(A - iT);
     }
   }
   e += 2;
-  line_sync<double>(logH);
-  cq v[16];
+  line_sync<double>(lg);
+  cq v[E];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = buf[spad(lane + m * G)];
-  q_fft<true, 1, false, REM>(v, e, buf, logH, lane, tw, logH + 1, true, slots, si);
+  for (int m = 0; m < E; ++m) v[m] = buf[spad(lane + m * G)];
+  q_fft<true, 1, false, REM, E>(v, e, buf, logH, lane, tw, logH + 1, true, slots, si);
   if (!valid) return;
   double* dst = out + (size_t)line * n;
   const bool pair_aligned = (reinterpret_cast<uintptr_t>(dst) % sizeof(double2)) == 0;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+  for (int m = 0; m < E / 2; ++m) {
     const int q = lane + m * G;
     if (2 * q < n) {
       const double a = q_out_any(v[m].x, e), b = q_out_any(v[m].y, e);
@@ -581,15 +587,40 @@ static cudaError_t q_launch(K kern, unsigned grid, int B, int threads, size_t sm
 struct QShape {
   int tl, threads, tiles;
   size_t sm;
+  bool thin;  // four entries a thread (q_fft4)
 };
-static QShape q_shape(int tuned, int L, long long lines_total, int lines_per_group) {
-  const int G = L >> 4;
+// Four entries a thread where, at sixteen, a vector's lines leave seven eighths of the chip's 608 sub-partitions
+// without a warp.  The line depends on the plan alone, so that a batch equals its vectors' applies bit for bit; a
+// batch of 8 then still has at most a warp per sub-partition.  One F64 vector, us per stage (with its launch),
+// sixteen -> four: 32^2 12.2, 10.8, 10.2 -> 9.6, 7.9, 7.2 (r2c, colmul, c2r), 128^2 13.1, 11.9, 10.2 -> 10.6, 8.9,
+// 8.2; 8 x 128^2 4.7 -> 4.1 a vector.  In larger launches the extra stages and barriers cost more: 8 x 256^2 7.1
+// -> 8.9 a vector.
+constexpr long long kQThinThreads = 152 * 16;
+static QShape q_shape(int tuned, int L, long long lines, int B, int lines_per_group, bool may_thin = true) {
   QShape q;
-  q.tl = pick_tl_tuned(tuned, sline(L), 16, G, 96 * 1024, lines_total);
+  q.thin = may_thin && L <= (1 << kQThinLog) && lines * (L >> 4) <= kQThinThreads;
+  const int G = q.thin ? L >> 2 : L >> 4;
+  q.tl = pick_tl_tuned(q.thin ? 0 : tuned, sline(L), 16, G, 96 * 1024, lines * B);
   q.threads = q.tl * G;
   q.tiles = (lines_per_group + q.tl - 1) / q.tl;
   q.sm = (size_t)q.tl * sline(L) * 16;
   return q;
+}
+
+// f(tag) for the kernel instance of a line of 2^logL points: tag::rem, tag::logp and tag::e entries a thread.
+template <int R, int L, int E>
+struct QTag : ShapeTag<R, L> {
+  static constexpr int e = E;
+};
+template <typename F>
+static cudaError_t q_with_shape(const QShape& q, int logL, F&& f) {
+  return with_line_shape(logL, [&](auto tag) {
+    constexpr int R = decltype(tag)::rem, L = decltype(tag)::logp;
+    if constexpr (L <= kQThinLog) {
+      if (q.thin) return f(QTag<R, L, 4>{});
+    }
+    return f(QTag<R, L, 16>{});
+  });
 }
 
 static LamMap q_lam_map(const Plan& p) {
@@ -616,53 +647,56 @@ template <bool DYN>
 static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const double* u, size_t ustride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
   const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
-  const QShape q = q_shape(tuned, H, (long long)nrows * B, nrows);
+  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows);
   Batch b;
   b.in = ustride;
   b.out = w.stride;
   b.skip = skip_stride;
-  return with_line_shape(p.logP[0] - 1, [&](auto tag) {
-    return q_launch(k_q_r2c<DYN, decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, u, w.S1,
-                    w.row, nrows, p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b,
-                    w.ex_stride);
+  return q_with_shape(q, p.logP[0] - 1, [&](auto tag) {
+    using K = decltype(tag);
+    return q_launch(k_q_r2c<DYN, K::rem, K::logp, K::e>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row,
+                    nrows, p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
   });
 }
 static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
                                   cudaStream_t s) {
   const int Py = p.P[1], ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1;
-  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1 * B, nz);
+  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1, B, nz);
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
-  return with_line_shape(p.logP[1], [&](auto tag) {
-    return q_launch(k_q_c2cT_fwd<decltype(tag)::rem, decltype(tag)::logp>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, w.S2,
-                    (const int*)w.row, w.line, nz, q.tiles, ny, (size_t)nz * ny, ny, (size_t)Py * nz, nz, p.logP[1],
+  return q_with_shape(q, p.logP[1], [&](auto tag) {
+    using K = decltype(tag);
+    return q_launch(k_q_c2cT_fwd<K::rem, K::logp, K::e>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1,
+                    w.S2, (const int*)w.row, w.line, nz, q.tiles, ny, (size_t)nz * ny, ny, (size_t)Py * nz, nz, p.logP[1],
                     q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
   });
 }
 static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
                                   cudaStream_t s) {
   const int Py = p.P[1], ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1;
-  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1 * B, nz);
+  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1, B, nz);
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
-  return with_line_shape(p.logP[1], [&](auto tag) {
-    return q_launch(k_q_c2cT_inv<decltype(tag)::rem, decltype(tag)::logp>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S2, w.S1,
-                    (const int*)w.col, w.line, nz, q.tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, p.logP[1],
+  return q_with_shape(q, p.logP[1], [&](auto tag) {
+    using K = decltype(tag);
+    return q_launch(k_q_c2cT_inv<K::rem, K::logp, K::e>, Hx1 * q.tiles, B, q.threads, q.sm, s, (const cq*)w.S2,
+                    w.S1, (const int*)w.col, w.line, nz, q.tiles, ny, (size_t)Py * nz, nz, (size_t)nz * ny, ny, p.logP[1],
                     q.tl, (const int4*)p.twq[1], skip, b, w.ex_stride);
   });
 }
 static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, size_t ystride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
   const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
-  const QShape q = q_shape(tuned, H, (long long)nrows * B, nrows);
+  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows);
   Batch b;
   b.in = w.stride;
   b.out = ystride;
   b.skip = skip_stride;
-  return with_line_shape(p.logP[0] - 1, [&](auto tag) {
-    return q_launch(k_q_c2r<decltype(tag)::rem, decltype(tag)::logp>, q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, y,
+  return q_with_shape(q, p.logP[0] - 1, [&](auto tag) {
+    using K = decltype(tag);
+    return q_launch(k_q_c2r<K::rem, K::logp, K::e>, q.tiles, B, q.threads, q.sm, s, (const cq*)w.S1, y,
                     (const int*)(p.d == 3 ? w.line : w.col), p.d == 3 ? p.n[2] : 1, p.d == 3 ? p.n[1] : nrows, nrows,
                     p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
   });
@@ -707,7 +741,7 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, s
   if ((e = q_stage_r2c<DYN>(p, w, B, u, vstride, tuned[0], skip, skip_stride, s)) != cudaSuccess) return e;
   if ((e = mark()) != cudaSuccess) return e;
   if (p.d == 2 && p.P[1] > kMaxLine) {
-    const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1 * B, Hx1);
+    const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1, B, Hx1, false);
     int* ex_tmp = w.col + Hx1;
     e = q_launch(k_q_colmul_split<false>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col, ex_tmp,
                  Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);
@@ -723,10 +757,10 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, s
     // the middle stage: columns over y in S1 (2D), over z in S2 (3D)
     const int ax = p.d == 3 ? 2 : 1;
     const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-    const QShape q = q_shape(tuned[p.d == 3 ? 2 : 1], p.P[ax], (long long)ncols * B, ncols);
-    e = with_line_shape(p.logP[ax], [&](auto tag) {
-      constexpr int REM = decltype(tag)::rem, LP = decltype(tag)::logp;
-      return q_launch(k_q_colmul<REM, LP>, q.tiles, B, q.threads, q.sm, s, p.d == 3 ? w.S2 : w.S1,
+    const QShape q = q_shape(tuned[p.d == 3 ? 2 : 1], p.P[ax], (long long)ncols, B, ncols);
+    e = q_with_shape(q, p.logP[ax], [&](auto tag) {
+      using K = decltype(tag);
+      return q_launch(k_q_colmul<K::rem, K::logp, K::e>, q.tiles, B, q.threads, q.sm, s, p.d == 3 ? w.S2 : w.S1,
                       (const int*)(p.d == 3 ? w.line : w.row), w.col, ncols, p.n[ax], (size_t)(p.d == 3 ? nz : nrows),
                       p.logP[ax], q.tl, lam, map, nz, (const int4*)p.twq[ax], skip, b, w.ex_stride);
     });

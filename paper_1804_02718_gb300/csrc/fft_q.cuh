@@ -343,16 +343,88 @@ __device__ __forceinline__ void q_last_stage(cq* v, int lane, int G, const int4*
 
 // Bits that a line's transform of log2 length = REM mod 4 ends below 2^62.5: a last stage of radix 2 or 4
 // grows by that, but its products divide by 16.
-template <int REM>
-constexpr int kQDrop = REM == 1 ? 3 : REM == 2 ? 2 : 0;
+template <int REM, int E = 16>
+constexpr int kQDrop = E == 4 ? ((REM & 1) ? 3 : 2) : REM == 1 ? 3 : REM == 2 ? 2 : 0;
+
+// Transforms with four entries a thread, for launches of few lines: every thread of a sixteen-entry line issues
+// some 1500 instructions a stage, and with less than a warp per SM sub-partition their latency is the time.
+// Four entries take radix-4 stages: a quarter of the entries and a fifth of the instructions a stage, twice the
+// stages, four times the threads.  Lines of at most 2^kQThinLog points; v[m] = x[lane + m L/4] on entry and
+// X[lane + m L/4] on exit, scaled as in q_fft (magnitudes below 2^(62.5 - kQDrop<REM, 4>)).  With DYN = false
+// the line is shifted by the stage's growth, 2, instead.
+constexpr int kQThinLog = 10;
+// What stands for log2 of the line length where that tells the threads of a line (line_sync, q_reduce).
+template <int E>
+__host__ __device__ constexpr int q_lg(int logL) {
+  return E == 4 ? logL + 2 : logL;
+}
+template <bool DYN, int SIGN, bool ZIN>
+__device__ __forceinline__ void q_fft4(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
+                                       int logPtab, bool sync_first, unsigned* slots, int& si) {
+  const int G = 1 << (logL - 2), lg = q_lg<4>(logL);
+  if constexpr (ZIN) v[2] = v[3] = {0, 0};
+  q_dft4<SIGN>(v[0], v[1], v[2], v[3]);
+  int logNs = 0;  // of the stage whose results v holds
+  while (true) {
+    const int nextNs = logNs + 2;
+    // the next stage's twiddles, in flight over the exchange
+    const bool last2 = nextNs + 1 == logL;
+    int4 w[3];
+    if (last2) {
+#pragma unroll
+      for (int b = 0; b < 2; ++b) w[b] = q_ld_tw(tw + ((lane + b * G) << (logPtab - logL)));
+    } else {
+      const int k = lane & ((1 << nextNs) - 1);
+#pragma unroll
+      for (int r = 1; r < 4; ++r) w[r - 1] = q_ld_tw(tw + ((r * k) << (logPtab - nextNs - 2)));
+    }
+    unsigned o = 0u;
+    if (DYN) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) o |= q_bits(v[m]);
+      o = q_publish<false>(o, lg, slots + si);
+    }
+    if (logNs > 0 || sync_first) line_sync<double>(lg);
+    const int Ns = 1 << logNs, kw = lane & (Ns - 1), ob = (lane - kw) * 4 + kw;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) buf[spad(ob + r * Ns)] = v[r];
+    line_sync<double>(lg);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = buf[spad(lane + m * G)];
+    const int sh = DYN ? q_fill_shift(q_fetch(o, lg, slots + si)) : 2;
+    if (DYN) ++si;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = {q_shl(v[m].x, sh), q_shl(v[m].y, sh)};
+    e += 4 - sh;
+    logNs = nextNs;
+    if (last2) {
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const cq s = q_shr_round<4>(v[b]), t = q_cmul<(SIGN > 0)>(v[b + 2], w[b]);
+        v[b] = s + t;
+        v[b + 2] = s - t;
+      }
+      return;
+    }
+    v[0] = q_shr_round<4>(v[0]);
+#pragma unroll
+    for (int r = 1; r < 4; ++r) v[r] = q_cmul<(SIGN > 0)>(v[r], w[r - 1]);
+    q_dft4<SIGN>(v[0], v[1], v[2], v[3]);
+    if (logNs + 2 == logL) return;
+  }
+}
 
 // As fft_regs: v[m] = x[lane + m G] on entry (components below 2^58), X[lane + m G] on exit (magnitudes
 // below 2^(62.5 - kQDrop)); e, the line's exponent, follows.  DYN: the scale follows the data between stages;
-// else it stays as set on entry (lines with three twiddled stages excepted).  ZIN: v[8..15] are zero.  slots: the line's reduction
-// words, used from index si on.
-template <bool DYN, int SIGN, bool ZIN, int REM>
+// else it stays as set on entry (lines with three twiddled stages excepted).  ZIN: v[8..15] are zero.  slots:
+// the line's reduction words, used from index si on.  E = 4: see q_fft4.
+template <bool DYN, int SIGN, bool ZIN, int REM, int E = 16>
 __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
                                       int logPtab, bool sync_first, unsigned* slots, int& si) {
+  if constexpr (E == 4) {
+    q_fft4<DYN, SIGN, ZIN>(v, e, buf, logL, lane, tw, logPtab, sync_first, slots, si);
+    return;
+  } else {
   const int G = 1 << (logL - 4);
   const bool dyn = DYN || (REM == 1 && logL > 12);
   if constexpr (ZIN) {
@@ -427,6 +499,7 @@ __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane
     if (logNs + 4 == logL) return;
     exchange(logNs, false, true);
     logNs += 4;
+  }
   }
 }
 

@@ -136,3 +136,28 @@ def test_df64_first_stage_entries(frlap, Ns):
         a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
         ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
         assert abs(float(ys[0][tuple(i)] - ref)) < 2.0 ** -48 * lam_max
+
+
+@pytest.mark.parametrize("prec,bound", [("f64", 2.0 ** -49), ("df64", 2.0 ** -48)])
+@pytest.mark.parametrize("Ns", [(16, 52, 52), (32, 52, 52), (64, 40, 40), (128, 40, 40), (256, 300), (64, 609),
+                                (64, 610), (40, 16, 40), (40, 40, 16), (16, 40, 130), (9, 600), (100, 512),
+                                (30, 512)])
+def test_lines_on_both_sides_of_four_and_sixteen_entries_a_thread(frlap, Ns, prec, bound):
+    """Plans of few lines give a thread four entries, others sixteen (2432 threads at sixteen, the edge: 608 and
+    609 rows of 64 points): against the defining sum at the bounds above, and a batch of 9 bit for bit its vectors'
+    applies."""
+    import torch
+
+    plan, coef, c, lam_max = _operator(frlap, Ns, 1.3, getattr(frlap, "FRLAP_" + prec.upper()))
+    us = torch.from_numpy(np.stack([inp.normal_field(Ns, seed=s) for s in range(9)])).cuda()
+    ys = frlap.frlap_apply_batch(plan, us)
+    for u, y in zip(us, ys):
+        assert torch.equal(y, frlap.frlap_apply(plan, u.clone()))
+    ul, y = us[0].cpu().numpy().astype(np.longdouble), ys[0].cpu().numpy()
+    rng = np.random.default_rng(5)
+    grids = [np.arange(k) for k in ul.shape]
+    for _ in range(40):
+        i = [int(rng.integers(k)) for k in ul.shape]
+        a = coef[np.ix_(*[np.abs(g - k) for g, k in zip(grids, i)])]
+        ref = -np.longdouble(c) * np.sum(a.astype(np.longdouble) * ul)
+        assert abs(float(y[tuple(i)] - ref)) < bound * lam_max
