@@ -259,7 +259,7 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
     const size_t ntw = (size_t)twiddle_entries(p->P[r]);
     o_tw64[r] = reserve(ntw * sizeof(double2));
     o_tw32[r] = reserve(ntw * sizeof(float2));
-    o_twq[r] = prec != FRLAP_F32 ? reserve(ntw * sizeof(int4)) : 0;
+    o_twq[r] = prec != FRLAP_F32 ? reserve((size_t)twq_entries(p->P[r]) * sizeof(int4)) : 0;
   }
   unsigned char* scratch = nullptr;
   auto cleanup = [&](frlap_status code, const std::string& msg) {
@@ -278,13 +278,12 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   p->lamL64 = reinterpret_cast<double*>(t + o_lamL64);
   if (prec != FRLAP_F64) p->lam32 = reinterpret_cast<float*>(t + o_lam32);
   for (int r = 0; r < d; ++r) {
-    const size_t ntw = (size_t)twiddle_entries(p->P[r]);
     p->tw64[r] = reinterpret_cast<double2*>(t + o_tw64[r]);
     p->tw32[r] = reinterpret_cast<float2*>(t + o_tw32[r]);
     cudaError_t e = twiddle_launch(p->P[r], p->tw64[r], p->tw32[r], s);
     if (e == cudaSuccess && prec != FRLAP_F32) {
       p->twq[r] = reinterpret_cast<int4*>(t + o_twq[r]);
-      e = to_q_launch(p->tw64[r], p->twq[r], ntw, s);
+      e = to_q_launch(p->tw64[r], p->twq[r], p->P[r], s);
     }
     if (e != cudaSuccess) return cleanup(FRLAP_ECUDA, std::string("twiddles: ") + cudaGetErrorString(e));
   }

@@ -37,7 +37,7 @@ namespace {
 // Spectrum columns of the learned preconditioner: columns of n entries -> zero-pad to P, forward FFT, all P
 // outputs in FP64 (stride ldo).
 template <int REM, int LOGP, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_col_fwd(const cq* __restrict__ in, const int* __restrict__ ex, double2* __restrict__ out, int ncols, int n,
                 size_t ld, size_t ldo, int logP, int TL, int cols_per, const int4* __restrict__ tw,
                 const int* __restrict__ skip, Batch bt, size_t ex_inst) {
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(512, 1)
 
 // Columns of P FP64 spectrum values times a multiplier (natural octant order) -> inverse FFT, crop to n.
 template <int REM, int LOGP, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_col_mulinv(const double2* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int ncols, int n,
                    size_t ld, size_t ldo, int logP, int TL, const double* __restrict__ lam, LamMap map,
                    const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(512, 1)
   for (int m = 0; m < E; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
   int e = qs.e;
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  q_store_scale<REM, E, E / 2>(v, e);
+  q_store_scale<REM, E, LOGP, E / 2>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex + col, e);
   store_line<E>(v, out, ncols, n, ldo, logP, TL);
 }

@@ -431,7 +431,7 @@ __device__ __forceinline__ void store_line(const C* v, C* __restrict__ data, int
                                            int TL) {
   unsigned tid;
   asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
-  constexpr int LE = E == 4 ? 2 : 4;
+  constexpr int LE = E == 4 ? 2 : E == 8 ? 3 : 4;
   const int G = 1 << (logP - LE);
   const int lane = (int)tid & (G - 1);
   const int col = (int)blockIdx.x * TL + ((int)tid >> (logP - LE));

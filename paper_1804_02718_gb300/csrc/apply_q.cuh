@@ -38,9 +38,9 @@ inline QExpLayout q_exp_layout(const Plan& p) {
 }
 
 // A transform's output v[0..N) to what is stored, components below 2^58, and its exponent.
-template <int REM, int E, int N>
+template <int REM, int E, int LOGL, int N>
 __device__ __forceinline__ void q_store_scale(cq* v, int& e) {
-  constexpr int SH = 5 - kQDrop<REM, E>;
+  constexpr int SH = 5 - kQDrop<REM, E, LOGL>;
 #pragma unroll
   for (int m = 0; m < N; ++m) v[m] = q_shr_even<SH>(v[m]);
   e += SH;
@@ -68,7 +68,7 @@ __device__ __forceinline__ cq q_align(cq v, int e, int top, bool up) {
   cq* smem = reinterpret_cast<cq*>(smem_raw);
 
 template <bool DYN, int REM, int LOGL, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_r2c(const double* __restrict__ in, cq* __restrict__ out, int* __restrict__ ex, int nlines, int n, size_t ldo,
             int logH, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
   logH = LOGL;
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(512, 1)
   // D = kQDrop (0 after q_fill).  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of
   // the downward shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in
   // a + b.
-  constexpr int D = DYN ? kQDrop<REM, E> : 0;
+  constexpr int D = DYN ? kQDrop<REM, E, LOGL> : 0;
   auto split = [&](int k, const int4 wk) {
     const int km = H - k;
     const cq a = buf[spad(k)];
@@ -245,7 +245,7 @@ __device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict
 
 // A column's entries of one line: element i of instance-local column col at data[col ld + i].
 template <int REM, int LOGP, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_colmul(cq* __restrict__ data, const int* __restrict__ ex_in, int* __restrict__ ex_out, int ncols, int n,
                size_t ld, int logP, int TL, const double* __restrict__ lam, LamMap map, int nz,
                const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt, size_t ex_inst) {
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(512, 1)
   q_symbol<E>(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, lg, slots + si);
   ++si;
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  q_store_scale<REM, E, E / 2>(v, e);
+  q_store_scale<REM, E, LOGP, E / 2>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex_out + col, e);
   store_line<E>(v, data, ncols, n, ld, logP, TL);
 }
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(512, 1)
 
 // groups of contiguous lines of length n -> pad, FFT, transposed store out[g][k][line]
 template <int REM, int LOGL, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_c2cT_fwd(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
                  int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
                  int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(512, 1)
                             lg, slots + si);
   ++si;
   q_fft<true, -1, true, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  q_store_scale<REM, E, E>(v, e);
+  q_store_scale<REM, E, LOGL, E>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
   line_sync<double>(lg);
 #pragma unroll
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(512, 1)
 
 // transposed in[g][k][line] (k < P) -> IFFT along k, crop to n, store out[g][line][i]
 template <int REM, int LOGL, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_c2cT_inv(const cq* __restrict__ in, cq* __restrict__ out, const int* __restrict__ ex_in,
                  int* __restrict__ ex_out, int nlines, int tiles, int n, size_t gin, int ldi, size_t gout, int ldo,
                  int logP, int TL, const int4* __restrict__ tw, const int* __restrict__ skip, Batch bt,
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
   for (int m = 0; m < E; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  q_store_scale<REM, E, E / 2>(v, e);
+  q_store_scale<REM, E, LOGL, E / 2>(v, e);
   if (line < nlines) {
     if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
     cq* dst = out + g * gout + (size_t)line * ldo;
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(512, 1)
 
 // Last stage.  Bin k of row r has exponent ex[k ex_k + (r / rows_per) ].
 template <int REM, int LOGL, int E>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(kQCta<E>, 1)
     k_q_c2r(const cq* __restrict__ in, double* __restrict__ out, const int* __restrict__ ex, int ex_k, int rows_per,
             int nlines, int n, size_t ldi, int logH, int TL, const int4* __restrict__ tw,
             const int* __restrict__ skip, Batch bt, size_t ex_inst) {
@@ -587,20 +587,30 @@ static cudaError_t q_launch(K kern, unsigned grid, int B, int threads, size_t sm
 struct QShape {
   int tl, threads, tiles;
   size_t sm;
-  bool thin;  // four entries a thread (q_fft4)
+  int e;  // entries a thread
 };
-// Four entries a thread where, at sixteen, a vector's lines leave seven eighths of the chip's 608 sub-partitions
-// without a warp.  The line depends on the plan alone, so that a batch equals its vectors' applies bit for bit; a
-// batch of 8 then still has at most a warp per sub-partition.  One F64 vector, us per stage (with its launch),
-// sixteen -> four: 32^2 12.2, 10.8, 10.2 -> 9.6, 7.9, 7.2 (r2c, colmul, c2r), 128^2 13.1, 11.9, 10.2 -> 10.6, 8.9,
-// 8.2; 8 x 128^2 4.7 -> 4.1 a vector.  In larger launches the extra stages and barriers cost more: 8 x 256^2 7.1
-// -> 8.9 a vector.
-constexpr long long kQThinThreads = 152 * 16;
-static QShape q_shape(int tuned, int L, long long lines, int B, int lines_per_group, bool may_thin = true) {
+// Entries a thread.  Sixteen (the fewest stages, exchanges and barriers) for launches that fill the chip.  Fewer
+// where, at sixteen, a vector's lines leave most of the 608 sub-partitions without a warp: then a thread's chain of
+// instructions is the time.  The lines depend on the plan alone, so that a batch equals its vectors' applies bit for
+// bit; a batch of 8 at the first line still has at most a warp per sub-partition.  One F64 vector, us per stage (with
+// its launch; r2c, colmul, c2r), sixteen -> four: 32^2 12.2, 10.8, 10.2 -> 9.6, 7.9, 7.2, 128^2 13.1, 11.9, 10.2 ->
+// 10.6, 8.9, 8.2; 8 x 128^2 4.7 -> 4.1 a vector.  Sixteen -> eight: 256^2 14.2, 14.9, 11.6 -> 11.7, 11.3, 10.2; above
+// the second line the further stage costs more: 512^2 colmul 17.0 -> 19.3, 8 x 255^2 3.2 -> 3.4
+// a vector, 8 x 2048^2 165 -> 206 a vector.  Rows of at most
+// 128 points are bound by their loads and conversions: with eight entries and twice the warps 128^3 r2c 36.9 -> 33.0,
+// c2r 32.7 -> 28.7.
+constexpr long long kQThin4 = 152 * 16, kQThin8 = 152 * 64;
+enum class QKind { Line, Row, Split };
+static QShape q_shape(int tuned, int L, long long lines, int B, int lines_per_group, QKind k = QKind::Line) {
   QShape q;
-  q.thin = may_thin && L <= (1 << kQThinLog) && lines * (L >> 4) <= kQThinThreads;
-  const int G = q.thin ? L >> 2 : L >> 4;
-  q.tl = pick_tl_tuned(q.thin ? 0 : tuned, sline(L), 16, G, 96 * 1024, lines * B);
+  const long long t16 = lines * (L >> 4);
+  q.e = k == QKind::Split || L > (1 << kQThinLog) ? 16
+        : t16 <= kQThin4                          ? 4
+        : t16 <= kQThin8 || (k == QKind::Row && L <= 128) ? 8
+                                                          : 16;
+  const int G = L / q.e;
+  q.tl = pick_tl_tuned(q.e == 4 ? 0 : tuned, sline(L), 16, G, 96 * 1024, lines * B);
+  while (q.tl > 1 && q.tl * G > 512) q.tl /= 2;  // (a tuned choice is one for sixteen entries)
   q.threads = q.tl * G;
   q.tiles = (lines_per_group + q.tl - 1) / q.tl;
   q.sm = (size_t)q.tl * sline(L) * 16;
@@ -617,7 +627,8 @@ static cudaError_t q_with_shape(const QShape& q, int logL, F&& f) {
   return with_line_shape(logL, [&](auto tag) {
     constexpr int R = decltype(tag)::rem, L = decltype(tag)::logp;
     if constexpr (L <= kQThinLog) {
-      if (q.thin) return f(QTag<R, L, 4>{});
+      if (q.e == 4) return f(QTag<R, L, 4>{});
+      if (q.e == 8) return f(QTag<R, L, 8>{});
     }
     return f(QTag<R, L, 16>{});
   });
@@ -637,7 +648,7 @@ static LamMap q_lam_map(const Plan& p) {
 #ifdef FRLAP_BOUNDS_CHECK
 static cudaError_t q_register(const Plan& p, BcRanges r, void* work, int B, cudaStream_t s) {
   r.add(work, (size_t)B * apply_work_bytes(p, 8));
-  for (int a = 0; a < p.d; ++a) r.add(p.twq[a], (size_t)twiddle_entries(p.P[a]) * sizeof(int4));
+  for (int a = 0; a < p.d; ++a) r.add(p.twq[a], (size_t)twq_entries(p.P[a]) * sizeof(int4));
   return r.commit(s);
 }
 #endif
@@ -647,7 +658,7 @@ template <bool DYN>
 static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const double* u, size_t ustride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
   const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
-  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows);
+  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows, QKind::Row);
   Batch b;
   b.in = ustride;
   b.out = w.stride;
@@ -689,7 +700,7 @@ static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tune
 static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, size_t ystride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
   const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
-  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows);
+  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows, QKind::Row);
   Batch b;
   b.in = w.stride;
   b.out = ystride;
@@ -741,7 +752,7 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, s
   if ((e = q_stage_r2c<DYN>(p, w, B, u, vstride, tuned[0], skip, skip_stride, s)) != cudaSuccess) return e;
   if ((e = mark()) != cudaSuccess) return e;
   if (p.d == 2 && p.P[1] > kMaxLine) {
-    const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1, B, Hx1, false);
+    const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1, B, Hx1, QKind::Split);
     int* ex_tmp = w.col + Hx1;
     e = q_launch(k_q_colmul_split<false>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col, ex_tmp,
                  Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);

@@ -572,17 +572,18 @@ __device__ __forceinline__ int2 q60(double x) {
   const int l = (int)v;
   return make_int2((int)((v - (long long)l) >> 32), l);
 }
-__global__ void k_to_q(const double2* __restrict__ src, int4* dst, size_t n) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int2 a = q60(src[i].x), b = q60(src[i].y);
+__global__ void k_to_q(const double2* __restrict__ src, int4* dst, int P) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, n = twiddle_entries(P);
+  if (i >= twq_entries(P)) return;
+  const double2 w = src[i < n ? i : ((i - n) / (P / 8) + 1) * ((i - n) % (P / 8))];
+  const int2 a = q60(w.x), b = q60(w.y);
   dst[i] = make_int4(a.x, a.y, b.x, b.y);
 }
 }  // namespace
 
-// fixed-point copy of a complex table (twiddles), n values, in the layout of Plan::twq
-cudaError_t to_q_launch(const double2* src, int4* dst, size_t n, cudaStream_t st) {
-  k_to_q<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(src, dst, n);
+// the fixed-point table of embedding size P from its FP64 one, in the layout of Plan::twq
+cudaError_t to_q_launch(const double2* src, int4* dst, int P, cudaStream_t st) {
+  k_to_q<<<(twq_entries(P) + 255) / 256, 256, 0, st>>>(src, dst, P);
   return cudaGetLastError();
 }
 

@@ -291,14 +291,17 @@ cudaError_t generator_octant_launch(const Plan& p, const double* coef, double* l
 // P + 15 (Ns - 1) + (r - 1) Ns + k, so a warp's 32 consecutive k of one r are 32 consecutive
 // entries (one load over a few cache lines instead of one line per lane).  The stage entries
 // are copies of plain entries (W_{16 Ns}^{r k} = W_P^{r k P / (16 Ns)}), so both give the same bits.
-inline int twiddle_entries(int P) { return P + 15 * (P / 8 - 1); }
+__host__ __device__ inline int twiddle_entries(int P) { return P + 15 * (P / 8 - 1); }
+// Entries of a fixed-point table: those, then W_P^{r k}, r = 1..7, k < P/8, at (r - 1) P/8 + k (the last stage of
+// radix 8 of a P-point line; its others read the radix-16 entries).
+__host__ __device__ inline int twq_entries(int P) { return twiddle_entries(P) + 7 * (P / 8); }
 // fills tw64 and tw32 (twiddle_entries(P) entries each; tw32 may be null)
 cudaError_t twiddle_launch(int P, double2* tw64, float2* tw32, cudaStream_t s);
 cudaError_t scale_symbol_launch(double* lam64, float* lam32, size_t n, double s, cudaStream_t st);
 // dst (line-major, converted to To) = s * oct (natural order); To = double or float
 template <typename To>
 cudaError_t line_symbol_launch(const Plan& p, const double* oct, To* dst, double s, cudaStream_t st);
-cudaError_t to_q_launch(const double2* src, int4* dst, size_t n, cudaStream_t st);
+cudaError_t to_q_launch(const double2* src, int4* dst, int P, cudaStream_t st);
 // even DFT of the octant along every axis (used for both the operator and preconditioner symbols)
 cudaError_t symbol_axes_launch(const Plan& p, double* lam_oct, cudaStream_t s);
 

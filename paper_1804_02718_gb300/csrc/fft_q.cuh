@@ -343,86 +343,127 @@ __device__ __forceinline__ void q_last_stage(cq* v, int lane, int G, const int4*
 
 // Bits that a line's transform of log2 length = REM mod 4 ends below 2^62.5: a last stage of radix 2 or 4
 // grows by that, but its products divide by 16.
-template <int REM, int E = 16>
-constexpr int kQDrop = E == 4 ? ((REM & 1) ? 3 : 2) : REM == 1 ? 3 : REM == 2 ? 2 : 0;
+template <int REM, int E = 16, int LOGL = 0>
+constexpr int kQDrop = E == 4 ? ((REM & 1) ? 3 : 2) : E == 8 ? (LOGL % 3 == 0 ? 1 : LOGL % 3 == 1 ? 3 : 2)
+                                                    : REM == 1 ? 3 : REM == 2 ? 2 : 0;
 
-// Transforms with four entries a thread, for launches of few lines: every thread of a sixteen-entry line issues
-// some 1500 instructions a stage, and with less than a warp per SM sub-partition their latency is the time.
-// Four entries take radix-4 stages: a quarter of the entries and a fifth of the instructions a stage, twice the
-// stages, four times the threads.  Lines of at most 2^kQThinLog points; v[m] = x[lane + m L/4] on entry and
-// X[lane + m L/4] on exit, scaled as in q_fft (magnitudes below 2^(62.5 - kQDrop<REM, 4>)).  With DYN = false
-// the line is shifted by the stage's growth, 2, instead.
+// Transforms with E = 4 or 8 entries a thread, in stages of radix E (a last one of 2 or 4 for the rest).
+// For launches of few lines: every thread of a sixteen-entry line issues some 1500 instructions a stage, and with
+// less than a warp per SM sub-partition their latency is the time.  E = 4 has a quarter of the entries and a fifth
+// of the instructions a stage, twice the stages and four times the threads; E = 8 lies between.  Lines of at most
+// 2^kQThinLog points.
+// v[m] = x[lane + m L/E] on entry and X[lane + m L/E] on exit, scaled as in q_fft (magnitudes below
+// 2^(62.5 - kQDrop<REM, E, LOGL>)).  With DYN = false the line is shifted by what its stage leaves free instead.
 constexpr int kQThinLog = 10;
+template <int E>
+constexpr int kQCta = E == 8 ? 1024 : 512;  // threads per CTA the kernels are compiled for
+template <int E>
+constexpr int kQLogE = E == 4 ? 2 : E == 8 ? 3 : 4;
 // What stands for log2 of the line length where that tells the threads of a line (line_sync, q_reduce).
 template <int E>
 __host__ __device__ constexpr int q_lg(int logL) {
-  return E == 4 ? logL + 2 : logL;
+  return logL + 4 - kQLogE<E>;
 }
-template <bool DYN, int SIGN, bool ZIN>
-__device__ __forceinline__ void q_fft4(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
-                                       int logPtab, bool sync_first, unsigned* slots, int& si) {
-  const int G = 1 << (logL - 2), lg = q_lg<4>(logL);
-  if constexpr (ZIN) v[2] = v[3] = {0, 0};
-  q_dft4<SIGN>(v[0], v[1], v[2], v[3]);
+template <int E, bool DYN, int SIGN, bool ZIN>
+__device__ __forceinline__ void q_fft_e(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
+                                        int logPtab, bool sync_first, unsigned* slots, int& si) {
+  constexpr int LE = kQLogE<E>;
+  const int G = 1 << (logL - LE), lg = q_lg<E>(logL);
+  if constexpr (ZIN) {
+#pragma unroll
+    for (int m = E / 2; m < E; ++m) v[m] = {0, 0};
+  }
+  q_dftR<E, SIGN>(v);
   int logNs = 0;  // of the stage whose results v holds
   while (true) {
-    const int nextNs = logNs + 2;
-    // the next stage's twiddles, in flight over the exchange
-    const bool last2 = nextNs + 1 == logL;
+    const int next = logNs + LE;
+    // E = 4: the next stage's twiddles are in flight over the exchange (E = 8 has no registers for them)
     int4 w[3];
-    if (last2) {
+    if constexpr (E == 4) {
+      if (next + 1 == logL) {
 #pragma unroll
-      for (int b = 0; b < 2; ++b) w[b] = q_ld_tw(tw + ((lane + b * G) << (logPtab - logL)));
-    } else {
-      const int k = lane & ((1 << nextNs) - 1);
+        for (int b = 0; b < 2; ++b) w[b] = q_ld_tw(tw + ((lane + b * G) << (logPtab - logL)));
+      } else {
+        const int k = lane & ((1 << next) - 1);
 #pragma unroll
-      for (int r = 1; r < 4; ++r) w[r - 1] = q_ld_tw(tw + ((r * k) << (logPtab - nextNs - 2)));
+        for (int r = 1; r < 4; ++r) w[r - 1] = q_ld_tw(tw + ((r * k) << (logPtab - next - 2)));
+      }
     }
     unsigned o = 0u;
     if (DYN) {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) o |= q_bits(v[m]);
+      for (int m = 0; m < E; ++m) o |= q_bits(v[m]);
       o = q_publish<false>(o, lg, slots + si);
     }
     if (logNs > 0 || sync_first) line_sync<double>(lg);
-    const int Ns = 1 << logNs, kw = lane & (Ns - 1), ob = (lane - kw) * 4 + kw;
+    const int Ns = 1 << logNs, kw = lane & (Ns - 1), ob = (lane - kw) * E + kw;
+    const bool ns16 = (Ns & 15) == 0;
+    const int obase = spad(ob), sstep = Ns + (Ns >> 4);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) buf[spad(ob + r * Ns)] = v[r];
+    for (int r = 0; r < E; ++r) buf[ns16 ? obase + r * sstep : spad(ob + r * Ns)] = v[r];
     line_sync<double>(lg);
+    const bool g16 = (G & 15) == 0;
+    const int rbase = spad(lane), rstep = G + (G >> 4);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) v[m] = buf[spad(lane + m * G)];
-    const int sh = DYN ? q_fill_shift(q_fetch(o, lg, slots + si)) : 2;
+    for (int m = 0; m < E; ++m) v[m] = buf[g16 ? rbase + m * rstep : spad(lane + m * G)];
+    const int sh = DYN ? q_fill_shift(q_fetch(o, lg, slots + si)) : 4 - LE;
     if (DYN) ++si;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) v[m] = {q_shl(v[m].x, sh), q_shl(v[m].y, sh)};
+    for (int m = 0; m < E; ++m) v[m] = {q_shl(v[m].x, sh), q_shl(v[m].y, sh)};
     e += 4 - sh;
-    logNs = nextNs;
-    if (last2) {
+    logNs = next;
+    if (logNs + 1 == logL) {  // radix 2
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const cq s = q_shr_round<4>(v[b]), t = q_cmul<(SIGN > 0)>(v[b + 2], w[b]);
+      for (int b = 0; b < E / 2; ++b) {
+        const int4 wb = E == 4 ? w[b & 1] : q_ld_tw(tw + ((lane + b * G) << (logPtab - logL)));
+        const cq s = q_shr_round<4>(v[b]), t = q_cmul<(SIGN > 0)>(v[b + E / 2], wb);
         v[b] = s + t;
-        v[b + 2] = s - t;
+        v[b + E / 2] = s - t;
       }
       return;
     }
-    v[0] = q_shr_round<4>(v[0]);
+    if constexpr (E == 8) {
+      if (logNs + 2 == logL) {  // radix 4
 #pragma unroll
-    for (int r = 1; r < 4; ++r) v[r] = q_cmul<(SIGN > 0)>(v[r], w[r - 1]);
-    q_dft4<SIGN>(v[0], v[1], v[2], v[3]);
-    if (logNs + 2 == logL) return;
+        for (int b = 0; b < 2; ++b) {
+          const int j = lane + b * G;
+          v[b] = q_shr_round<4>(v[b]);
+#pragma unroll
+          for (int r = 1; r < 4; ++r)
+            v[b + 2 * r] = q_cmul<(SIGN > 0)>(v[b + 2 * r], q_ld_tw(tw + ((r * j) << (logPtab - logL))));
+          q_dft4<SIGN>(v[b], v[b + 2], v[b + 4], v[b + 6]);
+        }
+        return;
+      }
+    }
+    v[0] = q_shr_round<4>(v[0]);
+    if constexpr (E == 4) {
+#pragma unroll
+      for (int r = 1; r < 4; ++r) v[r] = q_cmul<(SIGN > 0)>(v[r], w[r - 1]);
+    } else {
+      // W_{8 Ns}^{r k} = W_{16 Ns}^{2 r k}, in the table's radix-16 stage entries, or in its last part
+      const int k = lane & ((1 << logNs) - 1);
+      const bool st16 = logNs + 4 <= logPtab;
+      const int4* st = st16 ? tw + (1 << logPtab) + 15 * ((1 << logNs) - 1) - (1 << logNs) + k
+                            : tw + twiddle_entries(1 << logPtab) - (1 << logNs) + k;
+      const int step = st16 ? 2 << logNs : 1 << logNs;
+#pragma unroll
+      for (int r = 1; r < 8; ++r) v[r] = q_cmul<(SIGN > 0)>(v[r], q_ld_tw(st + r * step));
+    }
+    q_dftR<E, SIGN>(v);
+    if (logNs + LE == logL) return;
   }
 }
 
 // As fft_regs: v[m] = x[lane + m G] on entry (components below 2^58), X[lane + m G] on exit (magnitudes
 // below 2^(62.5 - kQDrop)); e, the line's exponent, follows.  DYN: the scale follows the data between stages;
 // else it stays as set on entry (lines with three twiddled stages excepted).  ZIN: v[8..15] are zero.  slots:
-// the line's reduction words, used from index si on.  E = 4: see q_fft4.
+// the line's reduction words, used from index si on.  E < 16: see q_fft_e.
 template <bool DYN, int SIGN, bool ZIN, int REM, int E = 16>
 __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
                                       int logPtab, bool sync_first, unsigned* slots, int& si) {
-  if constexpr (E == 4) {
-    q_fft4<DYN, SIGN, ZIN>(v, e, buf, logL, lane, tw, logPtab, sync_first, slots, si);
+  if constexpr (E < 16) {
+    q_fft_e<E, DYN, SIGN, ZIN>(v, e, buf, logL, lane, tw, logPtab, sync_first, slots, si);
     return;
   } else {
   const int G = 1 << (logL - 4);

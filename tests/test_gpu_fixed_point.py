@@ -141,11 +141,11 @@ def test_df64_first_stage_entries(frlap, Ns):
 @pytest.mark.parametrize("prec,bound", [("f64", 2.0 ** -49), ("df64", 2.0 ** -48)])
 @pytest.mark.parametrize("Ns", [(16, 52, 52), (32, 52, 52), (64, 40, 40), (128, 40, 40), (256, 300), (64, 609),
                                 (64, 610), (40, 16, 40), (40, 40, 16), (16, 40, 130), (9, 600), (100, 512),
-                                (30, 512)])
-def test_lines_on_both_sides_of_four_and_sixteen_entries_a_thread(frlap, Ns, prec, bound):
-    """Plans of few lines give a thread four entries, others sixteen (2432 threads at sixteen, the edge: 608 and
-    609 rows of 64 points): against the defining sum at the bounds above, and a batch of 9 bit for bit its vectors'
-    applies."""
+                                (30, 512), (100, 200), (250, 250), (12, 40, 40)])
+def test_four_eight_and_sixteen_entries_a_thread(frlap, Ns, prec, bound):
+    """Plans of few lines give a thread four or eight entries, others sixteen (the first edge, 2432 threads at
+    sixteen: 608 and 609 rows of 64 points): against the defining sum at the bounds above, and a batch of 9 bit for
+    bit its vectors' applies."""
     import torch
 
     plan, coef, c, lam_max = _operator(frlap, Ns, 1.3, getattr(frlap, "FRLAP_" + prec.upper()))
