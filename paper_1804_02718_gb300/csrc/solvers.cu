@@ -10,6 +10,7 @@
 // between chunks.  Inner products are accumulated in FP64 with a fixed
 // reduction order (per-block partials, then the last block to finish sums them
 // in block order), so results are deterministic.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <type_traits>
@@ -20,13 +21,16 @@
 
 namespace frlap {
 
+namespace cg = cooperative_groups;
+
 namespace {
 
 constexpr int kBlocks = 2 * 152;  // largest grid of the vector kernels: two CTAs per SM (four measured slower)
 constexpr int kThreads = 512;
 // CTA size and grid for n elements (the reductions use gridDim.x).  A CTA's FP64 tree costs each of its warps
 // five additions at 76 cycles, so a short vector takes CTAs of 128 threads, one warp per SM sub-partition,
-// with up to four elements a thread: 127^2 k_cg_update 9.2 -> 6.1 us, k_cg_pq 7.2 -> 4.8 us.
+// with up to four elements a thread: 127^2 k_cg_update 9.2 -> 6.1 us, k_cg_pq 7.2 -> 4.8 us (CG on vectors that
+// short now runs k_cg_small; initial residuals and k_resid take these sizes).
 inline unsigned vthreads(size_t n) { return n <= (size_t)kBlocks * 128 * 4 ? 128u : (unsigned)kThreads; }
 inline unsigned vgrid(size_t n) {
   const size_t t = vthreads(n), b = (n + t - 1) / t;
@@ -366,6 +370,134 @@ __global__ void k_cg_dir(const TZ* __restrict__ z, T* p, size_t n, CgState* S, L
   }
 }
 
+// The vector part of an iteration in one kernel, for short vectors: k_cg_pq, k_cg_update and, without a
+// preconditioner, k_cg_dir.  Those three take 13 us at 127^2, nearly all of it launches, loads and the two passes
+// through memory that make each sum known to all blocks (partials, fence, ticket).  One cluster of 16 CTAs holds
+// the vectors' entries in registers (at most 8 a thread) and exchanges its sums over distributed shared memory:
+// plain CG iteration at 127^2 28.9 -> 25.1 us, at 181^2 37.4 -> 32.2, 23^3 39.7 -> 35.7.  More entries would wait
+// for 16 SMs' FP64 pipes instead.
+constexpr int kSmallCtas = 16, kSmallThreads = 256, kSmallE = 8;
+constexpr size_t kSmallMax = (size_t)kSmallCtas * kSmallThreads * kSmallE;
+
+// Sum of v over the cluster, in thread 0 of every CTA (others: unspecified), in a fixed order.  slot: 16 doubles
+// of shared memory, used once per launch; red: block_sum's.
+__device__ __forceinline__ double cluster_sum(double v, double* red, double* slot, cg::cluster_group& cl) {
+  const double t = block_sum(v, red);
+  if (threadIdx.x < 32) {
+    const double s = __shfl_sync(0xffffffffu, t, 0);
+    if (threadIdx.x < kSmallCtas) *cl.map_shared_rank(slot + cl.block_rank(), threadIdx.x) = s;
+  }
+  cl.sync();
+  double w = 0.0;
+  if (threadIdx.x < 32) {
+    w = threadIdx.x < kSmallCtas ? slot[threadIdx.x] : 0.0;
+    for (int o = kSmallCtas / 2; o > 0; o >>= 1) w += __shfl_down_sync(0xffffffffu, w, o);
+  }
+  return w;
+}
+
+template <typename T>
+__global__ void __cluster_dims__(kSmallCtas) __launch_bounds__(kSmallThreads)
+    k_cg_small(T* __restrict__ x, T* __restrict__ r, T* __restrict__ p, T* __restrict__ q, int n, CgState* S,
+               int maxit, int precond, float* __restrict__ r32, LoopControl lc) {
+  using A = acc_t<T>;
+  __shared__ double red[32], slots[2 * kSmallCtas], bc[2];
+  __shared__ int ok;
+  if (S->done) {  // (set by an earlier kernel: the same for every CTA)
+    loop_control(S, lc);
+    return;
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+  const A sg = (A)S->sigma, sc = (A)S->s;
+  const bool plain = S->sigma == 0.0 && S->s == 1.0;
+  const double rz = S->rz;
+  const int i0 = blockIdx.x * kSmallThreads + threadIdx.x;
+  constexpr int kStep = kSmallCtas * kSmallThreads;
+  T pv[kSmallE], qv[kSmallE], xv[kSmallE], rv[kSmallE];
+#pragma unroll
+  for (int u = 0; u < kSmallE; ++u) {
+    const int i = i0 + u * kStep;
+    if (i < n) {
+      pv[u] = p[i];
+      qv[u] = q[i];
+      xv[u] = x[i];
+      rv[u] = r[i];
+    }
+  }
+  A a = 0;
+#pragma unroll
+  for (int u = 0; u < kSmallE; ++u) {
+    const int i = i0 + u * kStep;
+    if (i < n) {
+      if (!plain) {
+        qv[u] = (T)(sg * (A)pv[u] + sc * (A)qv[u]);
+        q[i] = qv[u];
+      }
+      a += (A)pv[u] * (A)qv[u];
+    }
+  }
+  const double pq = cluster_sum((double)a, red, slots, cl);
+  if (threadIdx.x == 0) {
+    ok = pq > 0.0 && isfinite(pq);
+    bc[0] = rz / pq;
+  }
+  __syncthreads();
+  if (!ok) {  // the same in every CTA
+    if (first) {
+      S->pq = pq;
+      S->status = isfinite(pq) ? FRLAP_EBREAKDOWN : FRLAP_ENAN;
+      S->done = 1;
+    }
+    loop_control(S, lc);
+    return;
+  }
+  const double alpha = bc[0];
+  const A al = (A)alpha;
+  a = 0;
+#pragma unroll
+  for (int u = 0; u < kSmallE; ++u) {
+    const int i = i0 + u * kStep;
+    if (i < n) {
+      x[i] = (T)((A)xv[u] + al * (A)pv[u]);
+      rv[u] = (T)((A)rv[u] - al * (A)qv[u]);
+      r[i] = rv[u];
+      if (r32) r32[i] = (float)rv[u];
+      a += (A)rv[u] * (A)rv[u];
+    }
+  }
+  const double rr = cluster_sum((double)a, red, slots + kSmallCtas, cl);
+  if (!precond) {
+    if (threadIdx.x == 0) bc[1] = rr / rz;
+    __syncthreads();
+    const A be = (A)bc[1];
+#pragma unroll
+    for (int u = 0; u < kSmallE; ++u) {
+      const int i = i0 + u * kStep;
+      if (i < n) p[i] = (T)((A)rv[u] + be * (A)pv[u]);
+    }
+  }
+  if (first) {
+    S->pq = pq;
+    S->alpha = alpha;
+    if (!precond) {
+      S->beta = bc[1];
+      S->rz = rr;
+    }
+    S->rr = rr;
+    S->iters += 1;
+    if (!isfinite(rr)) {
+      S->status = FRLAP_ENAN;
+      S->done = 1;
+    } else if (rr <= S->tol2) {
+      S->done = 1;
+    } else if (S->iters >= maxit) {
+      S->status = FRLAP_ENOCONV;
+      S->done = 1;
+    }
+  }
+  loop_control(S, lc);
+}
 
 __global__ void k_set_state(CgState* S, double sigma, double s) {
   S->sigma = sigma;
@@ -580,12 +712,20 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
   FRLAP_LAUNCH_CHECK("k_pcg_start");
   if (snap && nsnap > 0) FRLAP_CUDA_TRY(cudaMemcpyAsync(snap, x, n * sizeof(T), cudaMemcpyDeviceToDevice, st));
   const int* done = &S->done;
+  const bool small = n <= kSmallMax;
+  if (small)  // 16 CTAs a cluster are more than the portable 8
+    FRLAP_CUDA_TRY(cudaFuncSetAttribute(k_cg_small<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   // one iteration on stream `ss`; the snapshot copy (training pairs) needs the host's count
   auto iteration = [&](cudaStream_t ss, int it, LoopControl lc = LoopControl{}) -> cudaError_t {
     cudaError_t e = apply_T<T>(p, pv, q, b.awork, ss, done);
     if (e != cudaSuccess) return e;
-    k_cg_pq<T><<<vgrid(n), vthreads(n), 0, ss>>>(pv, q, n, b.partials, S);
-    k_cg_update<T><<<vgrid(n), vthreads(n), 0, ss>>>(x, r, pv, q, n, b.partials, S, maxit, mu != nullptr, r32);
+    if (small) {
+      k_cg_small<T><<<kSmallCtas, kSmallThreads, 0, ss>>>(x, r, pv, q, (int)n, S, maxit, mu != nullptr, r32,
+                                                          mu ? LoopControl{} : lc);
+    } else {
+      k_cg_pq<T><<<vgrid(n), vthreads(n), 0, ss>>>(pv, q, n, b.partials, S);
+      k_cg_update<T><<<vgrid(n), vthreads(n), 0, ss>>>(x, r, pv, q, n, b.partials, S, maxit, mu != nullptr, r32);
+    }
     if (snap && it + 1 < nsnap) {
       e = cudaMemcpyAsync(snap + (size_t)(it + 1) * n, x, n * sizeof(T), cudaMemcpyDeviceToDevice, ss);
       if (e != cudaSuccess) return e;
@@ -595,7 +735,7 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
       if (e != cudaSuccess) return e;
       k_pcg_beta<T, float><<<vgrid(n), vthreads(n), 0, ss>>>(r, b.z32, q, n, b.partials, S);
       k_cg_dir<T, float><<<vgrid(n), vthreads(n), 0, ss>>>(b.z32, pv, n, S, lc);
-    } else {
+    } else if (!small) {
       k_cg_dir<T, T><<<vgrid(n), vthreads(n), 0, ss>>>(r, pv, n, S, lc);
     }
     return cudaGetLastError();
