@@ -3,9 +3,9 @@
 
 Default workload: 2D, alpha = 1.5, Omega = (-1,1)^2, h = 2/2048 (2047 x 2047 interior
 unknowns), an FP64-precision apply y = A u through libfrlap (the 2D throughput case
-of the 3D FP64 CG configuration), computed by the double-float FFT engine
-(FP64 vectors; FFT stages in FP32 pairs, parity 1e-12 normwise against the FP64
-oracle, like native FP64).  One step = one batched apply (frlap_apply_batch, one
+of the 3D FP64 CG configuration), computed by the DF64 engine
+(FP64 vectors; FFT stages in 64-bit block fixed point, parity 1e-12 normwise against
+the FP64 oracle, as the F64 engine).  One step = one batched apply (frlap_apply_batch, one
 launch per stage) to 8 distinct seeded N(0,1) vectors (268 MB of inputs, more than
 the 129 MB L2).  Reported: apply
 unknowns/s over all ranks, the HBM roofline of the dominant kernel (pass-model bytes
@@ -13,7 +13,7 @@ over its measured duration, against the measured HBM copy rate), the same metric
 end to end through host buffers, and the CPU oracle timed on all host cores.  After
 the timed region: the metric's second half (time to a 1e-10 residual for plain FP64
 CG, Strang and learned PCG and FP32-inner refinement at 2047^2 and 255^3, each with
-its solution error against a tighter reference solve), native FP64, FP32 and 3D
+its solution error against a tighter reference solve), F64, FP32 and 3D
 applies, cuFFT as a comparison, and the radix-16 FFT stage on CUDA cores against its
 split-TF32 tensor-core form.  `--suite solvers` instead runs the solver configurations
 (time to 1e-10 for plain CG, refinement, Strang and learned preconditioning; the
@@ -46,7 +46,7 @@ BATCH = 8  # vectors per step of the 2D workload
 BATCH_2D = BATCH
 NGRID_3D, ALPHA_3D, BATCH_3D = 256, 1.0, 2
 # vectors per chunk of the host-buffer pipeline, per engine, as measured at 2047^2 (chunks of 1, 2, 4, 8;
-# three device slots; first and last chunk of one vector): double-float 11.2, 10.6, 9.0, 6.9 G unknowns/s;
+# three device slots; first and last chunk of one vector): DF64 11.2, 10.6, 9.0, 6.9 G unknowns/s;
 # FP32 24.2, 24.0, 22.0, 18.2 (the copies share about 215 GB/s of host link)
 E2E_CHUNK = {"df64": 1, "f64": 1, "f32": 2}
 METRIC = "apply unknowns/s & %HBM peak; PCG time to 1e-10 of FP64 sol vs plain FP64 CG"
@@ -66,8 +66,7 @@ def peaks():
 # kernel, engine): dram__bytes_read.sum + dram__bytes_write.sum from the ncu captures summarised in
 # profiles/apply_2d_2047_batch8.md and profiles/apply_3d_255_batch2.md; an entry is dropped when its
 # kernel changes after the capture
-MEASURED_TRAFFIC = {(2, "colmul", "df64"): 1285.1e6, (2, "colmul", "f32"): 588.4e6,
-                    (3, "colmul", "df64"): 2457.5e6, (3, "colmul", "f32"): 1219.4e6}
+MEASURED_TRAFFIC = {(2, "colmul", "f32"): 588.4e6, (3, "colmul", "f32"): 1219.4e6}
 
 
 def measure_fp32_fma_tflops(torch, tf32=False):
@@ -460,15 +459,13 @@ def main():
             "peak_source": f"{hbm_src} hbm_gbs (of measured)" if hbm_src == "measured" else "fallback 6800 GB/s",
             "bytes_per_launch": sb[dom] * BATCH}
     # the same kernel's pruned algorithmic flops against the measured FP32 FMA rate (cuBLAS SGEMM);
-    # for the double-float engine each counted flop is an FP64-class operation executed as a
-    # sequence of FP32 instructions
+    # for the FP64-class engines each counted flop is executed as a sequence of integer instructions
     fp32_peak = measure_fp32_fma_tflops(torch)
     fl_ach = sf[dom] / (stage_ms[dom] / 1e3) / 1e12
     roof["pruned_flops_vs_fp32_fma"] = {
         "flops_per_launch": sf[dom] * BATCH, "achieved_tflops": fl_ach, "fp32_fma_tflops_measured": fp32_peak,
         "frac": fl_ach / fp32_peak,
-        "note": "FP64-class flops executed as double-float FP32 sequences" if args.prec == "df64" else
-                ("native FP64 flops (FP64 pipe, about 1/62 of FP32)" if args.prec == "f64" else "FP32 flops")}
+        "note": "FP32 flops" if args.prec == "f32" else "FP64-class flops executed in 64-bit block fixed point"}
     roof["instances_per_launch"] = BATCH
     roof["launch_ms"] = stage_ms[dom] * BATCH
     apply_ms = sum(stage_ms)
@@ -523,7 +520,7 @@ def main():
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": {"df64": "f32x2"}.get(args.prec, args.prec),
+            "scaling": "weak", "vs_baseline": None, "dtype": "f32" if args.prec == "f32" else "f64 (64-bit block fixed point)",
             "data": "synthetic",
             "config": {"workload": f"{D}D {NG - 1}^{D} alpha={AL} {args.prec.upper()} FFT Toeplitz apply",
                        "batch_per_step": BATCH, "launch": "frlap_apply_batch (one launch per stage for the batch)",
@@ -642,7 +639,7 @@ def train_learned(fl, torch, learned):
 def run_pcg_rows(fl, torch, params_trained, d, N, alpha, seed=1):
     """The metric's second half: time to a true relative residual of 1e-10 on the fractional Poisson
     problem with a seeded Gaussian-sum f, for plain FP64 CG and the preconditioned / mixed-precision
-    variants; each row also gives its solution error against a tighter reference (native FP64,
+    variants; each row also gives its solution error against a tighter reference (F64,
     Strang-preconditioned CG to 1e-11, whose solution error is far below 1e-10 for this f)."""
     from paper_1804_02718_gb300 import learned
     h = 2.0 / N
@@ -667,7 +664,7 @@ def run_pcg_rows(fl, torch, params_trained, d, N, alpha, seed=1):
             ("ir_tau_fp32inner", MX, IR, TAU, None)]
     out = {"workload": f"{d}D {N - 1}^{d} alpha={alpha} Gaussian-sum f (seed {seed}), rtol 1e-10 (true residual)",
            "reference": {"iters": it_ref, "relres": rel_ref, "status": code_ref,
-                         "how": "native FP64 plan, Strang PCG to 1e-11"}}
+                         "how": "F64 plan, Strang PCG to 1e-11"}}
     for name, prec, solver, pre, which in rows:
         plan = fl.Plan(d, alpha, h, Ns, prec=prec)
         fl.frlap_plan_autotune(plan, 1)  # launch shapes (not part of the solve time)
@@ -750,7 +747,7 @@ def run_solver_suite(args):
 
     def solve_row(d, N, alpha, seed, variants):
         """Each variant to a true relative residual of 1e-10, timed (preconditioned ones after one
-        warm-up solve), with its solution error against a reference: native FP64, Strang PCG to 1e-11."""
+        warm-up solve), with its solution error against a reference: F64, Strang PCG to 1e-11."""
         h = 2.0 / N
         f = torch.from_numpy(inp.gaussian_sum_field((N,) * d, h, seed=seed)).cuda()
         ref_plan = fl.Plan(d, alpha, h, (N,) * d, prec=fl.FRLAP_F64)
