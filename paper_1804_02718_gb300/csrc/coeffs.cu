@@ -270,9 +270,26 @@ __global__ void k_pyramid(int d, double p, double alpha, int N, GaussRules g, do
 }
 
 // a_k for k != 0 (scaled by h^-alpha) and the block partial sums of 2^(d-sigma) a_k
+// a_0 is minus the sum of all others, so its rounding moves every eigenvalue alike: relative to the smallest, by up to
+// lambda_max / lambda_min units of it (1e-11 at 2047^2, alpha = 1.5, in a solution).  So the sum carries its error: an
+// unevaluated pair of doubles.
+__device__ __forceinline__ double2 add2(double2 a, double2 b) {
+  const double s = a.x + b.x, t = s - a.x;
+  return make_double2(s, ((a.x - (s - t)) + (b.x - t)) + (a.y + b.y));
+}
+// red[0] = the sum over the CTA's 256 threads, in a fixed order
+__device__ __forceinline__ void block_sum2(double2* red, double2 v) {
+  red[threadIdx.x] = v;
+  __syncthreads();
+  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+    if ((int)threadIdx.x < st) red[threadIdx.x] = add2(red[threadIdx.x], red[threadIdx.x + st]);
+    __syncthreads();
+  }
+}
+
 template <int D>
 __global__ void k_assemble(const double* __restrict__ w, int N, double gamma, double hscale,
-                           const double* __restrict__ pyr, double* coef, double* partial) {
+                           const double* __restrict__ pyr, double* coef, double2* partial) {
   const int N1 = N + 1;
   const size_t total = (D == 2) ? (size_t)N1 * N1 : (size_t)N1 * N1 * N1;
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -319,29 +336,22 @@ __global__ void k_assemble(const double* __restrict__ w, int N, double gamma, do
     }
   }
   // block reduction of the a_0 terms (h = 1 units)
-  __shared__ double red[256];
-  red[threadIdx.x] = contrib;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-    __syncthreads();
-  }
+  __shared__ double2 red[256];
+  block_sum2(red, make_double2(contrib, 0.0));
   if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
 // a_0 = -(sum of partials) - 2^d W_D2, scaled; one block, fixed summation order
-__global__ void k_diag(const double* __restrict__ partial, int nparts, int d, const double* __restrict__ pyr,
+__global__ void k_diag(const double2* __restrict__ partial, int nparts, int d, const double* __restrict__ pyr,
                        double hscale, double* coef) {
-  __shared__ double red[256];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) s += partial[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-    __syncthreads();
+  __shared__ double2 red[256];
+  double2 s = make_double2(0.0, 0.0);
+  for (int i = threadIdx.x; i < nparts; i += blockDim.x) s = add2(s, partial[i]);
+  block_sum2(red, s);
+  if (threadIdx.x == 0) {
+    s = add2(red[0], make_double2(ldexp(pyr[1], d), 0.0));
+    coef[0] = -(s.x + s.y) * hscale;
   }
-  if (threadIdx.x == 0) coef[0] = (-red[0] - ldexp(pyr[1], d)) * hscale;
 }
 
 // symbol octant initialisation: t_k = -c a_k for k_r <= n_r - 1, 0 elsewhere in [0, P_r/2]
@@ -458,7 +468,7 @@ size_t coeffs_scratch_bytes(int d, int Nmax) {
   const size_t N1 = (size_t)Nmax + 1;
   const size_t nco = (d == 2) ? N1 * N1 : N1 * N1 * N1;
   const size_t nparts = (nco + 255) / 256;
-  return align256(nel * 8) + align256(nparts * 8) + 256;
+  return align256(nel * 8) + align256(nparts * 16) + 256;
 }
 
 cudaError_t coeffs_launch(int d, double alpha, double gamma, double h, int N, double* coef, void* scratch,
@@ -470,8 +480,8 @@ cudaError_t coeffs_launch(int d, double alpha, double gamma, double h, int N, do
   const int nparts = (int)((nco + 255) / 256);
   double* w = reinterpret_cast<double*>(sp);
   sp += align256(nel * 8);
-  double* partial = reinterpret_cast<double*>(sp);
-  sp += align256((size_t)nparts * 8);
+  double2* partial = reinterpret_cast<double2*>(sp);
+  sp += align256((size_t)nparts * 16);
   double* pyr = reinterpret_cast<double*>(sp);
   const double p = d + alpha - gamma;
   const double hscale = pow(h, -alpha);

@@ -19,3 +19,21 @@ def test_coefficients_across_the_rules(frlap, d, N, alpha, gamma):
     a = frlap.frlap_coeffs(d, alpha, gamma, h, (N,) * d).cpu().numpy()
     ref = scheme.coefficients(d, alpha, h, N, gamma)
     assert np.max(np.abs(a - ref) / np.abs(ref)) < 1e-13
+
+
+def test_diagonal_is_the_rounded_sum(frlap):
+    """a_0 = -(sum of all others) - the far field, to one unit in the last place: at h = 2^-10 and alpha = 1.5 the
+    scale h^-alpha is a power of two, so the only roundings are the sum's (half a unit) and the far field's."""
+    import math
+
+    import numpy as np
+    from scipy.integrate import quad
+
+    N, alpha, h = 2048, 1.5, 2.0 ** -10
+    a = frlap.frlap_coeffs(2, alpha, 2.0, h, (N, N)).cpu().numpy()
+    m = np.where(np.arange(a.shape[0]) > 0, 2.0, 1.0)
+    terms = a * m[:, None] * m[None, :]
+    terms[0, 0] = 0.0
+    far = 4.0 * 2.0 * N ** -alpha / alpha * quad(lambda t: (1 + t * t) ** (-(2 + alpha) / 2), 0.0, 1.0)[0] * 2.0 ** 15
+    ref = -math.fsum(terms.ravel().tolist() + [far])
+    assert abs(float(a[0, 0]) - ref) <= 2.0 ** -52 * abs(ref)
