@@ -380,7 +380,8 @@ constexpr int kSmallCtas = 16, kSmallThreads = 256, kSmallE = 8;
 constexpr size_t kSmallMax = (size_t)kSmallCtas * kSmallThreads * kSmallE;
 
 // Sum of v over the cluster, in thread 0 of every CTA (others: unspecified), in a fixed order.  slot: 16 doubles
-// of shared memory, used once per launch; red: block_sum's.
+// of shared memory, used once per launch; red: block_sum's.  Stores into the other CTAs' shared memory: the caller
+// has passed a cluster barrier since the kernel's start (a CTA of the cluster may not have begun before that).
 __device__ __forceinline__ double cluster_sum(double v, double* red, double* slot, cg::cluster_group& cl) {
   const double t = block_sum(v, red);
   if (threadIdx.x < 32) {
@@ -408,6 +409,7 @@ __global__ void __cluster_dims__(kSmallCtas) __launch_bounds__(kSmallThreads)
     return;
   }
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();  // this CTA runs; the others' shared memory is touched after the wait below
   const bool first = blockIdx.x == 0 && threadIdx.x == 0;
   const A sg = (A)S->sigma, sc = (A)S->s;
   const bool plain = S->sigma == 0.0 && S->s == 1.0;
@@ -437,6 +439,7 @@ __global__ void __cluster_dims__(kSmallCtas) __launch_bounds__(kSmallThreads)
       a += (A)pv[u] * (A)qv[u];
     }
   }
+  cl.barrier_wait();  // every CTA of the cluster has begun (arrived long since, behind the loads)
   const double pq = cluster_sum((double)a, red, slots, cl);
   if (threadIdx.x == 0) {
     ok = pq > 0.0 && isfinite(pq);
