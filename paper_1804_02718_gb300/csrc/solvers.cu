@@ -683,6 +683,27 @@ static cudaError_t precondition(const Plan& p, const CgBufs& b, const float* mu,
   }
 }
 
+// Whether a cluster of k_cg_small can run at all where stream st runs: 16 CTAs are more than the portable 8 and need
+// that much room in one GPC, which a part of a GPU may not have.  (If not, the kernels for longer vectors run.)
+template <typename T>
+static bool cg_small_fits(cudaStream_t st) {
+  cudaLaunchAttribute dims;
+  dims.id = cudaLaunchAttributeClusterDimension;
+  dims.val.clusterDim.x = kSmallCtas;
+  dims.val.clusterDim.y = dims.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kSmallCtas);
+  cfg.blockDim = dim3(kSmallThreads);
+  cfg.stream = st;
+  cfg.attrs = &dims;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  cudaError_t e = cudaFuncSetAttribute(k_cg_small<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, k_cg_small<T>, &cfg);
+  if (e != cudaSuccess) cudaGetLastError();  // (not the caller's)
+  return e == cudaSuccess && clusters > 0;
+}
+
 // (Flexible) PCG on B x = f, B = sigma I + s A, in precision T; x holds x0 on entry.
 // mu = FP32 preconditioner symbol (octant) or nullptr for plain CG.
 template <typename T>
@@ -715,9 +736,7 @@ static frlap_status run_cg(const Plan& p, const T* f, T* x, double sigma, double
   FRLAP_LAUNCH_CHECK("k_pcg_start");
   if (snap && nsnap > 0) FRLAP_CUDA_TRY(cudaMemcpyAsync(snap, x, n * sizeof(T), cudaMemcpyDeviceToDevice, st));
   const int* done = &S->done;
-  const bool small = n <= kSmallMax;
-  if (small)  // 16 CTAs a cluster are more than the portable 8
-    FRLAP_CUDA_TRY(cudaFuncSetAttribute(k_cg_small<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  const bool small = n <= kSmallMax && cg_small_fits<T>(st);
   // one iteration on stream `ss`; the snapshot copy (training pairs) needs the host's count
   auto iteration = [&](cudaStream_t ss, int it, LoopControl lc = LoopControl{}) -> cudaError_t {
     cudaError_t e = apply_T<T>(p, pv, q, b.awork, ss, done);

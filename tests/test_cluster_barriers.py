@@ -49,6 +49,20 @@ def test_remote_stores_are_followed_by_a_cluster_barrier():
     assert body.index("map_shared_rank") < body.index("cl.sync(")
 
 
+def test_the_cluster_kernel_runs_only_where_a_cluster_fits():
+    """A cluster of 16 CTAs may not fit where a GPU is shared out; its launch would fail there.  The solver asks first
+    and otherwise takes the kernels that need no cluster (which tests/test_gpu_cg_small.py covers, just above the
+    limit on the length)."""
+    src = _source("solvers.cu")
+    fits = _body(src, "cg_small_fits")
+    assert "cudaOccupancyMaxActiveClusters(" in fits
+    run = _body(src, "run_cg")
+    flag = re.search(r"const bool small = ([^;]*);", run).group(1)
+    assert "cg_small_fits" in flag
+    assert run.index("if (small)") < run.index("k_cg_small<T><<<")  # its one launch, under that flag
+    assert src.count("k_cg_small<T><<<") == 1
+
+
 def test_no_other_kernel_reaches_a_peers_shared_memory():
     for name in sorted(os.listdir(CSRC)):
         if name != "solvers.cu":
