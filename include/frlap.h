@@ -193,7 +193,7 @@ frlap_status frlap_apply_host(const frlap_plan* plan, int nbatch, int chunk, con
 frlap_status frlap_apply_profiled(const frlap_plan* plan, const void* d_u, void* d_y, void* d_work, void* stream,
                                   void* const* events);
 
-/* Size of the device array behind frlap_apply_noalloc: 32 MiB. */
+/* Largest spectra that frlap_apply_noalloc takes: 32 MiB. */
 #define FRLAP_NOALLOC_MAX_BYTES (32u << 20)
 
 /* frlap_apply for callers that must not allocate device memory at call time:
@@ -201,11 +201,14 @@ frlap_status frlap_apply_profiled(const frlap_plan* plan, const void* d_u, void*
  * cudaMalloc, and latency-bound loops that cannot afford the device-wide
  * synchronisation a cudaMalloc/cudaFree implies.  The paper has no counterpart;
  * this is a library convenience.  Same product, arguments and result as
- * frlap_apply, but the scratch is a fixed library-owned device array of
- * FRLAP_NOALLOC_MAX_BYTES, reserved on every GPU that loads the library until
+ * frlap_apply, but the scratch is a fixed library-owned device array (40 MiB:
+ * FRLAP_NOALLOC_MAX_BYTES for spectra, 8 MiB for the FP64-class engines' line
+ * exponents), reserved on every GPU that loads the library until
  * the process exits.  The call allocates nothing.
- *  - Limit: plans whose frlap_workspace_bytes(plan, FRLAP_OP_APPLY) exceeds
- *    FRLAP_NOALLOC_MAX_BYTES are rejected with FRLAP_EINVAL and a message.
+ *  - Limit: plans whose spectra exceed FRLAP_NOALLOC_MAX_BYTES are rejected with
+ *    FRLAP_EINVAL and a message.  With P_r = max(32, power of two >= 2 n_r - 1) and
+ *    c = 16 bytes (F32: 8), each term rounded up to 256: 2D c (P_x/2 + 1) n_y,
+ *    twice that if P_y = 16384; 3D c (P_x/2 + 1) n_z n_y + c (P_x/2 + 1) P_y n_z.
  *    In interior unknowns per axis (n = N - 1) for square and cubic grids:
  *    2D FP64-class plans (F64, MIXED, DF64, MIXED_DF64) n <= 1024, 2D F32 n <= 2047,
  *    3D FP64-class n <= 64, 3D F32 n <= 93.

@@ -4,10 +4,13 @@
 
 namespace frlap {
 
-size_t apply_work_bytes(const Plan& p, int real_bytes) {
+size_t apply_spectra_bytes(const Plan& p, int real_bytes) {
   const size_t cb = 2 * (size_t)real_bytes;
-  size_t b = align256(p.s1_elems * cb);
-  b += align256(p.s2_elems * cb);
+  return align256(p.s1_elems * cb) + align256(p.s2_elems * cb);
+}
+
+size_t apply_work_bytes(const Plan& p, int real_bytes) {
+  size_t b = apply_spectra_bytes(p, real_bytes);
   if (real_bytes == 8) b += q_exp_layout(p).total * sizeof(int);  // the fixed-point engines' exponents
   return b;
 }

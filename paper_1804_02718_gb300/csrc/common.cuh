@@ -258,6 +258,7 @@ cudaError_t apply_launch(const Plan& p, const io_t<T>* u, io_t<T>* y, void* work
 cudaError_t apply64(const Plan& p, const double* u, double* y, void* work, cudaStream_t s, const int* skip,
                     cudaEvent_t const* ev = nullptr);
 size_t apply_work_bytes(const Plan& p, int real_bytes);
+size_t apply_spectra_bytes(const Plan& p, int real_bytes);  // S1 and S2 alone, without the line exponents
 // times every admissible lines-per-CTA choice of each apply stage on a batch of B zero vectors
 // (u, y: B vectors each; work: B apply workspaces) and stores the fastest in p.tl_tuned
 template <typename T>

@@ -18,7 +18,12 @@
 
 namespace {
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[FRLAP_NOALLOC_MAX_BYTES];
+// FRLAP_NOALLOC_MAX_BYTES for the spectra, and behind them the line exponents of the FP64-class engines
+// (QExpLayout), 4 bytes each.  Spectra take 16 bytes an entry.  In 2D there are at most 3 * 8193 exponents.  In 3D,
+// with H = P_x/2 + 1 in 17..1025, H n_z (n_y + P_y) <= 2^21 entries leave at most 2^21 / 17 rows n_y n_z, 2^21 / 33 lines
+// H n_z and, as P_y < 4 n_y beyond P_y = 32, 2^21 * 4 / 5 columns H P_y: 7.5 MB.
+constexpr size_t kNoallocBytes = (size_t)FRLAP_NOALLOC_MAX_BYTES + ((size_t)8 << 20);
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -32,8 +37,9 @@ extern "C" frlap_status frlap_apply_noalloc(const frlap_plan* plan, const void* 
   if (!plan || !d_u || !d_y) return fail(FRLAP_EINVAL, "plan, d_u or d_y is NULL");
   const bool f32 = plan->prec == FRLAP_F32;
   if (ranges_overlap(d_u, d_y, vector_bytes(*plan, f32))) return fail(FRLAP_EINVAL, "d_u and d_y must not overlap");
-  const size_t need = apply_work_bytes(*plan, f32 ? 4 : 8);
-  if (need > (size_t)FRLAP_NOALLOC_MAX_BYTES)
+  // the limit is on the spectra, so that it does not move with what an engine keeps beside them
+  const size_t need = apply_spectra_bytes(*plan, f32 ? 4 : 8);
+  if (need > (size_t)FRLAP_NOALLOC_MAX_BYTES || apply_work_bytes(*plan, f32 ? 4 : 8) > kNoallocBytes)
     return fail(FRLAP_EINVAL, "frlap_apply_noalloc: this grid needs " + std::to_string(need) +
                                   " bytes of scratch, more than the " + std::to_string((size_t)FRLAP_NOALLOC_MAX_BYTES) +
                                   "-byte static buffer; use frlap_apply with a caller workspace");
