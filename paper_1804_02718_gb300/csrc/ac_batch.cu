@@ -24,15 +24,14 @@ namespace frlap {
 
 namespace {
 
-constexpr int kAcMaxBlocks = 304;  // CTAs per instance of the vector kernels, at most
+constexpr int kAcMaxBlocks = 152;  // CTAs per instance of the vector kernels, at most
 constexpr int kAcThreads = 256;
-// CTAs per instance for a group of B instances of M unknowns: about four per SM over the group, each with at
-// least one pass of kU elements a thread (32 per instance whatever the group left four 1023^2 instances 8
-// warps per SM in flight).  With the groups as parallel branches and k_ac_next for two kernels, 12 instances
-// x 4 steps on 255^2, 511^2 and 1023^2: 20.0 -> 14.4 ms.
-inline int ac_blocks(size_t M, size_t B) {
-  const size_t want = (4 * 152 + B - 1) / B, most = (M + 4 * kAcThreads - 1) / (4 * kAcThreads);
-  const size_t b = want < most ? want : most;
+// CTAs per instance of M unknowns: one per SM, each with at least one pass of kU elements a thread.  A rule on M
+// alone: the sums' order, and so an instance's bits, must not depend on the others of its group.  DF64, 4 steps, ms:
+// 4 each of 255^2, 511^2 and 1023^2 18.2 (with 304: 18.4; with four per SM over the group: 18.2), 1023^2 alone 2.38
+// (2.40, 2.39), 8 x 1023^2 22.1 (22.5, 22.6), 32 x 255^2 4.96 (4.95, 4.97), 64 in turn 76.1 (78.6, 80.5).
+inline int ac_blocks(size_t M) {
+  const size_t b = (M + 4 * kAcThreads - 1) / (4 * kAcThreads);
   return (int)(b < 1 ? 1 : b > (size_t)kAcMaxBlocks ? (size_t)kAcMaxBlocks : b);
 }
 #ifdef FRLAP_BOUNDS_CHECK
@@ -549,7 +548,7 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
       const int B = (int)g.idx.size();
       const cudaStream_t gs = gi % (ns + 1) == 0 ? s : side[gi % (ns + 1) - 1];
       eb = batch_apply(p, B, g.p, g.q, g.vs, g.awork, gs, &g.S[0].done, sstride, g.lam, align256(p.lam_count * 8) / 8);
-      const dim3 grid(ac_blocks(g.M, B), B);
+      const dim3 grid(ac_blocks(g.M), B);
       k_ac_pq<<<grid, kAcThreads, 0, gs>>>(g.p, g.q, g.M, g.vs, g.S, g.partials, sc);
       k_ac_update<<<grid, kAcThreads, 0, gs>>>(g.x, g.r, g.p, g.q, g.M, g.vs, g.S, g.partials, maxit);
       k_ac_next<<<grid, kAcThreads, 0, gs>>>(g.u, g.x, g.r, g.p, g.M, g.vs, g.S, g.partials, g.partials2, nsteps, tau,
