@@ -16,48 +16,16 @@
 
 #include "common.cuh"
 #include "fft.cuh"
+#include "gauss_rules.h"
 
 namespace frlap {
 
 namespace {
 
-// Gauss-Legendre rules of the orders below on [0, 1], weights summing to 1, one after another; a kernel
-// argument (read as constants).  Newton's method on the three-term recurrence, on the host once per process:
-// on the device, 83 threads of one warp group in serial FP64 took 1.7 ms of each plan's creation.
-constexpr int kNumQ = 6;
-__host__ __device__ constexpr int rule_q(int r) {
-  return r == 0 ? 4 : r == 1 ? 5 : r == 2 ? 8 : r == 3 ? 14 : r == 4 ? 20 : 32;
-}
-__host__ __device__ constexpr int rule_off(int r) { return r == 0 ? 0 : rule_off(r - 1) + rule_q(r - 1); }
-constexpr int kQTotal = rule_off(kNumQ);
-struct GaussRules {
-  double x[kQTotal], w[kQTotal];
-};
-GaussRules make_gauss_rules() {
-  GaussRules g;
-  for (int r = 0; r < kNumQ; ++r) {
-    const int q = rule_q(r);
-    for (int i = 0; i < q; ++i) {
-      // in extended precision: an error of a rule is one of every element's integral alike
-      long double x = cosl(3.14159265358979323846L * (i + 0.75L) / (q + 0.5L)), dP = 1.0L;
-      for (int it = 0; it < 12; ++it) {  // quadratic: five steps reach the rounding level
-        long double p0 = 1.0L, p1 = x;
-        for (int k = 2; k <= q; ++k) {
-          const long double p2 = ((2.0L * k - 1.0L) * x * p1 - (k - 1.0L) * p0) / k;
-          p0 = p1;
-          p1 = p2;
-        }
-        dP = q * (x * p1 - p0) / (x * x - 1.0L);
-        x -= p1 / dP;
-      }
-      g.x[rule_off(r) + i] = (double)(0.5L * (1.0L - x));
-      g.w[rule_off(r) + i] = (double)(1.0L / ((1.0L - x * x) * dP * dP));  // (2 / ((1 - x^2) P'^2)) / 2
-    }
-  }
-  return g;
-}
+// The quadrature rules, a kernel argument (read as constants); on the host, once per process: on the device, 83
+// threads of one warp group in serial FP64 took 1.7 ms of each plan's creation.
 const GaussRules& gauss_rules() {
-  static const GaussRules g = make_gauss_rules();
+  static const GaussRules g = make_gauss_rules<long double>();
   return g;
 }
 
