@@ -173,7 +173,8 @@ frlap_status frlap_apply_batch(const frlap_plan* plan, int nbatch, const void* d
 /* Autotuner of the apply's launch shapes.  For each stage of the apply, and for each
  * engine the plan uses (FP32, and F64 or DF64), times every admissible
  * number of FFT lines per CTA (powers of two up to 512 threads and 227 KB of shared
- * memory) on a batch of nbatch zero vectors, and keeps the fastest in the plan;
+ * memory) on a batch of nbatch vectors of values in [-1, 1), and keeps the fastest in the plan
+ * (F64 and DF64: as launched; stages of few lines have a fixed number, then kept as it is);
  * later applies, batched applies, solves and Allen-Cahn runs on the plan use it.
  * The stages are timed independently (one launch each), so the search is exact
  * per stage.  d_work: frlap_autotune_workspace_bytes(plan, nbatch) bytes, 256-byte

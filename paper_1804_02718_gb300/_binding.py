@@ -338,7 +338,7 @@ def frlap_apply_host(plan: Plan, U: torch.Tensor, Y: torch.Tensor = None, chunk:
 
 def frlap_plan_autotune(plan: Plan, nbatch: int = 8, stream=None):
     """Time every admissible lines-per-CTA choice of each apply stage (per engine of the plan) on
-    nbatch zero vectors and keep the fastest in the plan.  Returns (FP64-side choices, FP32 choices),
+    nbatch vectors of values in [-1, 1) and keep the fastest in the plan.  Returns (FP64-side choices, FP32 choices),
     5 ints each (0 = stage or engine absent)."""
     nbytes = int(lib().frlap_autotune_workspace_bytes(plan.handle, int(nbatch)))
     raw = torch.empty(nbytes + 256, dtype=torch.uint8, device="cuda")

@@ -617,6 +617,20 @@ static QShape q_shape(int tuned, int L, long long lines, int B, int lines_per_gr
   return q;
 }
 
+// The shape of apply stage st: 2D rows, middle, rows; 3D rows, y lines, middle, y lines, rows.
+static QShape q_stage_shape(const Plan& p, int st, int tuned, int B) {
+  const int Hx1 = p.P[0] / 2 + 1, nrows = p.n[1] * p.n[2];
+  if (st == 0 || st == (p.d == 2 ? 2 : 4)) return q_shape(tuned, p.P[0] / 2, nrows, B, nrows, QKind::Row);
+  if (p.d == 3 && st != 2) return q_shape(tuned, p.P[1], (long long)p.n[2] * Hx1, B, p.n[2]);
+  if (p.d == 2 && p.P[1] > kMaxLine) return q_shape(tuned, kMaxLine, Hx1, B, Hx1, QKind::Split);
+  const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
+  return q_shape(tuned, p.P[p.d - 1], ncols, B, ncols);
+}
+template <typename T>
+int q_stage_tl(const Plan& p, int st, int tuned, int B) {
+  return q_stage_shape(p, st, tuned, B).tl;
+}
+
 // f(tag) for the kernel instance of a line of 2^logL points: tag::rem, tag::logp and tag::e entries a thread.
 template <int R, int L, int E>
 struct QTag : ShapeTag<R, L> {
@@ -657,8 +671,8 @@ static cudaError_t q_register(const Plan& p, BcRanges r, void* work, int B, cuda
 template <bool DYN>
 static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const double* u, size_t ustride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
-  const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
-  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows, QKind::Row);
+  const int nrows = p.n[1] * p.n[2];
+  const QShape q = q_stage_shape(p, 0, tuned, B);
   Batch b;
   b.in = ustride;
   b.out = w.stride;
@@ -672,7 +686,7 @@ static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const doubl
 static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
                                   cudaStream_t s) {
   const int Py = p.P[1], ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1;
-  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1, B, nz);
+  const QShape q = q_stage_shape(p, 1, tuned, B);
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
@@ -686,7 +700,7 @@ static cudaError_t q_stage_yz_fwd(const Plan& p, const QWork& w, int B, int tune
 static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tuned, const int* skip, int skip_stride,
                                   cudaStream_t s) {
   const int Py = p.P[1], ny = p.n[1], nz = p.n[2], Hx1 = p.P[0] / 2 + 1;
-  const QShape q = q_shape(tuned, Py, (long long)nz * Hx1, B, nz);
+  const QShape q = q_stage_shape(p, 1, tuned, B);
   Batch b;
   b.in = b.out = w.stride;
   b.skip = skip_stride;
@@ -699,8 +713,8 @@ static cudaError_t q_stage_yz_inv(const Plan& p, const QWork& w, int B, int tune
 }
 static cudaError_t q_stage_c2r(const Plan& p, const QWork& w, int B, double* y, size_t ystride, int tuned,
                                const int* skip, int skip_stride, cudaStream_t s) {
-  const int H = p.P[0] / 2, nrows = p.n[1] * p.n[2];
-  const QShape q = q_shape(tuned, H, (long long)nrows, B, nrows, QKind::Row);
+  const int nrows = p.n[1] * p.n[2];
+  const QShape q = q_stage_shape(p, p.d == 2 ? 2 : 4, tuned, B);
   Batch b;
   b.in = w.stride;
   b.out = ystride;
@@ -752,7 +766,7 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, s
   if ((e = q_stage_r2c<DYN>(p, w, B, u, vstride, tuned[0], skip, skip_stride, s)) != cudaSuccess) return e;
   if ((e = mark()) != cudaSuccess) return e;
   if (p.d == 2 && p.P[1] > kMaxLine) {
-    const QShape q = q_shape(tuned[1], kMaxLine, (long long)Hx1, B, Hx1, QKind::Split);
+    const QShape q = q_stage_shape(p, 1, tuned[1], B);
     int* ex_tmp = w.col + Hx1;
     e = q_launch(k_q_colmul_split<false>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col, ex_tmp,
                  Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);
@@ -768,7 +782,7 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, s
     // the middle stage: columns over y in S1 (2D), over z in S2 (3D)
     const int ax = p.d == 3 ? 2 : 1;
     const int ncols = p.d == 3 ? Hx1 * p.P[1] : Hx1;
-    const QShape q = q_shape(tuned[p.d == 3 ? 2 : 1], p.P[ax], (long long)ncols, B, ncols);
+    const QShape q = q_stage_shape(p, ax, tuned[ax], B);
     e = q_with_shape(q, p.logP[ax], [&](auto tag) {
       using K = decltype(tag);
       return q_launch(k_q_colmul<K::rem, K::logp, K::e>, q.tiles, B, q.threads, q.sm, s, p.d == 3 ? w.S2 : w.S1,
