@@ -551,14 +551,14 @@ def frlap_bounds_check_report():
 
 
 def frlap_async_wait_report() -> int:
-    """Bounded asynchronous-copy waits of the apply kernels that gave up since the last report."""
+    """Bounded waits of frlap_dft16_stages' tensor-core kernel that gave up since the last report."""
     n = ctypes.c_ulonglong(0)
     _check(lib().frlap_async_wait_report(ctypes.byref(n)), "frlap_async_wait_report")
     return int(n.value)
 
 
 def frlap_async_wait_selftest() -> int:
-    """Runs one bounded wait that nothing completes; returns the waits that gave up (1 expected)."""
+    """Runs that wait where nothing completes it; returns the waits that gave up (1 expected)."""
     n = ctypes.c_ulonglong(0)
     _check(lib().frlap_async_wait_selftest(ctypes.byref(n)), "frlap_async_wait_selftest")
     return int(n.value)

@@ -95,10 +95,7 @@ const char* frlap_last_error(void) { return g_last_error.c_str(); }
 
 frlap_status frlap_async_wait_report(unsigned long long* timeouts) {
   if (!timeouts) return fail(FRLAP_EINVAL, "timeouts is NULL");
-  unsigned long long c = 0ull, cd = 0ull;
-  FRLAP_CUDA_TRY(wait_collect(&c));
-  FRLAP_CUDA_TRY(dft16_wait_collect(&cd));
-  *timeouts = c + cd;
+  FRLAP_CUDA_TRY(dft16_wait_collect(timeouts));
   return FRLAP_OK;
 }
 

@@ -231,67 +231,4 @@ cudaError_t bc_selftest(unsigned long long* flagged) {
 #endif
 }
 
-namespace {
-
-// ---- the bounded mbarrier wait
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned arrivals) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(arrivals) : "memory");
-  // the initialised barrier is visible to the asynchronous proxy that completes its transactions
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-
-// Waits until the phase of `bar` with the given parity has completed.  Each try suspends the
-// thread for at most about kWaitHintNs; after kWaitTries tries (about a second) it gives up and
-// returns false.
-constexpr unsigned kWaitHintNs = 1000;
-constexpr int kWaitTries = 1 << 20;
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
-  const unsigned a = smem_addr(bar);
-  for (int i = 0; i < kWaitTries; ++i) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(a), "r"(parity), "r"(kWaitHintNs)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
-// Waits that gave up (wait_collect reads and resets it).
-__device__ unsigned long long g_wait_timeouts = 0ull;
-
-}  // namespace
-
-cudaError_t wait_collect(unsigned long long* count) {
-  cudaError_t e = cudaMemcpyFromSymbol(count, g_wait_timeouts, sizeof(*count));
-  if (e != cudaSuccess) return e;
-  const unsigned long long z = 0ull;
-  return cudaMemcpyToSymbol(g_wait_timeouts, &z, sizeof(z));
-}
-
-// The give-up path of the bounded mbarrier wait: one warp waits on a phase that nothing
-// completes (no arrival, no copy in flight), gives up after the wait's bound, and records it.
-__global__ void k_wait_selftest() {
-  __shared__ unsigned long long bar;
-  if (threadIdx.x == 0) mbar_init(&bar, 1);
-  __syncthreads();
-  const bool ok = mbar_wait(&bar, 0u);
-  if (!__syncthreads_and(ok) && threadIdx.x == 0) atomicAdd(&g_wait_timeouts, 1ull);
-}
-
-cudaError_t wait_selftest(unsigned long long* timeouts) {
-  unsigned long long c = 0;
-  cudaError_t e = wait_collect(&c);  // reset
-  if (e != cudaSuccess) return e;
-  k_wait_selftest<<<1, 32>>>();
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
-  return wait_collect(timeouts);
-}
-
 }  // namespace frlap

@@ -232,9 +232,6 @@ struct Plan {
   int tl_tuned[3][5] = {};
 };
 
-// The bounded mbarrier waits of wait_selftest's kernel that gave up since the last call (the counter is reset).
-cudaError_t wait_collect(unsigned long long* count);
-
 // Bounds-checked builds: accesses outside the registered ranges since the last call, summed per
 // engine's translation unit (the counters are reset); ordinary builds report zero.
 template <typename T>
@@ -242,10 +239,11 @@ cudaError_t bc_collect(unsigned long long* count, unsigned long long* first);
 // Bounds-checked builds: registers one 8-double range and probes 8 loads inside it and 5 just past
 // it (memory the library owns, so the probes are safe even unchecked); *flagged = accesses flagged.
 cudaError_t bc_selftest(unsigned long long* flagged);
-// Runs one bounded mbarrier wait that nothing completes; *timeouts = waits that gave up (1 expected).
+// Runs dft16_tc.cu's bounded mbarrier wait where nothing completes it; *timeouts = waits that gave up (1 expected).
 cudaError_t wait_selftest(unsigned long long* timeouts);
 // radix-16 stages on CUDA cores (engine 0) or tensor cores (engine 1); see dft16_tc.cu
 cudaError_t dft16_stages_launch(int engine, const float* in, float* out, int ntiles, int reps, cudaStream_t s);
+// that kernel's bounded waits that gave up since the last call (the counter is reset)
 cudaError_t dft16_wait_collect(unsigned long long* count);
 
 // apply pipeline (apply_impl.cuh, apply_q.cuh); work must hold apply_work_bytes(plan, sizeof(io_t<T>)) bytes

@@ -89,7 +89,8 @@ __device__ __forceinline__ void ld_row32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Bounded wait on an mbarrier phase (as the apply's waits: about a second, then false).
+// Bounded wait on an mbarrier phase: each try suspends the thread for at most about a microsecond; after 2^20 of them
+// (about a second) it gives up and returns false.
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   for (int i = 0; i < (1 << 20); ++i) {
     uint32_t done;
@@ -266,6 +267,19 @@ __global__ void __launch_bounds__(128) k_dft16_tc(const float* __restrict__ in, 
   }
 }
 
+// The give-up path of that wait: one warp waits on a phase that nothing completes (no arrival, no product in flight),
+// gives up after the bound, and records it.
+__global__ void k_wait_selftest() {
+  __shared__ unsigned long long bar;
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(&bar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncthreads();
+  const bool ok = bar_wait(smem_addr(&bar), 0u);
+  if (!__syncthreads_and(ok) && threadIdx.x == 0) atomicAdd(&g_tc_wait_timeouts, 1ull);
+}
+
 }  // namespace
 
 cudaError_t dft16_stages_launch(int engine, const float* in, float* out, int ntiles, int reps, cudaStream_t s) {
@@ -288,6 +302,16 @@ cudaError_t dft16_wait_collect(unsigned long long* count) {
   e = cudaMemcpyToSymbol(g_tc_wait_timeouts, &z, sizeof(z));
   *count = c;
   return e;
+}
+
+cudaError_t wait_selftest(unsigned long long* timeouts) {
+  unsigned long long c = 0;
+  cudaError_t e = dft16_wait_collect(&c);  // reset
+  if (e != cudaSuccess) return e;
+  k_wait_selftest<<<1, 32>>>();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+  return dft16_wait_collect(timeouts);
 }
 
 }  // namespace frlap
