@@ -364,7 +364,7 @@ struct Group {
 };
 
 bool same_shape(const Plan& a, const Plan& b) {
-  if (a.d != b.d || a.df64 != b.df64) return false;
+  if (a.d != b.d || a.df64 != b.df64 || a.lam_plain != b.lam_plain) return false;
   for (int r = 0; r < a.d; ++r)
     if (a.n[r] != b.n[r] || a.P[r] != b.P[r]) return false;
   return true;

@@ -210,6 +210,8 @@ frlap_status frlap_plan_create(int d, double alpha, double gamma, double h, cons
   p->prec = prec;
   p->df64 = (prec == FRLAP_DF64 || prec == FRLAP_MIXED_DF64);
   p->c = c_dalpha_host(d, alpha);
+  // lambda = h^-alpha times at least 8192^-2 / 100 and at most 100, over prod P_r <= 2^33
+  p->lam_plain = alpha > 1e-100 && fabs(alpha * log2(h)) < 900.0;
   p->Nmax = 0;
   p->M = 1;
   p->lam_count = 1;

@@ -61,6 +61,7 @@ struct LamMap {
   int Hx1;     // P_x/2 + 1
   int Hy1;     // P_y/2 + 1
   int Hz1;     // P_z/2 + 1 (3D)
+  bool plain = true;  // Plan::lam_plain (read by the fixed-point stages)
 };
 
 // Global loads are issued in unrolled batches before their shared-memory stores, so that

@@ -209,12 +209,15 @@ __device__ __forceinline__ double q_ld(const double* p) {
 
 // The symbol product v <- lambda v at a common exponent for the line, components below 2^58.  lambda enters by
 // its mantissa, so every entry has full precision whatever lambda's range along the line; the line's
-// exponent is what its largest |lambda_k| |v_k| needs.  lambda is positive: A is strictly diagonally dominant
-// and so is its circulant embedding (a zero from underflow acts as 2^-1022).
+// exponent is what its largest |lambda_k| |v_k| needs.  lambda is not negative: A is strictly diagonally dominant
+// and so is its circulant embedding (a rounding below zero is cut off in the table).
+// plain: every lambda is finite and normal (Plan::lam_plain).  Otherwise a subnormal or zero lambda has no leading bit,
+// and a non-finite one makes its line NaN, even one of zeros.  A flag of the plan, because to look at each
+// lambda costs a single 2047^2 apply 1%.
 // lrow[idx(m)] is entry m's lambda; its words are read twice (the second time from L1), since held over the
 // reduction they spill.
 template <int E, typename I>
-__device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict__ lrow, I idx, int logL,
+__device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict__ lrow, I idx, bool plain, int logL,
                                          unsigned* slot) {
   int top = 0;
 #pragma unroll
@@ -224,22 +227,32 @@ __device__ __forceinline__ void q_symbol(cq* v, int& e, const double* __restrict
     const int pos = __float_as_int(__uint2float_rn(q_bits(v[m]))) >> 23;
     top = max(top, (int)(h >> 20) + max(pos, 126));
   }
-  top = (int)q_reduce<true>((unsigned)top, logL, slot);
-#pragma unroll
-  for (int m = 0; m < E; ++m) {
-    // lambda v = (mant v / 2^64) 2^(el - 1020), 2^61 <= mant < 2^62, and |v| 2^(el - top + 127) < 2^33: the
-    // shift s = el - top + 152 brings the product below 2^58.  A right shift is one of the mantissa (its
-    // dropped bits weigh less than a unit of the product), a left one is one of v.
-    const double lam = q_ld(lrow + idx(m));
-    const unsigned h = (unsigned)__double2hiint(lam), l = (unsigned)__double2loint(lam);
-    const int s = (int)(h >> 20) - top + 152;
-    unsigned long long mant =
-        ((unsigned long long)__funnelshift_l(l, (h & 0xfffffu) | 0x100000u, 9) << 32) | (l << 9);
-    mant >>= min(max(-s, 0), 63);
-    const int sl = min(max(s, 0), 31);
-    const QHalf w = q_half((long long)mant);
-    v[m] = {q_rmul(q_half(q_shl(v[m].x, sl)), w), q_rmul(q_half(q_shl(v[m].y, sl)), w)};
+  if (!plain) {
+#pragma unroll 1
+    for (int m = 0; m < E; ++m)
+      if (q_ld_hi(lrow + idx(m)) >= 0x7ff00000u) top = 2 * kQNan;
   }
+  top = (int)q_reduce<true>((unsigned)top, logL, slot);
+  auto product = [&](auto normal) {
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      // lambda v = (mant v / 2^64) 2^(el - 1020), 2^61 <= mant < 2^62, and |v| 2^(el - top + 127) < 2^33: the
+      // shift s = el - top + 152 brings the product below 2^58.  A right shift is one of the mantissa (its
+      // dropped bits weigh less than a unit of the product), a left one is one of v.
+      const double lam = q_ld(lrow + idx(m));
+      const unsigned h = (unsigned)__double2hiint(lam), l = (unsigned)__double2loint(lam);
+      const int s = (int)(h >> 20) - top + 152;
+      unsigned long long mant =
+          ((unsigned long long)__funnelshift_l(l, (h & 0xfffffu) | 0x100000u, 9) << 32) | (l << 9);
+      if (!decltype(normal)::value && h < 0x100000u) mant = (mant - (1ull << 61)) << 1;  // el = 0 stands for 1
+      mant >>= min(max(-s, 0), 63);
+      const int sl = min(max(s, 0), 31);
+      const QHalf w = q_half((long long)mant);
+      v[m] = {q_rmul(q_half(q_shl(v[m].x, sl)), w), q_rmul(q_half(q_shl(v[m].y, sl)), w)};
+    }
+  };
+  if (plain) product(std::true_type{});
+  else product(std::false_type{});
   e += top - 1172;
 }
 
@@ -277,7 +290,8 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   const int ky = c & (map.Py - 1);
   const double* lrow = map.d == 2 ? lam + (size_t)c * map.Hy1
                                   : lam + ((size_t)kx * map.Hy1 + min(ky, map.Py - ky)) * map.Hz1;
-  q_symbol<E>(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, lg, slots + si);
+  q_symbol<E>(v, e, lrow, [&](int m) { return min(lane + m * G, P - lane - m * G); }, map.plain, lg,
+              slots + si);
   ++si;
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
   q_store_scale<REM, E, LOGP, E / 2>(v, e);
@@ -291,7 +305,7 @@ template <bool ODD>
 __global__ void __launch_bounds__(512, 1)
     k_q_colmul_split(cq* __restrict__ data, cq* __restrict__ tmp, const int* __restrict__ ex_in,
                      int* __restrict__ ex_out, int* __restrict__ ex_tmp, int ncols, int n, size_t ld, int TL,
-                     const double* __restrict__ lam, int Hy1, const int4* __restrict__ tw,
+                     const double* __restrict__ lam, int Hy1, bool plain, const int4* __restrict__ tw,
                      const int* __restrict__ skip, Batch bt, size_t ex_inst) {
   constexpr int logL = 13, L = 1 << logL, P = 2 * L, G = L >> 4, REM = logL & 3;
   {
@@ -330,7 +344,7 @@ __global__ void __launch_bounds__(512, 1)
         const int k = 2 * (lane + m * G) + (ODD ? 1 : 0);
         return min(k, P - k);
       },
-      logL, slots + si);
+      plain, logL, slots + si);
   ++si;
   q_fft<true, 1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, true, slots, si);
   if (!valid) return;
@@ -656,6 +670,7 @@ static LamMap q_lam_map(const Plan& p) {
   map.Py = p.P[1];
   map.Hy1 = p.P[1] / 2 + 1;
   map.Hz1 = p.d == 3 ? p.P[2] / 2 + 1 : 1;
+  map.plain = p.lam_plain;
   return map;
 }
 
@@ -769,10 +784,10 @@ cudaError_t q_apply_launch_b(const Plan& p, int B, const double* u, double* y, s
     const QShape q = q_stage_shape(p, 1, tuned[1], B);
     int* ex_tmp = w.col + Hx1;
     e = q_launch(k_q_colmul_split<false>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col, ex_tmp,
-                 Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);
+                 Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, map.plain, (const int4*)p.twq[1], skip, b, w.ex_stride);
     if (e == cudaSuccess)
       e = q_launch(k_q_colmul_split<true>, q.tiles, B, q.threads, q.sm, s, w.S1, w.S2, (const int*)w.row, w.col,
-                   ex_tmp, Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, (const int4*)p.twq[1], skip, b, w.ex_stride);
+                   ex_tmp, Hx1, ny, (size_t)nrows, q.tl, lam, map.Hy1, map.plain, (const int4*)p.twq[1], skip, b, w.ex_stride);
     if (e != cudaSuccess) return e;
   } else {
     if (p.d == 3) {

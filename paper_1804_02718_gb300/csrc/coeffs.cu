@@ -573,6 +573,7 @@ cudaError_t scale_symbol_launch(double* lam64, float* lam32, size_t n, double s,
 namespace {
 template <typename To>
 __device__ __forceinline__ To from_double(double v) {
+  if constexpr (std::is_same<To, double>::value) return v < 0.0 ? 0.0 : v;  // (a rounding below zero; NaN stays)
   return (To)v;
 }
 

@@ -211,6 +211,7 @@ struct Plan {
   // one column is contiguous.
   double* lam64 = nullptr;     // natural order, FP64 (always built)
   double* lamL64 = nullptr;    // line-major, FP64 (always built)
+  bool lam_plain = true;       // no entry of lamL64 can be subnormal, zero or non-finite
   float* lam32 = nullptr;      // line-major, FP32 (all plans but F64)
   // exp(-2 pi i m / P_r), m < P_r, followed by the radix-16 stage table of
   // twiddle_entries(P_r): see there
