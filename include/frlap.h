@@ -61,9 +61,10 @@ typedef enum {
  * precision FFT stages and symbol.  MIXED: a plan that holds both, so
  * that the iterative-refinement solver can run FP32 inner applies and FP64
  * outer residuals (coefficients and symbol are always generated in FP64).
- * DF64: FP64 vectors and symbol as F64; the first stage sets a row's scale once
- * instead of following its values: slightly faster, normwise within 2.1e-15 of F64
- * (rows of one spike above noise; N(0,1) and smooth vectors 2.3e-16).  A non-finite
+ * DF64: FP64 vectors and symbol as F64; on x axes of at most 512 intervals the first stage
+ * sets a row's scale once instead of following its values, normwise within 2e-15
+ * lambda_max ||u|| of F64 (rows of one spike above noise; N(0,1) and smooth vectors 2e-16);
+ * on longer ones DF64 and F64 give the same bits.  A non-finite
  * right-hand side of frlap_pcg_solve returns FRLAP_ENAN; the system is solved
  * scaled by the power of two at or below 1/max|f_i| (exactly, undone on the
  * solution), so that FP32 preconditioners see values they can hold.

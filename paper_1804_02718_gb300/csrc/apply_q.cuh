@@ -1,6 +1,6 @@
 // The apply's stages in the FP64 and the DF64 engine: the pipeline of apply_impl.cuh on 64-bit block fixed point
-// (fft_q.cuh).  Vectors and symbol are FP64.  The DF64 engine's first stage sets a row's scale once (DYN =
-// false); the other stages are common.  In the workspace a complex value is two 64-bit integers
+// (fft_q.cuh).  Vectors and symbol are FP64.  The DF64 engine's first stage sets the scale of a row of at most 512 points
+// once (DYN = false); all else is common.  In the workspace a complex value is two 64-bit integers
 // below 2^58, in the same S1 / S2 layout and 16 bytes as an FP64 pair, and each line that a kernel wrote
 // has its exponent in an array behind S1 and S2:
 //   ex_row[row]           after the first stage, for S1[.][row]
@@ -694,7 +694,7 @@ static cudaError_t q_stage_r2c(const Plan& p, const QWork& w, int B, const doubl
   b.skip = skip_stride;
   return q_with_shape(q, p.logP[0] - 1, [&](auto tag) {
     using K = decltype(tag);
-    return q_launch(k_q_r2c<DYN, K::rem, K::logp, K::e>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row,
+    return q_launch(k_q_r2c<DYN || ((1 << K::logp) > kQStaticMax), K::rem, K::logp, K::e>, q.tiles, B, q.threads, q.sm, s, u, w.S1, w.row,
                     nrows, p.n[0], (size_t)nrows, p.logP[0] - 1, q.tl, (const int4*)p.twq[0], skip, b, w.ex_stride);
   });
 }

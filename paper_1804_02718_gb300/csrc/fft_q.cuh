@@ -14,11 +14,12 @@
 // FP64's 2^-53.  The scale follows the data and not a growth bound, so lines whose spectra are concentrated
 // (smooth fields) lose nothing.
 //
-// The DF64 engine sets the scale of the first stage's rows once, on entry, which saves the reductions and shifts
-// between its stages (a sixth of their integer operations): 1.6e-16 for N(0,1) data.  A smooth row loses
-// nothing, since its largest value grows by the bound; rows of one spike lose most (4096-point
-// axis, normwise against the FP64 engine: 5.8e-16, over noise at 1e-3 2.0e-15; the double-float arithmetic that
-// this replaced 5e-15 throughout).  (Columns and inverse transforms need the data's scale: the
+// The DF64 engine sets the scale of the first stage's rows of at most kQStaticMax points once, on entry.  The unit
+// after the last butterfly is then 2^-60 L times the row's largest value: N(0,1) and smooth rows lose
+// nothing to speak of, since their largest value grows with the transform, rows of one spike over noise most.
+// Normwise difference from the F64 engine over lambda_max ||u||, at worst over spikes, noise and alpha: 1.3e-15 at L =
+// 512; it was 1.9e-15 at 1024 and 3.9e-15 at 2048 and 4096 (double-float arithmetic: 5e-15), where the scale now
+// follows the data and both engines agree bit for bit.  (Columns and inverse transforms need the data's scale: the
 // columns of a smooth field at high frequencies, and spectra, lost up to 28 bits without it.)
 //
 // Between kernels a line's values are stored as integers below 2^58 with the line's exponent beside them
@@ -355,6 +356,8 @@ constexpr int kQDrop = E == 4 ? ((REM & 1) ? 3 : 2) : E == 8 ? (LOGL % 3 == 0 ? 
 // v[m] = x[lane + m L/E] on entry and X[lane + m L/E] on exit, scaled as in q_fft (magnitudes below
 // 2^(62.5 - kQDrop<REM, E, LOGL>)).  With DYN = false the line is shifted by what its stage leaves free instead.
 constexpr int kQThinLog = 10;
+// Longest line whose scale may be set once (DYN = false): see above.
+constexpr int kQStaticMax = 512;
 template <int E>
 constexpr int kQCta = E == 8 ? 1024 : 512;  // threads per CTA the kernels are compiled for
 template <int E>
@@ -457,7 +460,7 @@ __device__ __forceinline__ void q_fft_e(cq* v, int& e, cq* buf, int logL, int la
 
 // As fft_regs: v[m] = x[lane + m G] on entry (components below 2^58), X[lane + m G] on exit (magnitudes
 // below 2^(62.5 - kQDrop)); e, the line's exponent, follows.  DYN: the scale follows the data between stages;
-// else it stays as set on entry (lines with three twiddled stages excepted).  ZIN: v[8..15] are zero.  slots:
+// else it stays as set on entry (lines of at most kQStaticMax points).  ZIN: v[8..15] are zero.  slots:
 // the line's reduction words, used from index si on.  E < 16: see q_fft_e.
 template <bool DYN, int SIGN, bool ZIN, int REM, int E = 16>
 __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane, const int4* __restrict__ tw,
@@ -467,7 +470,6 @@ __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane
     return;
   } else {
   const int G = 1 << (logL - 4);
-  const bool dyn = DYN || (REM == 1 && logL > 12);
   if constexpr (ZIN) {
 #pragma unroll
     for (int m = 8; m < 16; ++m) v[m] = {0, 0};
@@ -475,7 +477,7 @@ __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane
   // between stages: write, agree on the scale, read, shift
   auto exchange = [&](int logNs, bool first8, bool pre_sync) {
     unsigned o = 0u;
-    if (dyn) {
+    if (DYN) {
 #pragma unroll
       for (int m = 0; m < 16; ++m) o |= q_bits(v[m]);
       o = q_publish<false>(o, logL, slots + si);
@@ -502,7 +504,7 @@ __device__ __forceinline__ void q_fft(cq* v, int& e, cq* buf, int logL, int lane
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = buf[g16 ? rbase + m * rstep : spad(lane + m * G)];
     e += 4;
-    if (dyn) {
+    if (DYN) {
       const int sh = q_fill_shift(q_fetch(o, logL, slots + si));
       ++si;
 #pragma unroll
