@@ -452,15 +452,15 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
   // the graph runs on its own stream, ordered after the caller's work
   cudaStream_t s;
   FRLAP_CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-  cudaEvent_t ev0, ev1;
-  cudaEventCreateWithFlags(&ev0, cudaEventDisableTiming);
-  cudaEventCreateWithFlags(&ev1, cudaEventDisableTiming);
+  cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  cudaError_t made = cudaEventCreateWithFlags(&ev0, cudaEventDisableTiming);
+  if (made == cudaSuccess) made = cudaEventCreateWithFlags(&ev1, cudaEventDisableTiming);
   const int ns = (int)(groups.size() < (size_t)kAcStreams ? groups.size() : (size_t)kAcStreams) - 1;  // side streams
   cudaStream_t side[kAcStreams] = {};
   cudaEvent_t ev_side[kAcStreams] = {};
-  for (int k = 0; k < ns; ++k) {
-    cudaStreamCreateWithFlags(&side[k], cudaStreamNonBlocking);
-    cudaEventCreateWithFlags(&ev_side[k], cudaEventDisableTiming);
+  for (int k = 0; k < ns && made == cudaSuccess; ++k) {
+    made = cudaStreamCreateWithFlags(&side[k], cudaStreamNonBlocking);
+    if (made == cudaSuccess) made = cudaEventCreateWithFlags(&ev_side[k], cudaEventDisableTiming);
   }
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -468,16 +468,20 @@ frlap_status ac_batch_impl(int nb, const frlap_plan* const* plans, double* const
   auto cleanup = [&]() {
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
+    if (ev0) cudaEventDestroy(ev0);
+    if (ev1) cudaEventDestroy(ev1);
     for (int k = 0; k < ns; ++k) {
-      cudaEventDestroy(ev_side[k]);
-      cudaStreamDestroy(side[k]);
+      if (ev_side[k]) cudaEventDestroy(ev_side[k]);
+      if (side[k]) cudaStreamDestroy(side[k]);
     }
     cudaStreamDestroy(s);
   };
   do {
-    cudaError_t e;
+    cudaError_t e = made;
+    if (e != cudaSuccess) {
+      rc = cuda_fail(e, "streams and events");  // (on a stream that is not there, kernels would run outside the graph)
+      break;
+    }
     if ((e = cudaEventRecord(ev0, user)) != cudaSuccess || (e = cudaStreamWaitEvent(s, ev0, 0)) != cudaSuccess) {
       rc = cuda_fail(e, "stream ordering");
       break;
