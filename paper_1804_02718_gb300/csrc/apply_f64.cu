@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   for (int m = 0; m < E; ++m) v[m] = {q_in(x[m].x, qs), q_in(x[m].y, qs)};
   int e = qs.e;
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  q_store_scale<REM, E, LOGP, E / 2>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex + col, e);
   store_line<E>(v, out, ncols, n, ldo, logP, TL);
 }

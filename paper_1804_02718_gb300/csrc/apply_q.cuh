@@ -1,13 +1,13 @@
 // The apply's stages in the FP64 and the DF64 engine: the pipeline of apply_impl.cuh on 64-bit block fixed point
 // (fft_q.cuh).  Vectors and symbol are FP64.  The DF64 engine's first stage sets the scale of a row of at most 512 points
 // once (DYN = false); all else is common.  In the workspace a complex value is two 64-bit integers
-// below 2^58, in the same S1 / S2 layout and 16 bytes as an FP64 pair, and each line that a kernel wrote
+// below 2^62.5, as a transform leaves them, in the same S1 / S2 layout and 16 bytes as an FP64 pair, and each line that a kernel wrote
 // has its exponent in an array behind S1 and S2:
 //   ex_row[row]           after the first stage, for S1[.][row]
 //   ex_line[kx n_z + z]   3D, for the y lines of both directions
 //   ex_col[kx] (2D), ex_col[kx P_y + ky] (3D) after the middle stage
-// A kernel whose lines run across those shifts its entries to the largest of their exponents as it loads
-// them: the bits it drops are below the rounding unit of the line that set that exponent.
+// A kernel whose lines run across those shifts its entries to a common exponent as it loads them: the bits it drops
+// are below the rounding unit of its own line.
 //
 // Native FP64 stages were bound by the FP64 pipe (84% busy) at a ninth of these stages' rate; conversions
 // from and to FP64 (64 cycles a warp) remain only at the vectors.
@@ -37,25 +37,21 @@ inline QExpLayout q_exp_layout(const Plan& p) {
   return l;
 }
 
-// A transform's output v[0..N) to what is stored, components below 2^58, and its exponent.
-template <int REM, int E, int LOGL, int N>
-__device__ __forceinline__ void q_store_scale(cq* v, int& e) {
-  constexpr int SH = 5 - kQDrop<REM, E, LOGL>;
-#pragma unroll
-  for (int m = 0; m < N; ++m) v[m] = q_shr_even<SH>(v[m]);
-  e += SH;
-}
-
 __device__ __forceinline__ unsigned q_ord(int e) { return (unsigned)e ^ 0x80000000u; }
 __device__ __forceinline__ int q_unord(unsigned u) { return (int)(u ^ 0x80000000u); }
-// v 2^(e - top), e <= top, rounded down or, with up, up.  Callers alternate up with the parity of a frequency
-// index along which a line's exponent (and so the offset of a rounding) is the same: the offset then sits at
-// the middle of the axis' embedding, outside the box, instead of adding up at its first point.
-__device__ __forceinline__ cq q_align(cq v, int e, int top, bool up) {
+// v 2^(e - top), e <= top, to nearest, ties up or, with down, down.  Ties are frequent where few bits go.  Callers
+// alternate down with the parity of a frequency index along which a line's exponent (and so the offset of a rounding) is
+// the same: the offset then sits at the middle of the axis' embedding, outside the box, instead of adding up at its first
+// point.
+__device__ __forceinline__ cq q_align(cq v, int e, int top, bool down) {
   const int d = min(top - e, 63);
-  const unsigned c = up ? (1u << min(d, 31)) - 1u : 0u;
+  const unsigned c = ((1u << min(d, 31)) - (down ? 1u : 0u)) >> 1;
   return {(v.x + c) >> d, (v.y + c) >> d};
 }
+
+// The shift that brings a line with magnitude bits o of its components' high words to components below 2^58, what a
+// transform starts from.
+__device__ __forceinline__ int q_excess(unsigned o) { return max(6 - __clz((int)o), 0); }
 
 #define FRLAP_Q_PROLOGUE(logLine)                                        \
   extern __shared__ __align__(16) unsigned char smem_raw[];              \
@@ -128,32 +124,40 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   for (int j = 0; j < E / 2; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
   line_sync<double>(lg);
   // Real-data split in place, one product per pair (see r2c_tile): X[k] = s + W^k d,
-  // X[H-k] = conj(s - W^k d), s = (a + b) / 2, d = -i (a - b) / 2; stored below 2^57.5, that is over 2^(6 - D),
-  // D = kQDrop (0 after q_fill).  With D = 0, a + b can take 64 bits, so both are shifted first: the offsets of
-  // the downward shifts cancel in a - b, and + 4 makes up for them (mean -0.75, and -3.5 in the last shift) in
-  // a + b.
-  constexpr int D = DYN ? kQDrop<REM, E, LOGL> : 0;
+  // X[H-k] = conj(s - W^k d), s = (a + b) / 2, d = -i (a - b) / 2, over 2^F, below 2^61.5 (D = kQDrop, 0 after q_fill:
+  // a and b are below 2^(62.5 - D)).  A product's unit is 16: where a and b leave the room, a - b goes in 16 times
+  // larger, so that the high frequencies of a smooth row, which the symbol weighs most, carry units of 2^-61.5 of the
+  // row's largest value and not of 2^-58 (stored at 58 bits, F64 applies of smooth fields had 2.4e-16 lambda_max ||u|| on
+  // 4096-interval rows, native FP64 8.8e-17; now 3.8e-17).  With D = 0, a + b can take 64 bits, so both are shifted first.
+  constexpr int D = DYN ? kQDrop<REM, E, LOGL> : 0, F = D < 2 ? 2 - D : 0;
   auto split = [&](int k, const int4 wk) {
     const int km = H - k;
     const cq a = buf[spad(k)];
     const cq b = conjg(buf[spad(km & (H - 1))]);
+    const bool room = (q_bits(a) | q_bits(b)) < (1u << (25 + F));
+    constexpr int kRoom = 3 - F, kElse = D - 1;  // shifts of a - b
     cq d, s;
     if constexpr (D == 0) {
-      d = {(a.x >> 1) - (b.x >> 1), (a.y >> 1) - (b.y >> 1)};
-      s = {((a.x >> 2) + (b.x >> 2) + 4) >> 3, ((a.y >> 2) + (b.y >> 2) + 4) >> 3};
+      const int r = room ? 0 : 1;
+      d = {(a.x >> r) - (b.x >> r), (a.y >> r) - (b.y >> r)};
+      if (room) d = {d.x << kRoom, d.y << kRoom};
+      s = {((a.x >> 2) + (b.x >> 2) + 1) >> 1, ((a.y >> 2) + (b.y >> 2) + 1) >> 1};
     } else {
+      const int r = room ? kRoom : kElse;
       d = a - b;
-      d = {d.x << (D - 1), d.y << (D - 1)};
-      s = q_shr_even<5 - D>(a + b);
+      d = {d.x << r, d.y << r};
+      s = q_shr_even<1 + F>(a + b);
     }
-    const cq t = q_cmul<false>(mul_i<-1>(d), wk);
-    buf[spad(k)] = q_shr_even<2>(s + t);
-    if (k != km) buf[spad(km)] = conjg(q_shr_even<2>(s - t));
+    cq t = q_cmul<false>(mul_i<-1>(d), wk);
+    const int up = room ? 0 : kRoom - kElse;
+    t = {t.x << up, t.y << up};
+    buf[spad(k)] = s + t;
+    if (k != km) buf[spad(km)] = conjg(s - t);
   };
 #pragma unroll
   for (int j = 0; j < E / 2; ++j) split(lane + j * G, wk[j]);
   if (lane == 0) split(H / 2, FRLAP_GLD(tw + H / 2));
-  if (valid && lane == 0) FRLAP_GST(ex + line, e + 6 - D);
+  if (valid && lane == 0) FRLAP_GST(ex + line, e + F);
   __syncthreads();
   const int logTL = __ffs(TL) - 1;
   const int lt = threadIdx.x & (TL - 1);
@@ -167,10 +171,11 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   }
 }
 
-// Entries v[m], m < M, of a line that runs across lines of other exponents: v = line[lane + m G] aligned to
-// the largest, which it returns (up: see q_align).
+// Entries v[m], m < M, of a line that runs across lines of other exponents, aligned to an exponent at which all fit 58
+// bits, which it returns (down: see q_align).  Entries are stored with up to 63 bits: what a line drops here is below the
+// unit of its own largest value, where dropped before it was stored it would be one of the crossing line's.
 template <int M>
-__device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* ex, bool up, int lane, int G, int n,
+__device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* ex, bool down, int lane, int G, int n,
                                               bool valid, int logL, unsigned* slot) {
   int e[M];
   int top = kQZero;
@@ -182,10 +187,10 @@ __device__ __forceinline__ int q_load_aligned(cq* v, const cq* line, const int* 
     e[m] = ok ? FRLAP_GLD(ex + i) : kQZero;
   }
 #pragma unroll
-  for (int m = 0; m < M; ++m) top = max(top, e[m]);
+  for (int m = 0; m < M; ++m) top = max(top, e[m] + q_excess(q_bits(v[m])));
   top = q_unord(q_reduce<true>(q_ord(top), logL, slot));
 #pragma unroll
-  for (int m = 0; m < M; ++m) v[m] = q_align(v[m], e[m], top, up);
+  for (int m = 0; m < M; ++m) v[m] = q_align(v[m], e[m], top, down);
   return top;
 }
 
@@ -294,7 +299,6 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
               slots + si);
   ++si;
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  q_store_scale<REM, E, LOGP, E / 2>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex_out + col, e);
   store_line<E>(v, data, ncols, n, ld, logP, TL);
 }
@@ -349,26 +353,23 @@ __global__ void __launch_bounds__(512, 1)
   q_fft<true, 1, false, REM>(v, e, buf, logL, lane, tw, logL + 1, true, slots, si);
   if (!valid) return;
   if constexpr (!ODD) {
-    constexpr int SH = 5 - kQDrop<REM>;
-    if (lane == 0) FRLAP_GST(ex_tmp + col, e + SH);
+    if (lane == 0) FRLAP_GST(ex_tmp + col, e);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int j = lane + m * G;
-      if (j < n) FRLAP_GST(tline + j, q_shr_even<SH>(v[m]));
+      if (j < n) FRLAP_GST(tline + j, v[m]);
     }
   } else {
-    // y_j = even_j + W_P^-j odd_j, magnitudes below 2^58 each at exponents et and eo: the odd half, below
-    // 2^59.5, up by 2 before its product (which divides by 16)
+    // y_j = even_j + W_P^-j odd_j: the product divides by 16, and the even half is aligned to that
     const int et = FRLAP_GLD(ex_tmp + col);
-    const int eo = e + 2;
-    const int top = max(et, eo);
-    if (lane == 0) FRLAP_GST(ex_out + col, top + 1);
+    const int eo = e + 4, top = max(et + 4, eo);
+    if (lane == 0) FRLAP_GST(ex_out + col, top);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int j = lane + m * G;
       if (j < n) {
-        const cq o = q_cmul<true>(cq{v[m].x << 2, v[m].y << 2}, FRLAP_GLD(tw + j));
-        FRLAP_GST(line + j, q_shr_even<1>(q_align(o, eo, top, col & 1) + q_align(FRLAP_GLD(tline + j), et, top, col & 1)));
+        const cq o = q_cmul<true>(v[m], FRLAP_GLD(tw + j));
+        FRLAP_GST(line + j, q_align(o, eo, top, col & 1) + q_align(FRLAP_GLD(tline + j), et, top, col & 1));
       }
     }
   }
@@ -407,7 +408,6 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
                             lg, slots + si);
   ++si;
   q_fft<true, -1, true, REM, E>(v, e, buf, logP, lane, tw, logP, false, slots, si);
-  q_store_scale<REM, E, LOGL, E>(v, e);
   if (valid && lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
   line_sync<double>(lg);
 #pragma unroll
@@ -464,8 +464,15 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   cq v[E];
 #pragma unroll
   for (int m = 0; m < E; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
+  o = 0u;
+#pragma unroll
+  for (int m = 0; m < E; ++m) o |= q_bits(v[m]);
+  const int drop = q_excess(q_reduce<false>(o, lg, slots + si));
+  ++si;
+#pragma unroll
+  for (int m = 0; m < E; ++m) v[m] = q_align(v[m], 0, drop, (lane + m * G) & 1);
+  e += drop;
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
-  q_store_scale<REM, E, LOGL, E / 2>(v, e);
   if (line < nlines) {
     if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
     cq* dst = out + g * gout + (size_t)line * ldo;
@@ -520,8 +527,12 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   __syncthreads();
   e = q_unord(q_fetch(o, lg, slots));
   int si = 1;
-  // repack in place (see k_c2r_T), over 4: Z[k] = A + i T, Z[H-k] = conj(A - i T), A = X[k] + conj X[H-k],
-  // T = W^-k (X[k] - conj X[H-k])
+  // Repack in place (see k_c2r_T): Z[k] = A + i T, Z[H-k] = conj(A - i T), A = X[k] + conj X[H-k],
+  // T = W^-k (X[k] - conj X[H-k]), with two bits' room for the sums.  A product's unit is 16: where the pair leaves
+  // the room, its difference goes in 16 times larger, so that small bins keep a unit of 2^-60 of the row's largest.
+  // Then the line is shifted to what the transform takes, by its own largest value.
+  e += 2;
+  o = 0u;
 #pragma unroll
   for (int j = 0; j < E / 2 + 1; ++j) {
     const int k = lane + j * G;
@@ -529,18 +540,28 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
       const int km = H - k;
       const cq xk = q_align(buf[spad(k)], ea[j], e, k & 1);
       const cq b = conjg(q_align(buf[spad(km)], eb[j], e, k & 1));
-      const cq A = q_shr_even<2>(xk + b), d = xk - b;
+      const int r = (q_bits(xk) | q_bits(b)) < (1u << 24) ? 4 : 0;
+      const cq A = xk + b, d = xk - b;
       const int4 w = j < E / 2 ? wk[j & (E / 2 - 1)] : FRLAP_GLD(tw + k);
-      const cq iT = mul_i<1>(q_cmul<true>(cq{d.x << 2, d.y << 2}, w));
-      buf[spad(k)] = A + iT;
-      if (k != km && km != H) buf[spad(km)] = conjg(A - iT);
+      const cq t = q_cmul<true>(cq{d.x << r, d.y << r}, w);
+      const cq iT = mul_i<1>(cq{t.x << (4 - r), t.y << (4 - r)});
+      const cq z0 = A + iT, z1 = conjg(A - iT);
+      buf[spad(k)] = z0;
+      o |= q_bits(z0);
+      if (k != km && km != H) {
+        buf[spad(km)] = z1;
+        o |= q_bits(z1);
+      }
     }
   }
-  e += 2;
+  o = q_publish<false>(o, lg, slots + si);
   line_sync<double>(lg);
+  const int drop = q_excess(q_fetch(o, lg, slots + si));
+  ++si;
   cq v[E];
 #pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = buf[spad(lane + m * G)];
+  for (int m = 0; m < E; ++m) v[m] = q_align(buf[spad(lane + m * G)], 0, drop, (lane + m * G) & 1);
+  e += drop;
   q_fft<true, 1, false, REM, E>(v, e, buf, logH, lane, tw, logH + 1, true, slots, si);
   if (!valid) return;
   double* dst = out + (size_t)line * n;

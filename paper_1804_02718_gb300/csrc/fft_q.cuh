@@ -22,7 +22,7 @@
 // follows the data and both engines agree bit for bit.  (Columns and inverse transforms need the data's scale: the
 // columns of a smooth field at high frequencies, and spectra, lost up to 28 bits without it.)
 //
-// Between kernels a line's values are stored as integers below 2^58 with the line's exponent beside them
+// Between kernels a line's values are stored as integers with the line's exponent beside them
 // (apply_q.cuh); a kernel whose lines run across those aligns their exponents as it loads.
 #pragma once
 
