@@ -67,23 +67,6 @@ struct LamMap {
 // Global loads are issued in unrolled batches before their shared-memory stores, so that
 // each thread keeps many loads in flight (the kernels are latency-bound otherwise).
 
-// One line of P = 16 G elements, zero beyond n (or all zero if !valid): lane loads lane + j G.
-template <typename C>
-__device__ __forceinline__ void load_line(C* buf, const C* __restrict__ src, int lane, int G, int n, bool valid) {
-  constexpr int U = sizeof(C) <= 8 ? 16 : 8;
-#pragma unroll 1
-  for (int j0 = 0; j0 < 16; j0 += U) {
-    C t[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int i = lane + (j0 + u) * G;
-      t[u] = (valid && i < n) ? FRLAP_GLD(src + i) : czero<C>();
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) buf[spad(lane + (j0 + u) * G)] = t[u];
-  }
-}
-
 // Asynchronous copy of one 8- or 16-byte element from global to shared memory (cp.async;
 // with pred false it writes zeros and reads nothing).  The copies of a thread complete at
 // cp_async_wait_all(); a CTA barrier after it makes them visible to the other threads.
