@@ -126,8 +126,8 @@ __device__ __forceinline__ V ld_stream(const V* p) {
 
 
 // Engines of the apply: float (FP32), double (FP64 vectors and symbol, transforms in 64-bit fixed point whose
-// scale follows the data between stages) and this tag for the DF64 plans' one (the same with the scale set
-// once per transform).  io_t: the type of the engine's grid vectors and symbol.
+// scale follows the data between stages) and this tag for the DF64 plans' one (the same, with the scale of first-stage
+// rows of at most 512 points set once).  io_t: the type of the engine's grid vectors and symbol.
 struct df64 {};
 template <typename T> struct io_t_ { using type = T; };
 template <> struct io_t_<df64> { using type = double; };
