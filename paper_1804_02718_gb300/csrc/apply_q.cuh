@@ -450,28 +450,22 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   unsigned* slots = q_slot_words + (l & (kQLines - 1)) * kQSlots;
   cq* buf = smem + (size_t)l * LS;
   int ek[E];
-  int e = kQZero;
+#pragma unroll
+  for (int m = 0; m < E; ++m) ek[m] = FRLAP_GLD(ex_in + (size_t)g * P + lane + m * G);
+  load_transposed<cq>(smem, in + g * gin, TL * P, TL, LS, ldi, line0, nlines);
+  __syncthreads();
+  int si = 0;
+  cq v[E];
+  int e = kQZero;  // (by the entries, as in q_load_aligned: a column's exponent is that of its largest line)
 #pragma unroll
   for (int m = 0; m < E; ++m) {
-    ek[m] = FRLAP_GLD(ex_in + (size_t)g * P + lane + m * G);
-    e = max(e, ek[m]);
+    v[m] = buf[spad(lane + m * G)];
+    e = max(e, ek[m] + q_excess(q_bits(v[m])));
   }
-  load_transposed<cq>(smem, in + g * gin, TL * P, TL, LS, ldi, line0, nlines);
-  unsigned o = q_publish<true>(q_ord(e), lg, slots);
-  __syncthreads();
-  e = q_unord(q_fetch(o, lg, slots));
-  int si = 1;
-  cq v[E];
-#pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = q_align(buf[spad(lane + m * G)], ek[m], e, (lane + m * G) & 1);
-  o = 0u;
-#pragma unroll
-  for (int m = 0; m < E; ++m) o |= q_bits(v[m]);
-  const int drop = q_excess(q_reduce<false>(o, lg, slots + si));
+  e = q_unord(q_reduce<true>(q_ord(e), lg, slots + si));
   ++si;
 #pragma unroll
-  for (int m = 0; m < E; ++m) v[m] = q_align(v[m], 0, drop, (lane + m * G) & 1);
-  e += drop;
+  for (int m = 0; m < E; ++m) v[m] = q_align(v[m], ek[m], e, (lane + m * G) & 1);
   q_fft<true, 1, false, REM, E>(v, e, buf, logP, lane, tw, logP, true, slots, si);
   if (line < nlines) {
     if (lane == 0) FRLAP_GST(ex_out + (size_t)g * nlines + line, e);
@@ -508,7 +502,6 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
   cq* buf = smem + (size_t)l * LS;
   // this thread's pairs (k, H - k): k = lane + j G <= H/2 (j = E/2: lane 0 alone)
   int ea[E / 2 + 1], eb[E / 2 + 1];
-  int e = kQZero;
   const int* exl = ex + (valid ? line / rows_per : 0);
 #pragma unroll
   for (int j = 0; j < E / 2 + 1; ++j) {
@@ -516,23 +509,33 @@ __global__ void __launch_bounds__(kQCta<E>, 1)
     if (k <= H / 2) {
       ea[j] = FRLAP_GLD(exl + (size_t)k * ex_k);
       eb[j] = FRLAP_GLD(exl + (size_t)(H - k) * ex_k);
-      e = max(e, max(ea[j], eb[j]));
     }
   }
   load_transposed<cq>(smem, in, TL * (H + 1), TL, LS, ldi, line0, nlines);
-  unsigned o = q_publish<true>(q_ord(e), lg, slots);
   int4 wk[E / 2];  // W^k of this thread's pairs, in flight over the barrier
 #pragma unroll
   for (int j = 0; j < E / 2; ++j) wk[j] = FRLAP_GLD(tw + lane + j * G);
   __syncthreads();
-  e = q_unord(q_fetch(o, lg, slots));
-  int si = 1;
+  int si = 0;
+  // The row's exponent, at which its bins fit 60 bits, by the bins themselves: a column's exponent is that of its largest
+  // row, and a row that crosses one with a high wall in another row lost what that one is above it (a wall of height 1
+  // over noise of 1e-3, 2047 x 511: 1.6e-15 lambda_max ||u||, now 4.6e-16).
+  int e = kQZero;
+#pragma unroll
+  for (int j = 0; j < E / 2 + 1; ++j) {
+    const int k = lane + j * G;
+    if (k <= H / 2) {
+      e = max(e, ea[j] + max(4 - __clz((int)q_bits(buf[spad(k)])), 0));
+      e = max(e, eb[j] + max(4 - __clz((int)q_bits(buf[spad(H - k)])), 0));
+    }
+  }
+  e = q_unord(q_reduce<true>(q_ord(e), lg, slots + si));
+  ++si;
   // Repack in place (see k_c2r_T): Z[k] = A + i T, Z[H-k] = conj(A - i T), A = X[k] + conj X[H-k],
-  // T = W^-k (X[k] - conj X[H-k]), with two bits' room for the sums.  A product's unit is 16: where the pair leaves
+  // T = W^-k (X[k] - conj X[H-k]), magnitudes below 2^62.5.  A product's unit is 16: where the pair leaves
   // the room, its difference goes in 16 times larger, so that small bins keep a unit of 2^-60 of the row's largest.
   // Then the line is shifted to what the transform takes, by its own largest value.
-  e += 2;
-  o = 0u;
+  unsigned o = 0u;
 #pragma unroll
   for (int j = 0; j < E / 2 + 1; ++j) {
     const int k = lane + j * G;
