@@ -55,8 +55,9 @@ typedef enum {
 
 /* Arithmetic of the FFT apply.  F64: IEEE double vectors and symbol; the transforms
  * run in 64-bit fixed point with one exponent per line (58 to 62 bits below a line's
- * largest value; normwise errors of an apply, over lambda_max ||u||, 1e-17 to 1e-16), which GB300's integer pipes do several
- * times faster than its FP64 pipe.  Vectors of any finite scale; a non-finite
+ * largest value), which GB300's integer pipes do several times faster than its FP64 pipe.
+ * Normwise errors of an apply over lambda_max ||u||: 1e-17 to 1e-16 for smooth and N(0,1)
+ * vectors, up to 5e-16 where one grid line or point dominates.  Vectors of any finite scale; a non-finite
  * entry makes the whole product NaN.  F32: single
  * precision FFT stages and symbol.  MIXED: a plan that holds both, so
  * that the iterative-refinement solver can run FP32 inner applies and FP64
